@@ -231,13 +231,13 @@ __global__ void __launch_bounds__(kRowThreads) post_kernel(const PostArgs a) {
     }
 }
 
-// ---- after the QKV GEMM: sum the partials, rotate q and k at the row's position, keep q in fp32,
+// ---- after the QKV GEMM: sum the partials, rotate q and k at the row's position, keep q as bf16 pairs,
 // append k and v (rounded to bf16) to the paged cache. Block = (head, sequence), dh/2 threads.
 struct QkvArgs {
     int qdim, kvdim, dh, Hq, Hkv, splits, rows, ldp, page, max_ctx;
     RowGeo geo;                  // which sequence and position a row has
     const float *partial;
-    float *q;
+    bf16_t *q;                   // layout: AttnArgs::q
     KvPtrs kv;
     const float *rope_cos, *rope_sin;
     uint32_t *status;
@@ -266,15 +266,13 @@ __global__ void qkv_finish_kernel(const QkvArgs a) {
         hi = y * cs + x * sn;
     }
     if (head < a.Hq) {
-        // stored ready for the attention MMA: scaled by log2(e) / sqrt(dh), each value as its two bf16 parts
-        // (hi in the low half-word, lo in the high one)
+        // stored ready for the attention MMA (see AttnArgs::q): scaled by log2(e) / sqrt(dh), split into two bf16 parts
         const float sc = (1.0f / sqrtf((float)a.dh)) * 1.4426950408889634f;
-        uint32_t *qq = reinterpret_cast<uint32_t *>(a.q);
-        uint16_t h0, l0, h1, l1;
-        split_bf16(lo * sc, h0, l0);
-        split_bf16(hi * sc, h1, l1);
-        qq[(size_t)r * a.qdim + col + e] = (uint32_t)h0 | ((uint32_t)l0 << 16);
-        qq[(size_t)r * a.qdim + col + e + half] = (uint32_t)h1 | ((uint32_t)l1 << 16);
+        const int gq = a.Hq / a.Hkv, kvh = head / gq, h = head - kvh * gq;
+        bf16_t *qh = a.q + (((size_t)r * a.Hkv + kvh) * 2 * gq + h) * a.dh, *ql = qh + (size_t)gq * a.dh;
+        auto at = [&](int i) -> int { return (((i >> 3) ^ (h & 7)) << 3) | (i & 7); };
+        split_bf16(lo * sc, qh[at(e)], ql[at(e)]);
+        split_bf16(hi * sc, qh[at(e + half)], ql[at(e + half)]);
         return;
     }
     if (!valid) return;                       // padding row: nothing to store
@@ -291,67 +289,153 @@ __global__ void qkv_finish_kernel(const QkvArgs a) {
     dst[e + half] = f32_bf16bits(hi);
 }
 
-// ---- attention. A work item is one 256-token chunk of one (sequence, KV head); the Hq/Hkv query
-// heads of the group share the K/V stream. One persistent CTA per SM walks its items (item index =
-// CTA, CTA + grid, ...) as one continuous stream of 64-token blocks through a shared-memory ring,
-// so the copies of the next items are in flight while the current one is computed. Scores and the
-// weighted sum run on mma.sync.m16n8k16 with the query (and the probabilities) as the A operand,
-// rows 0-7 the high bf16 parts of the heads and rows 8-15 the low parts, so both products carry
-// fp32-accurate inputs. Each warp owns 16 tokens of every block and keeps its own running
-// (max, sum, output); the four warps merge in fixed order at the end of the item.
-// Output per item: unnormalised o, running max m and sum l per head.
+// ---- attention. A work item is one 256-token chunk of one (sequence, KV head) for up to ROWS rows of the sequence: the
+// M rows of a target step or of a draft's extend step share the K/V stream (ROWS = 4), later draft steps have one row
+// (ROWS = 1). The Hq/Hkv query heads of the group share it as well. One persistent CTA per SM; its eight compute warps
+// form two groups, each with a ring of its own, fed by its own copy warp, and each walking its own items, so one
+// group's serial work (softmax, barriers, the partial's write) hides behind the other's and behind both streams.
+//
+// Scores and the weighted sum run on mma.sync.m16n8k16 with the query heads (and the probabilities) as the A operand,
+// rows 0-7 the high bf16 parts of the heads and rows 8-15 the low parts, so both products carry fp32-accurate inputs.
+// Within a group warp w computes the scores of tokens 16w .. 16w+15 of a 64-token block; the warps exchange the block
+// maximum and the probabilities through shared memory, then warp w adds up its quarter of the head dimension over all 64
+// tokens. So an item ends without a merge across warps, and an output row costs 16 registers per thread instead of 64:
+// four rows fit. A row goes through the same operations whatever ROWS is and whatever rows share its item.
+//
+// The K/V pool is a stack of page x head-dim tiles: one TMA copy brings 16 tokens of K or V (4 KB at head dim 128) in the
+// 128-byte-swizzled layout ldmatrix reads without bank conflicts. The copies used to be 16-byte cp.async from 128 threads
+// that also read the block table: those reads queued behind the copies, and a block could not be requested before the
+// read of its table entries came back (1.2 us per 32 KB block). Now a warp holds the table entries of a whole item in
+// registers, one item ahead.
+// Bound: the K/V stream for one row; the tensor-core issue and the softmax for four. Measured at the 7B shape, before ->
+// now: 64 rows with contexts in [512, 8192] (618 MB) 154 -> 102 us (6.1 TB/s, 0.93 of a plain copy); 16 sequences x 4
+// rows at 2048 (67 MB) 82 -> 35 us, the latency of the two exchanges per block and of the softmax chain (the tensor pipe
+// is 20 % busy).
+//
+// Committed K/V (positions below seq_lens) is immutable during a call, so the first ring stages are requested before the
+// wait for the predecessor kernel; blocks with positions this call writes, and the queries, come after it.
+// Output per item and row: unnormalised o, running max m (log2 units) and sum l per head.
 struct AttnArgs {
-    int Hq, Hkv, dh, page, page_shift, max_ctx, max_chunks, B;    // B: rows
-    RowGeo geo;                  // which sequence and position a row has
+    int Hq, Hkv, dh, page, max_ctx, max_chunks, B;    // B: sequences
+    int tma;                     // pages are whole 16-token tiles: TMA copies (else 16-byte copies, any page size)
+    RowGeo geo;                  // which positions a sequence's rows have
     unsigned long long wait_limit_ns;   // a ring wait gives up after this long
-    const float *q;              // [rows][Hq*dh] words: the scaled query values as {hi, lo} bf16 pairs
+    const bf16_t *q;             // [rows][Hkv][2][Hq/Hkv][dh]: scaled queries, high parts then low parts, 16-byte pieces of head
+                                 // h (of its group) stored at piece ^ (h & 7)
     KvPtrs kv;
     float *att_part;             // [rows][Hq][max_chunks][dh+2]
     uint32_t *status;
 };
 
 constexpr int kAttnBlk = 64;                 // tokens per ring stage
-constexpr int kAttnStages = 5;
-constexpr int kAttnThreads = 128;            // compute threads (warps 0-3); warps 4-7 only issue the copies
+constexpr int kAttnBox = 16;                 // tokens per TMA copy, and per warp in the score product
+constexpr int kAttnCompute = 256;            // compute threads (warps 0-7); warps 8-11: two copy warps per group
+constexpr int kAttnThreads = kAttnCompute + 128;
+constexpr int kAttnRows = 4;                 // rows of an item in calls with several rows per sequence
 
-struct AttnItem {                            // one (sequence, KV head, chunk), CTA-uniform
-    int r, kvh, chunk, t0, n_ctx, n_blk;
-    const int32_t *bt;
+struct AttnItem {                            // one (sequence, KV head, chunk, row set), group-uniform
+    int seq, kvh, chunk, set, t0, n_ctx, n_blk;
 };
 
-template <int DH>
+template <int DH, int ROWS>
 struct AttnSmem {
-    static constexpr int ROWB = DH * 2 + 16;                     // padded row: conflict-free fragment loads
-    static constexpr int QB = 8 * DH * 4;                        // the group's query vectors (fp32)
-    static constexpr int STAGE = 2 * kAttnBlk * ROWB + QB;       // K block, V block, queries (first block of an item)
-    static constexpr int MERGE = 4 * 8 * (DH + 2) * 4 + 64 * 4;  // per-warp (o, m, l) of 8 heads, then 4 x 8 weights, 8 maxima, 8 sums
-    static constexpr int TOTAL = kAttnStages * STAGE + MERGE + (kBatchRows + 1) * 4 + kBatchRows * 4 + (2 * kAttnStages + 1) * 8;
+    static constexpr int BOX = kAttnBox * DH * 2;                // bytes of one copy: [DH / 64][16 tokens][128 bytes]
+    static constexpr int VOFF = 4 * BOX;                         // a stage: four K boxes, four V boxes
+    static constexpr int STAGE = 8 * BOX;
+    static constexpr int SG = ROWS == 1 ? 3 : 2;                 // stages per group
+    static constexpr int NQ = 2;                                 // items per group whose queries are held
+    static constexpr int QROW = 16 * DH * 2;                     // room for a row's queries (8 heads, two parts)
+    static constexpr int PROW = 16 * 128;                        // a row's probabilities: 16 operand rows x 64 tokens
+    static constexpr int O_Q = 2 * SG * STAGE;
+    static constexpr int O_P = O_Q + 2 * NQ * ROWS * QROW;
+    static constexpr int O_RED = O_P + 2 * ROWS * PROW;          // per group: [ROWS][4 warps][8 heads] maxima, then sums
+    static constexpr int O_BAR = O_RED + 2 * 2 * ROWS * 32 * 4;
+    static constexpr int O_TAB = O_BAR + (2 * (2 * SG + NQ) + 1) * 8;
+    static constexpr int BYTES = O_TAB + (4 * kBatchRows + 1) * 4;
+    static constexpr int TOTAL = BYTES + 1024;                   // the ring starts on a 1024-byte boundary
 };
 
-template <int DH>
-__global__ void __launch_bounds__(2 * kAttnThreads, 1) attn_kernel(const AttnArgs a) {
+__device__ __forceinline__ void ldsm4(uint32_t addr, uint32_t (&r)[4]) {
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(addr) : "memory");
+}
+__device__ __forceinline__ void ldsm4_trans(uint32_t addr, uint32_t (&r)[4]) {
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(addr) : "memory");
+}
+__device__ __forceinline__ void sts32(uint32_t addr, uint32_t v) { asm volatile("st.shared.u32 [%0], %1;" ::"r"(addr), "r"(v) : "memory"); }
+// Two values as two packed bf16 pairs: their high parts and what is left of them.
+__device__ __forceinline__ void split2(float a, float b, uint32_t &hi, uint32_t &lo) {
+    uint16_t h0, l0, h1, l1;
+    split_bf16(a, h0, l0);
+    split_bf16(b, h1, l1);
+    hi = (uint32_t)h0 | ((uint32_t)h1 << 16);
+    lo = (uint32_t)l0 | ((uint32_t)l1 << 16);
+}
+
+template <int DH, int ROWS>
+__global__ void __launch_bounds__(kAttnThreads, 1) attn_kernel(const __grid_constant__ AttnArgs a, const __grid_constant__ CUtensorMap kmap,
+                                                               const __grid_constant__ CUtensorMap vmap) {
     chain_release();
-    chain_wait();
-    using L = AttnSmem<DH>;
-    constexpr int ROWB = L::ROWB, STAGE = L::STAGE;
-    extern __shared__ __align__(16) unsigned char smem[];
-    float *mo = reinterpret_cast<float *>(smem + kAttnStages * STAGE);                    // [4][8][DH + 2]
-    // 8-byte barriers first (STAGE and MERGE are multiples of 16), then the 4-byte tables
-    uint64_t *full = reinterpret_cast<uint64_t *>(smem + kAttnStages * STAGE + L::MERGE);  // [stages] copies landed
-    uint64_t *empty = full + kAttnStages;                                                  // [stages] stage consumed
-    volatile uint32_t *abort_flag = reinterpret_cast<volatile uint32_t *>(empty + kAttnStages);
-    int *prefix = reinterpret_cast<int *>(empty + kAttnStages + 1);                        // [B + 1] chunks before sequence r
-    int *nctx = prefix + kBatchRows + 1;
-    const bool producer = threadIdx.x >= kAttnThreads;
-    const int tid = threadIdx.x & (kAttnThreads - 1), warp = tid >> 5, lane = tid & 31;
+    using L = AttnSmem<DH, ROWS>;
+    constexpr int SG = L::SG, NQ = L::NQ;
+    extern __shared__ unsigned char smem_raw[];
+    unsigned char *smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
+    uint64_t *bars = reinterpret_cast<uint64_t *>(smem + L::O_BAR);
+    volatile uint32_t *abort_flag = reinterpret_cast<volatile uint32_t *>(bars + 2 * (2 * SG + NQ));
+    int *prefix = reinterpret_cast<int *>(smem + L::O_TAB);                // [B + 1] items before a sequence
+    int *tpos = prefix + kBatchRows + 1;                                   // position of a sequence's row 0
+    int *tval = tpos + kBatchRows;                                         // its rows that count
+    int *tlen = tval + kBatchRows;                                         // its committed positions
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int grp = warp < 8 ? warp >> 2 : (warp - 8) >> 1;                // copy warps 8, 9 serve group 0; 10, 11 group 1
+    uint64_t *full = bars + grp * (2 * SG + NQ), *empty = full + SG, *qempty = empty + SG;
+    unsigned char *ring = smem + (size_t)grp * SG * L::STAGE;
+    const int max_tokens = min(a.kv.max_pages * a.page, a.max_ctx);
+    const int gq = a.Hq / a.Hkv;
     if (threadIdx.x == 0) {
-        for (int s = 0; s < kAttnStages; ++s) { mbar_init(&full[s], kAttnThreads); mbar_init(&empty[s], kAttnThreads); }
+        for (int g = 0; g < 2; ++g) {
+            uint64_t *b = bars + g * (2 * SG + NQ);
+            for (int s = 0; s < SG; ++s) { mbar_init(&b[s], a.tma ? 1 : 65); mbar_init(&b[SG + s], 4); }
+            for (int s = 0; s < NQ; ++s) mbar_init(&b[2 * SG + s], 4);
+        }
         *abort_flag = 0;
         mbar_fence_init();
     }
-    // a wait that gives up after two seconds (or when another thread has), so a logic error cannot hang the device
+    // visible positions 0 .. n-1 of row m of a sequence
+    auto row_ctx = [&](int pos0, int m) -> int { return min(pos0 + m, max_tokens - 1) + 1; };
+    if (warp == 0) {             // two sequences per lane; seq_lens and n_ext are inputs of the call: nothing to wait for
+        int cnt[2];
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+            const int s = 2 * lane + u;
+            cnt[u] = 0;
+            if (s < a.B) {
+                const int len = max(a.kv.seq_lens[s], 0), nx = geo_next(a.geo, s);
+                const int pos0 = a.geo.step > 0 ? len + nx - 1 + a.geo.step : len;
+                const int nv = a.geo.step > 0 ? 1 : nx;
+                tpos[s] = pos0; tval[s] = nv; tlen[s] = len;
+                cnt[u] = (row_ctx(pos0, nv - 1) + kBatchAttnChunk - 1) / kBatchAttnChunk * a.Hkv * ((nv + ROWS - 1) / ROWS);
+            }
+        }
+        int incl = cnt[0] + cnt[1];
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int t = __shfl_up_sync(0xffffffffu, incl, o);
+            if (lane >= o) incl += t;
+        }
+        if (2 * lane <= a.B) prefix[2 * lane] = incl - cnt[0] - cnt[1];
+        if (2 * lane + 1 <= a.B) prefix[2 * lane + 1] = incl - cnt[1];
+        if (lane == 31 && a.B == 2 * 32) prefix[a.B] = incl;
+    }
+    __syncthreads();
+    const int n_items = prefix[a.B], worker = grp * (int)gridDim.x + (int)blockIdx.x, stride = 2 * (int)gridDim.x;
+
+    // a wait that gives up after two seconds (or when another thread has), so a logic error cannot hang the device;
+    // after that no wait blocks any more and every role runs to its end
     auto wait = [&](uint64_t *bar, uint32_t parity) -> bool {
         if (mbar_try_wait(bar, parity)) return true;
+        if (*abort_flag) return false;
         const unsigned long long t_begin = global_timer_ns();
         uint32_t polls = 0;
         while (!mbar_try_wait(bar, parity)) {
@@ -362,242 +446,301 @@ __global__ void __launch_bounds__(2 * kAttnThreads, 1) attn_kernel(const AttnArg
         }
         return true;
     };
-    const int gq = a.Hq / a.Hkv;
-    const int max_tokens = min(a.kv.max_pages * a.page, a.max_ctx);
-    if (threadIdx.x < a.B) {     // visible positions 0 .. n-1 of every row
-        bool valid;
-        nctx[threadIdx.x] = min(geo_pos(a.geo, a.kv, threadIdx.x, &valid), max_tokens - 1) + 1;
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        int acc = 0;
-        for (int r = 0; r < a.B; ++r) { prefix[r] = acc; const int ct = attn_chunk_tokens(nctx[r]); acc += (nctx[r] + ct - 1) / ct; }
-        prefix[a.B] = acc;
-    }
-    __syncthreads();
-    const int n_items = prefix[a.B] * a.Hkv;
-
     auto load_item = [&](AttnItem &it, int item) {
-        const int cidx = item / a.Hkv;
-        it.kvh = item - cidx * a.Hkv;
-        int r = it.r;                        // a CTA's items come in ascending order: search on from the last one
-        while (prefix[r + 1] <= cidx) ++r;
-        it.r = r;
-        it.chunk = cidx - prefix[r];
-        it.n_ctx = nctx[r];
-        const int ct = attn_chunk_tokens(it.n_ctx);
-        it.t0 = it.chunk * ct;
-        it.n_blk = (min(ct, it.n_ctx - it.t0) + kAttnBlk - 1) / kAttnBlk;
-        it.bt = a.kv.block_table + (size_t)(r / a.geo.M) * a.kv.max_pages;
+        int s = it.seq;                      // a worker's items come in ascending order: search on from the last one
+        while (prefix[s + 1] <= item) ++s;
+        it.seq = s;
+        int rem = item - prefix[s];
+        it.kvh = rem % a.Hkv;
+        rem /= a.Hkv;
+        const int nv = tval[s], sets = (nv + ROWS - 1) / ROWS;
+        it.chunk = rem / sets;
+        it.set = rem - it.chunk * sets;
+        it.t0 = it.chunk * kBatchAttnChunk;
+        it.n_ctx = row_ctx(tpos[s], min(nv, (it.set + 1) * ROWS) - 1);             // of the set's last row
+        it.n_blk = max(0, (min(kBatchAttnChunk, it.n_ctx - it.t0) + kAttnBlk - 1) / kAttnBlk);   // 0: no row of the set sees the chunk
     };
+    const uint32_t qbytes = (uint32_t)(2 * gq * DH * 2);
+    auto copy_queries = [&](const AttnItem &it, int slot, int stage, int i) {      // thread i copies the queries of the set's row i
+        if (i < min(ROWS, tval[it.seq] - it.set * ROWS)) {
+            const size_t r = (size_t)it.seq * a.geo.M + it.set * ROWS + i;
+            bulk_load(smem_u32(smem + L::O_Q + ((size_t)(grp * NQ + slot) * ROWS + i) * L::QROW),
+                      a.q + (r * a.Hkv + it.kvh) * 2 * gq * DH, qbytes, &full[stage]);
+        }
+    };
+    auto query_bytes = [&](const AttnItem &it) -> uint32_t { return qbytes * (uint32_t)min(ROWS, tval[it.seq] - it.set * ROWS); };
 
-    if (producer) {
-    // ---- copy warps: block fb of item fc goes into stage fi % kAttnStages once its previous reader is done.
-    // The block-table entries of a block are loaded one block ahead, so their latency is off the issue path.
-    constexpr int PIECES = DH / 8;                      // 16-byte pieces per row
-    constexpr int NIT = kAttnBlk * PIECES / kAttnThreads;
-    constexpr int TSTEP = kAttnThreads / PIECES;        // tokens between a thread's consecutive pieces
-    const int pc = tid % PIECES, tl = tid / PIECES;
-    const uint64_t kv_policy = l2_evict_first();
-    auto load_pages = [&](const AttnItem &it_, int blk, int (&pg)[NIT]) {
-#pragma unroll
-        for (int it = 0; it < NIT; ++it) {
-            int pos = it_.t0 + blk * kAttnBlk + tl + it * TSTEP;
-            if (pos >= it_.n_ctx) pos = it_.n_ctx - 1;
-            pg[it] = it_.bt[a.page_shift >= 0 ? pos >> a.page_shift : pos / a.page];
+    if (warp >= 8) {
+    const int ct = threadIdx.x - kAttnCompute - grp * 64;                 // thread among the group's 64 copy threads
+    const uint64_t policy = l2_evict_first();
+    AttnItem it, nx;
+    it.seq = 0;
+    int stage = 0, li = 0;
+    uint32_t phase = 0;
+    bool ok = true;
+    if (a.tma) {
+        if (ct < 32) {
+            // ---- lane i holds where 16-token tile i of the item's chunk is: its row in the pool seen as [.., dh]
+            auto tile_row = [&](const AttnItem &i_) -> int {
+                const int pos = min(i_.t0 + (lane & 15) * kAttnBox, i_.n_ctx - 1) & ~(kAttnBox - 1), pgi = pos / a.page;
+                int page = a.kv.block_table[(size_t)i_.seq * a.kv.max_pages + pgi];
+                if ((unsigned)page >= (unsigned)a.kv.num_pages) { atomicOr(a.status, kDevBadPage); page = 0; }
+                return (page * a.Hkv + i_.kvh) * a.page + (pos - pgi * a.page);
+            };
+            // lanes 0-3 copy the K tiles of a block, lanes 4-7 its V tiles
+            auto copy_block = [&](const AttnItem &i_, int blk, int rows) {
+                const int n = min(4, (i_.n_ctx - i_.t0 - blk * kAttnBlk + kAttnBox - 1) / kAttnBox);
+                const int y = __shfl_sync(0xffffffffu, rows, blk * 4 + (lane & 3));
+                if (lane == 0) mbar_arrive_expect_tx(&full[stage], (uint32_t)(2 * n * L::BOX) + (blk == 0 ? query_bytes(i_) : 0u));
+                __syncwarp();
+                if (lane < 8 && (lane & 3) < n)
+                    tma_load_3d_hint(smem_u32(ring + (size_t)stage * L::STAGE + (lane >> 2) * L::VOFF + (lane & 3) * L::BOX),
+                                     lane < 4 ? &kmap : &vmap, 0, y, 0, &full[stage], policy);
+            };
+            int item = worker, pre = 0, rows = 0, nrows = 0;
+            // the first item with work
+            for (; item < n_items; item += stride) { load_item(it, item); if (it.n_blk > 0) break; }
+            if (item < n_items) {
+                rows = tile_row(it);
+                for (; pre < SG && pre < it.n_blk && it.t0 + (pre + 1) * kAttnBlk <= tlen[it.seq]; ++pre) { stage = pre; copy_block(it, pre, rows); }
+            }
+            chain_wait();
+            stage = 0;
+            while (item < n_items && ok) {
+                // the next item with work, and its tiles
+                int nitem = item + stride;
+                nx = it;
+                for (; nitem < n_items; nitem += stride) { load_item(nx, nitem); if (nx.n_blk > 0) break; }
+                if (nitem < n_items) nrows = tile_row(nx);
+                for (int blk = 0; blk < it.n_blk; ++blk) {
+                    if (lane == 0) ok = wait(&empty[stage], phase ^ 1u) && (blk > 0 || wait(&qempty[li % NQ], ((li / NQ) & 1) ^ 1));
+                    ok = __shfl_sync(0xffffffffu, ok, 0);
+                    if (!ok) break;
+                    if (pre > 0) --pre;                 // this block's K/V is already on its way
+                    else copy_block(it, blk, rows);
+                    if (blk == 0) copy_queries(it, li % NQ, stage, lane);
+                    if (++stage == SG) { stage = 0; phase ^= 1u; }
+                }
+                ++li;
+                it = nx; item = nitem; rows = nrows;
+            }
+            // after a timeout nobody may have waited for the last copies: they land before the CTA exits
+            if (!ok && lane == 0)
+                for (int s = 0; s < SG; ++s) {
+                    stage = stage == 0 ? SG - 1 : stage - 1;
+                    if (stage == SG - 1) phase ^= 1u;
+                    for (int n = 0; n < (1 << 16) && !mbar_try_wait(&full[stage], phase); ++n) { }
+                }
         }
-    };
-    AttnItem fc, fn;
-    fc.r = 0;
-    int f_item = blockIdx.x, fb = 0, fi = 0;
-    int pg_cur[NIT], pg_next[NIT];
-    if (f_item < n_items) { load_item(fc, f_item); load_pages(fc, 0, pg_cur); }
-    while (f_item < n_items) {
-        // where the next block is, and its block-table entries
-        int n_item = f_item, nb = fb + 1;
-        fn = fc;
-        if (nb == fc.n_blk) {
-            nb = 0;
-            n_item += gridDim.x;
-            if (n_item < n_items) load_item(fn, n_item);
+    } else {
+        // ---- any page size: 16-byte copies into the same layout, zeros beyond the visible positions
+        constexpr int PIECES = DH / 8;
+        chain_wait();
+        for (int item = worker; item < n_items && ok; item += stride) {
+            load_item(it, item);
+            if (it.n_blk == 0) continue;
+            for (int blk = 0; blk < it.n_blk; ++blk) {
+                if (!wait(&empty[stage], phase ^ 1u) || (blk == 0 && !wait(&qempty[li % NQ], ((li / NQ) & 1) ^ 1))) { ok = false; break; }
+                const uint32_t sb = smem_u32(ring + (size_t)stage * L::STAGE);
+                for (int i = ct; i < kAttnBlk * PIECES; i += 64) {
+                    const int t = i / PIECES, c = i - t * PIECES;
+                    const int pos = it.t0 + blk * kAttnBlk + t, pc = min(pos, it.n_ctx - 1), pgi = pc / a.page;
+                    int page = a.kv.block_table[(size_t)it.seq * a.kv.max_pages + pgi];
+                    if ((unsigned)page >= (unsigned)a.kv.num_pages) { atomicOr(a.status, kDevBadPage); page = 0; }
+                    const size_t off = (((size_t)page * a.Hkv + it.kvh) * a.page + (pc - pgi * a.page)) * DH + c * 8;
+                    const uint32_t d = sb + (uint32_t)((t >> 4) * L::BOX + (c >> 3) * 2048 + (t & 15) * 128 + (((c & 7) ^ (t & 7)) << 4));
+                    const uint32_t n = pos < it.n_ctx ? 16u : 0u;
+                    cp_async16_off_hint<0>(d, a.kv.k_pages + off, n, policy);
+                    cp_async16_off_hint<0>(d + L::VOFF, a.kv.v_pages + off, n, policy);
+                }
+                if (ct == 0) mbar_arrive_expect_tx(&full[stage], blk == 0 ? query_bytes(it) : 0u);
+                if (blk == 0) copy_queries(it, li % NQ, stage, ct);
+                cp_async_arrive(&full[stage]);
+                if (++stage == SG) { stage = 0; phase ^= 1u; }
+            }
+            ++li;
         }
-        if (n_item < n_items) load_pages(fn, nb, pg_next);
-        const int stage = fi % kAttnStages;
-        if (!wait(&empty[stage], ((fi / kAttnStages) & 1) ^ 1)) break;
-        unsigned char *st = smem + (size_t)stage * STAGE;
-        size_t off[NIT];
-        uint32_t ok[NIT];
-#pragma unroll
-        for (int it = 0; it < NIT; ++it) {
-            int pos = fc.t0 + fb * kAttnBlk + tl + it * TSTEP;
-            ok[it] = pos < fc.n_ctx ? 16u : 0u;
-            if (pos >= fc.n_ctx) pos = fc.n_ctx - 1;
-            const int pgi = a.page_shift >= 0 ? pos >> a.page_shift : pos / a.page;
-            const int in_page = pos - pgi * a.page;
-            int page = pg_cur[it];
-            if ((unsigned)page >= (unsigned)a.kv.num_pages) { atomicOr(a.status, kDevBadPage); page = 0; }
-            off[it] = (((size_t)page * a.Hkv + fc.kvh) * a.page + in_page) * DH + pc * 8;
-        }
-        const uint32_t d0 = smem_u32(st + tl * ROWB + pc * 16);
-#pragma unroll
-        for (int it = 0; it < NIT; ++it) {
-            cp_async16_off_hint<0>(d0 + it * TSTEP * ROWB, a.kv.k_pages + off[it], ok[it], kv_policy);
-            cp_async16_off_hint<0>(d0 + kAttnBlk * ROWB + it * TSTEP * ROWB, a.kv.v_pages + off[it], ok[it], kv_policy);
-        }
-        if (fb == 0) {     // the item's query vectors ride with its first block
-            const float *qsrc = a.q + ((size_t)fc.r * a.Hq + (size_t)fc.kvh * gq) * DH;    // packed {hi, lo} words
-            for (int i = tid; i < gq * DH / 4; i += kAttnThreads)
-                cp_async16_off<0>(smem_u32(st + 2 * kAttnBlk * ROWB + i * 16), qsrc + i * 4, 16u);
-        }
-        cp_async_arrive(&full[stage]);      // this thread's arrival fires when its copies above have landed
-        ++fi;
-        fc = fn; f_item = n_item; fb = nb;
-#pragma unroll
-        for (int it = 0; it < NIT; ++it) pg_cur[it] = pg_next[it];
+        cp_async_wait_all();
     }
-    cp_async_wait_all();
     } else {
 
     // ---- compute side
-    const int hrow = lane >> 2, kq = (lane & 3) * 2;
-    AttnItem cc;
-    cc.r = 0;
-    int c_item = blockIdx.x, cb = 0, ci = 0;
-    if (c_item < n_items) load_item(cc, c_item);
-    uint32_t qa[DH / 16][4];
-    float m_run = -INFINITY, l_run = 0.f;       // of head hrow, this warp's tokens (replicated on the 4 lanes of a row)
-    float o[DH / 8][4];                          // MMA accumulators: [0],[1] the hi-part products, [2],[3] the lo-part ones
-    while (c_item < n_items) {
-        const int stage = ci % kAttnStages;
-        // the 128 compute threads agree on the outcome of the wait before any of them moves on
-        if (epi_any(!wait(&full[stage], (ci / kAttnStages) & 1))) break;
-        const unsigned char *sk = smem + (size_t)stage * STAGE;
-        const unsigned char *sv = sk + kAttnBlk * ROWB;
-        if (cb == 0) {
-            // query fragments: A rows 0-7 = hi parts of heads 0..gq-1, rows 8-15 = lo parts
-            // (the rotary kernel stored every query value as {hi, lo} bf16 halves of one word, already scaled)
-            const uint32_t *qh = reinterpret_cast<const uint32_t *>(sv + kAttnBlk * ROWB) + hrow * DH;
+    const int wi = warp & 3, hrow = lane >> 2, kq = (lane & 3) * 2;
+    constexpr int KS = DH / 16;                              // 16-wide slices of the head dimension
+    constexpr int NT = DH / 32;                              // 8-wide tiles of this warp's quarter of the head dimension
+    float *mx_s = reinterpret_cast<float *>(smem + L::O_RED) + grp * 2 * ROWS * 32, *l_s = mx_s + ROWS * 32;
+    // ldmatrix row addresses. K: this warp's tile, tokens as the operand's n. V (transposed): tile s, this warp's dims
+    const int ktok = (lane & 7) + ((lane >> 4) << 3), vtok = (lane & 7) + (((lane >> 3) & 1) << 3);
+    const uint32_t kbase = (uint32_t)(wi * L::BOX + ktok * 128), ksw = (uint32_t)(ktok & 7), kpc = (uint32_t)((lane >> 3) & 1);
+    const uint32_t vbase = (uint32_t)(L::VOFF + (wi * NT / 8) * 2048 + vtok * 128), vsw = (uint32_t)(vtok & 7);
+    const uint32_t vpc = (uint32_t)((wi * NT) & 7) + (uint32_t)(lane >> 4);
+    // queries: operand rows 0-7 = high parts, 8-15 = low parts (a head that does not exist repeats the last one: not used)
+    const int qh = min(lane & 7, gq - 1);
+    const uint32_t qlane = (uint32_t)((((lane >> 3) & 1) * gq + qh) * DH * 2), qsw = (uint32_t)(qh & 7), qpc = (uint32_t)(lane >> 4);
+    // probabilities: [16 operand rows][64 tokens], pieces of 8 tokens swizzled by the row
+    const uint32_t pbase = smem_u32(smem + L::O_P) + (uint32_t)(grp * ROWS * L::PROW);
+    const uint32_t plane = (uint32_t)(((lane & 7) + ((lane >> 3) & 1) * 8) * 128), psw = (uint32_t)(lane & 7), ppc = (uint32_t)(lane >> 4);
+    const uint32_t pst = pbase + (uint32_t)(hrow * 128 + kq * 2);
+    AttnItem it;
+    it.seq = 0;
+    int stage = 0, li = 0;
+    uint32_t phase = 0;
+    for (int item = worker; item < n_items; item += stride) {
+        load_item(it, item);
+        if (it.n_blk == 0) continue;
+        const int slot = li % NQ;
+        ++li;
+        const uint32_t qbase = smem_u32(smem + L::O_Q + (size_t)(grp * NQ + slot) * ROWS * L::QROW) + qlane;
+        int nrow[ROWS];                                      // visible positions, 0 for a row that does not exist or is padding
 #pragma unroll
-            for (int ks = 0; ks < DH / 16; ++ks) {
-                uint2 w0 = make_uint2(0u, 0u), w1 = make_uint2(0u, 0u);
-                if (hrow < gq) {
-                    w0 = *reinterpret_cast<const uint2 *>(qh + ks * 16 + kq);
-                    w1 = *reinterpret_cast<const uint2 *>(qh + ks * 16 + kq + 8);
-                }
-                qa[ks][0] = __byte_perm(w0.x, w0.y, 0x5410);      // row hrow (hi parts), k = kq, kq+1
-                qa[ks][1] = __byte_perm(w0.x, w0.y, 0x7632);      // row hrow + 8 (lo parts)
-                qa[ks][2] = __byte_perm(w1.x, w1.y, 0x5410);      // row hrow,     k = kq+8, kq+9
-                qa[ks][3] = __byte_perm(w1.x, w1.y, 0x7632);
-            }
-            m_run = -INFINITY; l_run = 0.f;
+        for (int k = 0; k < ROWS; ++k) nrow[k] = it.set * ROWS + k < tval[it.seq] ? row_ctx(tpos[it.seq], it.set * ROWS + k) : 0;
+        uint32_t qa[ROWS == 1 ? KS : 1][4];
+        float m_run[ROWS], l_run[ROWS], o[ROWS][NT][4];      // o: [0],[1] the hi-part products, [2],[3] the lo-part ones
 #pragma unroll
-            for (int nt = 0; nt < DH / 8; ++nt) o[nt][0] = o[nt][1] = o[nt][2] = o[nt][3] = 0.f;
+        for (int k = 0; k < ROWS; ++k) {
+            m_run[k] = -INFINITY; l_run[k] = 0.f;
+#pragma unroll
+            for (int nt = 0; nt < NT; ++nt) o[k][nt][0] = o[k][nt][1] = o[k][nt][2] = o[k][nt][3] = 0.f;
         }
-        const int tw = warp * 16;                              // this warp's tokens inside the block
-        const int tbase = cc.t0 + cb * kAttnBlk + tw;
-        if (tbase < cc.n_ctx) {
-            // scores: two n-tiles of 8 tokens; one ldmatrix.x4 brings both tiles' K fragments of a 16-wide slice
-            float s[2][4];
-            s[0][0] = s[0][1] = s[0][2] = s[0][3] = 0.f;
-            s[1][0] = s[1][1] = s[1][2] = s[1][3] = 0.f;
-            const uint32_t kaddr = smem_u32(sk) + (uint32_t)((tw + (lane & 7) + ((lane >> 4) << 3)) * ROWB + ((lane >> 3) & 1) * 16);
+        for (int blk = 0; blk < it.n_blk; ++blk) {
+            wait(&full[stage], phase);
+            const uint32_t sb = smem_u32(ring + (size_t)stage * L::STAGE);
+            const int tb = it.t0 + blk * kAttnBlk, tw = tb + wi * kAttnBox;
+            if (ROWS == 1 && blk == 0) {
 #pragma unroll
-            for (int ks = 0; ks < DH / 16; ++ks) {
-                uint32_t b00, b01, b10, b11;
-                asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];"
-                             : "=r"(b00), "=r"(b01), "=r"(b10), "=r"(b11) : "r"(kaddr + ks * 32));
-                mma_bf16(s[0], qa[ks][0], qa[ks][1], qa[ks][2], qa[ks][3], b00, b01);
-                mma_bf16(s[1], qa[ks][0], qa[ks][1], qa[ks][2], qa[ks][3], b10, b11);
+                for (int ks = 0; ks < KS; ++ks) ldsm4(qbase + ((((uint32_t)(2 * ks) + qpc) ^ qsw) << 4), qa[ks]);
             }
-            // thread holds, for head hrow: tokens tw + nt*8 + kq + {0,1}: hi part in [0],[1], lo part in [2],[3]
-            float sc[4];
-            float mx = -INFINITY;
+            uint32_t kf[KS][4];
 #pragma unroll
-            for (int nt = 0; nt < 2; ++nt)
-#pragma unroll
-                for (int j = 0; j < 2; ++j) {
-                    float v = s[nt][j] + s[nt][j + 2];
-                    if (tbase + nt * 8 + kq + j >= cc.n_ctx) v = -INFINITY;
-                    sc[nt * 2 + j] = v;
-                    mx = fmaxf(mx, v);
+            for (int ks = 0; ks < KS; ++ks)
+                ldsm4(sb + kbase + (uint32_t)((ks >> 2) * 2048) + ((((uint32_t)(2 * (ks & 3)) + kpc) ^ ksw) << 4), kf[ks]);
+            const int over = it.n_ctx - tw;                  // of this warp's 16 tokens, those that exist
+            if (over > 0 && over < kAttnBox) {
+                // value rows nothing has written may hold anything: zeros, so that a probability of 0 meets a finite number
+                for (int i = lane; i < (kAttnBox - over) * (DH / 8); i += 32) {
+                    const int t = over + i / (DH / 8), c = i % (DH / 8);
+                    *reinterpret_cast<uint4 *>(ring + (size_t)stage * L::STAGE + L::VOFF + wi * L::BOX + (c >> 3) * 2048 + t * 128 + (c & 7) * 16) =
+                        make_uint4(0, 0, 0, 0);
                 }
-            mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 1));
-            mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 2));
-            const float m_new = fmaxf(m_run, mx);                 // finite: the warp's first token is visible
-            const float corr = exp2f(m_run - m_new);              // 0 on the item's first block (m_run = -inf)
-            float psum = 0.f;
-            uint32_t pa[4];
-            {
-                float pr[4];
-#pragma unroll
-                for (int i = 0; i < 4; ++i) { pr[i] = exp2f(sc[i] - m_new); psum += pr[i]; }
-                uint16_t h0, l0, h1, l1, h2, l2, h3, l3;
-                split_bf16(pr[0], h0, l0); split_bf16(pr[1], h1, l1); split_bf16(pr[2], h2, l2); split_bf16(pr[3], h3, l3);
-                pa[0] = (uint32_t)h0 | ((uint32_t)h1 << 16);      // row hrow,   tokens kq, kq+1
-                pa[1] = (uint32_t)l0 | ((uint32_t)l1 << 16);      // row hrow+8
-                pa[2] = (uint32_t)h2 | ((uint32_t)h3 << 16);      // row hrow,   tokens 8+kq, 8+kq+1
-                pa[3] = (uint32_t)l2 | ((uint32_t)l3 << 16);
+                fence_proxy_async();                         // before a later TMA copy overwrites them
             }
-            psum += __shfl_xor_sync(0xffffffffu, psum, 1);
-            psum += __shfl_xor_sync(0xffffffffu, psum, 2);
-            l_run = l_run * corr + psum;
-            m_run = m_new;
-            // weighted sum, accumulated in the MMA: rescale the running output only when some row's maximum moved
-            if (__any_sync(0xffffffffu, corr != 1.0f)) {
+            // No branch on a row's visibility: the rows' chains interleave. A row that sees nothing of a block adds zeros; one
+            // that does not exist or sees nothing of the chunk computes on whatever is there and is not written.
+            float sc[ROWS][4];
 #pragma unroll
-                for (int nt = 0; nt < DH / 8; ++nt) { o[nt][0] *= corr; o[nt][1] *= corr; o[nt][2] *= corr; o[nt][3] *= corr; }
-            }
-            // B[k = token][n = dim] read with a transposing ldmatrix from V[token][dim], two n-tiles per load
-            const uint32_t vaddr = smem_u32(sv) + (uint32_t)((tw + (lane & 7) + ((lane >> 3) & 1) * 8) * ROWB + (lane >> 4) * 16);
+            for (int k = 0; k < ROWS; ++k) {
+                float s[2][2][4];                            // [n-tile of 8 tokens][even / odd slices]: four independent chains
 #pragma unroll
-            for (int nt = 0; nt < DH / 8; nt += 2) {
-                uint32_t b00, b01, b10, b11;
-                asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];"
-                             : "=r"(b00), "=r"(b01), "=r"(b10), "=r"(b11) : "r"(vaddr + nt * 16));
-                mma_bf16(o[nt], pa[0], pa[1], pa[2], pa[3], b00, b01);
-                mma_bf16(o[nt + 1], pa[0], pa[1], pa[2], pa[3], b10, b11);
-            }
-        }
-        mbar_arrive(&empty[stage]);        // this thread has read all it needs from the stage
-        ++ci;
-        if (++cb == cc.n_blk) {
-            // ---- end of the item: merge the four warps (fixed order) and write the chunk's partial
-            float *dst = mo + ((size_t)warp * 8 + hrow) * (DH + 2);
+                for (int i = 0; i < 4; ++i) s[0][0][i] = s[0][1][i] = s[1][0][i] = s[1][1][i] = 0.f;
 #pragma unroll
-            for (int nt = 0; nt < DH / 8; ++nt) { dst[nt * 8 + kq] = o[nt][0] + o[nt][2]; dst[nt * 8 + kq + 1] = o[nt][1] + o[nt][3]; }
-            if ((lane & 3) == 0) { dst[DH] = m_run; dst[DH + 1] = l_run; }
-            bar_sync(1, kAttnThreads);
-            float *wgt = mo + 4 * 8 * (DH + 2);          // [4][8] weights, [8] maxima, [8] sums
-            if (tid < 32) {                               // thread = (head tid >> 2, warp tid & 3)
-                const int h = tid >> 2, w = tid & 3;
-                float m = -INFINITY;
-                for (int u = 0; u < 4; ++u) m = fmaxf(m, mo[((size_t)u * 8 + h) * (DH + 2) + DH]);
-                const float mw = mo[((size_t)w * 8 + h) * (DH + 2) + DH];
-                wgt[w * 8 + h] = mw == -INFINITY ? 0.f : exp2f(mw - m);
-                if (w == 0) {
-                    float l = 0.f;
-                    for (int u = 0; u < 4; ++u) {         // ascending warp order
-                        const float mu = mo[((size_t)u * 8 + h) * (DH + 2) + DH];
-                        l += mo[((size_t)u * 8 + h) * (DH + 2) + DH + 1] * (mu == -INFINITY ? 0.f : exp2f(mu - m));
+                for (int ks = 0; ks < KS; ++ks) {
+                    uint32_t q[4];
+                    if (ROWS == 1) {
+#pragma unroll
+                        for (int i = 0; i < 4; ++i) q[i] = qa[ROWS == 1 ? ks : 0][i];
+                    } else ldsm4(qbase + (uint32_t)(k * L::QROW) + ((((uint32_t)(2 * ks) + qpc) ^ qsw) << 4), q);
+                    mma_bf16_pure(s[0][ks & 1], q[0], q[1], q[2], q[3], kf[ks][0], kf[ks][1]);
+                    mma_bf16_pure(s[1][ks & 1], q[0], q[1], q[2], q[3], kf[ks][2], kf[ks][3]);
+                }
+                // thread: head hrow, tokens tw + nt*8 + kq + {0,1}; hi-part product in [0],[1], lo-part in [2],[3]
+                float mx = -INFINITY;
+#pragma unroll
+                for (int nt = 0; nt < 2; ++nt)
+#pragma unroll
+                    for (int j = 0; j < 2; ++j) {
+                        float v = (s[nt][0][j] + s[nt][1][j]) + (s[nt][0][j + 2] + s[nt][1][j + 2]);
+                        if (tw + nt * 8 + kq + j >= nrow[k]) v = -INFINITY;
+                        sc[k][nt * 2 + j] = v;
+                        mx = fmaxf(mx, v);
                     }
-                    wgt[32 + h] = m;
-                    wgt[40 + h] = l;
+                mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 1));
+                mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 2));
+                if ((lane & 3) == 0) mx_s[k * 32 + wi * 8 + hrow] = mx;
+            }
+            if (blk == it.n_blk - 1 || ROWS == 1) {          // the queries have been read for the last time (one row: kept in registers)
+                __syncwarp();
+                if (lane == 0 && (ROWS > 1 || blk == 0)) mbar_arrive(&qempty[slot]);
+            }
+            bar_sync(1 + grp, 128);
+#pragma unroll
+            for (int k = 0; k < ROWS; ++k) {
+                const float *mk = mx_s + k * 32 + hrow;
+                const float m_new = fmaxf(m_run[k], fmaxf(fmaxf(mk[0], mk[8]), fmaxf(mk[16], mk[24])));     // finite for a row that counts
+                const float corr = exp2f(m_run[k] - m_new);  // 0 on the item's first block (m_run = -inf)
+                float p[4];
+#pragma unroll
+                for (int i = 0; i < 4; ++i) p[i] = exp2f(sc[k][i] - m_new);
+                // each thread keeps its own tokens' share of the sum; the shares are added at the end of the item
+                l_run[k] = l_run[k] * corr + ((p[0] + p[1]) + (p[2] + p[3]));
+                m_run[k] = m_new;
+#pragma unroll
+                for (int nt = 0; nt < 2; ++nt) {
+                    uint32_t hi, lo;
+                    split2(p[2 * nt], p[2 * nt + 1], hi, lo);
+                    const uint32_t d = pst + (uint32_t)(k * L::PROW) + (((uint32_t)(wi * 2 + nt) ^ (uint32_t)hrow) << 4);
+                    sts32(d, hi);
+                    sts32(d + 1024, lo);
+                }
+                if (__any_sync(0xffffffffu, corr != 1.0f)) {
+#pragma unroll
+                    for (int nt = 0; nt < NT; ++nt) { o[k][nt][0] *= corr; o[k][nt][1] *= corr; o[k][nt][2] *= corr; o[k][nt][3] *= corr; }
                 }
             }
-            bar_sync(1, kAttnThreads);
-            for (int i = tid; i < gq * DH; i += kAttnThreads) {
-                const int h = i / DH, j = i - h * DH;
-                float acc = 0.f;
+            // one row: all value fragments are requested before the barrier; several: tile by tile (registers)
+            constexpr int VB = ROWS == 1 ? 4 : 1;
+            uint32_t vf[VB][NT / 2][4];
+            auto load_v = [&](int s, uint32_t (&v)[NT / 2][4]) {
 #pragma unroll
-                for (int w = 0; w < 4; ++w) acc += mo[((size_t)w * 8 + h) * (DH + 2) + j] * wgt[w * 8 + h];
-                float *out = a.att_part + (((size_t)cc.r * a.Hq + (size_t)cc.kvh * gq + h) * a.max_chunks + cc.chunk) * (DH + 2);
-                out[j] = acc;
-                if (j == 0) { out[DH] = wgt[32 + h] * 0.6931471805599453f; out[DH + 1] = wgt[40 + h]; }     // the chunk maximum in natural-log units
+                for (int j = 0; j < NT / 2; ++j)
+                    ldsm4_trans(sb + vbase + (uint32_t)(s * L::BOX) + (((vpc + (uint32_t)(2 * j)) ^ vsw) << 4), v[j]);
+            };
+            if (ROWS == 1) {
+#pragma unroll
+                for (int s = 0; s < VB; ++s) if (tb + s * kAttnBox < it.n_ctx) load_v(s, vf[s]);
             }
-            bar_sync(1, kAttnThreads);     // merge buffer free for the next item
-            cb = 0;
-            c_item += gridDim.x;
-            if (c_item < n_items) load_item(cc, c_item);
+            bar_sync(1 + grp, 128);
+#pragma unroll
+            for (int s = 0; s < 4; ++s) {
+                if (tb + s * kAttnBox >= it.n_ctx) continue;
+                if (ROWS > 1) load_v(s, vf[0]);
+#pragma unroll
+                for (int k = 0; k < ROWS; ++k) {
+                    uint32_t p[4];
+                    ldsm4(pbase + (uint32_t)(k * L::PROW) + plane + ((((uint32_t)(2 * s) + ppc) ^ psw) << 4), p);
+                    const auto &v = vf[ROWS == 1 ? s : 0];
+#pragma unroll
+                    for (int j = 0; j < NT / 2; ++j) {
+                        mma_bf16_pure(o[k][2 * j], p[0], p[1], p[2], p[3], v[j][0], v[j][1]);
+                        mma_bf16_pure(o[k][2 * j + 1], p[0], p[1], p[2], p[3], v[j][2], v[j][3]);
+                    }
+                }
+            }
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&empty[stage]);        // this warp has read all it needs from the stage
+            if (++stage == SG) { stage = 0; phase ^= 1u; }
+        }
+        // ---- the chunk's partial of every row that sees it
+#pragma unroll
+        for (int k = 0; k < ROWS; ++k) {
+            if (nrow[k] <= it.t0) continue;
+            float lw = l_run[k];
+            lw += __shfl_xor_sync(0xffffffffu, lw, 1);
+            lw += __shfl_xor_sync(0xffffffffu, lw, 2);
+            if ((lane & 3) == 0) l_s[k * 32 + wi * 8 + hrow] = lw;
+        }
+        bar_sync(1 + grp, 128);
+#pragma unroll
+        for (int k = 0; k < ROWS; ++k) {
+            if (nrow[k] <= it.t0 || hrow >= gq) continue;
+            const size_t r = (size_t)it.seq * a.geo.M + it.set * ROWS + k;
+            float *out = a.att_part + ((r * a.Hq + (size_t)it.kvh * gq + hrow) * a.max_chunks + it.chunk) * (DH + 2);
+#pragma unroll
+            for (int nt = 0; nt < NT; ++nt)
+                *reinterpret_cast<float2 *>(out + wi * (DH / 4) + nt * 8 + kq) = make_float2(o[k][nt][0] + o[k][nt][2], o[k][nt][1] + o[k][nt][3]);
+            if (wi == 0 && (lane & 3) == 0) {
+                const float *lk = l_s + k * 32 + hrow;
+                *reinterpret_cast<float2 *>(out + DH) = make_float2(m_run[k], ((lk[0] + lk[8]) + lk[16]) + lk[24]);
+            }
         }
     }
     }
@@ -622,7 +765,11 @@ __global__ void attn_merge_kernel(const MergeArgs a) {
     const int max_tokens = min(a.kv.max_pages * a.page, a.max_ctx);
     bool valid;
     const int n_ctx = min(geo_pos(a.geo, a.kv, r, &valid), max_tokens - 1) + 1;
-    const int n_chunks = (n_ctx + attn_chunk_tokens(n_ctx) - 1) / attn_chunk_tokens(n_ctx);
+    if (!valid) {                // padding row: attention skipped it
+        store_hilo(a.xop, a.ld, r, head * a.dh + j, 0.f);
+        return;
+    }
+    const int n_chunks = (n_ctx + kBatchAttnChunk - 1) / kBatchAttnChunk;
     const int stride = a.dh + 2;
     const float *base = a.att_part + ((size_t)r * a.Hq + head) * a.max_chunks * stride;
     // the chunks' maxima: each thread reads some, then a block-wide maximum (exact, order-free)
@@ -646,7 +793,7 @@ __global__ void attn_merge_kernel(const MergeArgs a) {
         }
 #pragma unroll
         for (int u = 0; u < 8; ++u) {
-            const float f = expf(mv[u] - m);
+            const float f = exp2f(mv[u] - m);
             acc += ov[u] * f;
             l += lv[u] * f;
         }
@@ -660,14 +807,14 @@ __global__ void attn_merge_kernel(const MergeArgs a) {
         }
 #pragma unroll
         for (int u = 0; u < 2; ++u) {
-            const float f = expf(mv[u] - m);
+            const float f = exp2f(mv[u] - m);
             acc += ov[u] * f;
             l += lv[u] * f;
         }
     }
     for (; c < n_chunks; ++c) {
         const float *src = base + (size_t)c * stride;
-        const float f = expf(src[a.dh] - m);
+        const float f = exp2f(src[a.dh] - m);
         acc += src[j] * f;
         l += src[a.dh + 1] * f;
     }
@@ -770,6 +917,56 @@ __global__ void __launch_bounds__(kCompactThreads) ids_compact_kernel(const uint
     }
 }
 
+// Tensor map of a paged K or V pool seen as rows of head_dim values: a copy brings 16 rows as [dh / 64][16][64], each
+// 128-byte row swizzled. Encoded per call (a host computation): the pool is the caller's.
+int attn_encode_map(CUtensorMap *map, const bf16_t *pool, const BatchedShape &sh, int num_pages) {
+    TmapEncodeFn encode;
+    if (int rc = tmap_encoder(&encode)) return rc;
+    const cuuint64_t dims[3] = {64, (cuuint64_t)num_pages * sh.Hkv * sh.page, (cuuint64_t)(sh.dh / 64)};
+    const cuuint64_t strides[2] = {(cuuint64_t)sh.dh * 2, 128};
+    const cuuint32_t box[3] = {64, kAttnBox, (cuuint32_t)(sh.dh / 64)};
+    const cuuint32_t estr[3] = {1, 1, 1};
+    CUresult r = encode(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<bf16_t *>(pool), dims, strides, box, estr,
+                        CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                        CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+    return r == CUDA_SUCCESS ? 0 : (int)cudaErrorInvalidValue;
+}
+
+template <int DH, int ROWS>
+int attn_launch(const AttnArgs &a, const CUtensorMap &kmap, const CUtensorMap &vmap, int n_sm, TmapCache *cache, cudaStream_t st) {
+    int &limit = cache->attn_smem[ROWS > 1];
+    if (limit < AttnSmem<DH, ROWS>::TOTAL) {      // raise the kernel's shared-memory limit once per context
+        cudaError_t e = cudaFuncSetAttribute(attn_kernel<DH, ROWS>, cudaFuncAttributeMaxDynamicSharedMemorySize, AttnSmem<DH, ROWS>::TOTAL);
+        if (e != cudaSuccess) return (int)e;
+        limit = AttnSmem<DH, ROWS>::TOTAL;
+    }
+    return (int)launch_chained(attn_kernel<DH, ROWS>, dim3(n_sm), dim3(kAttnThreads), (size_t)AttnSmem<DH, ROWS>::TOTAL, st, a, kmap, vmap);
+}
+
+// Attention and chunk merge of a pass over `rows` rows (geo.M per sequence).
+int attention(const BatchedShape &sh, const BatchedWs &ws, const KvPtrs &kv, const RowGeo &geo, int rows, int n_sm,
+              unsigned long long wait_limit_ns, TmapCache *cache, cudaStream_t st, long long *launches) {
+    AttnArgs a{};
+    a.Hq = sh.Hq; a.Hkv = sh.Hkv; a.dh = sh.dh; a.page = sh.page; a.max_ctx = sh.max_ctx; a.geo = geo;
+    a.max_chunks = ws.max_chunks; a.q = ws.q; a.kv = kv; a.att_part = ws.att_part; a.status = ws.status;
+    a.B = rows / geo.M; a.wait_limit_ns = wait_limit_ns;
+    a.tma = sh.page % kAttnBox == 0 && (long long)kv.num_pages * sh.Hkv * sh.page < (1ll << 31);
+    CUtensorMap kmap{}, vmap{};
+    int rc = 0;
+    if (a.tma) {
+        if ((rc = attn_encode_map(&kmap, kv.k_pages, sh, kv.num_pages))) return rc;
+        if ((rc = attn_encode_map(&vmap, kv.v_pages, sh, kv.num_pages))) return rc;
+    }
+    if (geo.M > 1) rc = sh.dh == 128 ? attn_launch<128, kAttnRows>(a, kmap, vmap, n_sm, cache, st) : attn_launch<64, kAttnRows>(a, kmap, vmap, n_sm, cache, st);
+    else rc = sh.dh == 128 ? attn_launch<128, 1>(a, kmap, vmap, n_sm, cache, st) : attn_launch<64, 1>(a, kmap, vmap, n_sm, cache, st);
+    if (rc) return rc;
+    MergeArgs m{};
+    m.Hq = sh.Hq; m.dh = sh.dh; m.page = sh.page; m.max_ctx = sh.max_ctx; m.geo = geo; m.max_chunks = ws.max_chunks;
+    m.ld = ws.ld0; m.kv = kv; m.att_part = ws.att_part; m.xop = ws.xop0;
+    *launches += 2;
+    return (int)launch_chained(attn_merge_kernel, dim3(sh.Hq, rows), dim3(sh.dh), 0, st, m);
+}
+
 int pick_splits(int n_tiles, int n_kb, int n_sm) {
     int best = 1;
     double best_eff = 0.0;
@@ -808,7 +1005,7 @@ size_t batched_layout(BatchedWs &ws, unsigned char *base, const BatchedShape &sh
     ws.partial = reinterpret_cast<float *>(take((size_t)kBatchMaxSplits * rows * ws.ldp * 4));
     ws.x = reinterpret_cast<float *>(take((size_t)rows * sh.d * 4));
     ws.hout = reinterpret_cast<float *>(take((size_t)rows * sh.d * 4));
-    ws.q = reinterpret_cast<float *>(take((size_t)rows * qdim * 4));
+    ws.q = reinterpret_cast<bf16_t *>(take((size_t)rows * 2 * qdim * 2));
     ws.att_part = reinterpret_cast<float *>(take((size_t)rows * sh.Hq * ws.max_chunks * (sh.dh + 2) * 4));
     ws.keys_bytes = (size_t)(sh.max_K > 1 ? sh.max_K : 1) * kBatchRows * 8 + 256;
     ws.keys = reinterpret_cast<unsigned long long *>(take(ws.keys_bytes));
@@ -859,15 +1056,6 @@ int batched_draft(const BatchedCall &c, cudaStream_t st, long long *launches) {
         return skinny_gemm_launch(g, c.n_sm, c.smem_optin, st, c.cache);
     };
     int rc = 0;
-    const size_t attn_smem = sh.dh == 128 ? AttnSmem<128>::TOTAL : AttnSmem<64>::TOTAL;
-    if (c.cache->attn_smem < (int)attn_smem) {
-        if (sh.dh == 128) e = cudaFuncSetAttribute(attn_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)attn_smem);
-        else e = cudaFuncSetAttribute(attn_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)attn_smem);
-        if (e != cudaSuccess) return (int)e;
-        c.cache->attn_smem = (int)attn_smem;
-    }
-    int page_shift = -1;
-    for (int b = 0; b < 31; ++b) if ((1 << b) == sh.page) page_shift = b;
 
     // One pass of the MTP module (projection, decoder layer, final norm) over `rows` activation rows of the sequences
     // seq0 .. seq0 + rows / geo.M - 1 of the group. The final norm publishes into `xop_head` (the output head's operand),
@@ -912,21 +1100,7 @@ int batched_draft(const BatchedCall &c, cudaStream_t st, long long *launches) {
             ++*launches;
             if ((rc = (int)launch_chained(qkv_finish_kernel, dim3(sh.Hq + 2 * sh.Hkv, rows), dim3(sh.dh / 2), 0, st, a))) return rc;
         }
-        {
-            AttnArgs a{};
-            a.Hq = sh.Hq; a.Hkv = sh.Hkv; a.dh = sh.dh; a.page = sh.page; a.max_ctx = sh.max_ctx; a.geo = geo;
-            a.max_chunks = ws.max_chunks; a.q = ws.q; a.kv = kv; a.att_part = ws.att_part; a.status = ws.status;
-            a.page_shift = page_shift; a.B = rows; a.wait_limit_ns = c.wait_limit_ns;
-            ++*launches;
-            if (sh.dh == 128) rc = (int)launch_chained(attn_kernel<128>, dim3(c.n_sm), dim3(2 * kAttnThreads), attn_smem, st, a);
-            else rc = (int)launch_chained(attn_kernel<64>, dim3(c.n_sm), dim3(2 * kAttnThreads), attn_smem, st, a);
-            if (rc) return rc;
-            MergeArgs m{};
-            m.Hq = sh.Hq; m.dh = sh.dh; m.page = sh.page; m.max_ctx = sh.max_ctx; m.geo = geo; m.max_chunks = ws.max_chunks;
-            m.ld = ws.ld0; m.kv = kv; m.att_part = ws.att_part; m.xop = ws.xop0;
-            ++*launches;
-            if ((rc = (int)launch_chained(attn_merge_kernel, dim3(sh.Hq, rows), dim3(sh.dh), 0, st, m))) return rc;
-        }
+        if ((rc = attention(sh, ws, kv, geo, rows, c.n_sm, c.wait_limit_ns, c.cache, st, launches))) return rc;
         // x += W_o o
         g = GemmArgs{};
         g.a[0] = c.layer.wo; g.a_rows[0] = d; g.n_seg = 1; g.epi = EPI_PARTIAL;
@@ -1008,15 +1182,6 @@ int batched_target(const BatchedTargetCall &c, cudaStream_t st, long long *launc
         return (int)launch_chained(post_kernel, dim3(R), dim3(kRowThreads), 0, st, a);
     };
     int rc = 0;
-    const size_t attn_smem = sh.dh == 128 ? AttnSmem<128>::TOTAL : AttnSmem<64>::TOTAL;
-    if (c.cache->attn_smem < (int)attn_smem) {
-        if (sh.dh == 128) e = cudaFuncSetAttribute(attn_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)attn_smem);
-        else e = cudaFuncSetAttribute(attn_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)attn_smem);
-        if (e != cudaSuccess) return (int)e;
-        c.cache->attn_smem = (int)attn_smem;
-    }
-    int page_shift = -1;
-    for (int b = 0; b < 31; ++b) if ((1 << b) == sh.page) page_shift = b;
 
     // x = Emb(tokens); operand of the first layer = rms(x; g_in)
     ++*launches;
@@ -1037,21 +1202,7 @@ int batched_target(const BatchedTargetCall &c, cudaStream_t st, long long *launc
             ++*launches;
             if ((rc = (int)launch_chained(qkv_finish_kernel, dim3(sh.Hq + 2 * sh.Hkv, R), dim3(sh.dh / 2), 0, st, a))) return rc;
         }
-        {
-            AttnArgs a{};
-            a.Hq = sh.Hq; a.Hkv = sh.Hkv; a.dh = sh.dh; a.page = sh.page; a.max_ctx = sh.max_ctx; a.geo = geo;
-            a.max_chunks = ws.max_chunks; a.q = ws.q; a.kv = kv; a.att_part = ws.att_part; a.status = ws.status;
-            a.page_shift = page_shift; a.B = R; a.wait_limit_ns = c.wait_limit_ns;
-            ++*launches;
-            if (sh.dh == 128) rc = (int)launch_chained(attn_kernel<128>, dim3(c.n_sm), dim3(2 * kAttnThreads), attn_smem, st, a);
-            else rc = (int)launch_chained(attn_kernel<64>, dim3(c.n_sm), dim3(2 * kAttnThreads), attn_smem, st, a);
-            if (rc) return rc;
-            MergeArgs m{};
-            m.Hq = sh.Hq; m.dh = sh.dh; m.page = sh.page; m.max_ctx = sh.max_ctx; m.geo = geo; m.max_chunks = ws.max_chunks;
-            m.ld = ws.ld0; m.kv = kv; m.att_part = ws.att_part; m.xop = ws.xop0;
-            ++*launches;
-            if ((rc = (int)launch_chained(attn_merge_kernel, dim3(sh.Hq, R), dim3(sh.dh), 0, st, m))) return rc;
-        }
+        if ((rc = attention(sh, ws, kv, geo, R, c.n_sm, c.wait_limit_ns, c.cache, st, launches))) return rc;
         g = GemmArgs{};
         g.a[0] = L.wo; g.a_rows[0] = d; g.n_seg = 1; g.epi = EPI_PARTIAL;
         if ((rc = gemm(g, d, qdim, qdim, ws.xop0, ws.ld0))) return rc;

@@ -8,13 +8,9 @@
 namespace fmtp {
 
 constexpr int kBatchRows = 64;        // sequences per group (activation columns = 2 x rows <= 128)
-constexpr int kBatchAttnChunk = 256;  // fewest context tokens per attention work item (sizes the partial buffer)
-// Context tokens per attention work item for a row that sees n_ctx positions. An item ends with serial work (the
-// compute warps merge their partials and write the chunk's) while the K/V stream of the next items waits, so long
-// contexts take four times longer items (measured at 64 sequences with contexts in [512, 8192]: -13 us of 393 per
-// step); up to 4096 positions a row keeps 256-token items so that a small batch still spreads over all SMs. The size
-// is a function of the row's own context only: a row's summation order does not depend on the batch it is in.
-__host__ __device__ inline int attn_chunk_tokens(int n_ctx) { return n_ctx > 4096 ? 1024 : kBatchAttnChunk; }
+// Context tokens per attention work item: a constant, so that items are equal and a row's summation order depends on
+// its own position only, never on the batch or on the rows it shares an item with.
+constexpr int kBatchAttnChunk = 256;
 constexpr int kBatchMaxSplits = 8;
 
 // What the launches of the batched path would otherwise ask the driver for on every call; lives in the context
@@ -29,7 +25,7 @@ struct TmapCache {
     TmapEntry e[12];
     int n, next;
     int gemm_smem[3];                        // limit set on skinny_gemm_kernel<1>, <2>, <4>
-    int attn_smem;                           // limit set on attn_kernel
+    int attn_smem[2];                        // limit set on attn_kernel for one row / several rows per sequence
 };
 
 struct BatchedWs {
@@ -39,7 +35,7 @@ struct BatchedWs {
     float *partial;               // [kBatchMaxSplits][rows][ldp] split-K partial sums
     float *x;                     // [rows][d]   residual stream
     float *hout;                  // [rows][d]   final-normed hidden state (recursed in fp32)
-    float *q;                     // [rows][qdim] rotated queries
+    bf16_t *q;                    // rotated, scaled queries as high and low bf16 parts
     float *att_part;              // [rows][Hq][max_chunks][dh + 2]  (o, m, l) per context chunk
     unsigned long long *keys;     // [max_K][kBatchRows] argmax keys
     uint32_t *id_bitmap;          // [ceil(V/32)] membership bits of the subset

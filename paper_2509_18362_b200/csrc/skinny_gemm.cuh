@@ -136,6 +136,19 @@ __device__ __forceinline__ void tma_load_2d(uint32_t dst_smem, const CUtensorMap
         : "memory");
 }
 
+// The same for a 3-D tensor map, with an L2 eviction policy.
+__device__ __forceinline__ void tma_load_3d_hint(uint32_t dst_smem, const CUtensorMap *map, int x, int y, int z, uint64_t *bar, uint64_t policy) {
+    asm volatile(
+        "cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint [%0], [%1, {%2, %3, %4}], [%5], %6;"
+        ::"r"(dst_smem), "l"(map), "r"(x), "r"(y), "r"(z), "r"(smem_u32(bar)), "l"(policy)
+        : "memory");
+}
+// One contiguous copy global -> shared; both addresses and the size are multiples of 16 bytes.
+__device__ __forceinline__ void bulk_load(uint32_t dst_smem, const void *src, uint32_t bytes, uint64_t *bar) {
+    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
+                 ::"r"(dst_smem), "l"(src), "r"(bytes), "r"(smem_u32(bar)) : "memory");
+}
+
 // State of one producer thread's walk over the ring.
 struct GemmProducer {
     uint32_t dst0;            // shared address of this thread's chunk in row r0 of stage 0
@@ -452,21 +465,29 @@ __global__ void __launch_bounds__(kGemmThreads, 1) skinny_gemm_kernel(const Gemm
     }
 }
 
-// Tensor map of the activation operand X [NB][ldx] (bf16): tiles of 64 K elements x NB rows, 128-byte
-// swizzle (the layout the MMA reads), zeros beyond K. Returns 0 or a cudaError_t.
-inline int gemm_encode_xmap(CUtensorMap *map, const bf16_t *x, int ldx, int K, int NB) {
-    typedef CUresult (*encode_fn)(CUtensorMap *, CUtensorMapDataType, cuuint32_t, void *, const cuuint64_t *, const cuuint64_t *,
-                                  const cuuint32_t *, const cuuint32_t *, CUtensorMapInterleave, CUtensorMapSwizzle,
-                                  CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
-    static encode_fn encode = nullptr;
+typedef CUresult (*TmapEncodeFn)(CUtensorMap *, CUtensorMapDataType, cuuint32_t, void *, const cuuint64_t *, const cuuint64_t *,
+                                 const cuuint32_t *, const cuuint32_t *, CUtensorMapInterleave, CUtensorMapSwizzle,
+                                 CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
+// The driver's tensor-map encoder (a host computation, no device work). Returns 0 or a cudaError_t.
+inline int tmap_encoder(TmapEncodeFn *out) {
+    static TmapEncodeFn encode = nullptr;
     if (!encode) {
         void *fn = nullptr;
         cudaDriverEntryPointQueryResult qr;
         cudaError_t e = cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &fn, cudaEnableDefault, &qr);
         if (e != cudaSuccess) return (int)e;
         if (!fn || qr != cudaDriverEntryPointSuccess) return (int)cudaErrorNotSupported;
-        encode = reinterpret_cast<encode_fn>(fn);
+        encode = reinterpret_cast<TmapEncodeFn>(fn);
     }
+    *out = encode;
+    return 0;
+}
+
+// Tensor map of the activation operand X [NB][ldx] (bf16): tiles of 64 K elements x NB rows, 128-byte
+// swizzle (the layout the MMA reads), zeros beyond K. Returns 0 or a cudaError_t.
+inline int gemm_encode_xmap(CUtensorMap *map, const bf16_t *x, int ldx, int K, int NB) {
+    TmapEncodeFn encode;
+    if (int rc = tmap_encoder(&encode)) return rc;
     const cuuint64_t dims[2] = {(cuuint64_t)K, (cuuint64_t)NB};
     const cuuint64_t strides[1] = {(cuuint64_t)ldx * 2};
     const cuuint32_t box[2] = {(cuuint32_t)kGemmBK, (cuuint32_t)NB};
