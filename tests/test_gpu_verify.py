@@ -130,3 +130,40 @@ def test_a_wait_that_runs_out_sets_the_timeout_flag_and_leaves_the_device_usable
     a, bonus, _ = _run(Bd, ctx, case["logits"], case["drafts"])
     assert np.array_equal(a, case["length"])
     ctx.close()
+
+
+@pytest.mark.parametrize("B,K,V", [
+    (1, 0, 1), (2, 1, 7), (3, 2, 8), (5, 3, 9),                 # rows shorter than, equal to and past one 16-byte vector
+    (1, 3, 2047), (3, 1, 2049), (64, 3, 2055),                  # around the shortest slice
+    (30, 3, 6001), (80, 1, 8193), (150, 0, 16393), (40, 7, 16384),   # every slice length, rows at every alignment
+])
+def test_scan_at_slice_edges(B, K, V):
+    """Maxima, ties, -inf and NaN on both sides of every slice and vector edge; exact."""
+    Bd, ctx = _ctx()
+    x = np.round(I.rng(B, f"edges.{V}").standard_normal((B, K + 1, V)).astype(np.float32) * 2) / 2      # many ties
+    bits = I.f32_to_bf16_bits(x).reshape(x.shape)
+    edges = sorted({e + d for n in (8, 2048, 4096, 8192, 16384, V) for e in range(0, V + 1, max(n, V // 7 // n * n, n)) for d in (-1, 0, 1)
+                    if 0 <= e + d < V})
+    flat = bits.reshape(-1, V)
+    for r, row in enumerate(flat):
+        at = [edges[(7 * r + 3 * i) % len(edges)] for i in range(3)]
+        if r % 5 == 0:
+            row[:] = 0xFF80                                      # -inf everywhere but a NaN and, every other time, one number
+            row[at[0]] = 0x7FC0
+            if r % 10 == 0:
+                row[at[1]] = 0xC000
+        elif r % 5 == 1:
+            row[at] = 0x4180                                     # the maximum up to three times
+        elif r % 5 == 2:
+            row[row == 0] = 0x8000                               # minus and plus zero are one value
+            row[(row & 0x8000) == 0] = 0x8000
+            row[at[0]] = 0x0000
+        elif r % 5 == 3:
+            row[at[:2]] = 0xFFC1                                 # NaNs of the other sign
+    drafts = I.token_ids(B, (B, K), V)
+    _, _, rg = O.verify_accept(bits, drafts)
+    drafts[::2] = rg[::2, :K]
+    a, bonus, g = _run(Bd, ctx, bits, drafts)
+    ra, rb, rg = O.verify_accept(bits, drafts)
+    assert np.array_equal(g, rg) and np.array_equal(a, ra) and np.array_equal(bonus, rb)
+    ctx.close()
