@@ -104,13 +104,17 @@ class FastMTPError(RuntimeError):
 
 
 def _ptr(t):
-    return None if t is None else C.c_void_p(t.data_ptr())
+    """Address of a tensor, as the plain integer the argtypes convert (None stays NULL)."""
+    return None if t is None else t.data_ptr()
+
+
+# Handle of the current stream. Building a torch Stream object for it cost 3.4 us a call, 0.3 us this way: a
+# verification of one sequence takes 7 us on the device and was bound by its 11 us on the host.
+_current_raw_stream = torch._C._cuda_getCurrentRawStream
 
 
 def _stream(stream):
-    if stream is None:
-        stream = torch.cuda.current_stream()
-    return C.c_void_p(stream.cuda_stream)
+    return _current_raw_stream(torch.cuda.current_device()) if stream is None else stream.cuda_stream
 
 
 def layer_w(t: dict) -> fmtp_layer_w:
