@@ -980,6 +980,25 @@ int pick_splits(int n_tiles, int n_kb, int n_sm) {
     return best;
 }
 
+// Rows and K ranges of a GEMM's work items; a function of the matrix and the SM count only, never of the batch.
+void pick_items(GemmArgs &g, int n_sm) {
+    const int n_kb = (g.K + kGemmBK - 1) / kGemmBK;
+    g.splits = 1;
+    g.item_rows = kGemmTileM;
+    g.n_ranges = 0;
+    if (g.epi == EPI_ARGMAX) {
+        // equal shares of the rows in the fewest rounds over the SMs
+        const int most = 2 * kGemmTileM, rounds = (g.n_rows + most * n_sm - 1) / (most * n_sm);
+        g.item_rows = ((g.n_rows + rounds * n_sm - 1) / (rounds * n_sm) + 7) / 8 * 8;
+        g.n_ranges = (g.n_rows + g.item_rows - 1) / g.item_rows;
+    } else {
+        for (int s = 0; s < g.n_seg; ++s) g.n_ranges += (g.a_rows[s] + g.item_rows - 1) / g.item_rows;
+        if (g.epi == EPI_PARTIAL) g.splits = pick_splits(g.n_ranges, n_kb, n_sm);
+    }
+    g.kb_per_split = (n_kb + g.splits - 1) / g.splits;
+    g.splits = (n_kb + g.kb_per_split - 1) / g.kb_per_split;      // no empty range
+}
+
 }  // namespace
 
 size_t batched_layout(BatchedWs &ws, unsigned char *base, const BatchedShape &sh) {
@@ -1047,10 +1066,7 @@ int batched_draft(const BatchedCall &c, cudaStream_t st, long long *launches) {
         g.wait_limit_ns = c.wait_limit_ns;
         g.extra_arrivals = inject_left > 0 ? 1 : 0;      // self-test: the call's first GEMM waits for a copy that never comes
         if (inject_left > 0) --inject_left;
-        const int n_tiles = (n_rows + kGemmTileM - 1) / kGemmTileM, n_kb = (Kdim + kGemmBK - 1) / kGemmBK;
-        g.splits = g.epi == EPI_PARTIAL ? pick_splits(n_tiles, n_kb, c.n_sm) : 1;
-        g.kb_per_split = (n_kb + g.splits - 1) / g.splits;
-        g.splits = (n_kb + g.kb_per_split - 1) / g.kb_per_split;      // no empty range
+        pick_items(g, c.n_sm);
         g.partial = ws.partial; g.ldp = ws.ldp;
         ++*launches;
         return skinny_gemm_launch(g, c.n_sm, c.smem_optin, st, c.cache);
@@ -1165,10 +1181,7 @@ int batched_target(const BatchedTargetCall &c, cudaStream_t st, long long *launc
         g.n_rows = n_rows; g.K = Kdim; g.lda = lda; g.x = x; g.ldx = ldx; g.NB = NB; g.R = R;
         g.status = ws.status;
         g.wait_limit_ns = c.wait_limit_ns;
-        const int n_tiles = (n_rows + kGemmTileM - 1) / kGemmTileM, n_kb = (Kdim + kGemmBK - 1) / kGemmBK;
-        g.splits = g.epi == EPI_PARTIAL ? pick_splits(n_tiles, n_kb, c.n_sm) : 1;
-        g.kb_per_split = (n_kb + g.splits - 1) / g.splits;
-        g.splits = (n_kb + g.kb_per_split - 1) / g.kb_per_split;
+        pick_items(g, c.n_sm);
         g.partial = ws.partial; g.ldp = ws.ldp;
         ++*launches;
         return skinny_gemm_launch(g, c.n_sm, c.smem_optin, st, c.cache);

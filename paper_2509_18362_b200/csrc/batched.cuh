@@ -24,7 +24,7 @@ struct TmapEntry {
 struct TmapCache {
     TmapEntry e[12];
     int n, next;
-    int gemm_smem[3];                        // limit set on skinny_gemm_kernel<1>, <2>, <4>
+    int gemm_smem[2];                        // limit set on skinny_gemm_kernel<2>, <4>
     int attn_smem[2];                        // limit set on attn_kernel for one row / several rows per sequence
 };
 

@@ -5,15 +5,21 @@
 //
 // The weight matrix is read exactly once from HBM; the activation operand X (bf16, row n = 2r is
 // the high part of activation row r and n = 2r + 1 the low part, so the pair carries an fp32
-// value) is small and re-read from L2 for every tile. One CTA per SM walks a static list of work
-// items (tile, K range). Roles: warps 0-3 epilogue (TMEM -> registers -> global), warp 4 issues
-// the MMAs, warps 5-12 copy A into a shared-memory ring with 16-byte cp.async, laid out as
-// the MMA's 128-byte-swizzled K-major tiles (64 K elements wide); the X block of a stage comes by
-// one TMA tile copy (same swizzle) through the copy engine, which leaves the load/store path's
-// ~64 GB/s per SM to the weights: with 64 rows the X bytes equal the weight bytes. A ring stage holds KA such
-// 64-wide blocks that are requested back to back, so a weight row is read in pieces of KA x 128
-// contiguous bytes. Accumulators are double buffered in TMEM so the epilogue of one item overlaps
-// the MMAs of the next.
+// value) is small and re-read from L2 for every item. One CTA per SM walks a static list of work
+// items (row range, K range). Roles: warps 0-3 epilogue (TMEM -> registers -> global), warp 4 issues
+// the MMAs, warp 5 the TMA tile copies of X, warps 6-13 copy A with 16-byte cp.async, laid out as the MMA's
+// 128-byte-swizzled K-major tiles (64 K elements wide). Accumulators are double buffered in TMEM so the epilogue of one
+// item overlaps the MMAs of the next.
+//
+// What bounds it. Up to 32 operand columns: HBM (7.5 TB/s between launches' fixed costs). At 64 activation rows the weight
+// bytes in flight: with A and X in one ring, half of the memory held X and 96 KB of weights were requested ahead per SM
+// (gate/up of the 7B shape 59 us, 65 with the MMAs and X taken out, against 49 at 4 rows with 192 KB). So A and X have
+// rings of their own (128-160 KB for A), and an item of gate/up or of the output head has two tiles that share every X
+// block; gate/up 56 us. The split-K matrices have too few rows for two tiles.
+// A stage is KA K blocks: four while three weight stages of that size fit, else two. Finer stages lose: a wait on a barrier
+// costs the MMA thread 200 cycles even when it is over, the four MMAs of a K block 190-260.
+// Weights by TMA lose too: the copy engine takes 47 GB/s per SM, and 128-byte pieces of rows 38 KB apart are slow at HBM
+// (down 28 -> 35 us); four gathered rows per copy cost 27 ns (head of 16384 ids 29 -> 80 us).
 //
 // A stage's barrier counts one asynchronous arrival per copy thread (cp.async.mbarrier.arrive), so a
 // stage is published the moment its bytes have landed.
@@ -28,14 +34,16 @@
 namespace fmtp {
 
 constexpr int kGemmProducers = 256;          // eight copy warps
-constexpr int kGemmThreads = 160 + kGemmProducers;
+constexpr int kGemmThreads = 192 + kGemmProducers;
 constexpr int kGemmBK = 64;                 // K elements per swizzled block: one 128-byte row
 constexpr int kGemmTileM = 128;
-constexpr int kGemmMaxStages = 10;
+constexpr int kGemmTileBytes = kGemmTileM * 128;    // a tile's 64-wide block
+constexpr int kGemmMaxStages = 6;
+constexpr int kGemmMaxXStages = 4;
 
 enum GemmEpilogue {
     EPI_PARTIAL = 0,   // fp32 partial sums  partial[split][r][m] = D[m,2r] + D[m,2r+1]
-    EPI_SWIGLU = 1,    // a tile holds 64 gate rows and the 64 up rows of the same indices: act = silu(g) * u, written as the
+    EPI_SWIGLU = 1,    // tile 0 holds gate rows, tile 1 the up rows of the same indices: act = silu(g) * u, written as the
                        // hi/lo operand of the next GEMM
     EPI_ARGMAX = 2,    // per activation row the maximum of (logit, row id) as a packed key (atomicMax), optional fp32 logits
 };
@@ -50,6 +58,7 @@ struct GemmArgs {
     int n_rows, K, lda;          // output rows (EPI_SWIGLU: ffn indices); K % 8 == 0
     const bf16_t *x;             // [NB][ldx] bf16
     int ldx, NB, R;              // NB % 16 == 0, 2R <= NB <= 128
+    int item_rows, n_ranges;     // output rows of an item (at most 128, EPI_ARGMAX 256) and number of such row ranges
     int splits, kb_per_split;    // K is cut into `splits` ranges of kb_per_split 64-wide blocks
     int epi;
     float *partial;              // [splits][R][ldp]
@@ -62,22 +71,18 @@ struct GemmArgs {
     bf16_t *logits_bf16;         // EPI_ARGMAX with round_bf16, optional: the logits as bf16, same indexing
     int round_bf16;              // 1: the argmax is decided on the logits rounded to bf16 (the values a caller sees)
     uint32_t *status;
-    int n_stages;
-    int force_ka;                // 0: pick the blocks per stage from the shared memory available
+    int n_stages, n_xstages;
     unsigned long long wait_limit_ns;   // every wait of the kernel gives up after this long
     int extra_arrivals;          // self-test only: arrivals a ring stage expects beyond the copies that are made
 };
 
 struct GemmSmem {
     uint64_t full[kGemmMaxStages], empty[kGemmMaxStages];
+    uint64_t xfull[kGemmMaxXStages], xempty[kGemmMaxXStages];
     uint64_t tfull[2], tempty[2], drain;
     uint32_t tmem_base, abort_flag;
     unsigned long long kmax[4][64];
-    float exch[64][17];          // EPI_SWIGLU: up-row sums handed to the gate rows' threads
 };
-
-__host__ __device__ inline int gemm_kblock_bytes(int NB) { return kGemmTileM * 128 + NB * 128; }
-__host__ __device__ inline int gemm_tile_rows(int epi) { return epi == EPI_SWIGLU ? 64 : kGemmTileM; }
 
 __device__ __forceinline__ bool gemm_wait(GemmSmem *sm, uint64_t *bar, uint32_t parity, unsigned long long limit_ns) {
     if (mbar_try_wait(bar, parity)) return true;
@@ -95,21 +100,41 @@ __device__ __forceinline__ bool gemm_wait(GemmSmem *sm, uint64_t *bar, uint32_t 
     return true;
 }
 
-// Work items of a CTA: items (tile of 128 rows, K range) are dealt round-robin over the CTAs. (Giving every CTA
-// an equal contiguous share of the output head's rows instead -- 221 rows as a full and a partial tile at the 7B
-// shape, where 256 tiles are 1.7 rounds of 148 CTAs -- was measured 3 % slower: the second round's 108 CTAs still
-// saturate HBM, and partial tiles cost issue slots.)
-struct GemmItem { int row0, row_end, split; };
-__device__ __forceinline__ int gemm_my_items(const GemmArgs &g, int n_items) {
+// After a timeout perhaps nobody has waited for the last copies of a ring (the next one would go to slot `pos` in phase
+// `phase`): wait for them, with a limit, before the CTA exits. Normally the MMA thread has seen all of them.
+__device__ __forceinline__ void gemm_drain(GemmSmem *sm, uint64_t *full, int n, int pos, uint32_t phase) {
+    const unsigned long long t0 = global_timer_ns();
+    for (int s = 0; s < n && *reinterpret_cast<volatile uint32_t *>(&sm->abort_flag); ++s) {
+        if (pos == 0) { pos = n; phase ^= 1u; }
+        --pos;
+        while (!mbar_try_wait(&full[pos], phase) && global_timer_ns() - t0 < 1000000ull) { }
+    }
+}
+
+// Work items of a CTA: items (row range, K range) are dealt round-robin over the CTAs. Ranges do not cross the
+// matrices of a concatenation.
+struct GemmItem { int row0, row_end, split, seg, src0; };       // output rows; matrix and its row of row0
+__device__ __forceinline__ int gemm_my_items(int n_items) {
     return (int)blockIdx.x < n_items ? (n_items - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x : 0;
 }
 __device__ __forceinline__ GemmItem gemm_my_item(const GemmArgs &g, int i) {
     GemmItem it;
     const int item = (int)blockIdx.x + i * (int)gridDim.x;
-    const int tile = item / g.splits, tile_rows = gemm_tile_rows(g.epi);
-    it.split = item - tile * g.splits;
-    it.row0 = tile * tile_rows;
-    it.row_end = min(it.row0 + tile_rows, g.n_rows);
+    int rng = item / g.splits, first = 0;
+    it.split = item - rng * g.splits;
+    it.seg = 0;
+    int rows = g.n_rows;
+    if (g.n_seg > 1) {
+        rows = g.a_rows[0];
+#pragma unroll
+        for (int s = 0; s < 2; ++s) {
+            const int n = (g.a_rows[s] + g.item_rows - 1) / g.item_rows;
+            if (it.seg == s && s + 1 < g.n_seg && rng >= n) { rng -= n; first += g.a_rows[s]; it.seg = s + 1; rows = g.a_rows[s + 1]; }
+        }
+    }
+    it.src0 = rng * g.item_rows;
+    it.row0 = first + it.src0;
+    it.row_end = first + min(it.src0 + g.item_rows, rows);
     return it;
 }
 
@@ -149,77 +174,28 @@ __device__ __forceinline__ void bulk_load(uint32_t dst_smem, const void *src, ui
                  ::"r"(dst_smem), "l"(src), "r"(bytes), "r"(smem_u32(bar)) : "memory");
 }
 
-// State of one producer thread's walk over the ring.
-struct GemmProducer {
-    uint32_t dst0;            // shared address of this thread's chunk in row r0 of stage 0
-    int stage_bytes, kblock_bytes, S, c;
-    int stage;
-    uint32_t phase;
-    bool tma_thread;          // the one producer thread that issues the X tile copies
-    uint32_t dst_x;           // shared address of the X tile in block 0 of stage 0
-    const CUtensorMap *xmap;
-    uint64_t *full;
-    uint64_t policy;          // L2 eviction policy of the weight stream
-};
-
-// Copies this thread's share of K block kb + J (if it is inside the item) into block J of the
-// current stage. Source addresses are the per-row pointers plus the immediate J * 128 bytes, so
-// all blocks of a stage go out before a pointer register is rewritten.
-// PART: 1 = the weight rows only, 2 = the activation rows only, 3 = both.
-template <int J, int PART>
-__device__ __forceinline__ void produce_kblock(const GemmArgs &g, const GemmProducer &pr, int kb, int kb1,
-                                               const bf16_t *(&ap)[4], const uint32_t (&aok)[4]) {
-    if (kb + J >= kb1) return;
-    if ((PART & 2) && pr.tma_thread)
-        tma_load_2d(pr.dst_x + (uint32_t)pr.stage * pr.stage_bytes + (uint32_t)J * pr.kblock_bytes, pr.xmap, (kb + J) * kGemmBK, 0,
-                    pr.full + pr.stage);
-    if (!(PART & 1)) return;
-    const bool kvalid = (kb + J) * kGemmBK + pr.c * 8 < g.K;
-    const uint32_t dst = pr.dst0 + (uint32_t)pr.stage * pr.stage_bytes + (uint32_t)J * pr.kblock_bytes;
-    if (kvalid && (aok[0] & aok[1] & aok[2] & aok[3]) != 0u) {      // the common case: plain 16-byte copies
-#pragma unroll
-        for (int i = 0; i < 4; ++i) cp_async16_full_hint<J * 128>(dst + i * 4096, ap[i], pr.policy);
-    } else if (kvalid) {
-#pragma unroll
-        for (int i = 0; i < 4; ++i) cp_async16_off_hint<J * 128>(dst + i * 4096, ap[i], aok[i], pr.policy);
-    } else {   // this chunk column lies beyond K: zeros, nothing is read
-#pragma unroll
-        for (int i = 0; i < 4; ++i) cp_async16_off<0>(dst + i * 4096, g.a[0], 0u);
-    }
-}
-
-template <int KA, int PART>
-__device__ __forceinline__ void produce_stage(const GemmArgs &g, const GemmProducer &pr, int kb, int kb1,
-                                              const bf16_t *(&ap)[4], const uint32_t (&aok)[4]) {
-    produce_kblock<0, PART>(g, pr, kb, kb1, ap, aok);
-    if constexpr (KA > 1) produce_kblock<1, PART>(g, pr, kb, kb1, ap, aok);
-    if constexpr (KA > 2) {
-        produce_kblock<2, PART>(g, pr, kb, kb1, ap, aok);
-        produce_kblock<3, PART>(g, pr, kb, kb1, ap, aok);
-    }
-}
-
-// KA 64-wide K blocks per ring stage; every stage of the ring can be in flight.
 template <int KA>
-__global__ void __launch_bounds__(kGemmThreads, 1) skinny_gemm_kernel(const GemmArgs g, const __grid_constant__ CUtensorMap xmap) {
-    extern __shared__ unsigned char smem_raw[];
-    const uint32_t raw = smem_u32(smem_raw);
-    unsigned char *ring = smem_raw + ((1024u - (raw & 1023u)) & 1023u);
-    const int S = g.n_stages;
-    const int kblock_bytes = gemm_kblock_bytes(g.NB);
-    const int stage_bytes = KA * kblock_bytes;
-    GemmSmem *sm = reinterpret_cast<GemmSmem *>(ring + (size_t)S * stage_bytes);
+__global__ void __launch_bounds__(kGemmThreads, 1) skinny_gemm_kernel(const __grid_constant__ GemmArgs g, const __grid_constant__ CUtensorMap xmap) {
+    extern __shared__ __align__(1024) unsigned char ring[];
+    const int S = g.n_stages, SX = g.n_xstages;
+    constexpr int kStage = KA * kGemmTileBytes;             // one tile, KA K blocks
+    const int xblock = g.NB * 128, xstage = KA * xblock;
+    unsigned char *xring = ring + (size_t)S * kStage;
+    GemmSmem *sm = reinterpret_cast<GemmSmem *>(xring + (size_t)SX * xstage);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const bool two = g.epi != EPI_PARTIAL;                  // items may have two tiles
 
-    const int buf_cols = (g.NB + 31) & ~31;                 // TMEM columns of one accumulator buffer
+    const int sub_cols = (g.NB + 31) & ~31;                 // TMEM columns of one tile's accumulator
+    const int buf_cols = two ? 2 * sub_cols : sub_cols;     // and of one accumulator buffer
     uint32_t alloc_cols = 32;
     while ((int)alloc_cols < 2 * buf_cols) alloc_cols <<= 1;
 
     if (tid == 0) {
-        for (int s = 0; s < S; ++s) { mbar_init(&sm->full[s], kGemmProducers + 1 + g.extra_arrivals); mbar_init(&sm->empty[s], 1); }
+        for (int s = 0; s < S; ++s) { mbar_init(&sm->full[s], kGemmProducers + g.extra_arrivals); mbar_init(&sm->empty[s], 1); }
+        for (int s = 0; s < SX; ++s) { mbar_init(&sm->xfull[s], 1); mbar_init(&sm->xempty[s], 1); }
         for (int b = 0; b < 2; ++b) { mbar_init(&sm->tfull[b], 1); mbar_init(&sm->tempty[b], 128); }
         mbar_init(&sm->drain, 1);
-        sm->abort_flag = 0;
+        sm->abort_flag = (smem_u32(ring) & 1023u) != 0u;    // swizzled tiles need the alignment: nothing runs without it
         mbar_fence_init();
     }
     if (warp == 4) {
@@ -232,130 +208,136 @@ __global__ void __launch_bounds__(kGemmThreads, 1) skinny_gemm_kernel(const Gemm
     tc_fence_after_sync();
     const uint32_t tmem_base = *reinterpret_cast<volatile uint32_t *>(&sm->tmem_base);
 
-    const int tile_rows = gemm_tile_rows(g.epi);
-    const int n_tiles = (g.n_rows + tile_rows - 1) / tile_rows;
-    const int n_items = n_tiles * g.splits;
+    const int n_items = *reinterpret_cast<volatile uint32_t *>(&sm->abort_flag) ? 0 : g.n_ranges * g.splits;
     const int n_kb = (g.K + kGemmBK - 1) / kGemmBK;
+    const int n_my = gemm_my_items(n_items);
+    auto tiles_of = [&](const GemmItem &gi) -> int { return g.epi == EPI_SWIGLU || gi.row_end - gi.row0 > kGemmTileM ? 2 : 1; };
 
-    if (warp >= 5) {
-        // ================= producers: thread pt copies chunk column c of tile rows r0 + 32 i
-        const int pt = tid - 160;
+    if (warp >= 6) {
+        // ================= weight copies: thread pt copies 16-byte column c of rows r0, r0 + 32, ... of a tile, KA K blocks at a
+        // time: the blocks are immediate offsets on the source, so a pointer register is rewritten only once per stage (a
+        // cp.async reads its address when it leaves the queue; rewriting it waits for that)
+        const int pt = tid - 192;
         const int c = pt & 7, r0 = pt >> 3;
-        GemmProducer pr;
-        pr.dst0 = smem_u32(ring) + (uint32_t)(r0 * 128 + ((c ^ (r0 & 7)) << 4));
-        pr.stage_bytes = stage_bytes; pr.kblock_bytes = kblock_bytes; pr.S = S; pr.c = c;
-        pr.stage = 0; pr.phase = 0;
-        pr.policy = l2_evict_first();
-        pr.tma_thread = pt == 0; pr.dst_x = smem_u32(ring) + 16384; pr.xmap = &xmap; pr.full = sm->full;
+        const uint32_t dst0 = smem_u32(ring) + (uint32_t)(r0 * 128 + ((c ^ (r0 & 7)) << 4));
+        const uint64_t policy = l2_evict_first();
+        int stage = 0;
+        uint32_t phase = 0;
         bool ok_run = true;
-        const bf16_t *ap[4];
-        uint32_t aok[4];
-        int kb0 = 0, kb1 = 0;
-        auto setup_item = [&](int i) {
-            const GemmItem gi = gemm_my_item(g, i);
-            kb0 = gi.split * g.kb_per_split;
-            kb1 = kb0 + g.kb_per_split;
-            if (kb1 > n_kb) kb1 = n_kb;
-#pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                const int tr = r0 + 32 * i;
-                const bf16_t *base = g.a[0];
-                int m;
-                if (g.epi == EPI_SWIGLU) {             // tile rows 0-63: gate rows, 64-127: the up rows of the same indices
-                    m = gi.row0 + (tr & 63);
-                    if (tr >= 64) base = g.a_up;
-                } else {
-                    m = gi.row0 + tr;
-                }
-                aok[i] = m < gi.row_end ? 16u : 0u;
-                if (m >= gi.row_end) m = gi.row_end - 1;
-                int row = m;
-                if (g.row_ids) {
-                    int id = g.row_ids[m];
-                    if ((unsigned)id >= (unsigned)g.V) { atomicOr(g.status, 0x1u); id = 0; }
-                    row = id;
-                } else if (g.n_seg > 1) {
-                    if (row >= g.a_rows[0]) {
-                        row -= g.a_rows[0];
-                        base = g.a[1];
-                        if (row >= g.a_rows[1]) { row -= g.a_rows[1]; base = g.a[2]; }
-                    }
-                }
-                ap[i] = base + (size_t)row * g.lda + (size_t)kb0 * kGemmBK + c * 8;
-            }
-        };
-        // The weights do not depend on the predecessor in the stream: the weight part of the first item's first
-        // stages goes out before waiting for it.
-        const int n_my = gemm_my_items(g, n_items);
         // The gathered head reads its row ids, which a kernel earlier in the same call wrote: that is a real
-        // dependency, so those GEMMs wait for the chain first (and give up the early weight requests below).
+        // dependency, so those GEMMs wait for the chain first. Plain weights depend on nothing in the stream, so
+        // these warps never wait for a predecessor.
         if (g.row_ids) chain_wait();
-        if (n_my > 0) setup_item(0);
-        int pre = 0;
-        for (int kb = kb0; kb < kb1 && pre < S; kb += KA, ++pre) {
-            pr.stage = pre;
-            produce_stage<KA, 1>(g, pr, kb, kb1, ap, aok);
-#pragma unroll
-            for (int i = 0; i < 4; ++i) ap[i] += KA * kGemmBK;
-        }
-        pr.stage = 0;
-        chain_wait();
         for (int i = 0; i < n_my && ok_run; ++i) {
-            if (i > 0) setup_item(i);
-            for (int kb = kb0; kb < kb1; kb += KA) {
-                if (!gemm_wait(sm, &sm->empty[pr.stage], pr.phase ^ 1u, g.wait_limit_ns)) { ok_run = false; break; }
-                if (pr.tma_thread) {   // the X tiles of this stage: their bytes are expected on the stage's barrier
-                    const int nv = kb1 - kb < KA ? kb1 - kb : KA;
-                    mbar_arrive_expect_tx(&sm->full[pr.stage], (uint32_t)(nv * g.NB * 128));
-                }
-                if (pre > 0) {      // weight part already in flight: add the activation part
-                    --pre;
-                    produce_stage<KA, 2>(g, pr, kb, kb1, ap, aok);
-                } else {
-                    produce_stage<KA, 3>(g, pr, kb, kb1, ap, aok);
+            const GemmItem gi = gemm_my_item(g, i);
+            const int kb0 = gi.split * g.kb_per_split, kb1 = min(kb0 + g.kb_per_split, n_kb), n_tiles = tiles_of(gi);
+            const bf16_t *ap[2][4];
+            uint32_t valid[2] = {0u, 0u};                   // bit q: row r0 + 32 q of the tile exists (the others stay stale: their
+#pragma unroll                                              // results are not used)
+            for (int u = 0; u < 2; ++u)
 #pragma unroll
-                    for (int i = 0; i < 4; ++i) ap[i] += KA * kGemmBK;
+                for (int q = 0; q < 4; ++q) {
+                    const int first = g.epi == EPI_SWIGLU ? 0 : u * kGemmTileM;
+                    int r = first + r0 + 32 * q;
+                    if (gi.row0 + r < gi.row_end) valid[u] |= 1u << q;
+                    else r = gi.row_end - gi.row0 - 1;
+                    int row = gi.src0 + r;
+                    if (g.row_ids) {
+                        row = g.row_ids[row];
+                        if ((unsigned)row >= (unsigned)g.V) { atomicOr(g.status, 0x1u); row = 0; }
+                    }
+                    ap[u][q] = (u == 1 && g.epi == EPI_SWIGLU ? g.a_up : g.a[gi.seg]) + (size_t)row * g.lda + (size_t)kb0 * kGemmBK + c * 8;
                 }
-                // this thread's arrival on the stage's barrier fires when its copies above have landed
-                cp_async_arrive(&sm->full[pr.stage]);
-                if (++pr.stage == S) { pr.stage = 0; pr.phase ^= 1u; }
+            for (int kb = kb0; kb < kb1 && ok_run; kb += KA) {
+#pragma unroll
+                for (int u = 0; u < 2; ++u) {
+                    if (u >= n_tiles) break;
+                    if (!gemm_wait(sm, &sm->empty[stage], phase ^ 1u, g.wait_limit_ns)) { ok_run = false; break; }
+                    const uint32_t d = dst0 + (uint32_t)stage * kStage;
+                    if ((kb + KA) * kGemmBK <= g.K && kb + KA <= kb1 && valid[u] == 15u) {      // the common case: plain 16-byte copies
+#pragma unroll
+                        for (int q = 0; q < 4; ++q) {
+                            cp_async16_full_hint<0>(d + (uint32_t)(q * 4096), ap[u][q], policy);
+                            cp_async16_full_hint<128>(d + (uint32_t)(q * 4096 + kGemmTileBytes), ap[u][q], policy);
+                            if (KA == 4) {
+                                cp_async16_full_hint<256>(d + (uint32_t)(q * 4096 + 2 * kGemmTileBytes), ap[u][q], policy);
+                                cp_async16_full_hint<384>(d + (uint32_t)(q * 4096 + 3 * kGemmTileBytes), ap[u][q], policy);
+                            }
+                        }
+                    } else {
+#pragma unroll
+                        for (int q = 0; q < 4; ++q)
+#pragma unroll
+                            for (int j = 0; j < KA; ++j) {
+                                if ((valid[u] >> q & 1u) && kb + j < kb1) {
+                                    // a column beyond K is filled with zeros, nothing is read
+                                    const uint32_t n = (kb + j) * kGemmBK + c * 8 < g.K ? 16u : 0u;
+                                    cp_async16_off_hint<0>(d + (uint32_t)(q * 4096 + j * kGemmTileBytes), n ? ap[u][q] + j * kGemmBK : g.a[0], n, policy);
+                                }
+                            }
+                    }
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) ap[u][q] += KA * kGemmBK;
+                    // this thread's arrival on the stage's barrier fires when its copies above have landed
+                    cp_async_arrive(&sm->full[stage]);
+                    if (++stage == S) { stage = 0; phase ^= 1u; }
+                }
             }
         }
         cp_async_wait_all();
-    } else if (warp == 4) {
-        // ================= MMA issue: one thread
+    } else if (warp == 5) {
+        // ================= X copies: one thread, one tile copy (64 K elements x NB columns) per K block, KA of them a stage
         chain_wait();
         if (lane == 0) {
-            const uint32_t idesc = umma_idesc_bf16(g.NB);
-            int stage = 0;
-            uint32_t phase = 0, tphase[2] = {0, 0};
-            int buf = 0;
+            int xs = 0;
+            uint32_t xphase = 0;
             bool ok_run = true;
-            const int n_my = gemm_my_items(g, n_items);
             for (int i = 0; i < n_my && ok_run; ++i) {
-                const int kb0 = gemm_my_item(g, i).split * g.kb_per_split;
-                int kb1 = kb0 + g.kb_per_split;
-                if (kb1 > n_kb) kb1 = n_kb;
+                const int kb0 = gemm_my_item(g, i).split * g.kb_per_split, kb1 = min(kb0 + g.kb_per_split, n_kb);
+                for (int kb = kb0; kb < kb1; kb += KA) {
+                    if (!gemm_wait(sm, &sm->xempty[xs], xphase ^ 1u, g.wait_limit_ns)) { ok_run = false; break; }
+                    const int nj = min(KA, kb1 - kb);
+                    mbar_arrive_expect_tx(&sm->xfull[xs], (uint32_t)(nj * xblock));
+                    for (int j = 0; j < nj; ++j)
+                        tma_load_2d(smem_u32(xring) + (uint32_t)(xs * xstage + j * xblock), &xmap, (kb + j) * kGemmBK, 0, &sm->xfull[xs]);
+                    if (++xs == SX) { xs = 0; xphase ^= 1u; }
+                }
+            }
+            gemm_drain(sm, sm->xfull, SX, xs, xphase);
+        }
+        __syncwarp();
+    } else if (warp == 4) {
+        // ================= MMA issue: one thread
+        if (lane == 0) {
+            const uint32_t idesc = umma_idesc_bf16(g.NB);
+            int stage = 0, xs = 0, buf = 0;
+            uint32_t phase = 0, xphase = 0, tphase[2] = {0, 0};
+            bool ok_run = true;
+            for (int i = 0; i < n_my && ok_run; ++i) {
+                const GemmItem gi = gemm_my_item(g, i);
+                const int kb0 = gi.split * g.kb_per_split, kb1 = min(kb0 + g.kb_per_split, n_kb), n_tiles = tiles_of(gi);
                 if (!gemm_wait(sm, &sm->tempty[buf], tphase[buf] ^ 1u, g.wait_limit_ns)) break;
                 tc_fence_after_sync();
                 const uint32_t d0 = tmem_base + (uint32_t)(buf * buf_cols);
-                for (int kb = kb0; kb < kb1; kb += KA) {
-                    if (!gemm_wait(sm, &sm->full[stage], phase, g.wait_limit_ns)) { ok_run = false; break; }
-                    fence_proxy_async();          // the copies' shared-memory writes, before the tensor core reads them
-                    tc_fence_after_sync();
+                for (int kb = kb0; kb < kb1 && ok_run; kb += KA) {
+                    ok_run = gemm_wait(sm, &sm->xfull[xs], xphase, g.wait_limit_ns);
+                    const uint32_t sb = umma_desc_lo(smem_u32(xring) + (uint32_t)(xs * xstage));
+                    for (int u = 0; u < n_tiles && ok_run; ++u) {
+                        if (!gemm_wait(sm, &sm->full[stage], phase, g.wait_limit_ns)) { ok_run = false; break; }
+                        fence_proxy_async();          // the copies' shared-memory writes, before the tensor core reads them
+                        tc_fence_after_sync();
+                        const uint32_t sa = umma_desc_lo(smem_u32(ring) + (uint32_t)stage * kStage);
 #pragma unroll
-                    for (int j = 0; j < KA; ++j) {
-                        if (kb + j < kb1) {
-                            const uint32_t sa = smem_u32(ring) + (uint32_t)stage * stage_bytes + (uint32_t)j * kblock_bytes;
-                            const uint32_t sb = sa + 16384;
-#pragma unroll
-                            for (int ks = 0; ks < 4; ++ks)
-                                umma_bf16(d0, umma_smem_desc(sa + ks * 32), umma_smem_desc(sb + ks * 32), idesc,
-                                          (kb + j > kb0) || (ks > 0));
-                        }
+                        for (int j = 0; j < KA; ++j)
+                            if (kb + j < kb1)
+                                umma_kblock(d0 + (uint32_t)(u * sub_cols), sa + (uint32_t)(j * (kGemmTileBytes >> 4)), sb + (uint32_t)(j * (xblock >> 4)),
+                                            idesc, kb + j > kb0);
+                        umma_commit(&sm->empty[stage]);
+                        if (++stage == S) { stage = 0; phase ^= 1u; }
                     }
-                    umma_commit(&sm->empty[stage]);
-                    if (++stage == S) { stage = 0; phase ^= 1u; }
+                    if (!ok_run) break;
+                    umma_commit(&sm->xempty[xs]);
+                    if (++xs == SX) { xs = 0; xphase ^= 1u; }
                 }
                 if (!ok_run) break;
                 umma_commit(&sm->tfull[buf]);
@@ -368,75 +350,81 @@ __global__ void __launch_bounds__(kGemmThreads, 1) skinny_gemm_kernel(const Gemm
         }
         __syncwarp();
     } else {
-        // ================= epilogue: thread = one row of the tile (TMEM lane 32*warp + lane)
+        // ================= epilogue: thread = one row of a tile (TMEM lane 32*warp + lane)
         chain_wait();
         uint32_t tphase[2] = {0, 0};
         int buf = 0;
-        const int n_my = gemm_my_items(g, n_items);
+        const int tr = warp * 32 + lane;
         for (int i = 0; i < n_my; ++i) {
             const GemmItem gi = gemm_my_item(g, i);
-            const int split = gi.split;
             // the 128 epilogue threads agree on the outcome of the wait before any of them moves on
             if (epi_any(!gemm_wait(sm, &sm->tfull[buf], tphase[buf], g.wait_limit_ns))) break;
             tc_fence_after_sync();
-            const int tr = warp * 32 + lane;
-            const int m = g.epi == EPI_SWIGLU ? gi.row0 + (tr & 63) : gi.row0 + tr;
-            const bool m_ok = m < gi.row_end;
             const uint32_t t0 = tmem_base + ((uint32_t)(warp * 32) << 16) + (uint32_t)(buf * buf_cols);
-            uint32_t row_id = (uint32_t)m;
-            if (g.epi == EPI_ARGMAX && g.row_ids && m_ok) {
-                int id = g.row_ids[m];
-                row_id = ((unsigned)id >= (unsigned)g.V) ? 0u : (uint32_t)id;
-            }
-            for (int c0 = 0; c0 < g.NB; c0 += 32) {
-                float v[32];
-                tmem_ld32(t0 + c0, v);
-                if (g.epi == EPI_PARTIAL) {
+            const int m0 = gi.row0 + tr;
+            if (g.epi == EPI_PARTIAL) {
+                const bool m_ok = m0 < gi.row_end;
+                for (int c0 = 0; c0 < g.NB; c0 += 32) {
+                    float v[32];
+                    tmem_ld32(t0 + c0, v);
 #pragma unroll
                     for (int j = 0; j < 16; ++j) {
                         const int r = (c0 >> 1) + j;
-                        if (r < g.R && m_ok) g.partial[((size_t)split * g.R + r) * g.ldp + m] = v[2 * j] + v[2 * j + 1];
+                        if (r < g.R && m_ok) g.partial[((size_t)gi.split * g.R + r) * g.ldp + m0] = v[2 * j] + v[2 * j + 1];
                     }
-                } else if (g.epi == EPI_SWIGLU) {
-                    if (warp >= 2) {
-#pragma unroll
-                        for (int j = 0; j < 16; ++j) sm->exch[tr - 64][j] = v[2 * j] + v[2 * j + 1];
-                    }
-                    bar_sync(1, 128);
-                    if (warp < 2) {
-#pragma unroll
-                        for (int j = 0; j < 16; ++j) {
-                            const int r = (c0 >> 1) + j;
-                            if (r < g.R && m_ok) {
-                                const float gv = v[2 * j] + v[2 * j + 1], uv = sm->exch[tr][j];
-                                const float act = gv / (1.0f + expf(-gv)) * uv;
-                                uint16_t hi, lo;
-                                split_bf16(act, hi, lo);
-                                g.xop_out[(size_t)(2 * r) * g.ld_out + m] = hi;
-                                g.xop_out[(size_t)(2 * r + 1) * g.ld_out + m] = lo;
-                            }
-                        }
-                    }
-                    bar_sync(1, 128);
-                } else {
+                }
+            } else if (g.epi == EPI_SWIGLU) {
+                const bool m_ok = m0 < gi.row_end;
+                for (int c0 = 0; c0 < g.NB; c0 += 32) {
+                    float v[32], u[32];
+                    tmem_ld32(t0 + c0, v);
+                    tmem_ld32(t0 + sub_cols + c0, u);
 #pragma unroll
                     for (int j = 0; j < 16; ++j) {
-                        const int r = (c0 >> 1) + j;           // warp-uniform
-                        if (r < g.R) {
-                            float logit = v[2 * j] + v[2 * j + 1];
-                            if (g.logits && m_ok) g.logits[(size_t)r * g.logits_stride + m] = logit;
-                            if (g.round_bf16) {
-                                const uint16_t b = f32_bf16bits(logit);
-                                if (g.logits_bf16 && m_ok) g.logits_bf16[(size_t)r * g.logits_stride + m] = b;
-                                logit = bf16bits_f32(b);
-                            }
-                            unsigned long long key = m_ok ? argmax_key(logit, row_id) : 0ull;
+                        const int r = (c0 >> 1) + j;
+                        if (r < g.R && m_ok) {
+                            const float gv = v[2 * j] + v[2 * j + 1], uv = u[2 * j] + u[2 * j + 1];
+                            const float act = gv / (1.0f + expf(-gv)) * uv;
+                            uint16_t hi, lo;
+                            split_bf16(act, hi, lo);
+                            g.xop_out[(size_t)(2 * r) * g.ld_out + m0] = hi;
+                            g.xop_out[(size_t)(2 * r + 1) * g.ld_out + m0] = lo;
+                        }
+                    }
+                }
+            } else {
+                const int n_tiles = tiles_of(gi);
+                for (int u = 0; u < n_tiles; ++u) {
+                    const int m = m0 + u * kGemmTileM;
+                    const bool m_ok = m < gi.row_end;
+                    uint32_t row_id = (uint32_t)m;
+                    if (g.row_ids && m_ok) {
+                        int id = g.row_ids[m];
+                        row_id = ((unsigned)id >= (unsigned)g.V) ? 0u : (uint32_t)id;
+                    }
+                    for (int c0 = 0; c0 < g.NB; c0 += 32) {
+                        float v[32];
+                        tmem_ld32(t0 + u * sub_cols + c0, v);
 #pragma unroll
-                            for (int o = 16; o > 0; o >>= 1) {
-                                const unsigned long long other = __shfl_xor_sync(0xffffffffu, key, o);
-                                key = other > key ? other : key;
+                        for (int j = 0; j < 16; ++j) {
+                            const int r = (c0 >> 1) + j;           // warp-uniform
+                            if (r < g.R) {
+                                float logit = v[2 * j] + v[2 * j + 1];
+                                if (g.logits && m_ok) g.logits[(size_t)r * g.logits_stride + m] = logit;
+                                if (g.round_bf16) {
+                                    const uint16_t b = f32_bf16bits(logit);
+                                    if (g.logits_bf16 && m_ok) g.logits_bf16[(size_t)r * g.logits_stride + m] = b;
+                                    logit = bf16bits_f32(b);
+                                }
+                                // the warp's maximum value, then the lowest id that has it (0: no value, never wins)
+                                const uint32_t key = m_ok ? float_order_key(logit) : 0u;
+                                const uint32_t top = __reduce_max_sync(0xffffffffu, key);
+                                const uint32_t id = __reduce_min_sync(0xffffffffu, m_ok && key == top ? row_id : 0xffffffffu);
+                                if (lane == 0) {
+                                    const unsigned long long k = ((unsigned long long)top << 32) | (0xffffffffu - id);
+                                    if (u == 0 || k > sm->kmax[warp][r]) sm->kmax[warp][r] = k;
+                                }
                             }
-                            if (lane == 0) sm->kmax[warp][r] = key;
                         }
                     }
                 }
@@ -483,17 +471,17 @@ inline int tmap_encoder(TmapEncodeFn *out) {
     return 0;
 }
 
-// Tensor map of the activation operand X [NB][ldx] (bf16): tiles of 64 K elements x NB rows, 128-byte
-// swizzle (the layout the MMA reads), zeros beyond K. Returns 0 or a cudaError_t.
-inline int gemm_encode_xmap(CUtensorMap *map, const bf16_t *x, int ldx, int K, int NB) {
+// Tensor map of a row-major bf16 matrix [rows][ld] for copies of 64 K elements x box_rows rows, 128-byte swizzle (the
+// layout the MMA reads), zeros beyond K. Returns 0 or a cudaError_t.
+inline int gemm_encode_map(CUtensorMap *map, const bf16_t *p, long long rows, int ld, int K, int box_rows) {
     TmapEncodeFn encode;
     if (int rc = tmap_encoder(&encode)) return rc;
-    const cuuint64_t dims[2] = {(cuuint64_t)K, (cuuint64_t)NB};
-    const cuuint64_t strides[1] = {(cuuint64_t)ldx * 2};
-    const cuuint32_t box[2] = {(cuuint32_t)kGemmBK, (cuuint32_t)NB};
+    const cuuint64_t dims[2] = {(cuuint64_t)K, (cuuint64_t)rows};
+    const cuuint64_t strides[1] = {(cuuint64_t)ld * 2};
+    const cuuint32_t box[2] = {(cuuint32_t)kGemmBK, (cuuint32_t)box_rows};
     const cuuint32_t estr[2] = {1, 1};
-    CUresult r = encode(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<bf16_t *>(x), dims, strides, box, estr,
-                        CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
+    CUresult r = encode(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<bf16_t *>(p), dims, strides, box, estr,
+                        CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                         CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     return r == CUDA_SUCCESS ? 0 : (int)cudaErrorInvalidValue;
 }
@@ -501,28 +489,27 @@ inline int gemm_encode_xmap(CUtensorMap *map, const bf16_t *x, int ldx, int K, i
 // Launches the GEMM on `stream` with one CTA per SM (fewer when there are fewer work items).
 // Returns the cudaError_t of the launch.
 inline int skinny_gemm_launch(GemmArgs g, int n_sm, int smem_optin, cudaStream_t stream, TmapCache *cache) {
-    const int avail = smem_optin - 1024 - (int)sizeof(GemmSmem);
-    const int kbb = gemm_kblock_bytes(g.NB);
-    // blocks per stage: as many as still leave a ring of three stages
-    int ka = g.force_ka > 0 ? g.force_ka : (avail / (4 * kbb) >= 3 ? 4 : avail / (2 * kbb) >= 3 ? 2 : 1);
-    int stages = avail / (ka * kbb);
+    const int avail = smem_optin - (int)sizeof(GemmSmem);
+    // K blocks per stage: four where a ring of three weight stages then still fits; X in flight for the latency of L2
+    // under a full HBM stream, the rest of the memory for the weights
+    const int ka = g.NB <= 32 ? 4 : 2, xstage = ka * g.NB * 128, wstage = ka * kGemmTileBytes;
+    const int want = ((g.epi == EPI_PARTIAL ? 96 : 64) * 1024 + xstage - 1) / xstage;
+    g.n_xstages = ka == 4 ? 2 : want < 2 ? 2 : want > kGemmMaxXStages ? kGemmMaxXStages : want;
+    int stages = (avail - g.n_xstages * xstage) / wstage;
     if (stages > kGemmMaxStages) stages = kGemmMaxStages;
     if (stages < 3) return (int)cudaErrorInvalidConfiguration;
     g.n_stages = stages;
-    const size_t smem = 1024 + (size_t)stages * ka * kbb + sizeof(GemmSmem);
-    const int tile_rows = gemm_tile_rows(g.epi);
-    const int n_items = ((g.n_rows + tile_rows - 1) / tile_rows) * g.splits;
+    void (*kern)(const GemmArgs, const CUtensorMap) = ka == 4 ? skinny_gemm_kernel<4> : skinny_gemm_kernel<2>;
+    int &limit = cache->gemm_smem[ka == 4];
+    const size_t smem = (size_t)stages * wstage + (size_t)g.n_xstages * xstage + sizeof(GemmSmem);
+    const int n_items = g.n_ranges * g.splits;
     const int grid = n_items < n_sm ? n_items : n_sm;
-    void (*kern)(const GemmArgs, const CUtensorMap) = ka == 4 ? skinny_gemm_kernel<4> : ka == 2 ? skinny_gemm_kernel<2> : skinny_gemm_kernel<1>;
-    if (ka != 1 && ka != 2 && ka != 4) return (int)cudaErrorInvalidConfiguration;
-    cudaError_t e = cudaSuccess;
-    int &limit = cache->gemm_smem[ka == 4 ? 2 : ka == 2 ? 1 : 0];
-    if ((int)smem > limit) {                  // raise the kernel's shared-memory limit once per footprint
-        e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if ((int)smem > limit) {       // raise the kernel's shared-memory limit once per footprint
+        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return (int)e;
         limit = (int)smem;
     }
-    // the operand's tensor map depends on (address, row pitch, K, rows) only: encoded once, then reused
+    // the activation operand is the library's own: its map depends on (address, row pitch, K, rows) only: encoded once, then reused
     CUtensorMap xmap;
     static_assert(sizeof(CUtensorMap) == 128, "tensor map size");
     TmapEntry *hit = nullptr;
@@ -530,15 +517,13 @@ inline int skinny_gemm_launch(GemmArgs g, int n_sm, int smem_optin, cudaStream_t
         if (cache->e[i].x == g.x && cache->e[i].ldx == g.ldx && cache->e[i].K == g.K && cache->e[i].NB == g.NB) { hit = &cache->e[i]; break; }
     if (hit) std::memcpy(&xmap, hit->map, sizeof(xmap));
     else {
-        int rc = gemm_encode_xmap(&xmap, g.x, g.ldx, g.K, g.NB);
-        if (rc) return rc;
+        if (int rc = gemm_encode_map(&xmap, g.x, g.NB, g.ldx, g.K, g.NB)) return rc;
         const int cap = (int)(sizeof(cache->e) / sizeof(cache->e[0]));
         TmapEntry &dst = cache->e[cache->n < cap ? cache->n++ : (cache->next++ % cap)];
         dst.x = g.x; dst.ldx = g.ldx; dst.K = g.K; dst.NB = g.NB;
         std::memcpy(dst.map, &xmap, sizeof(xmap));
     }
-    e = launch_chained(kern, dim3(grid), dim3(kGemmThreads), smem, stream, g, xmap);
-    return (int)e;
+    return (int)launch_chained(kern, dim3(grid), dim3(kGemmThreads), smem, stream, g, xmap);
 }
 
 }  // namespace fmtp

@@ -43,14 +43,28 @@ __host__ __device__ constexpr uint32_t umma_idesc_bf16(int n) {
            | (static_cast<uint32_t>(128 >> 4) << 24);
 }
 
-// D[tmem] (+)= A[smem] * B[smem]^T, one K = 16 slice; issued by ONE thread.
-__device__ __forceinline__ void umma_bf16(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc, bool accumulate) {
+// The same descriptor in two words: the high one is a constant, the low one moves with the address (16-byte units), so
+// stepping through a tile is one 32-bit add.
+constexpr uint32_t kUmmaDescHi = (1024u >> 4) | (1u << 14) | (2u << 29);
+__device__ __forceinline__ uint32_t umma_desc_lo(uint32_t saddr) { return ((saddr & 0x3ffffu) >> 4) | (1u << 16); }
+
+// D[tmem] (+)= A[smem] * B[smem]^T, one K = 16 slice; issued by ONE thread. What such an MMA costs is its issue: with the
+// 64-bit descriptors formed for every instruction it took 88 cycles whatever N was, with the two words 66 (76 at N = 128;
+// the tensor core itself 65).
+__device__ __forceinline__ void umma_bf16(uint32_t d_tmem, uint32_t a_lo, uint32_t b_lo, uint32_t idesc, bool accumulate) {
     asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "setp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"
-        ::"r"(d_tmem), "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate ? 1u : 0u)
+        "{\n\t.reg .pred p;\n\t.reg .b64 a, b;\n\t"
+        "setp.ne.u32 p, %5, 0;\n\t"
+        "mov.b64 a, {%1, %3};\n\tmov.b64 b, {%2, %3};\n\t"
+        "tcgen05.mma.cta_group::1.kind::f16 [%0], a, b, %4, p;\n\t}"
+        ::"r"(d_tmem), "r"(a_lo), "r"(b_lo), "r"(kUmmaDescHi), "r"(idesc), "r"(accumulate ? 1u : 0u)
         : "memory");
+}
+// The four slices of one 64-wide K block; without `accumulate` the first one overwrites D.
+__device__ __forceinline__ void umma_kblock(uint32_t d_tmem, uint32_t a_lo, uint32_t b_lo, uint32_t idesc, bool accumulate) {
+    umma_bf16(d_tmem, a_lo, b_lo, idesc, accumulate);
+#pragma unroll
+    for (int ks = 1; ks < 4; ++ks) umma_bf16(d_tmem, a_lo + ks * 2, b_lo + ks * 2, idesc, true);
 }
 // `bar` receives one arrival when every tcgen05.mma this thread issued so far has completed.
 __device__ __forceinline__ void umma_commit(uint64_t *bar) {
