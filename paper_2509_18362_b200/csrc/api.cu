@@ -95,7 +95,7 @@ size_t layout(fmtp_ctx *c, unsigned char *base) {
     s.ssB = cv.take<float>((size_t)c->n_sm * kMaxRows);
     s.ssC = cv.take<float>((size_t)c->n_sm * kMaxRows);
     s.ssD = cv.take<float>((size_t)c->n_sm * kMaxRows);
-    s.att_part = cv.take<float>((size_t)R * sh.n_q_heads * c->max_chunks * (sh.head_dim + 2));
+    s.att_part = cv.take<float>((size_t)R * sh.n_q_heads * c->max_chunks * (sh.head_dim + kPartPad));
     // control block, cleared by one memset before every launch
     cv.off = align_up(cv.off, 256);
     c->ctrl_off = cv.off;
@@ -154,7 +154,7 @@ int configure(fmtp_ctx *c, MegaParams &p, int mode, int B, int M) {
     // attention scratch: the rows' query vectors, then one (o, m, l) buffer per working warp group (the rows of a call
     // are dealt to two groups): [4 warps][8 heads][dh + 2] + 64 words
     size_t attn = (size_t)M * Gq * p.dh * 4 + (size_t)(M > 1 ? 2 : 1) * (4 * 8 * (p.dh + 2) + 64) * 4;
-    size_t mrg = ((size_t)2 * c->max_chunks + (size_t)kConsumerThreads + 64) * 4;      // chunk-merge scratch
+    size_t mrg = ((size_t)2 * c->max_chunks + 4 + (size_t)(4 * kConsumerThreads / p.dh) * (p.dh + kPartPad)) * 4;      // chunk-merge scratch
     if (mrg > attn) attn = mrg;
     size_t actd = (size_t)2 * R * act_stride(mode == 0 ? 2 * p.d : (p.d > p.qdim ? p.d : p.qdim)) * 2;
     size_t actq = (size_t)2 * R * act_stride(p.qdim) * 2;

@@ -17,6 +17,7 @@ constexpr int kProducerRegs = 96;
 constexpr int kConsumerRegs = 200;
 constexpr int kTileRows = 32;        // weight rows per pipeline stage (two 16-row MMA tiles)
 constexpr int kAttnChunk = 64;       // context tokens per attention work item
+constexpr int kPartPad = 4;          // words after a chunk partial's output vector: m, l, two unused (16-byte aligned vectors)
 constexpr int kMaxStages = 8;
 // Second staging level in tensor memory (see the kernel): a fourth warpgroup (one warp of it works) moves every landed
 // 32 KB weight stage from the shared-memory ring into one of eight 64-column slots of the SM's 256 KB tensor memory,
@@ -51,7 +52,7 @@ struct Scratch {
     bf16_t *actO_hi, *actO_lo;        // [R][qp]  attention output
     bf16_t *actF_hi, *actF_lo;        // [R][Fp]  SwiGLU activation
     float *ssA, *ssB, *ssC, *ssD;     // [grid][8] per-CTA partial sums of squares
-    float *att_part;                  // [R][Hq][max_chunks][dh + 2] (o, m, l) per context chunk
+    float *att_part;                  // [R][Hq][max_chunks][dh + kPartPad] (o, m, l) per context chunk
     unsigned long long *keys;         // [max_K or 1][8] argmax keys
     const float *rope_cos, *rope_sin; // [max_ctx][dh/2]
     uint32_t *barrier;                // grid barrier counter
