@@ -1235,30 +1235,29 @@ __device__ __forceinline__ void attention_phase(Cta &c, const KvPtrs &kv, int st
         bf16_t *sk = reinterpret_cast<bf16_t *>(c.ring + (size_t)slot * p.stage_bytes);
         bf16_t *sv = sk + (size_t)kAttnChunk * dh;
 
-        // -- rotated, pre-scaled queries of this KV head (independent of the stage); two elements per thread and
-        // round, all eight loads of a round issued before the first use (they are L2 round trips)
-        for (int i0 = c.tid; i0 < M * Gq * half; i0 += 2 * kConsumerThreads) {
-            float x[2], y[2], cs[2], sn[2];
-            int qi[2], e[2];
+        // -- rotated, pre-scaled queries of this KV head (independent of the stage); four element pairs per thread and round, by
+        // 16-byte loads (they are L2 round trips; four rows of seven heads are two rounds)
+        constexpr int q4 = half / 4;
+        for (int i = c.tid; i < M * Gq * q4; i += kConsumerThreads) {
+            const int qi = i / q4, e = (i - qi * q4) * 4;
+            const int m = qi / Gq, hq = kvh * Gq + (qi - m * Gq);
+            int pos = base + min(m, rows - 1);
+            if (pos >= max_tokens) pos = max_tokens - 1;
+            const float *q = p.s.qkv + (size_t)(b * M + m) * (p.qdim + 2 * p.kvdim) + hq * dh + e;
+            const uint4 xv = ldcg128(q), yv = ldcg128(q + half);
+            const float4 cs = *reinterpret_cast<const float4 *>(p.s.rope_cos + (size_t)pos * half + e);
+            const float4 sn = *reinterpret_cast<const float4 *>(p.s.rope_sin + (size_t)pos * half + e);
+            const float x[4] = {__uint_as_float(xv.x), __uint_as_float(xv.y), __uint_as_float(xv.z), __uint_as_float(xv.w)};
+            const float y[4] = {__uint_as_float(yv.x), __uint_as_float(yv.y), __uint_as_float(yv.z), __uint_as_float(yv.w)};
+            const float cc[4] = {cs.x, cs.y, cs.z, cs.w}, ss[4] = {sn.x, sn.y, sn.z, sn.w};
+            float lo[4], hi[4];
 #pragma unroll
-            for (int u = 0; u < 2; ++u) {
-                const int i = min(i0 + u * kConsumerThreads, M * Gq * half - 1);
-                qi[u] = i / half; e[u] = i - qi[u] * half;
-                const int m = qi[u] / Gq, hq = kvh * Gq + (qi[u] - m * Gq);
-                const int r = b * M + m;
-                int pos = base + min(m, rows - 1);
-                if (pos >= max_tokens) pos = max_tokens - 1;
-                const float *q = p.s.qkv + (size_t)r * (p.qdim + 2 * p.kvdim) + hq * dh;
-                x[u] = ldcg_f32(q + e[u]); y[u] = ldcg_f32(q + e[u] + half);
-                cs[u] = p.s.rope_cos[(size_t)pos * half + e[u]]; sn[u] = p.s.rope_sin[(size_t)pos * half + e[u]];
+            for (int u = 0; u < 4; ++u) {
+                lo[u] = (x[u] * cc[u] - y[u] * ss[u]) * qscale;
+                hi[u] = (y[u] * cc[u] + x[u] * ss[u]) * qscale;
             }
-#pragma unroll
-            for (int u = 0; u < 2; ++u) {
-                if (i0 + u * kConsumerThreads < M * Gq * half) {
-                    qs[qi[u] * dh + e[u]] = (x[u] * cs[u] - y[u] * sn[u]) * qscale;
-                    qs[qi[u] * dh + e[u] + half] = (y[u] * cs[u] + x[u] * sn[u]) * qscale;
-                }
-            }
+            *reinterpret_cast<float4 *>(qs + qi * dh + e) = make_float4(lo[0], lo[1], lo[2], lo[3]);
+            *reinterpret_cast<float4 *>(qs + qi * dh + e + half) = make_float4(hi[0], hi[1], hi[2], hi[3]);
         }
         PROF(c, ATTN * 8 + 3);
         wait_bar(c, &c.misc->full[slot], parity);
