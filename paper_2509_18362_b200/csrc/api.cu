@@ -150,31 +150,45 @@ int configure(fmtp_ctx *c, MegaParams &p, int mode, int B, int M) {
     p.max_ctx = sh.max_ctx;
     p.wait_limit_ns = kDefaultWaitNs;
     p.mode = mode; p.B = B; p.M = M; p.R = B * M;
-    const int R = p.R, Gq = p.Hq / p.Hkv;
-    // attention scratch: the rows' query vectors, then one (o, m, l) buffer per working warp group (the rows of a call
-    // are dealt to two groups): [4 warps][8 heads][dh + 2] + 64 words
-    size_t attn = (size_t)M * Gq * p.dh * 4 + (size_t)(M > 1 ? 2 : 1) * (4 * 8 * (p.dh + 2) + 64) * 4;
-    size_t mrg = ((size_t)2 * c->max_chunks + 4 + (size_t)(4 * kConsumerThreads / p.dh) * (p.dh + kPartPad)) * 4;      // chunk-merge scratch
-    if (mrg > attn) attn = mrg;
-    size_t actd = (size_t)2 * R * act_stride(mode == 0 ? 2 * p.d : (p.d > p.qdim ? p.d : p.qdim)) * 2;
-    size_t actq = (size_t)2 * R * act_stride(p.qdim) * 2;
-    size_t base = attn > actd ? attn : actd;
-    if (actq > base) base = actq;
-    base = align_up(base, 128);
-    size_t fixed = mega_fixed_smem(R);
-    size_t avail = (size_t)c->smem_optin;
-    // the ffn-wide input of the down projection is used once per CTA: it is read from global memory (L2), one
-    // stage ahead, and the shared memory goes to a deeper ring
+    // shared memory of a step with R rows (M per sequence): staging area in bytes, and how many ring stages are left
+    const int Gq = p.Hq / p.Hkv;
+    const size_t avail = (size_t)c->smem_optin;
+    auto plan = [&](int R, int M, size_t *scratch) -> int {
+        // attention scratch: the rows' query vectors, then one (o, m, l) buffer per working warp group (the rows of a call
+        // are dealt to two groups): [4 warps][8 heads][dh + 2] + 64 words
+        size_t attn = (size_t)M * Gq * p.dh * 4 + (size_t)(M > 1 ? 2 : 1) * (4 * 8 * (p.dh + 2) + 64) * 4;
+        size_t mrg = ((size_t)2 * c->max_chunks + 4 + (size_t)(4 * kConsumerThreads / p.dh) * (p.dh + kPartPad)) * 4;      // chunk-merge scratch
+        if (mrg > attn) attn = mrg;
+        size_t actd = (size_t)2 * R * act_stride(mode == 0 ? 2 * p.d : (p.d > p.qdim ? p.d : p.qdim)) * 2;
+        size_t actq = (size_t)2 * R * act_stride(p.qdim) * 2;
+        size_t base = attn > actd ? attn : actd;
+        if (actq > base) base = actq;
+        *scratch = align_up(base, 128);
+        // the ffn-wide input of the down projection is used once per CTA: it is read from global memory (L2), one
+        // stage ahead, and the shared memory goes to a deeper ring
+        const size_t used = mega_fixed_smem(R) + *scratch;
+        const int n = used < avail ? (int)((avail - used) / p.stage_bytes) : 0;
+        return n < kMaxStages ? n : kMaxStages;
+    };
+    const int R = p.R;
+    size_t base = 0;
+    int ns = plan(R, M, &base);
     p.scratch_smem = (int)base;
     // tensor memory as a second staging level: full-width stages only (every K a multiple of the stage width), at most
     // four activation rows, the down projection's slice ring inside the staging area
     p.use_tmem = c->tmem_staging && R <= 4 && p.KC == 512 && p.stage_bytes == kTileRows * 512 * 2 && p.d % 512 == 0 &&
                  p.qdim % 512 == 0 && p.F % 512 == 0 && (size_t)16 * R * 512 <= base;
-    size_t ring_off = fixed + base;
-    if (p.use_tmem) ring_off = align_up(ring_off, 1024) + 1024;        // as mega_smem_bytes lays it out
-    int ns = ring_off < avail ? (int)((avail - ring_off) / p.stage_bytes) : 0;
-    if (ns > kMaxStages) ns = kMaxStages;
+    if (p.use_tmem) {
+        const size_t ring_off = align_up(mega_fixed_smem(R) + base, 1024) + 1024;        // as mega_smem_bytes lays it out
+        ns = ring_off < avail ? (int)((avail - ring_off) / p.stage_bytes) : 0;
+        if (ns > kMaxStages) ns = kMaxStages;
+    }
     if (ns < 2) return FMTP_ESHAPE;
+    if (mode == 0 && M > 1 && !p.use_tmem) {      // later draft steps have one row per sequence: a layout of their own if it is deeper
+        size_t base2 = 0;
+        const int ns2 = plan(B, 1, &base2);
+        if (ns2 > ns) { p.n_stages2 = ns2; p.scratch_smem2 = (int)base2; }
+    }
     p.n_stages = ns;
     p.s = c->s;
     return FMTP_OK;

@@ -68,6 +68,7 @@ struct MegaParams {
     int KC;                           // k elements per pipeline stage
     int n_stages, stage_bytes;        // ring geometry: stages of stage_bytes (32 weight rows x KC elements, or one K/V chunk)
     int scratch_smem;                 // bytes of the per-phase shared scratch region
+    int n_stages2, scratch_smem2;     // the same for a draft's steps after the first when that has more rows; 0: one layout
     int max_chunks;                   // capacity of att_part's chunk dimension
     int max_ctx;                      // rows of the rotary table
     unsigned long long wait_limit_ns; // every device-side wait gives up after this long (2 s outside the self-test)

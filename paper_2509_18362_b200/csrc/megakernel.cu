@@ -58,8 +58,8 @@ enum Kind { PROJ = 0, QKV = 1, OPROJ = 2, GATEUP = 3, DOWN = 4, HEAD = 5, ATTN =
 struct Prog { int step, layer, kind; };
 
 struct Misc {   // small shared-memory block
-    uint64_t full[kMaxStages];
-    uint64_t empty[kMaxStages];
+    uint64_t full[2 * kMaxStages];    // second half: the ring of a draft's later steps (see switch_layout)
+    uint64_t empty[2 * kMaxStages];
     uint64_t tfull[kTmSlots];     // tensor-memory slots: filled by the mover's copies / read out by the four owning warps
     uint64_t tempty[kTmSlots];
     uint64_t tdrain;              // the mover's last copies, before the tensor memory is freed
@@ -110,6 +110,8 @@ struct Cta {
     float *red;            // [2][8 warps][32 rows][R]
     unsigned char *scr;    // per-phase scratch (activation staging / attention)
     unsigned char *ring;
+    uint64_t *full, *empty; // barriers of the ring
+    int n_stages, scr_bytes;
     int cta, grid, tid, warp, lane;
     int R, M;              // activation rows and rows per sequence of the current step (see set_step_rows)
     int slot;              // ring slot of the next stage (same sequence in producer and consumers)
@@ -122,7 +124,7 @@ struct Cta {
 };
 
 __device__ __forceinline__ void next_stage(Cta &c) {
-    if (++c.slot == c.p->n_stages) { c.slot = 0; c.parity ^= 1u; }
+    if (++c.slot == c.n_stages) { c.slot = 0; c.parity ^= 1u; }
 }
 __device__ __forceinline__ void next_tslot(Cta &c) {
     if (++c.tslot == kTmSlots) { c.tslot = 0; c.tparity ^= 1u; }
@@ -396,7 +398,7 @@ __device__ __forceinline__ void produce_phase(Cta &c, int kind, const LayerPtrs 
             const uint32_t parity = c.parity;
             bool ok = true;
             PROF_T0();
-            if (c.lane == 0) ok = wait_bar(c, &c.misc->empty[slot], parity ^ 1u);
+            if (c.lane == 0) ok = wait_bar(c, &c.empty[slot], parity ^ 1u);
             ok = __shfl_sync(0xffffffffu, ok, 0);
             PROF_ACC(c, 2, pw == 0 && c.lane == 0);
             if (!ok) return;   // abort: stop issuing copies
@@ -457,7 +459,7 @@ __device__ __forceinline__ void produce_phase(Cta &c, int kind, const LayerPtrs 
                     }
                 }
             }
-            cp_async_arrive(&c.misc->full[slot]);
+            cp_async_arrive(&c.full[slot]);
             PROF_ACC(c, 3, pw == 0 && c.lane == 0);
             next_stage(c);
         }
@@ -669,7 +671,7 @@ __device__ __forceinline__ void consume_tiles(Cta &c, const int kind, const ActS
         uint32_t xo[8];                                               // TM: where this lane's piece s of a 16 KB tile sits in its row
 #pragma unroll
         for (int s8 = 0; s8 < 8; ++s8) xo[s8] = (uint32_t)(32 * wi + c.lane) * 128u + (((uint32_t)s8 ^ ((uint32_t)c.lane & 7u)) << 4);
-        const bool gfast = !two_sets && !act.in_smem && 16 * R * 512 <= p.scratch_smem;      // the slice ring must fit the staging area
+        const bool gfast = !two_sets && !act.in_smem && 16 * R * 512 <= c.scr_bytes;      // the slice ring must fit the staging area
         // which half of the warps takes a stage depends only on the stage's index within the phase,
         // never on how many stages the CTA has seen before: the summation order of a row must not
         // depend on the batch or on earlier calls
@@ -718,7 +720,7 @@ __device__ __forceinline__ void consume_tiles(Cta &c, const int kind, const ActS
                         tmem_ld32_issue(ta, w0);
                         tmem_ld32_issue(ta + 32, w1);
                     } else {
-                        wait_bar(c, &c.misc->full[slot], c.parity);
+                        wait_bar(c, &c.full[slot], c.parity);
                         PROF_ACC(c, 0, c.tid == 0);
                     }
                     uint4 bq[kCpw];
@@ -774,7 +776,7 @@ __device__ __forceinline__ void consume_tiles(Cta &c, const int kind, const ActS
                         if (c.lane == 0) {
                             // counted before the arrival, so that the count of a use is never written after the slot's next use
                             if (wi == 0) { volatile uint32_t *ud = &c.misc->use_done[slot]; *ud = *ud + 1; }   // see the mover
-                            mbar_arrive(&c.misc->empty[slot]);
+                            mbar_arrive(&c.empty[slot]);
                         }
                     }
                     PROF_ACC(c, 1, c.tid == 0);
@@ -784,7 +786,7 @@ __device__ __forceinline__ void consume_tiles(Cta &c, const int kind, const ActS
                 const int slot = c.slot;
                 const uint32_t parity = c.parity;
                 PROF_T0();
-                wait_bar(c, &c.misc->full[slot], parity);
+                wait_bar(c, &c.full[slot], parity);
                 PROF_ACC(c, 0, c.tid == 0);
 
                 const StageK sk = stage_k(geo, ks);
@@ -836,7 +838,7 @@ __device__ __forceinline__ void consume_tiles(Cta &c, const int kind, const ActS
                     }
                 }
                 __syncwarp();
-                if (c.lane == 0) mbar_arrive(&c.misc->empty[slot]);
+                if (c.lane == 0) mbar_arrive(&c.empty[slot]);
                 PROF_ACC(c, 1, c.tid == 0);
             }
             next_stage(c);
@@ -900,6 +902,24 @@ __device__ __forceinline__ float reduce_partials(const float (&v)[kPartialRegs])
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
     return s;
+}
+
+// A draft call with several extend rows per sequence: step 0 carries B * M rows, whose staged vectors and partial sums
+// leave two to four ring stages, every later step B rows. So the shared memory is laid out anew between them, with a ring
+// of its own barriers: 7B shape, one sequence with up to four extend rows, the later steps stream from six stages
+// instead of two (draft call of three steps 556 -> 502 us). Consumers call this when they enter step 1 (behind a grid
+// barrier: the old layout is not read any more), producers wait for their arrival at the end of step 0 first.
+__device__ __forceinline__ size_t red_bytes(int R) { return ((size_t)2 * kConsumerWarps * kTileRows * R * sizeof(float) + 127) & ~size_t(127); }
+__device__ __forceinline__ void switch_layout(Cta &c) {
+    const MegaParams &p = *c.p;
+    c.scr = reinterpret_cast<unsigned char *>(c.red) + red_bytes(p.B);
+    c.ring = c.scr + p.scratch_smem2;
+    c.n_stages = p.n_stages2;
+    c.scr_bytes = p.scratch_smem2;
+    c.full = c.misc->full + kMaxStages;
+    c.empty = c.misc->empty + kMaxStages;
+    c.slot = 0;
+    c.parity = 0;
 }
 
 // Copies R rows of a hi/lo activation pair from global scratch into the shared staging area.
@@ -1178,7 +1198,7 @@ __device__ __forceinline__ void produce_attention(Cta &c, const KvPtrs &kv, int 
         const int slot = c.slot;
         const uint32_t parity = c.parity;
         bool ok = true;
-        if (c.lane == 0) ok = wait_bar(c, &c.misc->empty[slot], parity ^ 1u);
+        if (c.lane == 0) ok = wait_bar(c, &c.empty[slot], parity ^ 1u);
         ok = __shfl_sync(0xffffffffu, ok, 0);
         if (!ok) return;
         const uint32_t dst0 = smem_u32(c.ring + (size_t)slot * p.stage_bytes);
@@ -1207,7 +1227,7 @@ __device__ __forceinline__ void produce_attention(Cta &c, const KvPtrs &kv, int 
                 }
             }
         }
-        cp_async_arrive(&c.misc->full[slot]);
+        cp_async_arrive(&c.full[slot]);
         next_stage(c);
     }
 }
@@ -1260,7 +1280,7 @@ __device__ __forceinline__ void attention_phase(Cta &c, const KvPtrs &kv, int st
             *reinterpret_cast<float4 *>(qs + qi * dh + e + half) = make_float4(hi[0], hi[1], hi[2], hi[3]);
         }
         PROF(c, ATTN * 8 + 3);
-        wait_bar(c, &c.misc->full[slot], parity);
+        wait_bar(c, &c.full[slot], parity);
         PROF(c, ATTN * 8 + 4);
         // -- positions written earlier in this launch (previous draft steps): from the pages
         {
@@ -1315,7 +1335,7 @@ __device__ __forceinline__ void attention_phase(Cta &c, const KvPtrs &kv, int st
         attn_rows_mma<DH>(c, sk, sv, qs, part, b, kvh, chunk, base, max_tokens, rows);
         bar_sync(1, kConsumerThreads);   // every warp has read what it needs from the stage
         if (c.tid == 0) { volatile uint32_t *ud = &c.misc->use_done[slot]; *ud = *ud + 1; }   // see the mover of the tensor-memory path
-        if (c.warp < kConsumerWarps / 2 && c.lane == 0) mbar_arrive(&c.misc->empty[slot]);
+        if (c.warp < kConsumerWarps / 2 && c.lane == 0) mbar_arrive(&c.empty[slot]);
         next_stage(c);
         bar_sync(1, kConsumerThreads);   // the query / partial scratch is reused by the next item
     }
@@ -1393,9 +1413,13 @@ __global__ void __launch_bounds__(TM ? kTmThreads : kThreads, 1) mega_kernel(con
     c.misc = reinterpret_cast<Misc *>(smem);
     size_t off = (sizeof(Misc) + 127) & ~size_t(127);
     c.red = reinterpret_cast<float *>(smem + off);
-    off += ((size_t)2 * kConsumerWarps * kTileRows * p.R * sizeof(float) + 127) & ~size_t(127);
+    off += red_bytes(p.R);
     c.scr = smem + off;
     off += (size_t)p.scratch_smem;
+    c.full = c.misc->full;
+    c.empty = c.misc->empty;
+    c.n_stages = p.n_stages;
+    c.scr_bytes = p.scratch_smem;
     if (TM) off = (size_t)(((smem_u32(smem) + (uint32_t)off + 1023u) & ~1023u) - smem_u32(smem));   // swizzled tiles: 1024-byte aligned
     c.ring = smem + off;
     c.cta = blockIdx.x;
@@ -1416,9 +1440,9 @@ __global__ void __launch_bounds__(TM ? kTmThreads : kThreads, 1) mega_kernel(con
 #endif
 
     if (c.tid == 0) {
-        for (int i = 0; i < p.n_stages; ++i) {
-            mbar_init(&c.misc->full[i], kProducerWarps * 32);
-            mbar_init(&c.misc->empty[i], kConsumerWarps / 2);   // the four warps that own the stage (or the mover in their place)
+        for (int i = 0; i < 2 * kMaxStages; ++i) {
+            mbar_init(&c.full[i], kProducerWarps * 32);
+            mbar_init(&c.empty[i], kConsumerWarps / 2);   // the four warps that own the stage (or the mover in their place)
         }
         if (TM) {
             for (int i = 0; i < kTmSlots; ++i) {
@@ -1475,7 +1499,7 @@ __global__ void __launch_bounds__(TM ? kTmThreads : kThreads, 1) mega_kernel(con
                     if (g.kind == EMBED || g.kind == MERGE) continue;
                     if (g.kind == ATTN) {      // K/V stages stay in shared memory: skip this CTA's items
                         const int total = attn_total(c, p.kvs[g.layer], g.step);
-                        for (int item = c.cta; item < total; item += c.grid) { if (c.slot + 1 == p.n_stages) ++wraps; next_stage(c); }
+                        for (int item = c.cta; item < total; item += c.grid) { if (c.slot + 1 == c.n_stages) ++wraps; next_stage(c); }
                         continue;
                     }
                     const Geom geo = geom(c, g.kind);
@@ -1503,7 +1527,7 @@ __global__ void __launch_bounds__(TM ? kTmThreads : kThreads, 1) mega_kernel(con
                                 }
                                 __threadfence_block();
                             }
-                            ok = ok && wait_bar_idle(c, &c.misc->full[slot], c.parity) && wait_bar_idle(c, &c.misc->tempty[ts], c.tparity ^ 1u);
+                            ok = ok && wait_bar_idle(c, &c.full[slot], c.parity) && wait_bar_idle(c, &c.misc->tempty[ts], c.tparity ^ 1u);
                             if (!ok) break;
                             fence_proxy_async();          // the copies' shared-memory writes, before the tensor core reads them
                             tc_fence_after_sync();
@@ -1517,12 +1541,12 @@ __global__ void __launch_bounds__(TM ? kTmThreads : kThreads, 1) mega_kernel(con
                             // the stage may be overwritten once the copies have read it: the arrivals of the four warps that
                             // would have read it
 #pragma unroll
-                            for (int q = 0; q < kConsumerWarps / 2; ++q) umma_commit(&c.misc->empty[slot]);
+                            for (int q = 0; q < kConsumerWarps / 2; ++q) umma_commit(&c.empty[slot]);
                             umma_commit(&c.misc->tfull[ts]);
                             c.misc->use_done[slot] = wraps + 1;
                             next_tslot(c);
                         }
-                        if (c.slot + 1 == p.n_stages) ++wraps;
+                        if (c.slot + 1 == c.n_stages) ++wraps;
                         next_stage(c);
                     }
                 }
@@ -1543,6 +1567,10 @@ __global__ void __launch_bounds__(TM ? kTmThreads : kThreads, 1) mega_kernel(con
         Prog g;
         for (prog_begin(p, g); g.kind != DONE; prog_next(p, g)) {
             set_step_rows(c, g.step);
+            if (p.n_stages2 > 0 && g.step == 1 && g.kind == PROJ) {
+                bar_sync(5, kThreads);                // the consumers have left step 0's layout
+                switch_layout(c);
+            }
             if (g.kind == ATTN) produce_attention(c, p.kvs[g.layer], g.step);
             else if (g.kind != EMBED && g.kind != MERGE) produce_phase<TM>(c, g.kind, p.layers[g.layer]);
         }
@@ -1570,6 +1598,10 @@ __global__ void __launch_bounds__(TM ? kTmThreads : kThreads, 1) mega_kernel(con
         ex.to_next_layer = (p.mode == 1) && !last_layer;
         ex.gnext = ex.to_next_layer ? p.layers[g.layer + 1].g_in : p.g_final;
         PROF(c, kind * 8);
+        if (p.n_stages2 > 0 && step == 1 && kind == PROJ) {
+            switch_layout(c);
+            s_hi = reinterpret_cast<bf16_t *>(c.scr);
+        }
         if (kind == ATTN) {
             attention_phase<DH>(c, p.kvs[g.layer], step);
             PROF(c, kind * 8 + 2);
@@ -1744,6 +1776,7 @@ __global__ void __launch_bounds__(TM ? kTmThreads : kThreads, 1) mega_kernel(con
                 if (m != 0ull && orow >= 0) atomicMax(p.s.keys + (size_t)step * kMaxRows + orow, m);
             }
             ex.best = 0ull;
+            if (p.n_stages2 > 0 && step == 0 && p.K > 1) bar_arrive(5, kThreads);      // see switch_layout
         }
         PROF(c, kind * 8 + 2);
         grid_barrier(c);
@@ -1795,10 +1828,16 @@ extern "C" int fmtp_prof_read(unsigned long long *host, size_t bytes) {
 
 size_t mega_smem_bytes(const MegaParams &p) {
     size_t off = (sizeof(Misc) + 127) & ~size_t(127);
+    const size_t first = off;
     off += ((size_t)2 * kConsumerWarps * kTileRows * p.R * sizeof(float) + 127) & ~size_t(127);
     off += (size_t)p.scratch_smem;
     if (p.use_tmem) off = ((off + 1023) & ~size_t(1023)) + 1024;      // the ring starts on a 1024-byte boundary, wherever the base lies
     off += (size_t)p.n_stages * p.stage_bytes;
+    if (p.n_stages2 > 0) {
+        const size_t off2 = first + (((size_t)2 * kConsumerWarps * kTileRows * p.B * sizeof(float) + 127) & ~size_t(127)) +
+                            (size_t)p.scratch_smem2 + (size_t)p.n_stages2 * p.stage_bytes;
+        if (off2 > off) off = off2;
+    }
     return off;
 }
 
