@@ -44,7 +44,7 @@ struct fmtp_ctx {
     long long tmem_launches;
     int tmem_staging;          // the persistent kernel stages weights through tensor memory where the shape allows (env FMTP_TMEM=1)
     // answers that depend on the geometry only, kept so that the hot calls make no CUDA attribute / occupancy query:
-    struct { size_t smem; int grid; } mega_cfg[6];                 // per kernel instantiation: footprint its limit was raised to
+    struct { size_t smem; int grid; } mega_cfg[8];                 // per kernel instantiation: footprint its limit was raised to
     struct { int mode, B, M, G; } group_memo[16];                  // sequences per launch for (mode, B, M)
     int n_group_memo;
     TmapCache tmaps;                                               // tensor maps of the batched path's GEMM operands
@@ -153,13 +153,13 @@ int configure(fmtp_ctx *c, MegaParams &p, int mode, int B, int M) {
     // shared memory of a step with R rows (M per sequence): staging area in bytes, and how many ring stages are left
     const int Gq = p.Hq / p.Hkv;
     const size_t avail = (size_t)c->smem_optin;
-    auto plan = [&](int R, int M, size_t *scratch) -> int {
+    auto plan = [&](int R, int M, bool split, size_t *scratch) -> int {
         // attention scratch: the rows' query vectors, then one (o, m, l) buffer per working warp group (the rows of a call
         // are dealt to two groups): [4 warps][8 heads][dh + 2] + 64 words
         size_t attn = (size_t)M * Gq * p.dh * 4 + (size_t)(M > 1 ? 2 : 1) * (4 * 8 * (p.dh + 2) + 64) * 4;
         size_t mrg = ((size_t)2 * c->max_chunks + 4 + (size_t)(4 * kConsumerThreads / p.dh) * (p.dh + kPartPad)) * 4;      // chunk-merge scratch
         if (mrg > attn) attn = mrg;
-        size_t actd = (size_t)2 * R * act_stride(mode == 0 ? 2 * p.d : (p.d > p.qdim ? p.d : p.qdim)) * 2;
+        size_t actd = (size_t)2 * R * act_stride(mode == 0 && !split ? 2 * p.d : (p.d > p.qdim ? p.d : p.qdim)) * 2;
         size_t actq = (size_t)2 * R * act_stride(p.qdim) * 2;
         size_t base = attn > actd ? attn : actd;
         if (actq > base) base = actq;
@@ -172,13 +172,27 @@ int configure(fmtp_ctx *c, MegaParams &p, int mode, int B, int M) {
     };
     const int R = p.R;
     size_t base = 0;
-    int ns = plan(R, M, &base);
+    int ns = plan(R, M, false, &base);
+    if (mode == 0 && R <= 4 && (p.d + c->n_sm - 1) / c->n_sm <= kTileRows) {
+        // (more than four rows run the double-width stream, at which the batched path is faster: 189 against 247-278 us for
+        // one step of five to seven rows)
+        // restaging half way costs 2 us of the projection; worth it where the ring gets deeper (7B shape, four rows: four
+        // stages instead of two, draft call of three steps 502 -> 489 us)
+        size_t base_split = 0;
+        const int ns_split = plan(R, M, true, &base_split);
+        if (ns_split > ns && ns < 4) { ns = ns_split; base = base_split; p.proj_split = 1; }
+    }
     p.scratch_smem = (int)base;
     // tensor memory as a second staging level: full-width stages only (every K a multiple of the stage width), at most
     // four activation rows, the down projection's slice ring inside the staging area
     p.use_tmem = c->tmem_staging && R <= 4 && p.KC == 512 && p.stage_bytes == kTileRows * 512 * 2 && p.d % 512 == 0 &&
                  p.qdim % 512 == 0 && p.F % 512 == 0 && (size_t)16 * R * 512 <= base;
     if (p.use_tmem) {
+        if (p.proj_split) {                                       // that path stages both vectors at once
+            p.proj_split = 0;
+            ns = plan(R, M, false, &base);
+            p.scratch_smem = (int)base;
+        }
         const size_t ring_off = align_up(mega_fixed_smem(R) + base, 1024) + 1024;        // as mega_smem_bytes lays it out
         ns = ring_off < avail ? (int)((avail - ring_off) / p.stage_bytes) : 0;
         if (ns > kMaxStages) ns = kMaxStages;
@@ -186,7 +200,7 @@ int configure(fmtp_ctx *c, MegaParams &p, int mode, int B, int M) {
     if (ns < 2) return FMTP_ESHAPE;
     if (mode == 0 && M > 1 && !p.use_tmem) {      // later draft steps have one row per sequence: a layout of their own if it is deeper
         size_t base2 = 0;
-        const int ns2 = plan(B, 1, &base2);
+        const int ns2 = plan(B, 1, false, &base2);
         if (ns2 > ns) { p.n_stages2 = ns2; p.scratch_smem2 = (int)base2; }
     }
     p.n_stages = ns;

@@ -68,6 +68,8 @@ struct MegaParams {
     int KC;                           // k elements per pipeline stage
     int n_stages, stage_bytes;        // ring geometry: stages of stage_bytes (32 weight rows x KC elements, or one K/V chunk)
     int scratch_smem;                 // bytes of the per-phase shared scratch region
+    int proj_split;                   // the projection stages its second input vector over the first, half way through its stream:
+                                      // half the staging area, more ring stages (needs at most one tile of rows per CTA)
     int n_stages2, scratch_smem2;     // the same for a draft's steps after the first when that has more rows; 0: one layout
     int max_chunks;                   // capacity of att_part's chunk dimension
     int max_ctx;                      // rows of the rotary table
@@ -107,7 +109,7 @@ int mega_launch(const MegaParams &p, int grid, cudaStream_t stream);
 // grid for this footprint on the current device. The answer depends on (kernel, footprint) only: callers cache it.
 int mega_max_grid(const MegaParams &p, size_t smem_bytes, int *err);
 // Which of the kernel's instantiations (head dimension, more than four activation rows, tensor-memory staging) the
-// parameters select: 0..5.
+// parameters select: 0..7.
 int mega_kernel_index(const MegaParams &p);
 
 // Verification kernel (verify.cu).

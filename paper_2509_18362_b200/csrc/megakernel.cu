@@ -112,6 +112,7 @@ struct Cta {
     unsigned char *ring;
     uint64_t *full, *empty; // barriers of the ring
     int n_stages, scr_bytes;
+    int proj_split;        // the projection's two input vectors are staged one after the other (see MegaParams)
     int cta, grid, tid, warp, lane;
     int R, M;              // activation rows and rows per sequence of the current step (see set_step_rows)
     int slot;              // ring slot of the next stage (same sequence in producer and consumers)
@@ -620,6 +621,29 @@ __device__ __forceinline__ void park(float (&acc)[2][2][4], float (&acd)[2][2][4
         }
 }
 
+// The token embeddings of all rows over the first input vector in the staging area (projection with proj_split).
+__device__ __forceinline__ void restage_embeddings(const Cta &c, bf16_t *a_hi, bf16_t *a_lo, int st) {
+    const MegaParams &p = *c.p;
+    const int per_row = p.d >> 3;
+#pragma unroll 2
+    for (int i = c.tid; i < c.R * per_row; i += kConsumerThreads) {
+        const int r = i / per_row, k = (i - r * per_row) * 8;
+        const uint4 v = ldnc128(p.embed + (size_t)c.misc->tok[r] * p.d + k), g = ldnc128(p.g_enorm + k);
+        const uint32_t vw[4] = {v.x, v.y, v.z, v.w}, gw[4] = {g.x, g.y, g.z, g.w};
+        uint32_t h[4], l[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            uint16_t h0, l0, h1, l1;
+            split_bf16(bf16lo_f32(vw[q]) * bf16lo_f32(gw[q]), h0, l0);
+            split_bf16(bf16hi_f32(vw[q]) * bf16hi_f32(gw[q]), h1, l1);
+            h[q] = (uint32_t)h0 | ((uint32_t)h1 << 16);
+            l[q] = (uint32_t)l0 | ((uint32_t)l1 << 16);
+        }
+        *reinterpret_cast<uint4 *>(a_hi + (size_t)r * st + k) = make_uint4(h[0], h[1], h[2], h[3]);
+        *reinterpret_cast<uint4 *>(a_lo + (size_t)r * st + k) = make_uint4(l[0], l[1], l[2], l[3]);
+    }
+}
+
 // Runs all tiles of one matrix phase for this CTA and calls epilogue() once per valid (virtual
 // row, activation row), by exactly one thread. The kernel has a single call site per template
 // argument, so the streaming loop exists once in the instruction stream: this kernel is far
@@ -635,7 +659,7 @@ __device__ __forceinline__ void park(float (&acc)[2][2][4], float (&acd)[2][2][4
 // sixteen 16-byte pieces, already in fragment order, come by two tcgen05.ld of 32 registers each (the first eight
 // stages of a phase) or by sixteen conflict-free 128-bit loads from the shared-memory stage (the rest), and the
 // warp's four k chunks of a stage are 8*(j >> 1) + 2*wi + (j & 1), j = 0..3.
-template <bool two_sets, bool TM>
+template <bool two_sets, bool TM, bool SPLIT>
 __device__ __forceinline__ void consume_tiles(Cta &c, const int kind, const ActSrc &act, EpiCtx &ex) {
     const MegaParams &p = *c.p;
     const Geom geo = geom(c, kind);
@@ -702,6 +726,11 @@ __device__ __forceinline__ void consume_tiles(Cta &c, const int kind, const ActS
                 // the second input segment starts: every warp parks the sums of the first (whichever stages of it
                 // the warp owned)
                 park<two_sets>(acc, acd, acc0, acd0);
+                if (SPLIT && c.proj_split) {      // (one tile per CTA) the second input vector takes the place of the first
+                    bar_sync(1, kConsumerThreads);
+                    restage_embeddings(c, reinterpret_cast<bf16_t *>(c.scr), reinterpret_cast<bf16_t *>(c.scr) + (size_t)R * act.stride, act.stride);
+                    bar_sync(1, kConsumerThreads);
+                }
             }
             if (TM) {
                 // the first kTmSlots stages of a phase come through tensor memory (they land while the consumers are still
@@ -793,7 +822,7 @@ __device__ __forceinline__ void consume_tiles(Cta &c, const int kind, const ActS
                 const int nchunk = (sk.klen + 31) >> 5;
                 const uint32_t sb = smem_u32(c.ring + (size_t)slot * p.stage_bytes) + t * 16 + g * rs;
                 const int par = g & 1;                    // odd rows: 64-byte halves swapped
-                const size_t kbase = (size_t)sk.koff;
+                const size_t kbase = (size_t)sk.koff - (SPLIT && kind == PROJ && c.proj_split && ks >= geo.nks_seg ? (size_t)geo.seglen : 0);
                 if (!two_sets && nchunk == 16 && (act.in_smem || gfast)) {
                     // the stage width of the large shapes with at most four activation rows: this warp's chunks
                     // wi, wi + 4, wi + 8, wi + 12 in two batches of two, all loads of a batch issued before its MMAs,
@@ -916,6 +945,7 @@ __device__ __forceinline__ void switch_layout(Cta &c) {
     c.ring = c.scr + p.scratch_smem2;
     c.n_stages = p.n_stages2;
     c.scr_bytes = p.scratch_smem2;
+    c.proj_split = 0;
     c.full = c.misc->full + kMaxStages;
     c.empty = c.misc->empty + kMaxStages;
     c.slot = 0;
@@ -1402,11 +1432,12 @@ __device__ __forceinline__ void merge_phase(Cta &c, const KvPtrs &kv, int step) 
 }
 
 // ---- the kernel --------------------------------------------------------------------------------
-// One instantiation per (more than four activation rows?, head dimension): each contains only the
-// code it runs, which keeps it near the size of the instruction cache.
-template <bool TWO, int DH, bool TM>
+// One instantiation per (more than four activation rows?, head dimension, restaging projection): each contains only the
+// code it runs, which keeps it near the size of the instruction cache (with the restaging in every instantiation a
+// one-row draft call took 467 instead of 462 us).
+template <bool TWO, int DH, bool TM, bool SPLIT>
 __global__ void __launch_bounds__(TM ? kTmThreads : kThreads, 1) mega_kernel(const __grid_constant__ MegaParams p) {
-    static_assert(!(TM && TWO), "tensor-memory staging serves at most four activation rows");
+    static_assert(!(TM && (TWO || SPLIT)) && !(TWO && SPLIT), "tensor-memory staging and restaging serve at most four activation rows");
     extern __shared__ __align__(128) unsigned char smem[];
     Cta c;
     c.p = &p;
@@ -1420,6 +1451,7 @@ __global__ void __launch_bounds__(TM ? kTmThreads : kThreads, 1) mega_kernel(con
     c.empty = c.misc->empty;
     c.n_stages = p.n_stages;
     c.scr_bytes = p.scratch_smem;
+    c.proj_split = p.proj_split;
     if (TM) off = (size_t)(((smem_u32(smem) + (uint32_t)off + 1023u) & ~1023u) - smem_u32(smem));   // swizzled tiles: 1024-byte aligned
     c.ring = smem + off;
     c.cta = blockIdx.x;
@@ -1635,7 +1667,7 @@ __global__ void __launch_bounds__(TM ? kTmThreads : kThreads, 1) mega_kernel(con
         }
 
         // ============ matrix phases: stage the input vector(s) in shared memory ...
-        const int klen = (kind == PROJ) ? 2 * p.d : (kind == OPROJ) ? p.qdim : (kind == DOWN) ? p.F : p.d;
+        const int klen = (kind == PROJ) ? (SPLIT && c.proj_split ? p.d : 2 * p.d) : (kind == OPROJ) ? p.qdim : (kind == DOWN) ? p.F : p.d;
         const int st = ((klen + 31) & ~31) + 32;      // +64 B: rows land in different banks
         bf16_t *a_hi = s_hi, *a_lo = s_hi + (size_t)R * st;
         ActSrc act{a_hi, a_lo, st, true};
@@ -1685,8 +1717,10 @@ __global__ void __launch_bounds__(TM ? kTmThreads : kThreads, 1) mega_kernel(con
                     for (int i = 0; i < 4; ++i) {
                         float e0 = bf16lo_f32(ew[i]), e1 = bf16hi_f32(ew[i]);
                         sqe += e0 * e0 + e1 * e1;
-                        store_split(a_hi, a_lo, (size_t)r * st + p.d + k + 2 * i, e0 * bf16lo_f32(gw[i]));
-                        store_split(a_hi, a_lo, (size_t)r * st + p.d + k + 2 * i + 1, e1 * bf16hi_f32(gw[i]));
+                        if (!SPLIT || !c.proj_split) {
+                            store_split(a_hi, a_lo, (size_t)r * st + p.d + k + 2 * i, e0 * bf16lo_f32(gw[i]));
+                            store_split(a_hi, a_lo, (size_t)r * st + p.d + k + 2 * i + 1, e1 * bf16hi_f32(gw[i]));
+                        }
                     }
                     if (step == 0) {
                         uint4 hv = ldnc128(p.h_last + (size_t)r * p.d + k);
@@ -1754,7 +1788,7 @@ __global__ void __launch_bounds__(TM ? kTmThreads : kThreads, 1) mega_kernel(con
         PROF(c, kind * 8 + 1);
 
         // ============ ... stream the weights ...
-        consume_tiles<TWO, TM>(c, kind, act, ex);
+        consume_tiles<TWO, TM, SPLIT>(c, kind, act, ex);
 
         // ============ ... and publish what the next phase needs besides the vector
         if (kind == PROJ) flush_sq(c, ex.sq, p.s.ssA, nullptr);
@@ -1848,21 +1882,26 @@ size_t mega_fixed_smem(int R) {
 }
 
 namespace {
-const void *kernel_for(int R, int dh, int tm) {
-    if (tm) return dh == 128 ? (const void *)mega_kernel<false, 128, true> : (const void *)mega_kernel<false, 64, true>;
-    if (dh == 128) return R > 4 ? (const void *)mega_kernel<true, 128, false> : (const void *)mega_kernel<false, 128, false>;
-    return R > 4 ? (const void *)mega_kernel<true, 64, false> : (const void *)mega_kernel<false, 64, false>;
+template <int DH>
+const void *kernel_of(int R, int tm, int split) {
+    if (tm) return (const void *)mega_kernel<false, DH, true, false>;
+    if (split) return (const void *)mega_kernel<false, DH, false, true>;
+    return R > 4 ? (const void *)mega_kernel<true, DH, false, false> : (const void *)mega_kernel<false, DH, false, false>;
+}
+const void *kernel_for(const MegaParams &p) {
+    return p.dh == 128 ? kernel_of<128>(p.R, p.use_tmem, p.proj_split) : kernel_of<64>(p.R, p.use_tmem, p.proj_split);
 }
 }  // namespace
 
 int mega_kernel_index(const MegaParams &p) {
     if (p.use_tmem) return 4 + (p.dh == 128 ? 1 : 0);
+    if (p.proj_split) return 6 + (p.dh == 128 ? 1 : 0);
     return (p.dh == 128 ? 2 : 0) + (p.R > 4 ? 1 : 0);
 }
 
 int mega_max_grid(const MegaParams &p, size_t smem_bytes, int *err) {
     int dev = 0, sms = 0, per_sm = 0;
-    const void *fn = kernel_for(p.R, p.dh, p.use_tmem);
+    const void *fn = kernel_for(p);
     cudaError_t e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_bytes);
@@ -1874,7 +1913,7 @@ int mega_max_grid(const MegaParams &p, size_t smem_bytes, int *err) {
 
 int mega_launch(const MegaParams &p, int grid, cudaStream_t stream) {
     size_t smem = mega_smem_bytes(p);
-    const void *fn = kernel_for(p.R, p.dh, p.use_tmem);
+    const void *fn = kernel_for(p);
     void *args[] = {const_cast<MegaParams *>(&p)};
     return (int)cudaLaunchCooperativeKernel(fn, dim3(grid), dim3(p.use_tmem ? kTmThreads : kThreads), args, smem, stream);
 }
