@@ -695,7 +695,7 @@ __device__ __forceinline__ void consume_tiles(Cta &c, const int kind, const ActS
         uint32_t xo[8];                                               // TM: where this lane's piece s of a 16 KB tile sits in its row
 #pragma unroll
         for (int s8 = 0; s8 < 8; ++s8) xo[s8] = (uint32_t)(32 * wi + c.lane) * 128u + (((uint32_t)s8 ^ ((uint32_t)c.lane & 7u)) << 4);
-        const bool gfast = !two_sets && !act.in_smem && 16 * R * 512 <= c.scr_bytes;      // the slice ring must fit the staging area
+        const bool gfast = !act.in_smem && 16 * R * 512 <= c.scr_bytes;      // the slice ring must fit the staging area
         // which half of the warps takes a stage depends only on the stage's index within the phase,
         // never on how many stages the CTA has seen before: the summation order of a row must not
         // depend on the batch or on earlier calls
@@ -823,15 +823,18 @@ __device__ __forceinline__ void consume_tiles(Cta &c, const int kind, const ActS
                 const uint32_t sb = smem_u32(c.ring + (size_t)slot * p.stage_bytes) + t * 16 + g * rs;
                 const int par = g & 1;                    // odd rows: 64-byte halves swapped
                 const size_t kbase = (size_t)sk.koff - (SPLIT && kind == PROJ && c.proj_split && ks >= geo.nks_seg ? (size_t)geo.seglen : 0);
-                if (!two_sets && nchunk == 16 && (act.in_smem || gfast)) {
-                    // the stage width of the large shapes with at most four activation rows: this warp's chunks
+                if (nchunk == 16 && (act.in_smem || gfast)) {
+                    // the stage width of the large shapes: this warp's chunks
                     // wi, wi + 4, wi + 8, wi + 12 in two batches of two, all loads of a batch issued before its MMAs,
                     // nothing predicated (see the producer: this loop sets the stream rate)
-                    uint4 bq[kCpw];
+                    uint4 bq[kCpw], dq[two_sets ? kCpw : 1];
                     if (act.in_smem) {
-                        const uint32_t ab = smem_u32(abase + aoff0 + kbase);
+                        const uint32_t ab = smem_u32(abase + aoff0 + kbase), db = smem_u32(abase + aoff1 + kbase);
 #pragma unroll
-                        for (int j = 0; j < kCpw; ++j) bq[j] = has0 ? lds128_u32(ab + (wi + 4 * j) * 64) : zero;
+                        for (int j = 0; j < kCpw; ++j) {
+                            bq[j] = has0 ? lds128_u32(ab + (wi + 4 * j) * 64) : zero;
+                            if (two_sets) dq[two_sets ? j : 0] = has1 ? lds128_u32(db + (wi + 4 * j) * 64) : zero;
+                        }
                     } else {
                         // request the slices of the next owned stage, then wait for this stage's (requested one owned
                         // stage ago) and read the fragments from the slice ring
@@ -845,7 +848,10 @@ __device__ __forceinline__ void consume_tiles(Cta &c, const int kind, const ActS
                         __syncwarp();
                         const uint32_t sl = slice_slot(stage0 + ks) + (uint32_t)(arow * 512 + ((g & 1) * 4 + t) * 16);
 #pragma unroll
-                        for (int j = 0; j < kCpw; ++j) bq[j] = has0 ? lds128_u32(sl + j * 128) : zero;
+                        for (int j = 0; j < kCpw; ++j) {
+                            bq[j] = has0 ? lds128_u32(sl + j * 128) : zero;
+                            if (two_sets) dq[two_sets ? j : 0] = has1 ? lds128_u32(sl + 4 * 512 + j * 128) : zero;
+                        }
                     }
 #pragma unroll
                     for (int b2 = 0; b2 < 2; ++b2) {
@@ -853,7 +859,9 @@ __device__ __forceinline__ void consume_tiles(Cta &c, const int kind, const ActS
                         Frag f0 = load_frag(sb + (ch ^ par) * 64, rs);
                         Frag f1 = load_frag(sb + ((ch + 4) ^ par) * 64, rs);
                         mma_chunk(acc, f0, bq[2 * b2]);
+                        if (two_sets) mma_chunk(acd, f0, dq[two_sets ? 2 * b2 : 0]);
                         mma_chunk(acc, f1, bq[2 * b2 + 1]);
+                        if (two_sets) mma_chunk(acd, f1, dq[two_sets ? 2 * b2 + 1 : 0]);
                     }
                 } else {
 #pragma unroll 1
