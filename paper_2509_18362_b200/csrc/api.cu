@@ -41,6 +41,7 @@ struct fmtp_ctx {
     BatchedShape bsh;
     BatchedWs bws;
     int batched_min;           // calls with at least this many sequences take the batched path (env FMTP_BATCHED_MIN)
+    int persist_rows;          // a draft call whose step 0 has more rows takes the batched path, whatever its number of sequences
     long long tmem_launches;
     int tmem_staging;          // the persistent kernel stages weights through tensor memory where the shape allows (env FMTP_TMEM=1)
     // answers that depend on the geometry only, kept so that the hot calls make no CUDA attribute / occupancy query:
@@ -248,15 +249,16 @@ int launch_mega(fmtp_ctx *c, MegaParams &p, cudaStream_t st) {
 
 // Sequences per launch for a call of B sequences with M rows each: a call with more rows than one
 // launch takes runs as several launches over groups of whole sequences. The largest group is the
-// one whose input vectors still leave a ring of three stages (two at worst); 0 if even one
-// sequence does not fit.
+// one whose input vectors still leave a ring of three stages (two at worst; two at once in a target step,
+// where a launch streams all layers: 7B width, 4 layers, two sequences of four rows in one launch of two stages
+// 1000 us, in two launches 1232); 0 if even one sequence does not fit.
 int group_size(fmtp_ctx *c, int mode, int B, int M) {
     for (int i = 0; i < c->n_group_memo; ++i)
         if (c->group_memo[i].mode == mode && c->group_memo[i].B == B && c->group_memo[i].M == M) return c->group_memo[i].G;
     int gmax = kMaxRows / M;
     if (gmax > B) gmax = B;
     int G = 0;
-    for (int want = 3; want >= 2 && G == 0; --want)
+    for (int want = mode == 1 ? 2 : 3; want >= 2 && G == 0; --want)
         for (int g = gmax; g >= 1; --g) {
             MegaParams tmp;
             if (configure(c, tmp, mode, g, M) == FMTP_OK && tmp.n_stages >= want) { G = g; break; }
@@ -334,6 +336,10 @@ int fmtp_create(const fmtp_shape *sh, fmtp_ctx **out) {
         const double qd = (double)sh->n_q_heads * sh->head_dim, kvd = (double)sh->n_kv_heads * sh->head_dim;
         const double layer_bytes = 2.0 * (2.0 * sh->d * sh->d + sh->d * (qd + 2 * kvd) + qd * sh->d + 3.0 * sh->d * sh->ffn);
         if (layer_bytes >= 256e6 && c->batched_min > 3) c->batched_min = 3;
+        // more than four rows take a second set of accumulators and a shallow ring in the persistent kernel (7B shape, one
+        // step of five rows: 267 us against 189 on the batched path; two sequences of four extend rows, three steps: 974
+        // against 521)
+        c->persist_rows = layer_bytes >= 256e6 ? 4 : 1 << 30;
     }
     if (const char *v = std::getenv("FMTP_BATCHED_MIN")) { int n = std::atoi(v); if (n >= 1) c->batched_min = n; }
     c->tmem_staging = 0;       // measured slower than the plain ring so far: opt-in
@@ -427,7 +433,7 @@ int fastmtp_draft(fmtp_ctx *c, const fmtp_mtp_w *w, const fmtp_bf16 *h_last, con
     const int Neff = subset ? N : c->shape.vocab;
     const int d = c->shape.d;
     // the persistent kernel takes the call if its sequences are few and the extend rows of a group fit one launch
-    const int G = B < c->batched_min ? group_size(c, 0, B, max_ext) : 0;
+    const int G = B < c->batched_min && (long long)B * max_ext <= c->persist_rows ? group_size(c, 0, B, max_ext) : 0;
     if (G < 1) {
         // groups of up to 64 sequences, every weight streamed once per step and group by the tensor-core GEMM path
         for (int b0 = 0; b0 < B; b0 += kBatchRows) {
