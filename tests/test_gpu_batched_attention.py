@@ -20,9 +20,10 @@ EDGES = [0, 1, 14, 15, 16, 47, 63, 64, 250, 255, 256, 257, 511, 530]
     (64, 64, 6),                                               # two row sets per sequence
     (8, 128, 1), (5, 64, 4),                                   # pages that are not whole 16-token tiles: the 16-byte copies
 ])
-def test_batched_attention_edges(page, dh, M):
+def test_batched_attention_edges(page, dh, M, monkeypatch):
     """One layer over contexts at every tile edge. Cache slots that nothing has written hold NaN: they must not reach any
     result. Tolerances: gpu_util."""
+    monkeypatch.setenv("FMTP_BATCHED_MIN", "1")
     s = replace(I.TINY, head_dim=dh, page_size=page, n_layers=1)
     L = EDGES[:64 // M]
     kv = I.paged_kv(s, L, M, 41)
@@ -57,4 +58,22 @@ def test_batched_attention_edges(page, dh, M):
             assert np.array_equal(Bd.bf16_bits(l1[:, 0]), Bd.bf16_bits(l[:, i]))
             one.advance(1)
         one.close()
+    gpu.close()
+
+
+def test_merge_of_few_and_many_chunks(monkeypatch):
+    """Contexts around 8 and 32 items of 256 tokens, where the chunk merge changes its group size and starts a second group."""
+    s = replace(I.TINY, n_layers=1)
+    L, M = [2040, 2047, 2300, 8185, 8191, 8500], 2
+    kv = I.paged_kv(s, L, M, 51)
+    Wt = I.target_weights(s, 52)
+    gpu = GpuTarget(s, Wt, [kv], max(L) + M)
+    gpu.ctx.close()
+    monkeypatch.setenv("FMTP_BATCHED_MIN", "1")
+    gpu.ctx = Bd.Context(s, max_rows=64, max_K=1, max_ctx=max(L) + M)
+    t = I.token_ids(53, (len(L), M), s.vocab)
+    h, l, _ = gpu.step(t)
+    rh, rl = O.target_forward(s, Wt, t, [copy_kv(kv)])
+    close(h.float().cpu().numpy(), rh, "hidden states")
+    close(l.float().cpu().numpy(), rl, "logits")
     gpu.close()
