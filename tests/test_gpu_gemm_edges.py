@@ -1,8 +1,11 @@
 """Batched draft calls at the edges of the GEMM's tiles, items and operand widths, against the oracle."""
 import pytest
 
+from oracle import fastmtp_oracle as O
 from paper_2509_18362_b200 import inputs as I
+from tests.gpu_util import close, copy_kv
 from tests.test_gpu_draft import check_draft, run_draft_case
+from tests.test_gpu_target import GpuTarget
 
 pytestmark = pytest.mark.gpu
 
@@ -21,3 +24,23 @@ def test_gemm_edges(shape, B, N, monkeypatch):
     monkeypatch.setenv("FMTP_BATCHED_MIN", "1")
     got, ref = run_draft_case(shape, 70 + B, B, [5 * b % 90 for b in range(B)], 2, N, want_logits=False)
     check_draft(got, ref, f"B={B} N={N}")
+
+
+@pytest.mark.parametrize("d", [64, 4096, 4160, 8192, 8256])
+def test_row_kernels_by_width(d, monkeypatch):
+    """Widths at which a thread of the row-wise kernels owns one, two or more groups of columns."""
+    monkeypatch.setenv("FMTP_BATCHED_MIN", "1")
+    s = I.Shape(d=d, n_q_heads=2, n_kv_heads=1, head_dim=64, ffn=80, vocab=300, n_layers=2)
+    B, M = 3, 2
+    kvs = [I.paged_kv(s, [0, 7, 20], M, 91 + l) for l in range(2)]
+    Wt = I.target_weights(s, 90)
+    gpu = GpuTarget(s, Wt, kvs, 32)
+    t = I.token_ids(93, (B, M), s.vocab)
+    h, l, _ = gpu.step(t)
+    rh, rl = O.target_forward(s, Wt, t, [copy_kv(kv) for kv in kvs])
+    close(h.float().cpu().numpy(), rh, "hidden states")
+    close(l.float().cpu().numpy(), rl, "logits")
+    gpu.close()
+    if d <= 4160:                                  # the draft's first kernel too
+        got, ref = run_draft_case(s, 95, 2, [3, 40], 2, 200, want_logits=False)
+        check_draft(got, ref, f"d={d}")
