@@ -106,10 +106,23 @@ __device__ __forceinline__ void load_f32x8(const float *p, float (&v)[8]) {
 template <int U>
 __global__ void __launch_bounds__(kRowThreads) prologue_kernel(const PrologueArgs a) {
     chain_release();
-    chain_wait();
     __shared__ float red[32];
     __shared__ int s_tok;
     const int r = blockIdx.x, tid = threadIdx.x;
+    uint4 gh[U], ge[U];                          // weights, and in step 0 the caller's hidden state: nothing to wait for
+    float h[U][8];
+    if (!a.only_tokens) {
+#pragma unroll
+        for (int q = 0; q < U; ++q) {
+            const int j = (tid + q * kRowThreads) * 8;
+            if (j < a.d) {
+                gh[q] = *reinterpret_cast<const uint4 *>(a.g_h + j);
+                ge[q] = *reinterpret_cast<const uint4 *>(a.g_e + j);
+                if (a.step == 0) unpack_bf16x8(*reinterpret_cast<const uint4 *>(a.h_last + (size_t)r * a.d + j), h[q]);
+            }
+        }
+    }
+    chain_wait();
     if (tid == 0) {
         int tok;
         if (a.step == 0) {
@@ -138,17 +151,13 @@ __global__ void __launch_bounds__(kRowThreads) prologue_kernel(const PrologueArg
         return;
     }
     const bf16_t *erow = a.embed + (size_t)s_tok * a.d;
-    float h[U][8], e[U][8], sh = 0.f, se = 0.f;
-    uint4 gh[U], ge[U];
+    float e[U][8], sh = 0.f, se = 0.f;
 #pragma unroll
     for (int q = 0; q < U; ++q) {
         const int j = (tid + q * kRowThreads) * 8;
         if (j < a.d) {
-            if (a.step == 0) unpack_bf16x8(*reinterpret_cast<const uint4 *>(a.h_last + (size_t)r * a.d + j), h[q]);
-            else load_f32x8(a.hout + (size_t)r * a.d + j, h[q]);
+            if (a.step > 0) load_f32x8(a.hout + (size_t)r * a.d + j, h[q]);
             unpack_bf16x8(*reinterpret_cast<const uint4 *>(erow + j), e[q]);
-            gh[q] = *reinterpret_cast<const uint4 *>(a.g_h + j);
-            ge[q] = *reinterpret_cast<const uint4 *>(a.g_e + j);
         }
     }
 #pragma unroll
@@ -194,11 +203,14 @@ struct PostArgs {
 template <int U>
 __global__ void __launch_bounds__(kRowThreads) post_kernel(const PostArgs a) {
     chain_release();
-    chain_wait();
     __shared__ float red[32];
     const int r = blockIdx.x, tid = threadIdx.x;
     float v[U][8], ss = 0.f;
-    uint4 gn[U];
+    uint4 gn[U];                                 // (weights: nothing to wait for)
+#pragma unroll
+    for (int q = 0; q < U; ++q)
+        if ((tid + q * kRowThreads) * 8 < a.d) gn[q] = *reinterpret_cast<const uint4 *>(a.gain + (tid + q * kRowThreads) * 8);
+    chain_wait();
 #pragma unroll
     for (int q = 0; q < U; ++q) {
         const int j = (tid + q * kRowThreads) * 8;
@@ -208,7 +220,6 @@ __global__ void __launch_bounds__(kRowThreads) post_kernel(const PostArgs a) {
 #pragma unroll
             for (int s = 0; s < kBatchMaxSplits; ++s)
                 if (s < a.splits) load_f32x8(a.partial + ((size_t)s * a.rows + r) * a.ldp + j, part[s]);
-            gn[q] = *reinterpret_cast<const uint4 *>(a.gain + j);
             if (a.residual) load_f32x8(a.x + (size_t)r * a.d + j, v[q]);
             else {
 #pragma unroll
@@ -269,9 +280,9 @@ struct QkvArgs {
     uint32_t *status;
 };
 
+// Positions, rotary factors and the block table are inputs of the call: they are read before the wait for the predecessor.
 __global__ void qkv_finish_kernel(const QkvArgs a) {
     chain_release();
-    chain_wait();
     const int head = blockIdx.x, r = blockIdx.y, e = threadIdx.x, half = a.dh >> 1;
     const int max_tokens = min(a.kv.max_pages * a.page, a.max_ctx);
     const int seq = r / a.geo.M;
@@ -279,14 +290,25 @@ __global__ void qkv_finish_kernel(const QkvArgs a) {
     const int pos_true = geo_pos(a.geo, a.kv, r, &valid);
     const int pos = min(pos_true, max_tokens - 1);
     const int col = head * a.dh;              // q heads, then k heads, then v heads: the GEMM's row order
+    const bool rotate = head < a.Hq + a.Hkv;
+    const float cs = rotate ? a.rope_cos[(size_t)pos * half + e] : 1.f, sn = rotate ? a.rope_sin[(size_t)pos * half + e] : 0.f;
+    int page = head >= a.Hq ? a.kv.block_table[(size_t)seq * a.kv.max_pages + pos / a.page] : 0;
+    chain_wait();
     float lo = 0.f, hi = 0.f;
-    for (int s = 0; s < a.splits; ++s) {
-        const float *pp = a.partial + ((size_t)s * a.rows + r) * a.ldp + col;
-        lo += pp[e];
-        hi += pp[e + half];
+    {
+        float x[kBatchMaxSplits], y[kBatchMaxSplits];
+#pragma unroll
+        for (int s = 0; s < kBatchMaxSplits; ++s)
+            if (s < a.splits) {
+                const float *pp = a.partial + ((size_t)s * a.rows + r) * a.ldp + col;
+                x[s] = pp[e];
+                y[s] = pp[e + half];
+            }
+#pragma unroll
+        for (int s = 0; s < kBatchMaxSplits; ++s)
+            if (s < a.splits) { lo += x[s]; hi += y[s]; }
     }
-    if (head < a.Hq + a.Hkv) {
-        const float cs = a.rope_cos[(size_t)pos * half + e], sn = a.rope_sin[(size_t)pos * half + e];
+    if (rotate) {
         const float x = lo, y = hi;
         lo = x * cs - y * sn;
         hi = y * cs + x * sn;
@@ -306,9 +328,8 @@ __global__ void qkv_finish_kernel(const QkvArgs a) {
         if (head == a.Hq && e == 0) atomicOr(a.status, kDevBadPos);
         return;
     }
-    const bool is_k = head < a.Hq + a.Hkv;
+    const bool is_k = rotate;
     const int kvh = is_k ? head - a.Hq : head - a.Hq - a.Hkv;
-    int page = a.kv.block_table[(size_t)seq * a.kv.max_pages + pos / a.page];
     if ((unsigned)page >= (unsigned)a.kv.num_pages) { atomicOr(a.status, kDevBadPage); page = 0; }
     bf16_t *dst = (is_k ? a.kv.k_pages : a.kv.v_pages) + (((size_t)page * a.Hkv + kvh) * a.page + (pos % a.page)) * a.dh;
     dst[e] = f32_bf16bits(lo);
@@ -819,11 +840,11 @@ __device__ __forceinline__ float merge_chunks(const float *base, int n_chunks, i
 // Block = (head, row), a thread per output element.
 __global__ void attn_merge_kernel(const MergeArgs a) {
     chain_release();
-    chain_wait();
     const int head = blockIdx.x, r = blockIdx.y, j = threadIdx.x;
     const int max_tokens = min(a.kv.max_pages * a.page, a.max_ctx);
     bool valid;
     const int n_ctx = min(geo_pos(a.geo, a.kv, r, &valid), max_tokens - 1) + 1;
+    chain_wait();
     if (!valid) {                // padding row: attention skipped it
         store_hilo(a.xop, a.ld, r, head * a.dh + j, 0.f);
         return;
