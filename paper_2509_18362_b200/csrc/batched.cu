@@ -356,7 +356,7 @@ __global__ void qkv_finish_kernel(const QkvArgs a) {
 // registers, one item ahead.
 // Bound: the K/V stream for one row; the tensor-core issue and the softmax for four. Measured at the 7B shape, before ->
 // now: 64 rows with contexts in [512, 8192] (618 MB) 154 -> 102 us (6.1 TB/s, 0.93 of a plain copy); 16 sequences x 4
-// rows at 2048 (67 MB) 82 -> 35 us, the latency of the two exchanges per block and of the softmax chain (the tensor pipe
+// rows at 2048 (67 MB) 82 -> 30 us, the latency of the two exchanges per block and of the softmax chain (the tensor pipe
 // is 20 % busy).
 //
 // Committed K/V (positions below seq_lens) is immutable during a call, so the first ring stages are requested before the
@@ -411,13 +411,17 @@ __device__ __forceinline__ void ldsm4_trans(uint32_t addr, uint32_t (&r)[4]) {
                  : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(addr) : "memory");
 }
 __device__ __forceinline__ void sts32(uint32_t addr, uint32_t v) { asm volatile("st.shared.u32 [%0], %1;" ::"r"(addr), "r"(v) : "memory"); }
-// Two values as two packed bf16 pairs: their high parts and what is left of them.
+// Two values as two packed bf16 pairs: their high parts and what is left of them (two conversions for the four).
 __device__ __forceinline__ void split2(float a, float b, uint32_t &hi, uint32_t &lo) {
-    uint16_t h0, l0, h1, l1;
-    split_bf16(a, h0, l0);
-    split_bf16(b, h1, l1);
-    hi = (uint32_t)h0 | ((uint32_t)h1 << 16);
-    lo = (uint32_t)l0 | ((uint32_t)l1 << 16);
+    asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(hi) : "f"(b), "f"(a));
+    const float ra = a - bf16lo_f32(hi), rb = b - bf16hi_f32(hi);
+    asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(lo) : "f"(rb), "f"(ra));
+}
+// 2^x for x <= 0 (results below the normal range are zero, as is 2^-inf).
+__device__ __forceinline__ float exp2_fast(float x) {
+    float y;
+    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
 }
 
 template <int DH, int ROWS>
@@ -641,6 +645,7 @@ __global__ void __launch_bounds__(kAttnThreads, 1) attn_kernel(const __grid_cons
         int nrow[ROWS];                                      // visible positions, 0 for a row that does not exist or is padding
 #pragma unroll
         for (int k = 0; k < ROWS; ++k) nrow[k] = it.set * ROWS + k < tval[it.seq] ? row_ctx(tpos[it.seq], it.set * ROWS + k) : 0;
+        const int n_all = row_ctx(tpos[it.seq], it.set * ROWS);          // positions every row of the set sees
         uint32_t qa[ROWS == 1 ? KS : 1][4];
         float m_run[ROWS], l_run[ROWS], o[ROWS][NT][4];      // o: [0],[1] the hi-part products, [2],[3] the lo-part ones
 #pragma unroll
@@ -674,6 +679,7 @@ __global__ void __launch_bounds__(kAttnThreads, 1) attn_kernel(const __grid_cons
             // No branch on a row's visibility: the rows' chains interleave. A row that sees nothing of a block adds zeros; one
             // that does not exist or sees nothing of the chunk computes on whatever is there and is not written.
             float sc[ROWS][4];
+            const bool edge = tw + kAttnBox > n_all;         // some row does not see all of this warp's tokens
 #pragma unroll
             for (int k = 0; k < ROWS; ++k) {
                 float s[2][2][4];                            // [n-tile of 8 tokens][even / odd slices]: four independent chains
@@ -696,7 +702,7 @@ __global__ void __launch_bounds__(kAttnThreads, 1) attn_kernel(const __grid_cons
 #pragma unroll
                     for (int j = 0; j < 2; ++j) {
                         float v = (s[nt][0][j] + s[nt][1][j]) + (s[nt][0][j + 2] + s[nt][1][j + 2]);
-                        if (tw + nt * 8 + kq + j >= nrow[k]) v = -INFINITY;
+                        if (edge && tw + nt * 8 + kq + j >= nrow[k]) v = -INFINITY;
                         sc[k][nt * 2 + j] = v;
                         mx = fmaxf(mx, v);
                     }
@@ -713,10 +719,10 @@ __global__ void __launch_bounds__(kAttnThreads, 1) attn_kernel(const __grid_cons
             for (int k = 0; k < ROWS; ++k) {
                 const float *mk = mx_s + k * 32 + hrow;
                 const float m_new = fmaxf(m_run[k], fmaxf(fmaxf(mk[0], mk[8]), fmaxf(mk[16], mk[24])));     // finite for a row that counts
-                const float corr = exp2f(m_run[k] - m_new);  // 0 on the item's first block (m_run = -inf)
+                const float corr = exp2_fast(m_run[k] - m_new);  // 0 on the item's first block (m_run = -inf)
                 float p[4];
 #pragma unroll
-                for (int i = 0; i < 4; ++i) p[i] = exp2f(sc[k][i] - m_new);
+                for (int i = 0; i < 4; ++i) p[i] = exp2_fast(sc[k][i] - m_new);
                 // each thread keeps its own tokens' share of the sum; the shares are added at the end of the item
                 l_run[k] = l_run[k] * corr + ((p[0] + p[1]) + (p[2] + p[3]));
                 m_run[k] = m_new;
