@@ -351,6 +351,9 @@ __global__ void __launch_bounds__(kGemmThreads, 1) skinny_gemm_kernel(const __gr
         __syncwarp();
     } else {
         // ================= epilogue: thread = one row of a tile (TMEM lane 32*warp + lane)
+        // Four warps, one per scheduler: a chain of one activation row after the other is latency, exposed after the last item.
+        // So rows go in groups of eight or sixteen with one condition per group (64 rows, 3584-wide layer: exponential and
+        // divide 7 -> 5 us, warp maxima of the output head 18 -> 5, partial sums 2.6 -> 1).
         chain_wait();
         uint32_t tphase[2] = {0, 0};
         int buf = 0;
@@ -362,70 +365,109 @@ __global__ void __launch_bounds__(kGemmThreads, 1) skinny_gemm_kernel(const __gr
             tc_fence_after_sync();
             const uint32_t t0 = tmem_base + ((uint32_t)(warp * 32) << 16) + (uint32_t)(buf * buf_cols);
             const int m0 = gi.row0 + tr;
+            const bool m_ok = m0 < gi.row_end;
             if (g.epi == EPI_PARTIAL) {
-                const bool m_ok = m0 < gi.row_end;
-                for (int c0 = 0; c0 < g.NB; c0 += 32) {
+                float *out = g.partial + (size_t)gi.split * g.R * g.ldp + m0;
+                for (int c0 = 0; c0 < g.NB; c0 += 32, out += (size_t)16 * g.ldp) {
                     float v[32];
                     tmem_ld32(t0 + c0, v);
+                    const int nr = g.R - (c0 >> 1);         // activation rows from here on (warp-uniform)
+                    if (m_ok) {
+                        if (nr >= 16) {
 #pragma unroll
-                    for (int j = 0; j < 16; ++j) {
-                        const int r = (c0 >> 1) + j;
-                        if (r < g.R && m_ok) g.partial[((size_t)gi.split * g.R + r) * g.ldp + m0] = v[2 * j] + v[2 * j + 1];
+                            for (int j = 0; j < 16; ++j) out[(size_t)j * g.ldp] = v[2 * j] + v[2 * j + 1];
+                        } else {
+#pragma unroll
+                            for (int j = 0; j < 15; ++j)
+                                if (j < nr) out[(size_t)j * g.ldp] = v[2 * j] + v[2 * j + 1];
+                        }
                     }
+                    __syncwarp();
                 }
             } else if (g.epi == EPI_SWIGLU) {
-                const bool m_ok = m0 < gi.row_end;
-                for (int c0 = 0; c0 < g.NB; c0 += 32) {
+                bf16_t *out = g.xop_out + m0;
+                for (int c0 = 0; c0 < g.NB; c0 += 32, out += (size_t)32 * g.ld_out) {
                     float v[32], u[32];
                     tmem_ld32(t0 + c0, v);
                     tmem_ld32(t0 + sub_cols + c0, u);
+                    const int nr = g.R - (c0 >> 1);
 #pragma unroll
-                    for (int j = 0; j < 16; ++j) {
-                        const int r = (c0 >> 1) + j;
-                        if (r < g.R && m_ok) {
-                            const float gv = v[2 * j] + v[2 * j + 1], uv = u[2 * j] + u[2 * j + 1];
-                            const float act = gv / (1.0f + expf(-gv)) * uv;
-                            uint16_t hi, lo;
-                            split_bf16(act, hi, lo);
-                            g.xop_out[(size_t)(2 * r) * g.ld_out + m0] = hi;
-                            g.xop_out[(size_t)(2 * r + 1) * g.ld_out + m0] = lo;
+                    for (int j0 = 0; j0 < 16; j0 += 8) {
+                        if (j0 >= nr) break;
+                        float e[8], act[8];
+#pragma unroll
+                        for (int j = 0; j < 8; ++j) {
+                            v[j] = v[2 * (j0 + j)] + v[2 * (j0 + j) + 1];
+                            e[j] = 1.0f + expf(-v[j]);
+                        }
+#pragma unroll
+                        for (int j = 0; j < 8; ++j) act[j] = v[j] / e[j] * (u[2 * (j0 + j)] + u[2 * (j0 + j) + 1]);
+                        if (m_ok) {
+#pragma unroll
+                            for (int j = 0; j < 8; ++j)
+                                if (j0 + j < nr) {
+                                    uint16_t hi, lo;
+                                    split_bf16(act[j], hi, lo);
+                                    out[(size_t)(2 * (j0 + j)) * g.ld_out] = hi;
+                                    out[(size_t)(2 * (j0 + j) + 1) * g.ld_out] = lo;
+                                }
                         }
                     }
+                    __syncwarp();
                 }
             } else {
                 const int n_tiles = tiles_of(gi);
                 for (int u = 0; u < n_tiles; ++u) {
                     const int m = m0 + u * kGemmTileM;
-                    const bool m_ok = m < gi.row_end;
+                    const bool in = m < gi.row_end;
                     uint32_t row_id = (uint32_t)m;
-                    if (g.row_ids && m_ok) {
+                    if (g.row_ids && in) {
                         int id = g.row_ids[m];
                         row_id = ((unsigned)id >= (unsigned)g.V) ? 0u : (uint32_t)id;
                     }
                     for (int c0 = 0; c0 < g.NB; c0 += 32) {
                         float v[32];
                         tmem_ld32(t0 + u * sub_cols + c0, v);
+                        const int nr = g.R - (c0 >> 1);
+                        uint32_t top = 0u, top_id = 0u;             // lane j: activation row (c0 >> 1) + j
 #pragma unroll
-                        for (int j = 0; j < 16; ++j) {
-                            const int r = (c0 >> 1) + j;           // warp-uniform
-                            if (r < g.R) {
-                                float logit = v[2 * j] + v[2 * j + 1];
-                                if (g.logits && m_ok) g.logits[(size_t)r * g.logits_stride + m] = logit;
-                                if (g.round_bf16) {
-                                    const uint16_t b = f32_bf16bits(logit);
-                                    if (g.logits_bf16 && m_ok) g.logits_bf16[(size_t)r * g.logits_stride + m] = b;
-                                    logit = bf16bits_f32(b);
-                                }
-                                // the warp's maximum value, then the lowest id that has it (0: no value, never wins)
-                                const uint32_t key = m_ok ? float_order_key(logit) : 0u;
-                                const uint32_t top = __reduce_max_sync(0xffffffffu, key);
-                                const uint32_t id = __reduce_min_sync(0xffffffffu, m_ok && key == top ? row_id : 0xffffffffu);
-                                if (lane == 0) {
-                                    const unsigned long long k = ((unsigned long long)top << 32) | (0xffffffffu - id);
-                                    if (u == 0 || k > sm->kmax[warp][r]) sm->kmax[warp][r] = k;
+                        for (int j0 = 0; j0 < 16; j0 += 8) {
+                            if (j0 >= nr) break;                    // warp-uniform; rows beyond R in the eight are not used
+                            float x[8];
+#pragma unroll
+                            for (int j = 0; j < 8; ++j) x[j] = v[2 * (j0 + j)] + v[2 * (j0 + j) + 1];
+                            if (in && g.logits) {
+                                float *out = g.logits + (size_t)((c0 >> 1) + j0) * g.logits_stride + m;
+#pragma unroll
+                                for (int j = 0; j < 8; ++j)
+                                    if (j0 + j < nr) out[(size_t)j * g.logits_stride] = x[j];
+                            }
+                            if (g.round_bf16) {
+                                uint16_t b[8];
+#pragma unroll
+                                for (int j = 0; j < 8; ++j) { b[j] = f32_bf16bits(x[j]); x[j] = bf16bits_f32(b[j]); }
+                                if (in && g.logits_bf16) {
+                                    bf16_t *out = g.logits_bf16 + (size_t)((c0 >> 1) + j0) * g.logits_stride + m;
+#pragma unroll
+                                    for (int j = 0; j < 8; ++j)
+                                        if (j0 + j < nr) out[(size_t)j * g.logits_stride] = b[j];
                                 }
                             }
+                            // the warp's maximum value, then the lowest id that has it (0: no value, never wins)
+#pragma unroll
+                            for (int j = 0; j < 8; ++j) {
+                                const uint32_t key = in ? float_order_key(x[j]) : 0u;
+                                const uint32_t k = __reduce_max_sync(0xffffffffu, key);
+                                const uint32_t id = __reduce_min_sync(0xffffffffu, in && key == k ? row_id : 0xffffffffu);
+                                if (lane == j0 + j) { top = k; top_id = id; }
+                            }
                         }
+                        if (lane < 16 && lane < nr) {
+                            const unsigned long long k = ((unsigned long long)top << 32) | (0xffffffffu - top_id);
+                            unsigned long long &best = sm->kmax[warp][(c0 >> 1) + lane];
+                            if (u == 0 || k > best) best = k;
+                        }
+                        __syncwarp();
                     }
                 }
             }
