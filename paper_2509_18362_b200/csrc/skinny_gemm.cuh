@@ -9,7 +9,7 @@
 // items (row range, K range). Roles: warps 0-3 epilogue (TMEM -> registers -> global), warp 4 issues
 // the MMAs, warp 5 the TMA tile copies of X, warps 6-13 copy A with 16-byte cp.async, laid out as the MMA's
 // 128-byte-swizzled K-major tiles (64 K elements wide). Accumulators are double buffered in TMEM so the epilogue of one
-// item overlaps the MMAs of the next.
+// item overlaps the MMAs of the next; in the epilogue of the last item the copy warps help.
 //
 // What bounds it. Up to 32 operand columns: HBM (7.5 TB/s between launches' fixed costs). At 64 activation rows the weight
 // bytes in flight: with A and X in one ring, half of the memory held X and 96 KB of weights were requested ahead per SM
@@ -349,73 +349,68 @@ __global__ void __launch_bounds__(kGemmThreads, 1) skinny_gemm_kernel(const __gr
             gemm_wait(sm, &sm->drain, 0, g.wait_limit_ns);
         }
         __syncwarp();
-    } else {
-        // ================= epilogue: thread = one row of a tile (TMEM lane 32*warp + lane)
-        // Four warps, one per scheduler: a chain of one activation row after the other is latency, exposed after the last item.
-        // So rows go in groups of eight or sixteen with one condition per group (64 rows, 3584-wide layer: exponential and
-        // divide 7 -> 5 us, warp maxima of the output head 18 -> 5, partial sums 2.6 -> 1).
+    }
+    unsigned long long (*last_max)[64] = reinterpret_cast<unsigned long long (*)[64]>(ring);     // EPI_ARGMAX: maxima of the last item, per warp quarter
+    if (warp < 4 || warp >= 6) {
+        // ================= epilogue: thread = one row of a tile (TMEM lane 32*(warp % 4) + lane), eight activation rows at a time.
+        // One warp per scheduler would be a chain of latencies (64 rows, 3584-wide layer: 7 us of divides in gate/up, 18 us of
+        // warp maxima in the output head when the rows went one after the other, 5 and 5 us by eights), and after the last item
+        // nothing hides it. So the copy warps, which have nothing left to copy by then, take two thirds of the last item's rows.
         chain_wait();
-        uint32_t tphase[2] = {0, 0};
-        int buf = 0;
-        const int tr = warp * 32 + lane;
-        for (int i = 0; i < n_my; ++i) {
+        const int q = warp & 3, worker = warp < 4 ? 0 : 1 + ((warp - 6) >> 2), tr = q * 32 + lane;
+        for (int i = worker == 0 || n_my == 0 ? 0 : n_my - 1; i < n_my; ++i) {
+            const bool last = i == n_my - 1;
+            const int first = last ? worker * 8 : 0, step = last ? 24 : 8, buf = i & 1;
             const GemmItem gi = gemm_my_item(g, i);
-            // the 128 epilogue threads agree on the outcome of the wait before any of them moves on
-            if (epi_any(!gemm_wait(sm, &sm->tfull[buf], tphase[buf], g.wait_limit_ns))) break;
+            const bool late = !gemm_wait(sm, &sm->tfull[buf], (uint32_t)(i >> 1) & 1u, g.wait_limit_ns);
+            // before another item the 128 epilogue threads agree on the outcome; after the last one there is no barrier but the CTA's
+            if (last ? __any_sync(0xffffffffu, late) : epi_any(late)) break;
             tc_fence_after_sync();
-            const uint32_t t0 = tmem_base + ((uint32_t)(warp * 32) << 16) + (uint32_t)(buf * buf_cols);
+            const uint32_t t0 = tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(buf * buf_cols);
             const int m0 = gi.row0 + tr;
             const bool m_ok = m0 < gi.row_end;
             if (g.epi == EPI_PARTIAL) {
-                float *out = g.partial + (size_t)gi.split * g.R * g.ldp + m0;
-                for (int c0 = 0; c0 < g.NB; c0 += 32, out += (size_t)16 * g.ldp) {
-                    float v[32];
-                    tmem_ld32(t0 + c0, v);
-                    const int nr = g.R - (c0 >> 1);         // activation rows from here on (warp-uniform)
+                for (int r0 = first; r0 < g.R; r0 += step) {
+                    uint32_t v[16];
+                    tmem_ld16_issue(t0 + 2 * r0, v);
+                    tmem_ld_wait();
+                    float *out = g.partial + (size_t)(gi.split * g.R + r0) * g.ldp + m0;
                     if (m_ok) {
-                        if (nr >= 16) {
 #pragma unroll
-                            for (int j = 0; j < 16; ++j) out[(size_t)j * g.ldp] = v[2 * j] + v[2 * j + 1];
-                        } else {
-#pragma unroll
-                            for (int j = 0; j < 15; ++j)
-                                if (j < nr) out[(size_t)j * g.ldp] = v[2 * j] + v[2 * j + 1];
-                        }
+                        for (int j = 0; j < 8; ++j)
+                            if (r0 + j < g.R) out[(size_t)j * g.ldp] = __uint_as_float(v[2 * j]) + __uint_as_float(v[2 * j + 1]);
                     }
                     __syncwarp();
                 }
             } else if (g.epi == EPI_SWIGLU) {
-                bf16_t *out = g.xop_out + m0;
-                for (int c0 = 0; c0 < g.NB; c0 += 32, out += (size_t)32 * g.ld_out) {
-                    float v[32], u[32];
-                    tmem_ld32(t0 + c0, v);
-                    tmem_ld32(t0 + sub_cols + c0, u);
-                    const int nr = g.R - (c0 >> 1);
+                for (int r0 = first; r0 < g.R; r0 += step) {
+                    uint32_t v[16], u[16];
+                    tmem_ld16_issue(t0 + 2 * r0, v);
+                    tmem_ld16_issue(t0 + sub_cols + 2 * r0, u);
+                    tmem_ld_wait();
+                    float gv[8], e[8], act[8];
 #pragma unroll
-                    for (int j0 = 0; j0 < 16; j0 += 8) {
-                        if (j0 >= nr) break;
-                        float e[8], act[8];
+                    for (int j = 0; j < 8; ++j) {
+                        gv[j] = __uint_as_float(v[2 * j]) + __uint_as_float(v[2 * j + 1]);
+                        e[j] = 1.0f + expf(-gv[j]);
+                    }
 #pragma unroll
-                        for (int j = 0; j < 8; ++j) {
-                            v[j] = v[2 * (j0 + j)] + v[2 * (j0 + j) + 1];
-                            e[j] = 1.0f + expf(-v[j]);
-                        }
+                    for (int j = 0; j < 8; ++j) act[j] = gv[j] / e[j] * (__uint_as_float(u[2 * j]) + __uint_as_float(u[2 * j + 1]));
+                    bf16_t *out = g.xop_out + (size_t)(2 * r0) * g.ld_out + m0;
+                    if (m_ok) {
 #pragma unroll
-                        for (int j = 0; j < 8; ++j) act[j] = v[j] / e[j] * (u[2 * (j0 + j)] + u[2 * (j0 + j) + 1]);
-                        if (m_ok) {
-#pragma unroll
-                            for (int j = 0; j < 8; ++j)
-                                if (j0 + j < nr) {
-                                    uint16_t hi, lo;
-                                    split_bf16(act[j], hi, lo);
-                                    out[(size_t)(2 * (j0 + j)) * g.ld_out] = hi;
-                                    out[(size_t)(2 * (j0 + j) + 1) * g.ld_out] = lo;
-                                }
-                        }
+                        for (int j = 0; j < 8; ++j)
+                            if (r0 + j < g.R) {
+                                uint16_t hi, lo;
+                                split_bf16(act[j], hi, lo);
+                                out[(size_t)(2 * j) * g.ld_out] = hi;
+                                out[(size_t)(2 * j + 1) * g.ld_out] = lo;
+                            }
                     }
                     __syncwarp();
                 }
             } else {
+                unsigned long long *best = last ? last_max[q] : sm->kmax[q];
                 const int n_tiles = tiles_of(gi);
                 for (int u = 0; u < n_tiles; ++u) {
                     const int m = m0 + u * kGemmTileM;
@@ -425,56 +420,50 @@ __global__ void __launch_bounds__(kGemmThreads, 1) skinny_gemm_kernel(const __gr
                         int id = g.row_ids[m];
                         row_id = ((unsigned)id >= (unsigned)g.V) ? 0u : (uint32_t)id;
                     }
-                    for (int c0 = 0; c0 < g.NB; c0 += 32) {
-                        float v[32];
-                        tmem_ld32(t0 + u * sub_cols + c0, v);
-                        const int nr = g.R - (c0 >> 1);
-                        uint32_t top = 0u, top_id = 0u;             // lane j: activation row (c0 >> 1) + j
+                    for (int r0 = first; r0 < g.R; r0 += step) {        // rows beyond R of the eight are not used
+                        uint32_t v[16];
+                        tmem_ld16_issue(t0 + u * sub_cols + 2 * r0, v);
+                        tmem_ld_wait();
+                        float x[8];
 #pragma unroll
-                        for (int j0 = 0; j0 < 16; j0 += 8) {
-                            if (j0 >= nr) break;                    // warp-uniform; rows beyond R in the eight are not used
-                            float x[8];
+                        for (int j = 0; j < 8; ++j) x[j] = __uint_as_float(v[2 * j]) + __uint_as_float(v[2 * j + 1]);
+                        if (in && g.logits) {
+                            float *out = g.logits + (size_t)r0 * g.logits_stride + m;
 #pragma unroll
-                            for (int j = 0; j < 8; ++j) x[j] = v[2 * (j0 + j)] + v[2 * (j0 + j) + 1];
-                            if (in && g.logits) {
-                                float *out = g.logits + (size_t)((c0 >> 1) + j0) * g.logits_stride + m;
+                            for (int j = 0; j < 8; ++j)
+                                if (r0 + j < g.R) out[(size_t)j * g.logits_stride] = x[j];
+                        }
+                        if (g.round_bf16) {
+                            uint16_t b[8];
+#pragma unroll
+                            for (int j = 0; j < 8; ++j) { b[j] = f32_bf16bits(x[j]); x[j] = bf16bits_f32(b[j]); }
+                            if (in && g.logits_bf16) {
+                                bf16_t *out = g.logits_bf16 + (size_t)r0 * g.logits_stride + m;
 #pragma unroll
                                 for (int j = 0; j < 8; ++j)
-                                    if (j0 + j < nr) out[(size_t)j * g.logits_stride] = x[j];
-                            }
-                            if (g.round_bf16) {
-                                uint16_t b[8];
-#pragma unroll
-                                for (int j = 0; j < 8; ++j) { b[j] = f32_bf16bits(x[j]); x[j] = bf16bits_f32(b[j]); }
-                                if (in && g.logits_bf16) {
-                                    bf16_t *out = g.logits_bf16 + (size_t)((c0 >> 1) + j0) * g.logits_stride + m;
-#pragma unroll
-                                    for (int j = 0; j < 8; ++j)
-                                        if (j0 + j < nr) out[(size_t)j * g.logits_stride] = b[j];
-                                }
-                            }
-                            // the warp's maximum value, then the lowest id that has it (0: no value, never wins)
-#pragma unroll
-                            for (int j = 0; j < 8; ++j) {
-                                const uint32_t key = in ? float_order_key(x[j]) : 0u;
-                                const uint32_t k = __reduce_max_sync(0xffffffffu, key);
-                                const uint32_t id = __reduce_min_sync(0xffffffffu, in && key == k ? row_id : 0xffffffffu);
-                                if (lane == j0 + j) { top = k; top_id = id; }
+                                    if (r0 + j < g.R) out[(size_t)j * g.logits_stride] = b[j];
                             }
                         }
-                        if (lane < 16 && lane < nr) {
+                        // the warp's maximum value, then the lowest id that has it (0: no value, never wins); lane j keeps row r0 + j
+                        uint32_t top = 0u, top_id = 0u;
+#pragma unroll
+                        for (int j = 0; j < 8; ++j) {
+                            const uint32_t key = in ? float_order_key(x[j]) : 0u;
+                            const uint32_t k = __reduce_max_sync(0xffffffffu, key);
+                            const uint32_t id = __reduce_min_sync(0xffffffffu, in && key == k ? row_id : 0xffffffffu);
+                            if (lane == j) { top = k; top_id = id; }
+                        }
+                        if (lane < 8 && r0 + lane < g.R) {
                             const unsigned long long k = ((unsigned long long)top << 32) | (0xffffffffu - top_id);
-                            unsigned long long &best = sm->kmax[warp][(c0 >> 1) + lane];
-                            if (u == 0 || k > best) best = k;
+                            if (u == 0 || k > best[r0 + lane]) best[r0 + lane] = k;
                         }
                         __syncwarp();
                     }
                 }
             }
             tc_fence_before_sync();
+            if (last) break;
             mbar_arrive(&sm->tempty[buf]);
-            tphase[buf] ^= 1u;
-            buf ^= 1;
             if (g.epi == EPI_ARGMAX) {
                 bar_sync(1, 128);
                 if (tid < g.R && g.keys) {
@@ -488,7 +477,14 @@ __global__ void __launch_bounds__(kGemmThreads, 1) skinny_gemm_kernel(const __gr
         }
     }
     __syncthreads();
-    if (tid == 0 && *reinterpret_cast<volatile uint32_t *>(&sm->abort_flag)) atomicOr(g.status, 0x8u);
+    const bool aborted = *reinterpret_cast<volatile uint32_t *>(&sm->abort_flag) != 0u;
+    if (tid == 0 && aborted) atomicOr(g.status, 0x8u);
+    if (g.epi == EPI_ARGMAX && n_my > 0 && !aborted && tid < g.R && g.keys) {
+        unsigned long long k = last_max[0][tid];
+#pragma unroll
+        for (int w = 1; w < 4; ++w) k = last_max[w][tid] > k ? last_max[w][tid] : k;
+        atomicMax(&g.keys[tid], k);
+    }
     if (warp == 4) {
         tc_fence_after_sync();
         tmem_dealloc(tmem_base, alloc_cols);
