@@ -344,20 +344,20 @@ __global__ void qkv_finish_kernel(const QkvArgs a) {
 //
 // Scores and the weighted sum run on mma.sync.m16n8k16 with the query heads (and the probabilities) as the A operand,
 // rows 0-7 the high bf16 parts of the heads and rows 8-15 the low parts, so both products carry fp32-accurate inputs.
-// Within a group warp w computes the scores of tokens 16w .. 16w+15 of a 64-token block; the warps exchange the block
-// maximum and the probabilities through shared memory, then warp w adds up its quarter of the head dimension over all 64
-// tokens. So an item ends without a merge across warps, and an output row costs 16 registers per thread instead of 64:
-// four rows fit. A row goes through the same operations whatever ROWS is and whatever rows share its item.
+// One row: within a group warp w computes the scores of tokens 16w .. 16w+15 of a 64-token block; the warps exchange the
+// block maximum and the probabilities through shared memory, then warp w adds up its quarter of the head dimension over all
+// 64 tokens. Several rows: one warp per row, all 64 tokens and the whole head dimension, its probabilities never leave
+// its registers. A row goes through the same operations, in the same order, either way and whatever rows share its item.
 //
 // The K/V pool is a stack of page x head-dim tiles: one TMA copy brings 16 tokens of K or V (4 KB at head dim 128) in the
 // 128-byte-swizzled layout ldmatrix reads without bank conflicts. The copies used to be 16-byte cp.async from 128 threads
 // that also read the block table: those reads queued behind the copies, and a block could not be requested before the
 // read of its table entries came back (1.2 us per 32 KB block). Now a warp holds the table entries of a whole item in
 // registers, one item ahead.
-// Bound: the K/V stream for one row; the tensor-core issue and the softmax for four. Measured at the 7B shape, before ->
-// now: 64 rows with contexts in [512, 8192] (618 MB) 154 -> 102 us (6.1 TB/s, 0.93 of a plain copy); 16 sequences x 4
-// rows at 2048 (67 MB) 82 -> 30 us, the latency of the two exchanges per block and of the softmax chain (the tensor pipe
-// is 20 % busy).
+// Bound: the K/V stream for one row; the tensor-core issue, shared-memory reads and the softmax for four. Measured at the
+// 7B shape, before -> now: 64 rows with contexts in [512, 8192] (618 MB) 154 -> 95 us (6.5 TB/s); 16 sequences x 4 rows at
+// 2048 (67 MB) 82 -> 24 us (28 with four rows split over the warps like one: two barriers per block, and the queries
+// re-read from shared memory for every block).
 //
 // Committed K/V (positions below seq_lens) is immutable during a call, so the first ring stages are requested before the
 // wait for the predecessor kernel; blocks with positions this call writes, and the queries, come after it.
@@ -389,14 +389,14 @@ struct AttnSmem {
     static constexpr int BOX = kAttnBox * DH * 2;                // bytes of one copy: [DH / 64][16 tokens][128 bytes]
     static constexpr int VOFF = 4 * BOX;                         // a stage: four K boxes, four V boxes
     static constexpr int STAGE = 8 * BOX;
-    static constexpr int SG = ROWS == 1 ? 3 : 2;                 // stages per group
-    static constexpr int NQ = 2;                                 // items per group whose queries are held
+    static constexpr int SG = 3;                                 // stages per group
+    static constexpr int NQ = ROWS == 1 ? 2 : 1;                 // items per group whose queries are held (they go to registers at once)
     static constexpr int QROW = 16 * DH * 2;                     // room for a row's queries (8 heads, two parts)
-    static constexpr int PROW = 16 * 128;                        // a row's probabilities: 16 operand rows x 64 tokens
+    static constexpr int PROW = ROWS == 1 ? 16 * 128 : 0;        // a row's probabilities: 16 operand rows x 64 tokens
     static constexpr int O_Q = 2 * SG * STAGE;
     static constexpr int O_P = O_Q + 2 * NQ * ROWS * QROW;
-    static constexpr int O_RED = O_P + 2 * ROWS * PROW;          // per group: [ROWS][4 warps][8 heads] maxima, then sums
-    static constexpr int O_BAR = O_RED + 2 * 2 * ROWS * 32 * 4;
+    static constexpr int O_RED = O_P + 2 * PROW;                 // per group, one row: [4 warps][8 heads] maxima, then sums
+    static constexpr int O_BAR = O_RED + (ROWS == 1 ? 2 * 2 * 32 * 4 : 0);
     static constexpr int O_TAB = O_BAR + (2 * (2 * SG + NQ) + 1) * 8;
     static constexpr int BYTES = O_TAB + (4 * kBatchRows + 1) * 4;
     static constexpr int TOTAL = BYTES + 1024;                   // the ring starts on a 1024-byte boundary
@@ -618,153 +618,236 @@ __global__ void __launch_bounds__(kAttnThreads, 1) attn_kernel(const __grid_cons
     // ---- compute side
     const int wi = warp & 3, hrow = lane >> 2, kq = (lane & 3) * 2;
     constexpr int KS = DH / 16;                              // 16-wide slices of the head dimension
-    constexpr int NT = DH / 32;                              // 8-wide tiles of this warp's quarter of the head dimension
-    float *mx_s = reinterpret_cast<float *>(smem + L::O_RED) + grp * 2 * ROWS * 32, *l_s = mx_s + ROWS * 32;
-    // ldmatrix row addresses. K: this warp's tile, tokens as the operand's n. V (transposed): tile s, this warp's dims
+    // ldmatrix row addresses. K: tokens as the operand's n; V (transposed): tokens as its k
     const int ktok = (lane & 7) + ((lane >> 4) << 3), vtok = (lane & 7) + (((lane >> 3) & 1) << 3);
-    const uint32_t kbase = (uint32_t)(wi * L::BOX + ktok * 128), ksw = (uint32_t)(ktok & 7), kpc = (uint32_t)((lane >> 3) & 1);
-    const uint32_t vbase = (uint32_t)(L::VOFF + (wi * NT / 8) * 2048 + vtok * 128), vsw = (uint32_t)(vtok & 7);
-    const uint32_t vpc = (uint32_t)((wi * NT) & 7) + (uint32_t)(lane >> 4);
+    const uint32_t kbase = (uint32_t)(ktok * 128), ksw = (uint32_t)(ktok & 7), kpc = (uint32_t)((lane >> 3) & 1);
+    const uint32_t vbase = (uint32_t)(L::VOFF + vtok * 128), vsw = (uint32_t)(vtok & 7);
     // queries: operand rows 0-7 = high parts, 8-15 = low parts (a head that does not exist repeats the last one: not used)
     const int qh = min(lane & 7, gq - 1);
     const uint32_t qlane = (uint32_t)((((lane >> 3) & 1) * gq + qh) * DH * 2), qsw = (uint32_t)(qh & 7), qpc = (uint32_t)(lane >> 4);
-    // probabilities: [16 operand rows][64 tokens], pieces of 8 tokens swizzled by the row
-    const uint32_t pbase = smem_u32(smem + L::O_P) + (uint32_t)(grp * ROWS * L::PROW);
-    const uint32_t plane = (uint32_t)(((lane & 7) + ((lane >> 3) & 1) * 8) * 128), psw = (uint32_t)(lane & 7), ppc = (uint32_t)(lane >> 4);
-    const uint32_t pst = pbase + (uint32_t)(hrow * 128 + kq * 2);
     AttnItem it;
     it.seq = 0;
     int stage = 0, li = 0;
     uint32_t phase = 0;
+    auto load_q = [&](int row, int slot, uint32_t (&q)[KS][4]) {
+        const uint32_t b = smem_u32(smem + L::O_Q + ((size_t)(grp * NQ + slot) * ROWS + row) * L::QROW) + qlane;
+#pragma unroll
+        for (int ks = 0; ks < KS; ++ks) ldsm4(b + ((((uint32_t)(2 * ks) + qpc) ^ qsw) << 4), q[ks]);
+    };
+    auto load_k = [&](uint32_t sb, int tile, int ks, uint32_t (&k)[4]) {
+        ldsm4(sb + kbase + (uint32_t)(tile * L::BOX + (ks >> 2) * 2048) + ((((uint32_t)(2 * (ks & 3)) + kpc) ^ ksw) << 4), k);
+    };
+    auto load_v = [&](uint32_t sb, int tile, uint32_t half, uint32_t piece, uint32_t (&v)[4]) {    // 16 head dims from 64 half + 8 piece on
+        ldsm4_trans(sb + vbase + (uint32_t)(tile * L::BOX) + half * 2048u + (((piece + (uint32_t)(lane >> 4)) ^ vsw) << 4), v);
+    };
+    // scores of a tile's 16 tokens: thread: head hrow, tokens nt*8 + kq + {0,1} of the tile
+    auto scores = [&](const uint32_t (&q)[KS][4], const uint32_t (&kf)[KS][4], float (&sc)[4]) {
+        float s[2][2][4];                                    // [n-tile of 8 tokens][even / odd slices]: four independent chains
+#pragma unroll
+        for (int i = 0; i < 4; ++i) s[0][0][i] = s[0][1][i] = s[1][0][i] = s[1][1][i] = 0.f;
+#pragma unroll
+        for (int ks = 0; ks < KS; ++ks) {
+            mma_bf16_pure(s[0][ks & 1], q[ks][0], q[ks][1], q[ks][2], q[ks][3], kf[ks][0], kf[ks][1]);
+            mma_bf16_pure(s[1][ks & 1], q[ks][0], q[ks][1], q[ks][2], q[ks][3], kf[ks][2], kf[ks][3]);
+        }
+        // hi-part product in [0],[1], lo-part in [2],[3]
+#pragma unroll
+        for (int nt = 0; nt < 2; ++nt)
+#pragma unroll
+            for (int j = 0; j < 2; ++j) sc[nt * 2 + j] = (s[nt][0][j] + s[nt][1][j]) + (s[nt][0][j + 2] + s[nt][1][j + 2]);
+    };
+    // value rows nothing has written may hold anything: zeros, so that a probability of 0 meets a finite number
+    auto clear_values = [&](int tile, int tokens) {
+        for (int i = lane; i < (kAttnBox - tokens) * (DH / 8); i += 32) {
+            const int tok = tokens + i / (DH / 8), c = i % (DH / 8);
+            *reinterpret_cast<uint4 *>(ring + (size_t)stage * L::STAGE + L::VOFF + tile * L::BOX + (c >> 3) * 2048 + tok * 128 + (c & 7) * 16) =
+                make_uint4(0, 0, 0, 0);
+        }
+        fence_proxy_async();                                 // before a later TMA copy overwrites them
+    };
+
+    if constexpr (ROWS == 1) {
+    constexpr int NT = DH / 32;                              // 8-wide tiles of this warp's quarter of the head dimension
+    float *mx_s = reinterpret_cast<float *>(smem + L::O_RED) + grp * 64, *l_s = mx_s + 32;
+    const uint32_t vhalf = (uint32_t)(wi * NT / 8), vpiece = (uint32_t)((wi * NT) & 7);
+    // probabilities: [16 operand rows][64 tokens], pieces of 8 tokens swizzled by the row
+    const uint32_t pbase = smem_u32(smem + L::O_P) + (uint32_t)(grp * L::PROW);
+    const uint32_t plane = (uint32_t)(((lane & 7) + ((lane >> 3) & 1) * 8) * 128), psw = (uint32_t)(lane & 7), ppc = (uint32_t)(lane >> 4);
+    const uint32_t pst = pbase + (uint32_t)(hrow * 128 + kq * 2);
     for (int item = worker; item < n_items; item += stride) {
         load_item(it, item);
         if (it.n_blk == 0) continue;
         const int slot = li % NQ;
         ++li;
-        const uint32_t qbase = smem_u32(smem + L::O_Q + (size_t)(grp * NQ + slot) * ROWS * L::QROW) + qlane;
-        int nrow[ROWS];                                      // visible positions, 0 for a row that does not exist or is padding
+        uint32_t qa[KS][4];
+        float m_run = -INFINITY, l_run = 0.f, o[NT][4];      // o: [0],[1] the hi-part products, [2],[3] the lo-part ones
 #pragma unroll
-        for (int k = 0; k < ROWS; ++k) nrow[k] = it.set * ROWS + k < tval[it.seq] ? row_ctx(tpos[it.seq], it.set * ROWS + k) : 0;
-        const int n_all = row_ctx(tpos[it.seq], it.set * ROWS);          // positions every row of the set sees
-        uint32_t qa[ROWS == 1 ? KS : 1][4];
-        float m_run[ROWS], l_run[ROWS], o[ROWS][NT][4];      // o: [0],[1] the hi-part products, [2],[3] the lo-part ones
-#pragma unroll
-        for (int k = 0; k < ROWS; ++k) {
-            m_run[k] = -INFINITY; l_run[k] = 0.f;
-#pragma unroll
-            for (int nt = 0; nt < NT; ++nt) o[k][nt][0] = o[k][nt][1] = o[k][nt][2] = o[k][nt][3] = 0.f;
-        }
+        for (int nt = 0; nt < NT; ++nt) o[nt][0] = o[nt][1] = o[nt][2] = o[nt][3] = 0.f;
         for (int blk = 0; blk < it.n_blk; ++blk) {
             wait(&full[stage], phase);
             const uint32_t sb = smem_u32(ring + (size_t)stage * L::STAGE);
             const int tb = it.t0 + blk * kAttnBlk, tw = tb + wi * kAttnBox;
-            if (ROWS == 1 && blk == 0) {
-#pragma unroll
-                for (int ks = 0; ks < KS; ++ks) ldsm4(qbase + ((((uint32_t)(2 * ks) + qpc) ^ qsw) << 4), qa[ks]);
-            }
+            if (blk == 0) load_q(0, slot, qa);
             uint32_t kf[KS][4];
 #pragma unroll
-            for (int ks = 0; ks < KS; ++ks)
-                ldsm4(sb + kbase + (uint32_t)((ks >> 2) * 2048) + ((((uint32_t)(2 * (ks & 3)) + kpc) ^ ksw) << 4), kf[ks]);
+            for (int ks = 0; ks < KS; ++ks) load_k(sb, wi, ks, kf[ks]);
             const int over = it.n_ctx - tw;                  // of this warp's 16 tokens, those that exist
-            if (over > 0 && over < kAttnBox) {
-                // value rows nothing has written may hold anything: zeros, so that a probability of 0 meets a finite number
-                for (int i = lane; i < (kAttnBox - over) * (DH / 8); i += 32) {
-                    const int t = over + i / (DH / 8), c = i % (DH / 8);
-                    *reinterpret_cast<uint4 *>(ring + (size_t)stage * L::STAGE + L::VOFF + wi * L::BOX + (c >> 3) * 2048 + t * 128 + (c & 7) * 16) =
-                        make_uint4(0, 0, 0, 0);
-                }
-                fence_proxy_async();                         // before a later TMA copy overwrites them
+            if (over > 0 && over < kAttnBox) clear_values(wi, over);
+            float sc[4], mx = -INFINITY;
+            scores(qa, kf, sc);
+            const bool edge = over < kAttnBox;
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                if (edge && (i >> 1) * 8 + kq + (i & 1) >= over) sc[i] = -INFINITY;
+                mx = fmaxf(mx, sc[i]);
             }
-            // No branch on a row's visibility: the rows' chains interleave. A row that sees nothing of a block adds zeros; one
-            // that does not exist or sees nothing of the chunk computes on whatever is there and is not written.
-            float sc[ROWS][4];
-            const bool edge = tw + kAttnBox > n_all;         // some row does not see all of this warp's tokens
-#pragma unroll
-            for (int k = 0; k < ROWS; ++k) {
-                float s[2][2][4];                            // [n-tile of 8 tokens][even / odd slices]: four independent chains
-#pragma unroll
-                for (int i = 0; i < 4; ++i) s[0][0][i] = s[0][1][i] = s[1][0][i] = s[1][1][i] = 0.f;
-#pragma unroll
-                for (int ks = 0; ks < KS; ++ks) {
-                    uint32_t q[4];
-                    if (ROWS == 1) {
-#pragma unroll
-                        for (int i = 0; i < 4; ++i) q[i] = qa[ROWS == 1 ? ks : 0][i];
-                    } else ldsm4(qbase + (uint32_t)(k * L::QROW) + ((((uint32_t)(2 * ks) + qpc) ^ qsw) << 4), q);
-                    mma_bf16_pure(s[0][ks & 1], q[0], q[1], q[2], q[3], kf[ks][0], kf[ks][1]);
-                    mma_bf16_pure(s[1][ks & 1], q[0], q[1], q[2], q[3], kf[ks][2], kf[ks][3]);
-                }
-                // thread: head hrow, tokens tw + nt*8 + kq + {0,1}; hi-part product in [0],[1], lo-part in [2],[3]
-                float mx = -INFINITY;
-#pragma unroll
-                for (int nt = 0; nt < 2; ++nt)
-#pragma unroll
-                    for (int j = 0; j < 2; ++j) {
-                        float v = (s[nt][0][j] + s[nt][1][j]) + (s[nt][0][j + 2] + s[nt][1][j + 2]);
-                        if (edge && tw + nt * 8 + kq + j >= nrow[k]) v = -INFINITY;
-                        sc[k][nt * 2 + j] = v;
-                        mx = fmaxf(mx, v);
-                    }
-                mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 1));
-                mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 2));
-                if ((lane & 3) == 0) mx_s[k * 32 + wi * 8 + hrow] = mx;
-            }
-            if (blk == it.n_blk - 1 || ROWS == 1) {          // the queries have been read for the last time (one row: kept in registers)
+            mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 1));
+            mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 2));
+            if ((lane & 3) == 0) mx_s[wi * 8 + hrow] = mx;
+            if (blk == 0) {                                  // the queries are in registers
                 __syncwarp();
-                if (lane == 0 && (ROWS > 1 || blk == 0)) mbar_arrive(&qempty[slot]);
+                if (lane == 0) mbar_arrive(&qempty[slot]);
             }
             bar_sync(1 + grp, 128);
+            const float *mk = mx_s + hrow;
+            const float m_new = fmaxf(m_run, fmaxf(fmaxf(mk[0], mk[8]), fmaxf(mk[16], mk[24])));
+            const float corr = exp2_fast(m_run - m_new);     // 0 on the item's first block (m_run = -inf)
+            float p[4];
 #pragma unroll
-            for (int k = 0; k < ROWS; ++k) {
-                const float *mk = mx_s + k * 32 + hrow;
-                const float m_new = fmaxf(m_run[k], fmaxf(fmaxf(mk[0], mk[8]), fmaxf(mk[16], mk[24])));     // finite for a row that counts
-                const float corr = exp2_fast(m_run[k] - m_new);  // 0 on the item's first block (m_run = -inf)
-                float p[4];
+            for (int i = 0; i < 4; ++i) p[i] = exp2_fast(sc[i] - m_new);
+            // each thread keeps its own tokens' share of the sum; the shares are added at the end of the item
+            l_run = l_run * corr + ((p[0] + p[1]) + (p[2] + p[3]));
+            m_run = m_new;
 #pragma unroll
-                for (int i = 0; i < 4; ++i) p[i] = exp2_fast(sc[k][i] - m_new);
-                // each thread keeps its own tokens' share of the sum; the shares are added at the end of the item
-                l_run[k] = l_run[k] * corr + ((p[0] + p[1]) + (p[2] + p[3]));
-                m_run[k] = m_new;
-#pragma unroll
-                for (int nt = 0; nt < 2; ++nt) {
-                    uint32_t hi, lo;
-                    split2(p[2 * nt], p[2 * nt + 1], hi, lo);
-                    const uint32_t d = pst + (uint32_t)(k * L::PROW) + (((uint32_t)(wi * 2 + nt) ^ (uint32_t)hrow) << 4);
-                    sts32(d, hi);
-                    sts32(d + 1024, lo);
-                }
-                if (__any_sync(0xffffffffu, corr != 1.0f)) {
-#pragma unroll
-                    for (int nt = 0; nt < NT; ++nt) { o[k][nt][0] *= corr; o[k][nt][1] *= corr; o[k][nt][2] *= corr; o[k][nt][3] *= corr; }
-                }
+            for (int nt = 0; nt < 2; ++nt) {
+                uint32_t hi, lo;
+                split2(p[2 * nt], p[2 * nt + 1], hi, lo);
+                const uint32_t d = pst + (((uint32_t)(wi * 2 + nt) ^ (uint32_t)hrow) << 4);
+                sts32(d, hi);
+                sts32(d + 1024, lo);
             }
-            // one row: all value fragments are requested before the barrier; several: tile by tile (registers)
-            constexpr int VB = ROWS == 1 ? 4 : 1;
-            uint32_t vf[VB][NT / 2][4];
-            auto load_v = [&](int s, uint32_t (&v)[NT / 2][4]) {
+            if (__any_sync(0xffffffffu, corr != 1.0f)) {
 #pragma unroll
-                for (int j = 0; j < NT / 2; ++j)
-                    ldsm4_trans(sb + vbase + (uint32_t)(s * L::BOX) + (((vpc + (uint32_t)(2 * j)) ^ vsw) << 4), v[j]);
-            };
-            if (ROWS == 1) {
-#pragma unroll
-                for (int s = 0; s < VB; ++s) if (tb + s * kAttnBox < it.n_ctx) load_v(s, vf[s]);
+                for (int nt = 0; nt < NT; ++nt) { o[nt][0] *= corr; o[nt][1] *= corr; o[nt][2] *= corr; o[nt][3] *= corr; }
             }
+            uint32_t vf[4][NT / 2][4];                       // all value fragments are requested before the barrier
+#pragma unroll
+            for (int s = 0; s < 4; ++s)
+                if (tb + s * kAttnBox < it.n_ctx) {
+#pragma unroll
+                    for (int j = 0; j < NT / 2; ++j) load_v(sb, s, vhalf, vpiece + (uint32_t)(2 * j), vf[s][j]);
+                }
             bar_sync(1 + grp, 128);
 #pragma unroll
             for (int s = 0; s < 4; ++s) {
                 if (tb + s * kAttnBox >= it.n_ctx) continue;
-                if (ROWS > 1) load_v(s, vf[0]);
+                uint32_t pf[4];
+                ldsm4(pbase + plane + ((((uint32_t)(2 * s) + ppc) ^ psw) << 4), pf);
 #pragma unroll
-                for (int k = 0; k < ROWS; ++k) {
-                    uint32_t p[4];
-                    ldsm4(pbase + (uint32_t)(k * L::PROW) + plane + ((((uint32_t)(2 * s) + ppc) ^ psw) << 4), p);
-                    const auto &v = vf[ROWS == 1 ? s : 0];
+                for (int j = 0; j < NT / 2; ++j) {
+                    mma_bf16_pure(o[2 * j], pf[0], pf[1], pf[2], pf[3], vf[s][j][0], vf[s][j][1]);
+                    mma_bf16_pure(o[2 * j + 1], pf[0], pf[1], pf[2], pf[3], vf[s][j][2], vf[s][j][3]);
+                }
+            }
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&empty[stage]);        // this warp has read all it needs from the stage
+            if (++stage == SG) { stage = 0; phase ^= 1u; }
+        }
+        // ---- the chunk's partial
+        l_run += __shfl_xor_sync(0xffffffffu, l_run, 1);
+        l_run += __shfl_xor_sync(0xffffffffu, l_run, 2);
+        if ((lane & 3) == 0) l_s[wi * 8 + hrow] = l_run;
+        bar_sync(1 + grp, 128);
+        if (hrow < gq) {
+            const size_t r = (size_t)it.seq * a.geo.M + it.set;
+            float *out = a.att_part + ((r * a.Hq + (size_t)it.kvh * gq + hrow) * a.max_chunks + it.chunk) * (DH + 2);
 #pragma unroll
-                    for (int j = 0; j < NT / 2; ++j) {
-                        mma_bf16_pure(o[k][2 * j], p[0], p[1], p[2], p[3], v[j][0], v[j][1]);
-                        mma_bf16_pure(o[k][2 * j + 1], p[0], p[1], p[2], p[3], v[j][2], v[j][3]);
+            for (int nt = 0; nt < NT; ++nt)
+                *reinterpret_cast<float2 *>(out + wi * (DH / 4) + nt * 8 + kq) = make_float2(o[nt][0] + o[nt][2], o[nt][1] + o[nt][3]);
+            if (wi == 0 && (lane & 3) == 0) {
+                const float *lk = l_s + hrow;
+                *reinterpret_cast<float2 *>(out + DH) = make_float2(m_run, ((lk[0] + lk[8]) + lk[16]) + lk[24]);
+            }
+        }
+    }
+    } else {
+    // One warp per row: its scores are its own probabilities' operand (an accumulator's lanes are an A operand's), so nothing
+    // is exchanged and the group's warps meet nowhere but at the ring. The other group starts with another warp's
+    // scheduler, so that two rows use all four.
+    static_assert(ROWS == 4, "one row per warp");
+    constexpr int ND = DH / 16;
+    const int row = (wi + 2 * grp) & 3;
+    for (int item = worker; item < n_items; item += stride) {
+        load_item(it, item);
+        if (it.n_blk == 0) continue;
+        const int slot = li % NQ;
+        ++li;
+        const int m = it.set * ROWS + row;
+        const int n = m < tval[it.seq] ? row_ctx(tpos[it.seq], m) : 0;             // visible positions, 0 for a row that does not exist
+        const bool active = n > it.t0;
+        uint32_t qa[KS][4];
+        float m_run = -INFINITY, l_run[4], o[2 * ND][4];     // l_run: by tile of a block
+#pragma unroll
+        for (int s = 0; s < 4; ++s) l_run[s] = 0.f;
+#pragma unroll
+        for (int nt = 0; nt < 2 * ND; ++nt) o[nt][0] = o[nt][1] = o[nt][2] = o[nt][3] = 0.f;
+        for (int blk = 0; blk < it.n_blk; ++blk) {
+            wait(&full[stage], phase);
+            if (blk == 0) {
+                if (active) load_q(row, slot, qa);
+                __syncwarp();
+                if (lane == 0) mbar_arrive(&qempty[slot]);
+            }
+            const uint32_t sb = smem_u32(ring + (size_t)stage * L::STAGE);
+            const int left = n - (it.t0 + blk * kAttnBlk);   // positions of the block that the row sees
+            if (active && left > 0) {
+                float sc[4][4], mx = -INFINITY;
+#pragma unroll
+                for (int s = 0; s < 4; ++s) {                // a tile that was not copied is whatever is there: masked
+                    uint32_t kf[KS][4];
+#pragma unroll
+                    for (int ks = 0; ks < KS; ++ks) load_k(sb, s, ks, kf[ks]);
+                    scores(qa, kf, sc[s]);
+                }
+                const int exist = it.n_ctx - (it.t0 + blk * kAttnBlk);      // positions of the block that any row of the set sees
+                if (exist < kAttnBlk && (exist & (kAttnBox - 1))) { clear_values(exist / kAttnBox, exist & (kAttnBox - 1)); __syncwarp(); }
+                if (left < kAttnBlk) {
+#pragma unroll
+                    for (int s = 0; s < 4; ++s)
+#pragma unroll
+                        for (int i = 0; i < 4; ++i)
+                            if (s * kAttnBox + (i >> 1) * 8 + kq + (i & 1) >= left) sc[s][i] = -INFINITY;
+                }
+#pragma unroll
+                for (int s = 0; s < 4; ++s) mx = fmaxf(mx, fmaxf(fmaxf(sc[s][0], sc[s][1]), fmaxf(sc[s][2], sc[s][3])));
+                mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 1));
+                mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 2));
+                const float m_new = fmaxf(m_run, mx);
+                const float corr = exp2_fast(m_run - m_new);
+                m_run = m_new;
+                if (__any_sync(0xffffffffu, corr != 1.0f)) {
+#pragma unroll
+                    for (int nt = 0; nt < 2 * ND; ++nt) { o[nt][0] *= corr; o[nt][1] *= corr; o[nt][2] *= corr; o[nt][3] *= corr; }
+                }
+                uint32_t pf[4][4];
+#pragma unroll
+                for (int s = 0; s < 4; ++s) {
+                    float p[4];
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) p[i] = exp2_fast(sc[s][i] - m_new);
+                    l_run[s] = l_run[s] * corr + ((p[0] + p[1]) + (p[2] + p[3]));
+                    split2(p[0], p[1], pf[s][0], pf[s][1]);
+                    split2(p[2], p[3], pf[s][2], pf[s][3]);
+                }
+#pragma unroll
+                for (int s = 0; s < 4; ++s) {
+                    if (s * kAttnBox >= left) break;
+#pragma unroll
+                    for (int j = 0; j < ND; ++j) {
+                        uint32_t v[4];
+                        load_v(sb, s, (uint32_t)(j >> 2), (uint32_t)(2 * (j & 3)), v);
+                        mma_bf16_pure(o[2 * j], pf[s][0], pf[s][1], pf[s][2], pf[s][3], v[0], v[1]);
+                        mma_bf16_pure(o[2 * j + 1], pf[s][0], pf[s][1], pf[s][2], pf[s][3], v[2], v[3]);
                     }
                 }
             }
@@ -772,29 +855,22 @@ __global__ void __launch_bounds__(kAttnThreads, 1) attn_kernel(const __grid_cons
             if (lane == 0) mbar_arrive(&empty[stage]);        // this warp has read all it needs from the stage
             if (++stage == SG) { stage = 0; phase ^= 1u; }
         }
-        // ---- the chunk's partial of every row that sees it
+        if (!active) continue;
+        // ---- the chunk's partial of the row
 #pragma unroll
-        for (int k = 0; k < ROWS; ++k) {
-            if (nrow[k] <= it.t0) continue;
-            float lw = l_run[k];
-            lw += __shfl_xor_sync(0xffffffffu, lw, 1);
-            lw += __shfl_xor_sync(0xffffffffu, lw, 2);
-            if ((lane & 3) == 0) l_s[k * 32 + wi * 8 + hrow] = lw;
+        for (int s = 0; s < 4; ++s) {
+            l_run[s] += __shfl_xor_sync(0xffffffffu, l_run[s], 1);
+            l_run[s] += __shfl_xor_sync(0xffffffffu, l_run[s], 2);
         }
-        bar_sync(1 + grp, 128);
-#pragma unroll
-        for (int k = 0; k < ROWS; ++k) {
-            if (nrow[k] <= it.t0 || hrow >= gq) continue;
-            const size_t r = (size_t)it.seq * a.geo.M + it.set * ROWS + k;
+        if (hrow < gq) {
+            const size_t r = (size_t)it.seq * a.geo.M + m;
             float *out = a.att_part + ((r * a.Hq + (size_t)it.kvh * gq + hrow) * a.max_chunks + it.chunk) * (DH + 2);
 #pragma unroll
-            for (int nt = 0; nt < NT; ++nt)
-                *reinterpret_cast<float2 *>(out + wi * (DH / 4) + nt * 8 + kq) = make_float2(o[k][nt][0] + o[k][nt][2], o[k][nt][1] + o[k][nt][3]);
-            if (wi == 0 && (lane & 3) == 0) {
-                const float *lk = l_s + k * 32 + hrow;
-                *reinterpret_cast<float2 *>(out + DH) = make_float2(m_run[k], ((lk[0] + lk[8]) + lk[16]) + lk[24]);
-            }
+            for (int nt = 0; nt < 2 * ND; ++nt)
+                *reinterpret_cast<float2 *>(out + nt * 8 + kq) = make_float2(o[nt][0] + o[nt][2], o[nt][1] + o[nt][3]);
+            if ((lane & 3) == 0) *reinterpret_cast<float2 *>(out + DH) = make_float2(m_run, ((l_run[0] + l_run[1]) + l_run[2]) + l_run[3]);
         }
+    }
     }
     }
     __syncthreads();
