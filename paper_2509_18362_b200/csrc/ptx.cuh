@@ -39,12 +39,6 @@ __device__ __forceinline__ bool mbar_try_wait(uint64_t *bar, uint32_t parity) {
     return ok != 0;
 }
 
-// ---- 16-byte asynchronous copies global -> shared through the load/store path ----------------
-// (measured on B200: this path sustains ~65 GB/s per SM against ~47 GB/s for 1-D bulk copies, and has
-// no per-request cost, so any row length and any shared-memory layout stream at full speed)
-__device__ __forceinline__ void cp_async16(void *dst_smem, const void *src_gmem) {
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(dst_smem)), "l"(src_gmem) : "memory");
-}
 // The executing thread's earlier cp.async copies arrive on `bar` when they have all landed (the
 // barrier's expected count must include one arrival per calling thread).
 __device__ __forceinline__ void cp_async_arrive(uint64_t *bar) {

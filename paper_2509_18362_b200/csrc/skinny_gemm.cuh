@@ -11,11 +11,12 @@
 // 128-byte-swizzled K-major tiles (64 K elements wide). Accumulators are double buffered in TMEM so the epilogue of one
 // item overlaps the MMAs of the next; in the epilogue of the last item the copy warps help.
 //
-// What bounds it. Up to 32 operand columns: HBM (7.5 TB/s between launches' fixed costs). At 64 activation rows the weight
-// bytes in flight: with A and X in one ring, half of the memory held X and 96 KB of weights were requested ahead per SM
-// (gate/up of the 7B shape 59 us, 65 with the MMAs and X taken out, against 49 at 4 rows with 192 KB). So A and X have
-// rings of their own (128-160 KB for A), and an item of gate/up or of the output head has two tiles that share every X
-// block; gate/up 56 us. The split-K matrices have too few rows for two tiles.
+// What bounds it: HBM, plus the wait for the first X block and the last item's epilogue of every launch (3584-wide layer:
+// gate/up 40 us at 4 rows, 46 at 64 for 272 MB, 41.5 us at a plain copy's rate; down 20 and 23 for 136 MB). At 64 activation
+// rows it was the weight bytes in flight: with A and X in one ring, half of the memory held X and 96 KB of weights were
+// requested ahead per SM (gate/up 59 us). So A and X have rings of their own (128-160 KB for A; 56 us), an item of gate/up
+// or of the output head has two tiles that share every X block, and the epilogue is cut short (see there). The split-K
+// matrices have too few rows for two tiles.
 // A stage is KA K blocks: four while three weight stages of that size fit, else two. Finer stages lose: a wait on a barrier
 // costs the MMA thread 200 cycles even when it is over, the four MMAs of a K block 190-260.
 // Weights by TMA lose too: the copy engine takes 47 GB/s per SM, and 128-byte pieces of rows 38 KB apart are slow at HBM
