@@ -60,12 +60,12 @@ typedef enum {
  * d a multiple of 64; n_q_heads a multiple of n_kv_heads with at most 8 query heads per
  * KV head; max_rows <= 4096 (rows = batch x rows-per-sequence handled in one call).
  *
- * Two kernel paths sit behind the draft and target calls, chosen by the call's number of
+ * Two kernel paths sit behind the draft and target calls. A target call's is chosen by its number of
  * sequences B alone (never by rows per sequence, so a position scored as one of 1 or of K+1 rows
- * gives the same bits):
- *   - few sequences (as many as fit one launch: up to 8 rows; at most 2 sequences for models that
- *     stream >= 256 MB of layer weights per step): one persistent kernel launch per call, or per
- *     group of whole sequences when the rows exceed one launch;
+ * gives the same bits), a draft call's by B and its first step's rows:
+ *   - few sequences (as many as fit one launch: up to 8 rows; for models that stream >= 256 MB of layer
+ *     weights per step 2 sequences and 4 rows in a draft call, 1 sequence in a target call): one persistent
+ *     kernel launch per call, or per group of whole sequences when the rows exceed one launch;
  *   - more sequences: groups of up to 64 rows, each step a sequence of kernels on the caller's
  *     stream that read every weight once per group (tensor-core GEMMs).
  * Within a path a sequence's results do not depend on the batch it is in; between the two paths

@@ -1,5 +1,6 @@
 """Batched draft calls at the edges of the GEMM's tiles, items and operand widths, against the oracle."""
 import pytest
+import torch
 
 from oracle import fastmtp_oracle as O
 from paper_2509_18362_b200 import inputs as I
@@ -44,3 +45,27 @@ def test_row_kernels_by_width(d, monkeypatch):
     if d <= 4160:                                  # the draft's first kernel too
         got, ref = run_draft_case(s, 95, 2, [3, 40], 2, 200, want_logits=False)
         check_draft(got, ref, f"d={d}")
+
+
+@pytest.mark.parametrize("B", [1, 2, 3])
+def test_target_path_by_sequences(B):
+    """A model with more than 256 MB of weights per layer: target calls of two and more sequences take the batched path, whose
+    bits do not depend on the rows per call."""
+    s = I.Shape(d=2560, n_q_heads=2, n_kv_heads=1, head_dim=128, ffn=16384, vocab=300, n_layers=1)
+    M, L = 2, [40, 0, 70][:B]
+    kv = I.paged_kv(s, L, M, 94)
+    Wt = I.target_weights(s, 95)
+    gpu, one = GpuTarget(s, Wt, [kv], max(L) + M), GpuTarget(s, Wt, [kv], max(L) + M)
+    t = I.token_ids(96, (B, M), s.vocab)
+    n0 = gpu.ctx.launch_count
+    h, l, _ = gpu.step(t)
+    assert (gpu.ctx.launch_count - n0 == 1) == (B == 1)
+    rh, rl = O.target_forward(s, Wt, t, [copy_kv(kv)])
+    close(h.float().cpu().numpy(), rh, "hidden states")
+    close(l.float().cpu().numpy(), rl, "logits")
+    for i in range(M):
+        h1, l1, _ = one.step(t[:, i:i + 1].copy())
+        assert torch.equal(h1[:, 0], h[:, i]) and torch.equal(l1[:, 0], l[:, i])
+        one.advance(1)
+    gpu.close()
+    one.close()
