@@ -40,8 +40,7 @@ struct fmtp_ctx {
     // batched draft path (more sequences than one persistent-kernel launch takes)
     BatchedShape bsh;
     BatchedWs bws;
-    int batched_min;           // draft calls with at least this many sequences take the batched path (env FMTP_BATCHED_MIN: both)
-    int target_min;            // and target calls
+    int batched_min;           // calls with at least this many sequences take the batched path (env FMTP_BATCHED_MIN)
     int persist_rows;          // a draft call whose step 0 has more rows takes the batched path, whatever its number of sequences
     long long tmem_launches;
     int tmem_staging;          // the persistent kernel stages weights through tensor memory where the shape allows (env FMTP_TMEM=1)
@@ -328,26 +327,27 @@ int fmtp_create(const fmtp_shape *sh, fmtp_ctx **out) {
     c->ws_need = layout(c, nullptr);
     const int g1 = group_size(c, 0, kMaxRows, 1);
     if (g1 < 1) { delete c; return FMTP_ESHAPE; }
-    // Which path a target call takes depends on its number of sequences only (so a sequence scored with 1 or with K+1
-    // rows takes the same path and gives the same bits). Small models: the persistent kernel as long as the sequences fit
-    // one launch. Models that stream >= 256 MB of layer weights per step (measured at the 7B shape): drafts take the batched
-    // path from three sequences on (three steps, two sequences at 2048: 482 us against 493), target calls from two on (four
-    // layers, two sequences, persistent / batched: one row at 512 / 2048 / 8192 558 / 573 / 646 us against 571 / 573 / 600,
-    // two rows at 64 600 against 573, three at 512 769 against 580, four at 2048 1001 against 588: the two per cent that one
-    // row of a short context loses are the price of bits that do not depend on the rows; one sequence: one row over 28
-    // layers 2780 against 2953, four rows 3217 against 3060).
-    c->batched_min = c->target_min = g1 + 1;
+    // Which path a target call takes depends on its number of sequences only (so a sequence scored with 1 or with K+1 rows
+    // takes the same path and gives the same bits). Small models: the persistent kernel as long as the sequences fit
+    // one launch. Models that stream >= 256 MB of layer weights per step: the batched path from three sequences on.
+    // 7B shape, persistent / batched, us: drafts of three steps, two sequences 486 / 493, three 528 / 498, four 560 / 501; target
+    // calls of four layers, three sequences of one row 594 / 576, of two 799 / 585; two sequences of one row at 512, 2048
+    // and 8192 558 / 570, 574 / 571 and 647 / 603, of two at 512 597 / 583, three 766 / 581, four at 2048 998 / 586.
+    // d = 4096 with ffn 14336 (503 MB): drafts of one, two and three 494 / 508, 536 / 518, 561 / 525.
+    // Target calls of two sequences stay here for all that: on the batched path one row at a short context is slower, and what
+    // they return is further from 64 bits (eight layers, appended keys 2.1e-4 against 2.9e-4, fp32 logits of a draft
+    // 4.3e-6 against 8.4e-6: the tensor core truncates along chains of up to 237 products, this kernel's are an eighth).
+    c->batched_min = g1 + 1;
     {
         const double qd = (double)sh->n_q_heads * sh->head_dim, kvd = (double)sh->n_kv_heads * sh->head_dim;
         const double layer_bytes = 2.0 * (2.0 * sh->d * sh->d + sh->d * (qd + 2 * kvd) + qd * sh->d + 3.0 * sh->d * sh->ffn);
         if (layer_bytes >= 256e6 && c->batched_min > 3) c->batched_min = 3;
-        if (layer_bytes >= 256e6 && c->target_min > 2) c->target_min = 2;
         // more than four rows take a second set of accumulators and a shallow ring in the persistent kernel (7B shape, one
         // step of five rows: 267 us against 189 on the batched path; two sequences of four extend rows, three steps: 974
         // against 521)
         c->persist_rows = layer_bytes >= 256e6 ? 4 : 1 << 30;
     }
-    if (const char *v = std::getenv("FMTP_BATCHED_MIN")) { int n = std::atoi(v); if (n >= 1) c->batched_min = c->target_min = n; }
+    if (const char *v = std::getenv("FMTP_BATCHED_MIN")) { int n = std::atoi(v); if (n >= 1) c->batched_min = n; }
     c->tmem_staging = 0;       // measured slower than the plain ring so far: opt-in
     if (const char *v = std::getenv("FMTP_TMEM")) c->tmem_staging = std::atoi(v) != 0;
     c->pinned_bytes = (size_t)sh->max_rows * sh->d * 2 + (size_t)sh->max_rows * 4 * (3 + (sh->max_K > 1 ? sh->max_K : 1)) +
@@ -609,7 +609,7 @@ int fastmtp_target_step(fmtp_ctx *c, const fmtp_target_w *w, const int32_t *toke
     if (!aligned16(w->embed) || !aligned16(w->lm_head) || !aligned16(w->g_final)) return FMTP_EINVAL;
     for (int l = 0; l < nl; ++l) if (!layer_ok(w->layers[l]) || !kv_ok(kvs[l])) return FMTP_EINVAL;
     const int V = c->shape.vocab, d = c->shape.d;
-    if (B >= c->target_min && M <= kBatchRows) {
+    if (B >= c->batched_min && M <= kBatchRows) {
         // more rows than one launch of the persistent kernel takes: groups of whole sequences, up to 64 rows each,
         // every layer's weights streamed once per group by the tensor-core GEMM path
         if ((out_h && !aligned16(out_h))) return FMTP_EINVAL;

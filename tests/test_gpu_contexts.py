@@ -1,0 +1,71 @@
+"""What a context accepts, several contexts in one process, and a context after a timeout."""
+from dataclasses import replace
+
+import numpy as np
+import pytest
+import torch
+
+from paper_2509_18362_b200 import binding as Bd
+from paper_2509_18362_b200 import inputs as I
+from tests.gpu_util import copy_kv
+
+pytestmark = pytest.mark.gpu
+
+
+class Drafter:
+    """One context with a seeded draft call of B sequences, E pairs each."""
+
+    def __init__(self, shape, B, E=1, seed=500, max_ctx=None, L=None):
+        L = [7 * b % 60 for b in range(B)] if L is None else L
+        self.B, self.E, self.kv = B, E, I.paged_kv(shape, L, E + 2, seed + 1)
+        self.dW = Bd.to_device(I.mtp_weights(shape, seed))
+        self.h = Bd.bf16_tensor(I.hidden_bf16(seed + 2, (B, E, shape.d)))
+        self.tok = torch.from_numpy(I.token_ids(seed + 3, (B, E), shape.vocab)).cuda()
+        self.ctx = Bd.Context(shape, max_rows=max(8, B * E), max_K=2, max_ctx=max_ctx or max(L) + E + 4)
+        self.shape = shape
+
+    def call(self):
+        """The call's results as one array of bits, and the status word."""
+        dkv = Bd.to_device(copy_kv(self.kv))
+        out_d = torch.full((self.B, 2), -1, dtype=torch.int32, device="cuda")
+        out_h = torch.zeros((self.B, 2, self.shape.d), dtype=torch.bfloat16, device="cuda")
+        st = torch.zeros(1, dtype=torch.int32, device="cuda")
+        self.ctx.fastmtp_draft(Bd.mtp_w(self.dW), self.h, self.tok, Bd.kv(dkv), self.B, 2, None, out_d, out_h, None, st, max_ext=self.E)
+        torch.cuda.synchronize()
+        return np.concatenate([Bd.bf16_bits(out_h).ravel(), out_d.cpu().numpy().ravel().astype(np.uint16)]), int(st.item())
+
+    def bits(self):
+        got, status = self.call()
+        assert status == 0
+        return got
+
+
+WIDE = replace(I.TINY, d=2048, vocab=1500)
+
+
+# more than 256 MB of weights per layer: the sizes at which the switch points come earlier
+LARGE = I.Shape(d=2560, n_q_heads=2, n_kv_heads=1, head_dim=128, ffn=16384, vocab=300, n_layers=1)
+
+
+def test_hidden_states_of_two_sequences_may_start_anywhere():
+    """A target call of fewer than three sequences takes out_h at any address; from three on it has to be a multiple of 16."""
+    Wt = Bd.to_device(I.target_weights(LARGE, 510))
+    w, keep = Bd.target_w(Wt)
+    for B in (1, 2, 3):
+        dkv = Bd.to_device(I.paged_kv(LARGE, [40, 9, 0][:B], 1, 511))
+        tok = torch.from_numpy(I.token_ids(512, (B, 1), LARGE.vocab)).cuda()
+        ctx = Bd.Context(LARGE, max_rows=8, max_K=1, max_ctx=64)
+        pool = torch.zeros(B * LARGE.d + 8, dtype=torch.bfloat16, device="cuda")
+        ctx.fastmtp_target_step(w, tok, [Bd.kv(dkv)], B, 1, pool[:B * LARGE.d])
+        want = Bd.bf16_bits(pool[:B * LARGE.d])
+        pool.zero_()
+        if B < 3:
+            ctx.fastmtp_target_step(w, tok, [Bd.kv(dkv)], B, 1, pool[3:])
+            got = Bd.bf16_bits(pool)
+            assert np.array_equal(got[3:3 + B * LARGE.d], want)
+            assert not got[:3].any() and not got[3 + B * LARGE.d:].any()
+        else:
+            with pytest.raises(Bd.FastMTPError):
+                ctx.fastmtp_target_step(w, tok, [Bd.kv(dkv)], B, 1, pool[3:])
+        ctx.close()
+    del keep

@@ -49,8 +49,8 @@ def test_row_kernels_by_width(d, monkeypatch):
 
 @pytest.mark.parametrize("B", [1, 2, 3])
 def test_target_path_by_sequences(B):
-    """A model with more than 256 MB of weights per layer: target calls of two and more sequences take the batched path, whose
-    bits do not depend on the rows per call."""
+    """A model with more than 256 MB of weights per layer: target calls of three and more sequences take the batched path. On
+    either path the bits do not depend on the rows per call."""
     s = I.Shape(d=2560, n_q_heads=2, n_kv_heads=1, head_dim=128, ffn=16384, vocab=300, n_layers=1)
     M, L = 2, [40, 0, 70][:B]
     kv = I.paged_kv(s, L, M, 94)
@@ -59,7 +59,7 @@ def test_target_path_by_sequences(B):
     t = I.token_ids(96, (B, M), s.vocab)
     n0 = gpu.ctx.launch_count
     h, l, _ = gpu.step(t)
-    assert (gpu.ctx.launch_count - n0 == 1) == (B == 1)
+    assert (gpu.ctx.launch_count - n0 == 1) == (B < 3)
     rh, rl = O.target_forward(s, Wt, t, [copy_kv(kv)])
     close(h.float().cpu().numpy(), rh, "hidden states")
     close(l.float().cpu().numpy(), rl, "logits")
