@@ -363,7 +363,11 @@ __global__ void __launch_bounds__(kGemmThreads, 1) skinny_gemm_kernel(const __gr
             const bool last = i == n_my - 1;
             const int first = last ? worker * 8 : 0, step = last ? 24 : 8, buf = i & 1;
             const GemmItem gi = gemm_my_item(g, i);
-            const bool late = !gemm_wait(sm, &sm->tfull[buf], (uint32_t)(i >> 1) & 1u, g.wait_limit_ns);
+            // the copy warps come for the last item only: `drain` completes once, behind its MMAs (tfull's phase is no answer there,
+            // the parity also fits two items earlier, which a CTA whose ring holds its last items may not have begun). It
+            // completes after a timeout too, so they look at the flag as well
+            const bool late = worker == 0 ? !gemm_wait(sm, &sm->tfull[buf], (uint32_t)(i >> 1) & 1u, g.wait_limit_ns)
+                                          : !gemm_wait(sm, &sm->drain, 0, g.wait_limit_ns) || *reinterpret_cast<volatile uint32_t *>(&sm->abort_flag);
             // before another item the 128 epilogue threads agree on the outcome; after the last one there is no barrier but the CTA's
             if (last ? __any_sync(0xffffffffu, late) : epi_any(late)) break;
             tc_fence_after_sync();

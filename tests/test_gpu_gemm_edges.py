@@ -27,6 +27,18 @@ def test_gemm_edges(shape, B, N, monkeypatch):
     check_draft(got, ref, f"B={B} N={N}")
 
 
+@pytest.mark.parametrize("d,V,B", [(64, 75900, 17), (128, 75900, 64), (64, 152064, 64), (128, 152064, 17), (64, 152064, 5)])
+def test_head_of_three_and_more_items_per_cta(d, V, B, monkeypatch):
+    """So few K blocks that a CTA's ring holds its last items before the first one's MMAs have begun: whoever joins for the
+    last item's epilogue has to wait for that item, not for an earlier one in the same accumulator buffer."""
+    monkeypatch.setenv("FMTP_BATCHED_MIN", "1")
+    s = I.Shape(d=d, n_q_heads=2, n_kv_heads=1, head_dim=64, ffn=144, vocab=V, n_layers=1)
+    got, ref = run_draft_case(s, 60 + B, B, [3 * b % 50 for b in range(B)], 1, None, want_logits=True)
+    check_draft(got, ref, f"d={d} V={V} B={B}")
+    for b in range(B):
+        close(got["logits"][b, 0], O.head_logits(ref["h_out"][b, 0], ref["W"]["lm_head"]), f"logits b={b}")
+
+
 @pytest.mark.parametrize("d", [64, 4096, 4160, 8192, 8256])
 def test_row_kernels_by_width(d, monkeypatch):
     """Widths at which a thread of the row-wise kernels owns one, two or more groups of columns."""
