@@ -1051,11 +1051,11 @@ int attn_encode_map(CUtensorMap *map, const bf16_t *pool, const BatchedShape &sh
 
 template <int DH, int ROWS>
 int attn_launch(const AttnArgs &a, const CUtensorMap &kmap, const CUtensorMap &vmap, int n_sm, TmapCache *cache, cudaStream_t st) {
-    int &limit = cache->attn_smem[ROWS > 1];
-    if (limit < AttnSmem<DH, ROWS>::TOTAL) {      // raise the kernel's shared-memory limit once per context
+    bool &raised = cache->attn_raised[ROWS > 1];
+    if (!raised) {                                // once per context (every context of this kernel sets the same limit)
         cudaError_t e = cudaFuncSetAttribute(attn_kernel<DH, ROWS>, cudaFuncAttributeMaxDynamicSharedMemorySize, AttnSmem<DH, ROWS>::TOTAL);
         if (e != cudaSuccess) return (int)e;
-        limit = AttnSmem<DH, ROWS>::TOTAL;
+        raised = true;
     }
     return (int)launch_chained(attn_kernel<DH, ROWS>, dim3(n_sm), dim3(kAttnThreads), (size_t)AttnSmem<DH, ROWS>::TOTAL, st, a, kmap, vmap);
 }

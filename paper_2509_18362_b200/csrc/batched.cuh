@@ -24,8 +24,8 @@ struct TmapEntry {
 struct TmapCache {
     TmapEntry e[12];
     int n, next;
-    int gemm_smem[2];                        // limit set on skinny_gemm_kernel<2>, <4>
-    int attn_smem[2];                        // limit set on attn_kernel for one row / several rows per sequence
+    bool gemm_raised[2];                     // skinny_gemm_kernel<2>, <4>: shared-memory limit raised
+    bool attn_raised[2];                     // attn_kernel for one row / several rows per sequence
 };
 
 struct BatchedWs {

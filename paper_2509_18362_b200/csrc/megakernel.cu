@@ -1908,11 +1908,13 @@ int mega_kernel_index(const MegaParams &p) {
 }
 
 int mega_max_grid(const MegaParams &p, size_t smem_bytes, int *err) {
-    int dev = 0, sms = 0, per_sm = 0;
+    int dev = 0, sms = 0, optin = 0, per_sm = 0;
     const void *fn = kernel_for(p);
     cudaError_t e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_bytes);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+    // always the same limit: it is the device's, and a lower one would take away from contexts with a larger footprint
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, optin);
     if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, p.use_tmem ? kTmThreads : kThreads, smem_bytes);
     if (err) *err = (int)e;
     if (e != cudaSuccess) return 0;

@@ -543,14 +543,14 @@ inline int skinny_gemm_launch(GemmArgs g, int n_sm, int smem_optin, cudaStream_t
     if (stages < 3) return (int)cudaErrorInvalidConfiguration;
     g.n_stages = stages;
     void (*kern)(const GemmArgs, const CUtensorMap) = ka == 4 ? skinny_gemm_kernel<4> : skinny_gemm_kernel<2>;
-    int &limit = cache->gemm_smem[ka == 4];
+    bool &raised = cache->gemm_raised[ka == 4];
     const size_t smem = (size_t)stages * wstage + (size_t)g.n_xstages * xstage + sizeof(GemmSmem);
     const int n_items = g.n_ranges * g.splits;
     const int grid = n_items < n_sm ? n_items : n_sm;
-    if ((int)smem > limit) {       // raise the kernel's shared-memory limit once per footprint
-        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (!raised) {       // once per context, to the most there is: the limit is the device's, a lower one would take away from other contexts
+        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_optin);
         if (e != cudaSuccess) return (int)e;
-        limit = (int)smem;
+        raised = true;
     }
     // the activation operand is the library's own: its map depends on (address, row pitch, K, rows) only: encoded once, then reused
     CUtensorMap xmap;

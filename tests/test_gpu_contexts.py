@@ -43,6 +43,28 @@ class Drafter:
 WIDE = replace(I.TINY, d=2048, vocab=1500)
 
 
+@pytest.mark.parametrize("batched,first,second", [
+    (True, (I.TINY, 16), (I.TINY, 4)),                 # the operand's widths differ
+    (True, (I.TINY, 64), (I.TINY, 20)),
+    (False, (WIDE, 1), (I.TINY, 1)),                   # the persistent kernel: one instantiation, two footprints
+    (False, (WIDE, 1, 4), (I.TINY, 1, 4)),
+    (False, (WIDE, 6), (I.TINY, 8)),
+])
+def test_contexts_of_different_footprints_take_turns(batched, first, second, monkeypatch):
+    """A kernel's shared-memory limit belongs to the device: a context with a small footprint must not take away what another
+    one has been given. Same bits in every turn."""
+    monkeypatch.setenv("FMTP_BATCHED_MIN", "1" if batched else "99")
+    a, b = Drafter(*first), None
+    want = a.bits()
+    b = Drafter(*second)
+    other = b.bits()
+    for _ in range(2):
+        assert np.array_equal(a.bits(), want)
+        assert np.array_equal(b.bits(), other)
+    a.ctx.close()
+    b.ctx.close()
+
+
 # more than 256 MB of weights per layer: the sizes at which the switch points come earlier
 LARGE = I.Shape(d=2560, n_q_heads=2, n_kv_heads=1, head_dim=128, ffn=16384, vocab=300, n_layers=1)
 
