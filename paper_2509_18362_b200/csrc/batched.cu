@@ -656,6 +656,14 @@ __global__ void __launch_bounds__(kAttnThreads, 1) attn_kernel(const __grid_cons
 #pragma unroll
             for (int j = 0; j < 2; ++j) sc[nt * 2 + j] = (s[nt][0][j] + s[nt][1][j]) + (s[nt][0][j + 2] + s[nt][1][j + 2]);
     };
+    if constexpr (ROWS == 1) {
+    constexpr int NT = DH / 32;                              // 8-wide tiles of this warp's quarter of the head dimension
+    float *mx_s = reinterpret_cast<float *>(smem + L::O_RED) + grp * 64, *l_s = mx_s + 32;
+    const uint32_t vhalf = (uint32_t)(wi * NT / 8), vpiece = (uint32_t)((wi * NT) & 7);
+    // probabilities: [16 operand rows][64 tokens], pieces of 8 tokens swizzled by the row
+    const uint32_t pbase = smem_u32(smem + L::O_P) + (uint32_t)(grp * L::PROW);
+    const uint32_t plane = (uint32_t)(((lane & 7) + ((lane >> 3) & 1) * 8) * 128), psw = (uint32_t)(lane & 7), ppc = (uint32_t)(lane >> 4);
+    const uint32_t pst = pbase + (uint32_t)(hrow * 128 + kq * 2);
     // value rows nothing has written may hold anything: zeros, so that a probability of 0 meets a finite number
     auto clear_values = [&](int tile, int tokens) {
         for (int i = lane; i < (kAttnBox - tokens) * (DH / 8); i += 32) {
@@ -665,15 +673,6 @@ __global__ void __launch_bounds__(kAttnThreads, 1) attn_kernel(const __grid_cons
         }
         fence_proxy_async();                                 // before a later TMA copy overwrites them
     };
-
-    if constexpr (ROWS == 1) {
-    constexpr int NT = DH / 32;                              // 8-wide tiles of this warp's quarter of the head dimension
-    float *mx_s = reinterpret_cast<float *>(smem + L::O_RED) + grp * 64, *l_s = mx_s + 32;
-    const uint32_t vhalf = (uint32_t)(wi * NT / 8), vpiece = (uint32_t)((wi * NT) & 7);
-    // probabilities: [16 operand rows][64 tokens], pieces of 8 tokens swizzled by the row
-    const uint32_t pbase = smem_u32(smem + L::O_P) + (uint32_t)(grp * L::PROW);
-    const uint32_t plane = (uint32_t)(((lane & 7) + ((lane >> 3) & 1) * 8) * 128), psw = (uint32_t)(lane & 7), ppc = (uint32_t)(lane >> 4);
-    const uint32_t pst = pbase + (uint32_t)(hrow * 128 + kq * 2);
     for (int item = worker; item < n_items; item += stride) {
         load_item(it, item);
         if (it.n_blk == 0) continue;
@@ -809,8 +808,6 @@ __global__ void __launch_bounds__(kAttnThreads, 1) attn_kernel(const __grid_cons
                     for (int ks = 0; ks < KS; ++ks) load_k(sb, s, ks, kf[ks]);
                     scores(qa, kf, sc[s]);
                 }
-                const int exist = it.n_ctx - (it.t0 + blk * kAttnBlk);      // positions of the block that any row of the set sees
-                if (exist < kAttnBlk && (exist & (kAttnBox - 1))) { clear_values(exist / kAttnBox, exist & (kAttnBox - 1)); __syncwarp(); }
                 if (left < kAttnBlk) {
 #pragma unroll
                     for (int s = 0; s < 4; ++s)
@@ -841,13 +838,30 @@ __global__ void __launch_bounds__(kAttnThreads, 1) attn_kernel(const __grid_cons
                 }
 #pragma unroll
                 for (int s = 0; s < 4; ++s) {
-                    if (s * kAttnBox >= left) break;
+                    if ((s + 1) * kAttnBox > left) break;
 #pragma unroll
                     for (int j = 0; j < ND; ++j) {
                         uint32_t v[4];
                         load_v(sb, s, (uint32_t)(j >> 2), (uint32_t)(2 * (j & 3)), v);
                         mma_bf16_pure(o[2 * j], pf[s][0], pf[s][1], pf[s][2], pf[s][3], v[0], v[1]);
                         mma_bf16_pure(o[2 * j + 1], pf[s][0], pf[s][1], pf[s][2], pf[s][3], v[2], v[3]);
+                    }
+                }
+                if (left < kAttnBlk && (left & (kAttnBox - 1))) {
+                    // the tile in which the row's context ends: what lies beyond is another row's value, or what an unwritten
+                    // slot holds, and need not be finite. A probability of 0 meets a 0 there
+                    const int s = left / kAttnBox, seen = left & (kAttnBox - 1);
+                    const uint32_t keep0 = (kq < seen ? 0xffffu : 0u) | (kq + 1 < seen ? 0xffff0000u : 0u);
+                    const uint32_t keep1 = (kq + 8 < seen ? 0xffffu : 0u) | (kq + 9 < seen ? 0xffff0000u : 0u);
+                    uint32_t pe[4];
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) pe[i] = s == 0 ? pf[0][i] : s == 1 ? pf[1][i] : s == 2 ? pf[2][i] : pf[3][i];
+#pragma unroll
+                    for (int j = 0; j < ND; ++j) {
+                        uint32_t v[4];
+                        load_v(sb, s, (uint32_t)(j >> 2), (uint32_t)(2 * (j & 3)), v);
+                        mma_bf16_pure(o[2 * j], pe[0], pe[1], pe[2], pe[3], v[0] & keep0, v[1] & keep1);
+                        mma_bf16_pure(o[2 * j + 1], pe[0], pe[1], pe[2], pe[3], v[2] & keep0, v[3] & keep1);
                     }
                 }
             }

@@ -3,6 +3,7 @@ from dataclasses import replace
 
 import numpy as np
 import pytest
+import torch
 
 from oracle import fastmtp_oracle as O
 from paper_2509_18362_b200 import binding as Bd
@@ -77,3 +78,32 @@ def test_merge_of_few_and_many_chunks(monkeypatch):
     close(h.float().cpu().numpy(), rh, "hidden states")
     close(l.float().cpu().numpy(), rl, "logits")
     gpu.close()
+
+
+@pytest.mark.parametrize("batched", [True])
+@pytest.mark.parametrize("bits", [0x7FC0, 0x7F80])               # NaN, infinity
+@pytest.mark.parametrize("dh,M", [(64, 4), (128, 3), (64, 6)])
+def test_a_row_does_not_see_what_later_rows_hold(dh, M, bits, batched, monkeypatch):
+    """The last row's token has an embedding that is not finite, and so are its keys and values: the rows before it, which share
+    its K/V blocks, give the bits they give beside a finite one."""
+    monkeypatch.setenv("FMTP_BATCHED_MIN", "1" if batched else "99")
+    s = replace(I.TINY, head_dim=dh, n_layers=1)
+    L = [0, 3, 14, 30, 63, 250] if batched else [14 if M < 6 else 60]
+    kv = I.paged_kv(s, L, M, 61)
+    Wt = I.target_weights(s, 62)
+    t = I.token_ids(63, (len(L), M), s.vocab - 1)
+    t_odd = t.copy()
+    t_odd[:, -1] = s.vocab - 1
+    Wt["embed"][s.vocab - 1] = bits
+    got = []
+    for tokens in (t, t_odd):
+        gpu = GpuTarget(s, Wt, [kv], max(L) + M)
+        gpu.ctx.close()
+        gpu.ctx = Bd.Context(s, max_rows=64, max_K=1, max_ctx=max(L) + M)
+        h = torch.zeros((len(L), M, s.d), dtype=torch.bfloat16, device="cuda")
+        gpu.ctx.fastmtp_target_step(gpu.w, torch.from_numpy(tokens).cuda(), [Bd.kv(k) for k in gpu.dkvs], len(L), M, h)
+        torch.cuda.synchronize()
+        got.append(Bd.bf16_bits(h))
+        gpu.close()
+    assert np.isnan(O.bf16_to_f64(got[1][:, -1])).any()
+    assert np.array_equal(got[0][:, :-1], got[1][:, :-1])
