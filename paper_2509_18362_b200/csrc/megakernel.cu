@@ -1131,7 +1131,12 @@ __device__ __forceinline__ void attn_rows_mma(Cta &c, const bf16_t *sk, const bf
             }
             psum += __shfl_xor_sync(0xffffffffu, psum, 1);
             psum += __shfl_xor_sync(0xffffffffu, psum, 2);
-            // o[head][dim] = sum over the warp's tokens of p * V
+            // o[head][dim] = sum over the warp's tokens of p * V. Beyond the row's context the stage holds later rows' values or
+            // what nothing has written, which need not be finite: a probability of 0 meets a 0 there (masked in registers,
+            // and not by zeros in the stage besides: that cost 0.3 % of a draft)
+            const int seen = npos + 1 - (c0 + tw);
+            const uint32_t keep0 = (kq < seen ? 0xffffu : 0u) | (kq + 1 < seen ? 0xffff0000u : 0u);
+            const uint32_t keep1 = (kq + 8 < seen ? 0xffffu : 0u) | (kq + 9 < seen ? 0xffff0000u : 0u);
             float o[DH / 8][4];
 #pragma unroll
             for (int nt = 0; nt < DH / 8; ++nt) o[nt][0] = o[nt][1] = o[nt][2] = o[nt][3] = 0.f;
@@ -1140,8 +1145,8 @@ __device__ __forceinline__ void attn_rows_mma(Cta &c, const bf16_t *sk, const bf
                 uint32_t b00, b01, b10, b11;
                 asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];"
                              : "=r"(b00), "=r"(b01), "=r"(b10), "=r"(b11) : "r"(vrow + ((((uint32_t)(nt + vpc)) ^ vsw) << 4)));
-                mma_bf16(o[nt], pa[0], pa[1], pa[2], pa[3], b00, b01);
-                mma_bf16(o[nt + 1], pa[0], pa[1], pa[2], pa[3], b10, b11);
+                mma_bf16(o[nt], pa[0], pa[1], pa[2], pa[3], b00 & keep0, b01 & keep1);
+                mma_bf16(o[nt + 1], pa[0], pa[1], pa[2], pa[3], b10 & keep0, b11 & keep1);
             }
             // ---- merge the group's four warps (fixed order) -> chunk partial in global memory
             {
@@ -1357,14 +1362,6 @@ __device__ __forceinline__ void attention_phase(Cta &c, const KvPtrs &kv, int st
             kv.k_pages[o + e + half] = k1;
             kv.v_pages[o + e] = v0;
             kv.v_pages[o + e + half] = v1;
-        }
-        // -- value rows of the chunk's positions that nothing has written (beyond the last row of this call): zeros, so
-        // that a masked probability of 0 meets a finite number in the tensor-core product
-        {
-            const int last = min(base + rows - 1, max_tokens - 1);
-            const int nfill = max(0, min(kAttnChunk, last + 1 - c0));
-            for (int i = c.tid; i < (kAttnChunk - nfill) * upt; i += kConsumerThreads)
-                *reinterpret_cast<uint4 *>(sv + (size_t)nfill * dh + (size_t)i * 8) = make_uint4(0, 0, 0, 0);
         }
         bar_sync(1, kConsumerThreads);
         PROF(c, ATTN * 8 + 5);

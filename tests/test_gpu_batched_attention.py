@@ -80,7 +80,7 @@ def test_merge_of_few_and_many_chunks(monkeypatch):
     gpu.close()
 
 
-@pytest.mark.parametrize("batched", [True])
+@pytest.mark.parametrize("batched", [True, False])
 @pytest.mark.parametrize("bits", [0x7FC0, 0x7F80])               # NaN, infinity
 @pytest.mark.parametrize("dh,M", [(64, 4), (128, 3), (64, 6)])
 def test_a_row_does_not_see_what_later_rows_hold(dh, M, bits, batched, monkeypatch):
