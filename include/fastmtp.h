@@ -158,7 +158,8 @@ int fmtp_selftest_wait_timeout(uint32_t *dev_status, int limit_ms, unsigned long
  *   which = 1  the persistent kernel's grid barrier expects one arrival more than there are CTAs
  *              (takes effect if that call runs on the persistent path);
  *   which = 2  the first ring stage of the call's first tensor-core GEMM expects one copy more than is made
- *              (takes effect if that call runs on the batched path).
+ *              (takes effect if that call runs on the batched path);
+ *   which = 3  every ring stage of the call's first batched attention kernel does (likewise).
  * The wait runs out, the kernel ORs FMTP_DEV_TIMEOUT into the status word, every other CTA / role sees the abort
  * flag and stops waiting, copies in flight are drained, tensor memory is freed, and the launch -- and the rest of
  * the call's launches, on garbage that stays inside the caller's buffers -- ends normally: nothing hangs, traps or

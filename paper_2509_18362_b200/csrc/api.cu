@@ -51,7 +51,7 @@ struct fmtp_ctx {
     TmapCache tmaps;                                               // tensor maps of the batched path's GEMM operands
     // fmtp_selftest_inject_wait_timeout: the next draft call runs with this wait limit and one wait that cannot end
     unsigned long long inject_limit_ns;
-    int inject_which;                                              // 0 none, 1 grid barrier of the persistent kernel, 2 ring stage of a GEMM
+    int inject_which;                                              // 0 none, 1 grid barrier of the persistent kernel, 2 ring stage of a GEMM, 3 of the attention
 };
 
 namespace {
@@ -359,7 +359,7 @@ int fmtp_create(const fmtp_shape *sh, fmtp_ctx **out) {
 }
 
 int fmtp_selftest_inject_wait_timeout(fmtp_ctx *c, int limit_ms, int which) {
-    if (!c || (which != 1 && which != 2)) return FMTP_EINVAL;
+    if (!c || which < 1 || which > 3) return FMTP_EINVAL;
     if (limit_ms < 1 || limit_ms > 1000) return FMTP_EINVAL;      // bounded on purpose
     c->inject_limit_ns = (unsigned long long)limit_ms * 1000000ull;
     c->inject_which = which;
@@ -449,7 +449,7 @@ int fastmtp_draft(fmtp_ctx *c, const fmtp_mtp_w *w, const fmtp_bf16 *h_last, con
             bc.rope_cos = c->s.rope_cos; bc.rope_sin = c->s.rope_sin;
             bc.n_sm = c->n_sm; bc.smem_optin = c->smem_optin; bc.cache = &c->tmaps;
             bc.wait_limit_ns = kDefaultWaitNs;
-            if (c->inject_which == 2) { bc.wait_limit_ns = c->inject_limit_ns; bc.inject_gemm_timeout = 1; c->inject_which = 0; }
+            if (c->inject_which >= 2) { bc.wait_limit_ns = c->inject_limit_ns; bc.inject = c->inject_which; c->inject_which = 0; }
             bc.B = (B - b0 < kBatchRows) ? B - b0 : kBatchRows;
             bc.K = K; bc.N = Neff; bc.ids = subset;
             bc.M0 = max_ext; bc.n_ext = n_ext ? n_ext + b0 : nullptr;

@@ -365,6 +365,7 @@ __global__ void qkv_finish_kernel(const QkvArgs a) {
 struct AttnArgs {
     int Hq, Hkv, dh, page, max_ctx, max_chunks, B;    // B: sequences
     int tma;                     // pages are whole 16-token tiles: TMA copies (else 16-byte copies, any page size)
+    int extra_arrivals;          // self-test only: arrivals a ring stage expects beyond the copies that are made
     RowGeo geo;                  // which positions a sequence's rows have
     unsigned long long wait_limit_ns;   // a ring wait gives up after this long
     const bf16_t *q;             // [rows][Hkv][2][Hq/Hkv][dh]: scaled queries, high parts then low parts, 16-byte pieces of head
@@ -447,7 +448,7 @@ __global__ void __launch_bounds__(kAttnThreads, 1) attn_kernel(const __grid_cons
     if (threadIdx.x == 0) {
         for (int g = 0; g < 2; ++g) {
             uint64_t *b = bars + g * (2 * SG + NQ);
-            for (int s = 0; s < SG; ++s) { mbar_init(&b[s], a.tma ? 1 : 65); mbar_init(&b[SG + s], 4); }
+            for (int s = 0; s < SG; ++s) { mbar_init(&b[s], (a.tma ? 1 : 65) + a.extra_arrivals); mbar_init(&b[SG + s], 4); }
             for (int s = 0; s < NQ; ++s) mbar_init(&b[2 * SG + s], 4);
         }
         *abort_flag = 0;
@@ -575,13 +576,6 @@ __global__ void __launch_bounds__(kAttnThreads, 1) attn_kernel(const __grid_cons
                 ++li;
                 it = nx; item = nitem; rows = nrows;
             }
-            // after a timeout nobody may have waited for the last copies: they land before the CTA exits
-            if (!ok && lane == 0)
-                for (int s = 0; s < SG; ++s) {
-                    stage = stage == 0 ? SG - 1 : stage - 1;
-                    if (stage == SG - 1) phase ^= 1u;
-                    for (int n = 0; n < (1 << 16) && !mbar_try_wait(&full[stage], phase); ++n) { }
-                }
         }
     } else {
         // ---- any page size: 16-byte copies into the same layout, zeros beyond the visible positions
@@ -612,6 +606,16 @@ __global__ void __launch_bounds__(kAttnThreads, 1) attn_kernel(const __grid_cons
             ++li;
         }
         cp_async_wait_all();
+    }
+    // The copies of the last stages (K/V tiles, queries) land before the CTA exits, also after a timeout, when nobody else
+    // waits for them any more: 1 ms at most
+    if (ct == 0) {
+        const unsigned long long t_begin = global_timer_ns();
+        for (int s = 0; s < SG; ++s) {
+            stage = stage == 0 ? SG - 1 : stage - 1;
+            if (stage == SG - 1) phase ^= 1u;
+            while (!mbar_try_wait(&full[stage], phase) && global_timer_ns() - t_begin < 1000000ull) { }
+        }
     }
     } else {
 
@@ -1076,8 +1080,9 @@ int attn_launch(const AttnArgs &a, const CUtensorMap &kmap, const CUtensorMap &v
 
 // Attention and chunk merge of a pass over `rows` rows (geo.M per sequence).
 int attention(const BatchedShape &sh, const BatchedWs &ws, const KvPtrs &kv, const RowGeo &geo, int rows, int n_sm,
-              unsigned long long wait_limit_ns, TmapCache *cache, cudaStream_t st, long long *launches) {
+              unsigned long long wait_limit_ns, int extra_arrivals, TmapCache *cache, cudaStream_t st, long long *launches) {
     AttnArgs a{};
+    a.extra_arrivals = extra_arrivals;
     a.Hq = sh.Hq; a.Hkv = sh.Hkv; a.dh = sh.dh; a.page = sh.page; a.max_ctx = sh.max_ctx; a.geo = geo;
     a.max_chunks = ws.max_chunks; a.q = ws.q; a.kv = kv; a.att_part = ws.att_part; a.status = ws.status;
     a.B = rows / geo.M; a.wait_limit_ns = wait_limit_ns;
@@ -1182,7 +1187,7 @@ int batched_draft(const BatchedCall &c, cudaStream_t st, long long *launches) {
     const int B = c.B, K = c.K, d = sh.d;
     const int M0 = c.M0 > 1 ? c.M0 : 1;
     const bool ext = M0 > 1;                       // step 0 carries up to M0 extend rows per sequence
-    int inject_left = c.inject_gemm_timeout ? 1 : 0;
+    int inject_gemm = c.inject == 2 ? 1 : 0, inject_attn = c.inject == 3 ? 1 : 0;      // self-test: one launch each
     const int qdim = sh.Hq * sh.dh, kvdim = sh.Hkv * sh.dh;
     cudaError_t e = cudaMemsetAsync(ws.keys, 0, ws.keys_bytes, st);     // argmax keys and the status word
     if (e != cudaSuccess) return (int)e;
@@ -1205,8 +1210,8 @@ int batched_draft(const BatchedCall &c, cudaStream_t st, long long *launches) {
         g.n_rows = n_rows; g.K = Kdim; g.lda = lda; g.x = x; g.ldx = ldx; g.NB = (2 * rows + 15) / 16 * 16; g.R = rows;
         g.status = ws.status;
         g.wait_limit_ns = c.wait_limit_ns;
-        g.extra_arrivals = inject_left > 0 ? 1 : 0;      // self-test: the call's first GEMM waits for a copy that never comes
-        if (inject_left > 0) --inject_left;
+        g.extra_arrivals = inject_gemm;
+        inject_gemm = 0;
         pick_items(g, c.n_sm);
         g.partial = ws.partial; g.ldp = ws.ldp;
         ++*launches;
@@ -1257,7 +1262,8 @@ int batched_draft(const BatchedCall &c, cudaStream_t st, long long *launches) {
             ++*launches;
             if ((rc = (int)launch_chained(qkv_finish_kernel, dim3(sh.Hq + 2 * sh.Hkv, rows), dim3(sh.dh / 2), 0, st, a))) return rc;
         }
-        if ((rc = attention(sh, ws, kv, geo, rows, c.n_sm, c.wait_limit_ns, c.cache, st, launches))) return rc;
+        if ((rc = attention(sh, ws, kv, geo, rows, c.n_sm, c.wait_limit_ns, inject_attn, c.cache, st, launches))) return rc;
+        inject_attn = 0;
         // x += W_o o
         g = GemmArgs{};
         g.a[0] = c.layer.wo; g.a_rows[0] = d; g.n_seg = 1; g.epi = EPI_PARTIAL;
@@ -1356,7 +1362,7 @@ int batched_target(const BatchedTargetCall &c, cudaStream_t st, long long *launc
             ++*launches;
             if ((rc = (int)launch_chained(qkv_finish_kernel, dim3(sh.Hq + 2 * sh.Hkv, R), dim3(sh.dh / 2), 0, st, a))) return rc;
         }
-        if ((rc = attention(sh, ws, kv, geo, R, c.n_sm, c.wait_limit_ns, c.cache, st, launches))) return rc;
+        if ((rc = attention(sh, ws, kv, geo, R, c.n_sm, c.wait_limit_ns, 0, c.cache, st, launches))) return rc;
         g = GemmArgs{};
         g.a[0] = L.wo; g.a_rows[0] = d; g.n_seg = 1; g.epi = EPI_PARTIAL;
         if ((rc = gemm(g, d, qdim, qdim, ws.xop0, ws.ld0))) return rc;

@@ -60,7 +60,7 @@ struct BatchedCall {
     int n_sm, smem_optin;
     TmapCache *cache;
     unsigned long long wait_limit_ns;     // every device-side wait gives up after this long
-    int inject_gemm_timeout;              // self-test: the call's first GEMM expects a copy that is never made
+    int inject;                           // self-test: a copy that is never made is expected by the call's first GEMM (2) or attention (3)
     int B, K, N;
     const int32_t *ids;                   // subset or NULL
     int M0;                               // extend rows per sequence in step 0 (layout of h_last / tok_last), >= 1

@@ -1,4 +1,5 @@
 """What a context accepts, several contexts in one process, and a context after a timeout."""
+import time
 from dataclasses import replace
 
 import numpy as np
@@ -41,6 +42,23 @@ class Drafter:
 
 
 WIDE = replace(I.TINY, d=2048, vocab=1500)
+
+
+@pytest.mark.parametrize("which,shape,B,E", [
+    (3, I.TINY, 12, 1), (3, I.TINY, 12, 4),            # batched attention, one and several rows: tile copies
+    (3, replace(I.TINY, page_size=5), 12, 1), (3, replace(I.TINY, page_size=5), 12, 4),       # 16-byte copies
+])
+def test_a_wait_that_runs_out_leaves_the_context_usable(which, shape, B, E):
+    """A wait of the next call cannot end and is limited to 20 ms: the call returns soon after with the timeout flag, the next
+    one gives the bits of the one before."""
+    a = Drafter(shape, B, E)
+    want = a.bits()
+    a.ctx.fmtp_selftest_inject_wait_timeout(20, which)
+    t0 = time.time()
+    _, status = a.call()
+    assert status & Bd.DEV_TIMEOUT and 0.015 < time.time() - t0 < 2.0
+    assert np.array_equal(a.bits(), want)
+    a.ctx.close()
 
 
 @pytest.mark.parametrize("batched,first,second", [
