@@ -70,11 +70,12 @@ typedef enum {
  *     stream that read every weight once per group (tensor-core GEMMs).
  * Within a path a sequence's results do not depend on the batch it is in; between the two paths
  * results agree within the documented tolerances, not bit for bit (different summation order).
- * The environment variable FMTP_BATCHED_MIN (read at fmtp_create) overrides the switch point (at 2, target calls of two
- * sequences with several rows are up to 1.7 times faster at 7B width; the batched path's sums are half as exact); FMTP_TMEM=1
- * (also read at fmtp_create) lets the persistent kernel stage weights through tensor memory where the shape allows (results
- * agree with the default within the tolerances of the tests, not bit for bit: the k chunks are dealt to the warps
- * differently). */
+ * The environment variable FMTP_BATCHED_MIN (read at fmtp_create) overrides the switch point: calls of either kind with at
+ * least that many sequences take the batched path, those with fewer the persistent one as long as a sequence's rows fit
+ * one launch. (At 2, target calls of two sequences with several rows are up to 1.7 times faster at 7B width; the batched
+ * path's sums are half as exact.) FMTP_TMEM=1 (also read at fmtp_create) lets the persistent kernel stage weights through
+ * tensor memory where the shape allows (results agree with the default within the tolerances of the tests, not bit for
+ * bit: the k chunks are dealt to the warps differently). */
 typedef struct {
     int32_t d, n_q_heads, n_kv_heads, head_dim, ffn, vocab;
     int32_t n_layers;      /* target decoder depth (fastmtp_target_step); the MTP head has 1 */

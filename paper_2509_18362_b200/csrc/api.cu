@@ -40,8 +40,8 @@ struct fmtp_ctx {
     // batched draft path (more sequences than one persistent-kernel launch takes)
     BatchedShape bsh;
     BatchedWs bws;
-    int batched_min;           // calls with at least this many sequences take the batched path (env FMTP_BATCHED_MIN)
-    int persist_rows;          // a draft call whose step 0 has more rows takes the batched path, whatever its number of sequences
+    int batched_min;           // calls with at least this many sequences take the batched path
+    int persist_rows;          // so does a draft call whose step 0 has more rows (env FMTP_BATCHED_MIN: its value for the sequences, no rule on rows)
     long long tmem_launches;
     int tmem_staging;          // the persistent kernel stages weights through tensor memory where the shape allows (env FMTP_TMEM=1)
     // answers that depend on the geometry only, kept so that the hot calls make no CUDA attribute / occupancy query:
@@ -347,7 +347,10 @@ int fmtp_create(const fmtp_shape *sh, fmtp_ctx **out) {
         // against 521)
         c->persist_rows = layer_bytes >= 256e6 ? 4 : 1 << 30;
     }
-    if (const char *v = std::getenv("FMTP_BATCHED_MIN")) { int n = std::atoi(v); if (n >= 1) c->batched_min = n; }
+    if (const char *v = std::getenv("FMTP_BATCHED_MIN")) {
+        const int n = std::atoi(v);
+        if (n >= 1) { c->batched_min = n; c->persist_rows = 1 << 30; }
+    }
     c->tmem_staging = 0;       // measured slower than the plain ring so far: opt-in
     if (const char *v = std::getenv("FMTP_TMEM")) c->tmem_staging = std::atoi(v) != 0;
     c->pinned_bytes = (size_t)sh->max_rows * sh->d * 2 + (size_t)sh->max_rows * 4 * (3 + (sh->max_K > 1 ? sh->max_K : 1)) +

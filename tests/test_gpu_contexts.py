@@ -87,6 +87,20 @@ def test_contexts_of_different_footprints_take_turns(batched, first, second, mon
 LARGE = I.Shape(d=2560, n_q_heads=2, n_kv_heads=1, head_dim=128, ffn=16384, vocab=300, n_layers=1)
 
 
+def test_the_switch_point_variable_overrides_the_row_rule_of_drafts(monkeypatch):
+    """Five pairs of one sequence at a large width: several kernels by default, one launch where FMTP_BATCHED_MIN says so."""
+    monkeypatch.delenv("FMTP_BATCHED_MIN", raising=False)
+    a = Drafter(LARGE, 1, 5)
+    a.bits()
+    assert a.ctx.launch_count > 3
+    a.ctx.close()
+    monkeypatch.setenv("FMTP_BATCHED_MIN", "9")
+    b = Drafter(LARGE, 1, 5)
+    b.bits()
+    assert b.ctx.launch_count == 1
+    b.ctx.close()
+
+
 def test_hidden_states_of_two_sequences_may_start_anywhere():
     """A target call of fewer than three sequences takes out_h at any address; from three on it has to be a multiple of 16."""
     Wt = Bd.to_device(I.target_weights(LARGE, 510))
