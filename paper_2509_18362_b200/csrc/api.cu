@@ -158,7 +158,9 @@ int configure(fmtp_ctx *c, MegaParams &p, int mode, int B, int M) {
         // attention scratch: the rows' query vectors, then one (o, m, l) buffer per working warp group (the rows of a call
         // are dealt to two groups): [4 warps][8 heads][dh + 2] + 64 words
         size_t attn = (size_t)M * Gq * p.dh * 4 + (size_t)(M > 1 ? 2 : 1) * (4 * 8 * (p.dh + 2) + 64) * 4;
-        size_t mrg = ((size_t)2 * c->max_chunks + 4 + (size_t)(4 * kConsumerThreads / p.dh) * (p.dh + kPartPad)) * 4;      // chunk-merge scratch
+        // chunk merge: a context's maxima and sums. Its partial sums (4.3 KB) lie behind them only where something else asks for
+        // that much (see merge_phase), so that they take no length away from the longest contexts
+        size_t mrg = ((size_t)2 * c->max_chunks + 320) * 4;
         if (mrg > attn) attn = mrg;
         size_t actd = (size_t)2 * R * act_stride(mode == 0 && !split ? 2 * p.d : (p.d > p.qdim ? p.d : p.qdim)) * 2;
         size_t actq = (size_t)2 * R * act_stride(p.qdim) * 2;

@@ -58,10 +58,10 @@ enum Kind { PROJ = 0, QKV = 1, OPROJ = 2, GATEUP = 3, DOWN = 4, HEAD = 5, ATTN =
 struct Prog { int step, layer, kind; };
 
 struct Misc {   // small shared-memory block
-    uint64_t full[2 * kMaxStages];    // second half: the ring of a draft's later steps (see switch_layout)
-    uint64_t empty[2 * kMaxStages];
-    uint64_t tfull[kTmSlots];     // tensor-memory slots: filled by the mover's copies / read out by the four owning warps
-    uint64_t tempty[kTmSlots];
+    uint64_t full[kMaxStages];
+    uint64_t empty[kMaxStages];
+    uint64_t tfull[kTmSlots];     // tensor-memory slots: filled by the mover's copies / read out by the four owning warps.
+    uint64_t tempty[kTmSlots];    // Without tensor memory: the ring of a draft's later steps (see switch_layout)
     uint64_t tdrain;              // the mover's last copies, before the tensor memory is freed
     uint32_t tmem_base;
     uint32_t use_done[kMaxStages];   // per ring slot: uses whose data has been taken out (read by consumers or moved)
@@ -954,8 +954,9 @@ __device__ __forceinline__ void switch_layout(Cta &c) {
     c.n_stages = p.n_stages2;
     c.scr_bytes = p.scratch_smem2;
     c.proj_split = 0;
-    c.full = c.misc->full + kMaxStages;
-    c.empty = c.misc->empty + kMaxStages;
+    static_assert(kTmSlots == kMaxStages, "the tensor-memory slots' barriers serve this ring");
+    c.full = c.misc->tfull;
+    c.empty = c.misc->tempty;
     c.slot = 0;
     c.parity = 0;
 }
@@ -1393,7 +1394,9 @@ __device__ __forceinline__ void merge_phase(Cta &c, const KvPtrs &kv, int step) 
     const int max_tokens = min(kv.max_pages * p.page, p.max_ctx);
     float *ms = reinterpret_cast<float *>(c.scr);    // [max_chunks] chunk maxima
     float *ls = ms + p.max_chunks;                   // [max_chunks] chunk denominators
-    float *red = reinterpret_cast<float *>(c.scr) + ((2 * p.max_chunks + 3) & ~3);   // [ncg][stride] partial sums (+ denominators)
+    // [ncg][stride] partial sums (+ denominators), behind those where the staging area has the room, else in their place
+    const bool tight = (((2 * p.max_chunks + 3) & ~3) + ncg * stride) * 4 > c.scr_bytes;
+    float *red = reinterpret_cast<float *>(c.scr) + (tight ? 0 : (2 * p.max_chunks + 3) & ~3);
     const int units = c.R * p.Hq;
     const int el = (c.tid % q4) * 4, cg = c.tid / q4;
     for (int u = c.cta; u < units; u += c.grid) {
@@ -1424,6 +1427,7 @@ __device__ __forceinline__ void merge_phase(Cta &c, const KvPtrs &kv, int step) 
         for (int i = 0; i < kPre; ++i) if (cg + i * ncg < ncm) add(cg + i * ncg, pre[i]);
 #pragma unroll 4
         for (int ch = cg + kPre * ncg; ch < ncm; ch += ncg) add(ch, ldcg128(src + (size_t)ch * stride + el));
+        if (tight) bar_sync(1, kConsumerThreads);    // every thread has read the maxima and sums
         *reinterpret_cast<float4 *>(red + cg * stride + el) = make_float4(o0, o1, o2, o3);
         if (el == 0) red[cg * stride + dh] = l;
         bar_sync(1, kConsumerThreads);
@@ -1477,9 +1481,13 @@ __global__ void __launch_bounds__(TM ? kTmThreads : kThreads, 1) mega_kernel(con
 #endif
 
     if (c.tid == 0) {
-        for (int i = 0; i < 2 * kMaxStages; ++i) {
+        for (int i = 0; i < kMaxStages; ++i) {
             mbar_init(&c.full[i], kProducerWarps * 32);
             mbar_init(&c.empty[i], kConsumerWarps / 2);   // the four warps that own the stage (or the mover in their place)
+            if (!TM) {
+                mbar_init(&c.misc->tfull[i], kProducerWarps * 32);
+                mbar_init(&c.misc->tempty[i], kConsumerWarps / 2);
+            }
         }
         if (TM) {
             for (int i = 0; i < kTmSlots; ++i) {

@@ -83,6 +83,19 @@ def test_contexts_of_different_footprints_take_turns(batched, first, second, mon
     b.ctx.close()
 
 
+def test_the_longest_context_is_accepted_and_gives_the_same_bits():
+    """The persistent kernel keeps a context's chunk maxima and sums in shared memory, which bounds max_ctx: beside two ring
+    stages of 16 KB, 5.5 KB of fixed data and 1280 bytes, eight bytes per 64 positions fit up to this length at this width."""
+    most = 24096 * 64
+    a, b = Drafter(I.TINY, 1, L=[700]), Drafter(I.TINY, 1, L=[700], max_ctx=most)
+    assert np.array_equal(a.bits(), b.bits())
+    assert b.ctx.launch_count == 1
+    a.ctx.close()
+    b.ctx.close()
+    with pytest.raises(Bd.FastMTPError):
+        Drafter(I.TINY, 1, max_ctx=most + 16 * 64)
+
+
 # more than 256 MB of weights per layer: the sizes at which the switch points come earlier
 LARGE = I.Shape(d=2560, n_q_heads=2, n_kv_heads=1, head_dim=128, ffn=16384, vocab=300, n_layers=1)
 
