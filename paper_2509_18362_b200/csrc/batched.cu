@@ -44,11 +44,13 @@ struct RowGeo {
     int step;                // draft step (0 in a target step)
     const int32_t *n_ext;    // [sequences] or NULL (= M0 for every sequence)
 };
+constexpr int kMaxLen = 1 << 30;      // a longer committed length is the caller's error: flagged like any position without a slot
+__device__ __forceinline__ int geo_len(const KvPtrs &kv, int seq) { return min(max(kv.seq_lens[seq], 0), kMaxLen); }
 __device__ __forceinline__ int geo_next(const RowGeo &g, int seq) { return g.n_ext ? min(max(g.n_ext[seq], 1), g.M0) : g.M0; }
 // Position of row r (before clamping to the cache's capacity); *valid = false for a padding row.
 __device__ __forceinline__ int geo_pos(const RowGeo &g, const KvPtrs &kv, int r, bool *valid) {
     const int seq = r / g.M, m = r - seq * g.M;
-    const int L = max(kv.seq_lens[seq], 0);
+    const int L = geo_len(kv, seq);
     if (g.step > 0) { *valid = true; return L + geo_next(g, seq) - 1 + g.step; }
     const int n = geo_next(g, seq);
     *valid = m < n;
@@ -463,7 +465,7 @@ __global__ void __launch_bounds__(kAttnThreads, 1) attn_kernel(const __grid_cons
             const int s = 2 * lane + u;
             cnt[u] = 0;
             if (s < a.B) {
-                const int len = max(a.kv.seq_lens[s], 0), nx = geo_next(a.geo, s);
+                const int len = geo_len(a.kv, s), nx = geo_next(a.geo, s);
                 const int pos0 = a.geo.step > 0 ? len + nx - 1 + a.geo.step : len;
                 const int nv = a.geo.step > 0 ? 1 : nx;
                 tpos[s] = pos0; tval[s] = nv; tlen[s] = len;

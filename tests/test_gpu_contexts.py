@@ -136,3 +136,21 @@ def test_hidden_states_of_two_sequences_may_start_anywhere():
                 ctx.fastmtp_target_step(w, tok, [Bd.kv(dkv)], B, 1, pool[3:])
         ctx.close()
     del keep
+
+
+@pytest.mark.parametrize("batched", [False, True])
+@pytest.mark.parametrize("E", [1, 3])
+def test_a_committed_length_without_bounds_is_flagged(E, batched, monkeypatch):
+    """The largest length an int32 holds: no slot for the sequence's positions, the other sequence is not affected."""
+    monkeypatch.setenv("FMTP_BATCHED_MIN", "1" if batched else "99")
+    a, one = Drafter(I.TINY, 2, E, L=[5, 70]), Drafter(I.TINY, 1, E, L=[5])
+    a.kv["seq_lens"][1] = 2 ** 31 - 1
+    one.kv["k_pages"], one.kv["v_pages"] = a.kv["k_pages"], a.kv["v_pages"]
+    one.kv["block_table"] = a.kv["block_table"][:1]
+    one.h, one.tok = a.h[:1].contiguous(), a.tok[:1].contiguous()
+    (got, status), want = a.call(), one.bits()
+    n = 2 * I.TINY.d
+    assert status & Bd.DEV_BAD_POS and not status & Bd.DEV_TIMEOUT
+    assert np.array_equal(got[:n], want[:n]) and np.array_equal(got[2 * n:2 * n + 2], want[n:])
+    a.ctx.close()
+    one.ctx.close()
