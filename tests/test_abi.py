@@ -40,3 +40,20 @@ def test_host_argument_validation_needs_no_gpu():
     assert B.lib.fmtp_create(None, None) == -1
     assert B.lib.fmtp_workspace_bytes(None) == 0
     assert B.lib.fmtp_destroy(None) == -1
+
+
+def test_binding_needs_no_private_function_of_torch(monkeypatch):
+    """The short way to the current stream's handle is used where torch has it; without it the binding works all the same."""
+    import importlib.util
+    import torch
+    monkeypatch.delattr(torch._C, "_cuda_getCurrentRawStream", raising=False)
+    spec = importlib.util.spec_from_file_location("paper_2509_18362_b200.binding_without", os.path.join(ROOT, "paper_2509_18362_b200", "binding.py"))
+    B = importlib.util.module_from_spec(spec)
+    spec.loader.exec_module(B)
+
+    class Stream:
+        cuda_stream = 7
+
+    assert B._stream(Stream()) == 7
+    monkeypatch.setattr(torch.cuda, "current_stream", Stream)
+    assert B._stream(None) == 7
