@@ -177,8 +177,7 @@ int configure(fmtp_ctx *c, MegaParams &p, int mode, int B, int M) {
     size_t base = 0;
     int ns = plan(R, M, false, &base);
     if (mode == 0 && R <= 4 && (p.d + c->n_sm - 1) / c->n_sm <= kTileRows) {
-        // (more than four rows run the double-width stream, at which the batched path is faster: 189 against 247-278 us for
-        // one step of five to seven rows)
+        // (the kernel for more than four rows has no restaging form)
         // restaging half way costs 2 us of the projection; worth it where the ring gets deeper (7B shape, four rows: four
         // stages instead of two, draft call of three steps 502 -> 489 us)
         size_t base_split = 0;
@@ -252,8 +251,9 @@ int launch_mega(fmtp_ctx *c, MegaParams &p, cudaStream_t st) {
 // Sequences per launch for a call of B sequences with M rows each: a call with more rows than one
 // launch takes runs as several launches over groups of whole sequences. The largest group is the
 // one whose input vectors still leave a ring of three stages (two at worst; two at once in a target step,
-// where a launch streams all layers: 7B width, 4 layers, two sequences of four rows in one launch of two stages
-// 1000 us, in two launches 1232); 0 if even one sequence does not fit.
+// where a launch streams all layers. Four layers, two sequences of four rows, one launch of two stages against two launches:
+// 7B shape 1000 us / 1232, d = 3584 with ffn 4096 399 / 554, d = 4096 with ffn 2048 393 / 549); 0 if even one sequence does
+// not fit.
 int group_size(fmtp_ctx *c, int mode, int B, int M) {
     for (int i = 0; i < c->n_group_memo; ++i)
         if (c->group_memo[i].mode == mode && c->group_memo[i].B == B && c->group_memo[i].M == M) return c->group_memo[i].G;

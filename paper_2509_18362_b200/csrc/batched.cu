@@ -979,8 +979,9 @@ __global__ void __launch_bounds__(kRowThreads) embed_kernel(const int32_t *token
 // its rows, and gathering head rows in address order keeps the 128 rows of a GEMM tile within a few
 // memory pages (an unsorted subset spreads them over the whole matrix and the address translation
 // misses cost ~25 % of the head's stream rate). Membership bitmap, then a one-block compaction.
-// (The two kernels run under the first kernels of step 0; the head GEMM, the only reader of the sorted ids, waits
-// for the whole chain before it looks at them.)
+// (The two kernels stand before step 0: its first kernel waits for them as for any predecessor, and only its launch and the first
+// weight copies of the projection overlap them. The head GEMM, the only reader of the sorted ids, waits for the whole
+// chain before it looks at them.)
 __global__ void ids_mark_kernel(const int32_t *ids, int N, int V, uint32_t *bitmap, uint32_t *status) {
     chain_release();
     chain_wait();
@@ -1191,7 +1192,10 @@ int batched_draft(const BatchedCall &c, cudaStream_t st, long long *launches) {
     const bool ext = M0 > 1;                       // step 0 carries up to M0 extend rows per sequence
     int inject_gemm = c.inject == 2 ? 1 : 0, inject_attn = c.inject == 3 ? 1 : 0;      // self-test: one launch each
     const int qdim = sh.Hq * sh.dh, kvdim = sh.Hkv * sh.dh;
-    cudaError_t e = cudaMemsetAsync(ws.keys, 0, ws.keys_bytes, st);     // argmax keys and the status word
+    // Argmax keys and the status word. A memset is a full dependency on the stream's earlier work, the one that makes it safe for
+    // the call's kernels, which release each other at their first instruction, to read the call's inputs (hidden states,
+    // lengths, block table, cached K/V, weights) before they wait for their predecessor: something of this kind has to stay first.
+    cudaError_t e = cudaMemsetAsync(ws.keys, 0, ws.keys_bytes, st);
     if (e != cudaSuccess) return (int)e;
 
     // head rows in ascending id order (the debug logits keep the caller's order, so they skip this)
@@ -1324,7 +1328,8 @@ int batched_target(const BatchedTargetCall &c, cudaStream_t st, long long *launc
     const int qdim = sh.Hq * sh.dh, kvdim = sh.Hkv * sh.dh;
     const int NB = (2 * R + 15) / 16 * 16;
     const RowGeo geo{c.M, c.M, 0, nullptr};       // M rows per sequence at positions L .. L+M-1, all of them real
-    cudaError_t e = cudaMemsetAsync(ws.keys, 0, ws.keys_bytes, st);     // argmax keys and the status word
+    // argmax keys and the status word; also the full dependency that the reads ahead of a wait rely on (see batched_draft)
+    cudaError_t e = cudaMemsetAsync(ws.keys, 0, ws.keys_bytes, st);
     if (e != cudaSuccess) return (int)e;
     auto gemm = [&](GemmArgs &g, int n_rows, int Kdim, int lda, const bf16_t *x, int ldx) -> int {
         g.n_rows = n_rows; g.K = Kdim; g.lda = lda; g.x = x; g.ldx = ldx; g.NB = NB; g.R = R;

@@ -43,12 +43,14 @@ def test_batched_attention_edges(page, dh, M, monkeypatch):
     rh, rl = O.target_forward(s, Wt, t, okv)
     close(h.float().cpu().numpy(), rh, "hidden states")
     close(l.float().cpu().numpy(), rl, "logits")
-    for b, n in enumerate(L):                                  # the appended rows, and nothing else, changed
-        for i in range(M):
-            at = (kv["block_table"][b, (n + i) // page], slice(None), (n + i) % page)
-            for k in ("k_pages", "v_pages"):
-                got = Bd.bf16_bits(gpu.dkvs[0][k])
+    for k in ("k_pages", "v_pages"):                           # the appended rows, and nothing else, changed
+        got, want = Bd.bf16_bits(gpu.dkvs[0][k]), kv[k].copy()
+        for b, n in enumerate(L):
+            for i in range(M):
+                at = (kv["block_table"][b, (n + i) // page], slice(None), (n + i) % page)
                 close(O.bf16_to_f64(got[at]), O.bf16_to_f64(okv[0][k][at]), k)
+                want[at] = got[at]
+        assert np.array_equal(got, want)
     if M > 1:                                                  # rows one by one: the same bits
         one = GpuTarget(s, Wt, [kv], max(L) + M)
         one.ctx.close()

@@ -45,6 +45,8 @@ WIDE = replace(I.TINY, d=2048, vocab=1500)
 
 
 @pytest.mark.parametrize("which,shape,B,E", [
+    (1, WIDE, 1, 4),                                   # the persistent kernel changes its shared-memory layout between the steps
+    (1, replace(I.TINY, d=3072, vocab=1500), 1, 4),    # and its projection restages
     (3, I.TINY, 12, 1), (3, I.TINY, 12, 4),            # batched attention, one and several rows: tile copies
     (3, replace(I.TINY, page_size=5), 12, 1), (3, replace(I.TINY, page_size=5), 12, 4),       # 16-byte copies
 ])
