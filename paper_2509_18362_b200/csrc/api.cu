@@ -337,16 +337,17 @@ int fmtp_create(const fmtp_shape *sh, fmtp_ctx **out) {
     // and 8192 558 / 570, 574 / 571 and 647 / 603, of two at 512 597 / 583, three 766 / 581, four at 2048 998 / 586.
     // d = 4096 with ffn 14336 (503 MB): drafts of one, two and three 494 / 508, 536 / 518, 561 / 525.
     // Target calls of two sequences stay here for all that: on the batched path one row at a short context is slower, and what
-    // they return is further from 64 bits (eight layers, appended keys 2.1e-4 against 2.9e-4, fp32 logits of a draft
-    // 4.3e-6 against 8.4e-6: the tensor core truncates along chains of up to 237 products, this kernel's are an eighth).
+    // they return is further from 64 bits (eight layers, appended keys 2.1e-4 against 2.9e-4; fp32 logits of a draft
+    // 4.3e-6 against 8.4e-6; the likely cause: there up to 237 products of 16 go into one fp32 sum, here an eighth as many).
     c->batched_min = g1 + 1;
     {
         const double qd = (double)sh->n_q_heads * sh->head_dim, kvd = (double)sh->n_kv_heads * sh->head_dim;
         const double layer_bytes = 2.0 * (2.0 * sh->d * sh->d + sh->d * (qd + 2 * kvd) + qd * sh->d + 3.0 * sh->d * sh->ffn);
         if (layer_bytes >= 256e6 && c->batched_min > 3) c->batched_min = 3;
         // more than four rows take a second set of accumulators and a shallow ring in the persistent kernel (7B shape, one
-        // step of five rows: 267 us against 189 on the batched path; two sequences of four extend rows, three steps: 974
-        // against 521)
+        // step of five rows 268 us against 174 on the batched path, two sequences of three 357 against 174, of four over three
+        // steps 979 against 495; d = 4096 with ffn 14336, two of three 376 against 185). What such a call returns is as near to
+        // 64 bits either way (hidden states 1.67e-3, appended keys 1e-5), its optional fp32 logits are not (4.3e-6 / 8.4e-6)
         c->persist_rows = layer_bytes >= 256e6 ? 4 : 1 << 30;
     }
     if (const char *v = std::getenv("FMTP_BATCHED_MIN")) {
