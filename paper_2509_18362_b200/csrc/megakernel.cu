@@ -57,6 +57,12 @@ enum Kind { PROJ = 0, QKV = 1, OPROJ = 2, GATEUP = 3, DOWN = 4, HEAD = 5, ATTN =
 // walk it independently with this iterator, each from a single loop.
 struct Prog { int step, layer, kind; };
 
+// A matrix phase's rows x K, tile height, this CTA's row range, and how K is cut into ring stages:
+// into segments of seglen (the projection has two, one per input vector; every other phase one) and each
+// segment into nks_seg stages of kc = KC elements (the last one shorter).
+struct Geom { int rows, K, cap, nks, v0, v1, kc, rs, seglen, nks_seg; };
+constexpr int kMatrixKinds = 6;      // PROJ .. HEAD
+
 struct Misc {   // small shared-memory block
     uint64_t full[kMaxStages];
     uint64_t empty[kMaxStages];
@@ -68,16 +74,19 @@ struct Misc {   // small shared-memory block
     float scale0[kMaxRows];
     float scale1[kMaxRows];
     float ssred[kConsumerWarps][kMaxRows][2];
-    float colred[kTileRows][kMaxRows];
+    float colred[2 * kConsumerWarps][kMaxRows];
     unsigned long long keyred[kConsumerWarps][kMaxRows];
     int tok[kMaxRows];
     int outrow[kMaxRows];   // where the head publishes activation row r (out_row), set when the head's input is staged
     int seqlen[kMaxRows];   // committed length of every sequence and its number of extend rows, read once at kernel start:
     int next[kMaxRows];     // neither changes during a launch, and every phase that needs them saves an L2 round trip
+    Geom geo[kMatrixKinds];          // filled once per launch: row shares and stage counts take divisions, 800 cycles at every phase start
     unsigned long long rowptr[kProducerWarps][32];   // tile row pointers, one line per producer warp
     int flag;
     uint32_t aborted;
 };
+constexpr size_t kMiscBytes = 3584;          // its room in shared memory; what it takes, the longest contexts lack
+static_assert(sizeof(Misc) <= kMiscBytes, "a larger block refuses contexts that were accepted");
 
 // Development aid, compiled only with -DFMTP_PROF: consumer thread 0 of every CTA stamps the
 // global timer at phase boundaries, and warp 0 of each role accumulates the cycles it spends
@@ -261,20 +270,18 @@ __device__ __forceinline__ int out_row(const Cta &c, int r, int step) {
 }
 
 // ---- phase geometry ----------------------------------------------------------------------
-// rows x K of the phase's matrix, tile height, this CTA's row range, and how K is cut into ring stages:
-// into segments of seglen (the projection has two, one per input vector; every other phase one) and each
-// segment into nks_seg stages of kc = KC elements (the last one shorter).
-struct Geom { int rows, K, cap, nks, v0, v1, kc, rs, seglen, nks_seg; };
+// First column and width of stage ks of a tile. A matrix has one segment, the projection two: no division.
 struct StageK { int koff, klen; };
 __device__ __forceinline__ StageK stage_k(const Geom &g, int ks) {
-    const int seg = ks / g.nks_seg, j = ks - seg * g.nks_seg;
+    const bool second = ks >= g.nks_seg;
+    const int j = second ? ks - g.nks_seg : ks;
     StageK s;
-    s.koff = seg * g.seglen + j * g.kc;
+    s.koff = (second ? g.seglen : 0) + j * g.kc;
     s.klen = min(g.kc, g.seglen - j * g.kc);
     return s;
 }
 
-__device__ __forceinline__ Geom geom(const Cta &c, int kind) {
+__device__ __forceinline__ Geom make_geom(const Cta &c, int kind) {
     const MegaParams &p = *c.p;
     Geom g;
     switch (kind) {
@@ -295,6 +302,7 @@ __device__ __forceinline__ Geom geom(const Cta &c, int kind) {
     g.nks = ((kind == PROJ) ? 2 : 1) * g.nks_seg;
     return g;
 }
+__device__ __forceinline__ Geom geom(const Cta &c, int kind) { return c.misc->geo[kind]; }
 
 // Address of weight row `j` (0..31) of the tile whose first virtual row is vr0; nullptr if the
 // tile row is unused.
@@ -671,8 +679,11 @@ __device__ __forceinline__ void consume_tiles(Cta &c, const int kind, const ActS
     const bool has0 = arow < R, has1 = two_sets && (arow + 4 < R);
     const size_t aoff0 = (size_t)arow * act.stride + t * 8, aoff1 = (size_t)(arow + 4) * act.stride + t * 8;
     const uint32_t rs = (uint32_t)geo.rs;
+    const uint32_t ring0 = smem_u32(c.ring) + (uint32_t)(t * 16) + (uint32_t)g * rs;                  // this lane's fragments of ring slot 0
+    const uint32_t act0 = act.in_smem ? smem_u32(abase + aoff0) + (uint32_t)(wi * 64) : 0u;           // and of its warp's first chunk of the input
     const uint4 zero = make_uint4(0, 0, 0, 0);
-    for (int vr0 = geo.v0; vr0 < geo.v1; vr0 += geo.cap) {
+    int stage0 = 0;                                                  // stages of the phase before this tile
+    for (int vr0 = geo.v0; vr0 < geo.v1; vr0 += geo.cap, stage0 += geo.nks) {
         const int nv = min(geo.cap, geo.v1 - vr0);
         const int erow = c.tid >> 3, ecol = c.tid & 7;               // this thread's epilogue element
         const bool evalid = erow < ((kind == GATEUP) ? min(nv, 16) : nv) && ecol < R;
@@ -699,7 +710,6 @@ __device__ __forceinline__ void consume_tiles(Cta &c, const int kind, const ActS
         // which half of the warps takes a stage depends only on the stage's index within the phase,
         // never on how many stages the CTA has seen before: the summation order of a row must not
         // depend on the batch or on earlier calls
-        const int stage0 = ((vr0 - geo.v0) / geo.cap) * geo.nks;
         // slice ring: slot (stage index mod 4) x warp of the owning group x activation row x 512 bytes
         const uint32_t slice_base = smem_u32(c.scr) + (uint32_t)(wi * R) * 512u;
         auto slice_slot = [&](int sa) -> uint32_t { return slice_base + (uint32_t)((sa & 3) * 4 * R) * 512u; };
@@ -713,26 +723,25 @@ __device__ __forceinline__ void consume_tiles(Cta &c, const int kind, const ActS
                 asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst + (uint32_t)r * 512u), "l"(src + (size_t)r * act.stride) : "memory");
             asm volatile("cp.async.commit_group;" ::: "memory");
         };
-        if (gfast) {
-            const int ks0 = ((stage0 & 1) == grp) ? 0 : 1;          // first stage this warp owns
-            if (ks0 < geo.nks) {
-                const StageK s0 = stage_k(geo, ks0);
-                if (s0.klen == 512) slice_fetch(stage0 + ks0, s0);
-            }
+        const int first = ((stage0 & 1) == grp) ? 0 : 1;            // first stage this warp owns
+        if (gfast && first < geo.nks) {
+            const StageK s0 = stage_k(geo, first);
+            if (s0.klen == 512) slice_fetch(stage0 + first, s0);
         }
+        // the second input segment starts: every warp parks the sums of the first (whichever stages of it the warp owned)
+        auto second_segment = [&]() {
+            park<two_sets>(acc, acd, acc0, acd0);
+            if (SPLIT && c.proj_split) {          // (one tile per CTA) the second input vector takes the place of the first
+                bar_sync(1, kConsumerThreads);
+                restage_embeddings(c, reinterpret_cast<bf16_t *>(c.scr), reinterpret_cast<bf16_t *>(c.scr) + (size_t)R * act.stride, act.stride);
+                bar_sync(1, kConsumerThreads);
+            }
+        };
+        if constexpr (TM) {
 #pragma unroll 1
         for (int ks = 0; ks < geo.nks; ++ks) {
-            if (kind == PROJ && ks == geo.nks_seg) {
-                // the second input segment starts: every warp parks the sums of the first (whichever stages of it
-                // the warp owned)
-                park<two_sets>(acc, acd, acc0, acd0);
-                if (SPLIT && c.proj_split) {      // (one tile per CTA) the second input vector takes the place of the first
-                    bar_sync(1, kConsumerThreads);
-                    restage_embeddings(c, reinterpret_cast<bf16_t *>(c.scr), reinterpret_cast<bf16_t *>(c.scr) + (size_t)R * act.stride, act.stride);
-                    bar_sync(1, kConsumerThreads);
-                }
-            }
-            if (TM) {
+            if (kind == PROJ && ks == geo.nks_seg) second_segment();
+            {
                 // the first kTmSlots stages of a phase come through tensor memory (they land while the consumers are still
                 // busy with the previous phase's end), the rest is read from the shared-memory stage directly
                 const bool via_tmem = stage0 + ks < kTmSlots;
@@ -811,7 +820,22 @@ __device__ __forceinline__ void consume_tiles(Cta &c, const int kind, const ActS
                     PROF_ACC(c, 1, c.tid == 0);
                 }
                 if (via_tmem) next_tslot(c);
-            } else if (((stage0 + ks) & 1) == grp) {
+            }
+            next_stage(c);
+        }
+        } else {
+        // Only the stages this warp owns: every other one. What a stage costs beyond its loads and MMAs counts: the ring is full when
+        // a phase starts, its first stages go by at the consumers' rate, not HBM's, and the down projection all the way. With a
+        // division per stage and a pass over the others' stages a stage took 1400 cycles of a warp, now 1000: QKV and O-proj
+        // 5300 -> 4100 cycles, a one-row draft call of three steps 458 -> 448 us, a 28-layer call of four rows 3203 -> 3056.
+        auto skip_stages = [&](int n) { if ((c.slot += n) >= c.n_stages) { c.slot -= c.n_stages; c.parity ^= 1u; } };     // n <= 2 <= ring
+        bool parked = kind != PROJ;
+        skip_stages(first);
+        int ks = first;
+#pragma unroll 1
+        for (; ks < geo.nks; ks += 2, skip_stages(2)) {
+            if (!parked && ks >= geo.nks_seg) { second_segment(); parked = true; }
+            {
                 const int slot = c.slot;
                 const uint32_t parity = c.parity;
                 PROF_T0();
@@ -820,20 +844,20 @@ __device__ __forceinline__ void consume_tiles(Cta &c, const int kind, const ActS
 
                 const StageK sk = stage_k(geo, ks);
                 const int nchunk = (sk.klen + 31) >> 5;
-                const uint32_t sb = smem_u32(c.ring + (size_t)slot * p.stage_bytes) + t * 16 + g * rs;
+                const uint32_t sb = ring0 + (uint32_t)slot * (uint32_t)p.stage_bytes;
                 const int par = g & 1;                    // odd rows: 64-byte halves swapped
-                const size_t kbase = (size_t)sk.koff - (SPLIT && kind == PROJ && c.proj_split && ks >= geo.nks_seg ? (size_t)geo.seglen : 0);
+                const int kbase = sk.koff - (SPLIT && kind == PROJ && c.proj_split && ks >= geo.nks_seg ? geo.seglen : 0);
                 if (nchunk == 16 && (act.in_smem || gfast)) {
                     // the stage width of the large shapes: this warp's chunks
                     // wi, wi + 4, wi + 8, wi + 12 in two batches of two, all loads of a batch issued before its MMAs,
                     // nothing predicated (see the producer: this loop sets the stream rate)
                     uint4 bq[kCpw], dq[two_sets ? kCpw : 1];
                     if (act.in_smem) {
-                        const uint32_t ab = smem_u32(abase + aoff0 + kbase), db = smem_u32(abase + aoff1 + kbase);
+                        const uint32_t ab = act0 + (uint32_t)kbase * 2u, db = ab + (uint32_t)act.stride * 8u;
 #pragma unroll
                         for (int j = 0; j < kCpw; ++j) {
-                            bq[j] = has0 ? lds128_u32(ab + (wi + 4 * j) * 64) : zero;
-                            if (two_sets) dq[two_sets ? j : 0] = has1 ? lds128_u32(db + (wi + 4 * j) * 64) : zero;
+                            bq[j] = has0 ? lds128_u32(ab + j * 256) : zero;
+                            if (two_sets) dq[two_sets ? j : 0] = has1 ? lds128_u32(db + j * 256) : zero;
                         }
                     } else {
                         // request the slices of the next owned stage, then wait for this stage's (requested one owned
@@ -878,7 +902,12 @@ __device__ __forceinline__ void consume_tiles(Cta &c, const int kind, const ActS
                 if (c.lane == 0) mbar_arrive(&c.empty[slot]);
                 PROF_ACC(c, 1, c.tid == 0);
             }
-            next_stage(c);
+        }
+        if (!parked) second_segment();
+        if (ks > geo.nks) {                       // one stage too far
+            if (c.slot == 0) { c.slot = c.n_stages; c.parity ^= 1u; }
+            --c.slot;
+        }
         }
         // cross-warp reduction in a fixed order
         PROF_T0();
@@ -1451,7 +1480,7 @@ __global__ void __launch_bounds__(TM ? kTmThreads : kThreads, 1) mega_kernel(con
     Cta c;
     c.p = &p;
     c.misc = reinterpret_cast<Misc *>(smem);
-    size_t off = (sizeof(Misc) + 127) & ~size_t(127);
+    size_t off = kMiscBytes;
     c.red = reinterpret_cast<float *>(smem + off);
     off += red_bytes(p.R);
     c.scr = smem + off;
@@ -1500,6 +1529,7 @@ __global__ void __launch_bounds__(TM ? kTmThreads : kThreads, 1) mega_kernel(con
         c.misc->aborted = 0;
         mbar_fence_init();
     }
+    if (c.tid >= 32 && c.tid < 32 + kMatrixKinds) c.misc->geo[c.tid - 32] = make_geom(c, c.tid - 32);
     if (c.tid < p.B) {
         c.misc->seqlen[c.tid] = p.kvs[0].seq_lens[c.tid];
         c.misc->next[c.tid] = (p.mode == 0 && p.n_ext) ? min(max(p.n_ext[c.tid], 1), p.M) : p.M;
@@ -1874,7 +1904,7 @@ extern "C" int fmtp_prof_read(unsigned long long *host, size_t bytes) {
 #endif
 
 size_t mega_smem_bytes(const MegaParams &p) {
-    size_t off = (sizeof(Misc) + 127) & ~size_t(127);
+    size_t off = kMiscBytes;
     const size_t first = off;
     off += ((size_t)2 * kConsumerWarps * kTileRows * p.R * sizeof(float) + 127) & ~size_t(127);
     off += (size_t)p.scratch_smem;
@@ -1889,7 +1919,7 @@ size_t mega_smem_bytes(const MegaParams &p) {
 }
 
 size_t mega_fixed_smem(int R) {
-    size_t off = (sizeof(Misc) + 127) & ~size_t(127);
+    size_t off = kMiscBytes;
     off += ((size_t)2 * kConsumerWarps * kTileRows * R * sizeof(float) + 127) & ~size_t(127);
     return off;
 }
