@@ -63,6 +63,21 @@ struct Prog { int step, layer, kind; };
 struct Geom { int rows, K, cap, nks, v0, v1, kc, rs, seglen, nks_seg; };
 constexpr int kMatrixKinds = 6;      // PROJ .. HEAD
 
+// The addresses a matrix phase reads and writes. They are chosen, and the first tile's epilogue operands requested, between
+// a CTA's arrival at the barrier before the phase and the wait there: the parameter block is larger than the constant cache's
+// first level, so every phase met its pointers with misses (450 cycles at its start, 350 more at its first tile).
+struct PhaseIo {
+    const bf16_t *in_hi, *in_lo;     // input vector [R][in_stride], in_len elements
+    const float *sstab;              // partial sums of squares that normalise it, or NULL
+    const float *res;                // [R][d] added to the dot product, or NULL
+    const bf16_t *gain, *gain2;      // norm gains applied to the result for the next phase (gain2: to the recursed state), or NULL
+    const int32_t *ids;              // head: subset or NULL
+    float *out;                      // fp32 result [R][out_stride], or NULL
+    bf16_t *out_hi, *out_lo;         // result x gain [R][out_split], or NULL
+    int in_stride, in_len, out_stride, out_split;
+    int recurse;                     // down projection of a draft: publishes the recursed state as well
+};
+
 struct Misc {   // small shared-memory block
     uint64_t full[kMaxStages];
     uint64_t empty[kMaxStages];
@@ -80,6 +95,7 @@ struct Misc {   // small shared-memory block
     int outrow[kMaxRows];   // where the head publishes activation row r (out_row), set when the head's input is staged
     int seqlen[kMaxRows];   // committed length of every sequence and its number of extend rows, read once at kernel start:
     int next[kMaxRows];     // neither changes during a launch, and every phase that needs them saves an L2 round trip
+    PhaseIo io;                      // of the current matrix phase
     Geom geo[kMatrixKinds];          // filled once per launch: row shares and stage counts take divisions, 800 cycles at every phase start
     unsigned long long rowptr[kProducerWarps][32];   // tile row pointers, one line per producer warp
     int flag;
@@ -197,24 +213,27 @@ __device__ __forceinline__ void do_abort(const Cta &c) {
     atomicExch(c.p->s.abort_flag, 1u);
 }
 
-// Grid-wide barrier among the consumer threads of all CTAs (the producer warp never joins).
-__device__ __forceinline__ void grid_barrier(Cta &c) {
+// Grid-wide barrier among the consumer threads of all CTAs (the producer warps never join). `between` is what every
+// thread does after the CTA has arrived and before it waits.
+template <class F>
+__device__ __forceinline__ void grid_barrier(Cta &c, F &&between) {
     bar_sync(1, kConsumerThreads);
     c.bar_target += (uint32_t)(c.grid + c.p->extra_arrivals);     // extra_arrivals: 0, or 1 in the wait-timeout self-test
     if (c.tid == 0) {
         // the arrival is a release at device scope: it orders every write the CTA made before the bar.sync above
         // (the waiting side reads with acquire), so no separate fences are needed
         asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(c.p->s.barrier) : "memory");
-        if (!aborted(c)) {
-            uint32_t n = 0;
-            unsigned long long t0 = 0;
-            while ((int32_t)(ld_acquire_u32(c.p->s.barrier) - c.bar_target) < 0) {
-                if ((++n & 255u) == 255u) {
-                    if (ldcg_u32(c.p->s.abort_flag) != 0) { c.misc->aborted = 1; break; }
-                    unsigned long long now = global_timer_ns();
-                    if (t0 == 0) t0 = now;
-                    else if (now - t0 > c.p->wait_limit_ns) { do_abort(c); break; }
-                }
+    }
+    between();
+    if (c.tid == 0 && !aborted(c)) {
+        uint32_t n = 0;
+        unsigned long long t0 = 0;
+        while ((int32_t)(ld_acquire_u32(c.p->s.barrier) - c.bar_target) < 0) {
+            if ((++n & 255u) == 255u) {
+                if (ldcg_u32(c.p->s.abort_flag) != 0) { c.misc->aborted = 1; break; }
+                unsigned long long now = global_timer_ns();
+                if (t0 == 0) t0 = now;
+                else if (now - t0 > c.p->wait_limit_ns) { do_abort(c); break; }
             }
         }
     }
@@ -488,14 +507,17 @@ struct SqAcc {
     float a, b;
 };
 
-// What the per-row epilogue of a matrix phase needs besides the value.
+// Operands of the epilogue that do not depend on the dot product (residual value, norm gains, the
+// token id of a head row): loaded when the tile starts, so their latency hides behind the stream.
+struct EpiPre { float resid, g0, g1; int id; };
+struct Phase : Prog {
+    EpiPre pre;                      // of this thread's element of the first tile
+};
+
+// What the per-row epilogue of a matrix phase keeps.
 struct EpiCtx {
     SqAcc sq;
     unsigned long long best;     // running (logit, id) maximum of this thread (output head)
-    const LayerPtrs *L;
-    const bf16_t *gnext;         // gain applied after the down projection (next layer's or the final norm's)
-    int step;
-    bool to_next_layer;          // target mode, not the last layer: the result feeds the next layer
 };
 
 __device__ __forceinline__ void store_split(bf16_t *hi, bf16_t *lo, size_t idx, float v) {
@@ -505,73 +527,45 @@ __device__ __forceinline__ void store_split(bf16_t *hi, bf16_t *lo, size_t idx, 
     lo[idx] = l;
 }
 
-// Operands of the epilogue that do not depend on the dot product (residual value, norm gains, the
-// token id of a head row): loaded when the tile starts, so their latency hides behind the stream.
-struct EpiPre { float resid, g0, g1; int id; };
-__device__ __forceinline__ EpiPre epi_prefetch(const Cta &c, int kind, const EpiCtx &x, int row, int col, bool valid) {
-    const MegaParams &p = *c.p;
+__device__ __forceinline__ EpiPre epi_prefetch(const Cta &c, const PhaseIo &io, int row, int col, bool valid) {
     EpiPre e;
     e.resid = 0.f; e.g0 = 0.f; e.g1 = 0.f; e.id = row;
     if (!valid) return e;
-    switch (kind) {
-        case PROJ: e.g0 = bf16bits_f32(x.L->g_in[row]); break;
-        case OPROJ:
-            e.resid = ldcg_f32(p.s.x0 + (size_t)col * p.d + row);
-            e.g0 = bf16bits_f32(x.L->g_post[row]);
-            break;
-        case DOWN:
-            e.resid = ldcg_f32(p.s.x1 + (size_t)col * p.d + row);
-            e.g0 = bf16bits_f32(x.gnext[row]);
-            if (p.mode == 0) e.g1 = bf16bits_f32(p.g_hnorm[row]);
-            break;
-        case HEAD:
-            if (p.ids) e.id = p.ids[row];
-            break;
-        default: break;
-    }
+    // the residual was written by this very thread: rows are shared out alike in every phase whose result has d rows
+    if (io.res) e.resid = ldcg_f32(io.res + (size_t)col * c.p->d + row);
+    if (io.gain) e.g0 = bf16bits_f32(io.gain[row]);
+    if (io.gain2) e.g1 = bf16bits_f32(io.gain2[row]);
+    if (io.ids) e.id = io.ids[row];
     return e;
+}
+// Whether this thread has an element (row, activation row) of a tile of nv rows.
+__device__ __forceinline__ bool epi_valid(const Cta &c, int kind, int nv) {
+    return (c.tid >> 3) < (kind == GATEUP ? min(nv, kTileRows / 2) : nv) && (c.tid & 7) < c.R;
 }
 
 // Epilogue of one (virtual row, activation row): what the phase does with the finished dot product.
-__device__ __forceinline__ void epilogue(const Cta &c, int kind, EpiCtx &x, const EpiPre &pre, int row, int col, float v, float up) {
+__device__ __forceinline__ void epilogue(const Cta &c, const Phase &ph, EpiCtx &x, const EpiPre &pre, int row, int col, float v, float up) {
     const MegaParams &p = *c.p;
-    const Scratch &s = p.s;
-    switch (kind) {
-        case PROJ: {
-            s.x0[(size_t)col * p.d + row] = v;
-            store_split(s.actD_hi, s.actD_lo, (size_t)col * p.dp + row, v * pre.g0);
-            x.sq.a += v * v;
-            break;
-        }
+    const PhaseIo &io = c.misc->io;
+    switch (ph.kind) {
         case QKV:
-            s.qkv[(size_t)col * (p.qdim + 2 * p.kvdim) + row] = v * c.misc->scale0[col];
+            io.out[(size_t)col * io.out_stride + row] = v * c.misc->scale0[col];
             break;
-        case OPROJ: {
-            float r = pre.resid + v;
-            s.x1[(size_t)col * p.d + row] = r;
-            store_split(s.actP_hi, s.actP_lo, (size_t)col * p.dp + row, r * pre.g0);
-            x.sq.a += r * r;
-            break;
-        }
         case GATEUP: {
             float sc = c.misc->scale0[col];
             float gt = v * sc, u = up * sc;
-            store_split(s.actF_hi, s.actF_lo, (size_t)col * p.Fp + row, gt / (1.f + expf(-gt)) * u);
+            store_split(io.out_hi, io.out_lo, (size_t)col * io.out_split + row, gt / (1.f + expf(-gt)) * u);
             break;
         }
-        case DOWN: {
-            float r = pre.resid + v;
+        case PROJ: case OPROJ: case DOWN: {
+            float r = io.res ? pre.resid + v : v;
             float y = r * pre.g0;
             x.sq.a += r * r;
-            if (x.to_next_layer) {
-                s.x0[(size_t)col * p.d + row] = r;
-                store_split(s.actD_hi, s.actD_lo, (size_t)col * p.dp + row, y);
-            } else {
-                store_split(s.actH_hi, s.actH_lo, (size_t)col * p.dp + row, y);
-                if (p.mode == 0) {
-                    store_split(s.actR_hi, s.actR_lo, (size_t)col * p.dp + row, y * pre.g1);
-                    x.sq.b += y * y;
-                }
+            if (io.out) io.out[(size_t)col * io.out_stride + row] = r;
+            store_split(io.out_hi, io.out_lo, (size_t)col * io.out_split + row, y);
+            if (io.recurse) {
+                store_split(p.s.actR_hi, p.s.actR_lo, (size_t)col * p.dp + row, y * pre.g1);
+                x.sq.b += y * y;
             }
             break;
         }
@@ -586,13 +580,62 @@ __device__ __forceinline__ void epilogue(const Cta &c, int kind, EpiCtx &x, cons
                 lv = bf16bits_f32(lb);
             } else if (p.out_logits_f32) {
                 const int orow = c.misc->outrow[col];
-                if (orow >= 0) p.out_logits_f32[((size_t)orow * p.K + x.step) * p.N + row] = v * c.misc->scale0[col];
+                if (orow >= 0) p.out_logits_f32[((size_t)orow * p.K + ph.step) * p.N + row] = v * c.misc->scale0[col];
             }
             unsigned long long key = argmax_key(lv, (uint32_t)id);
             x.best = key > x.best ? key : x.best;
             break;
         }
     }
+}
+
+// The phase of program position g (c.R is its row count already); every consumer thread calls it, between two CTA barriers.
+// PRE: the first tile's epilogue operands are kept from here on (with two sets of accumulators there are no registers for them).
+template <bool PRE>
+__device__ __forceinline__ void make_phase(const Cta &c, Phase &g) {
+    const MegaParams &p = *c.p;
+    const Scratch &s = p.s;
+    if (g.kind >= kMatrixKinds) return;
+    PhaseIo io;
+    io.in_hi = s.actH_hi; io.in_lo = s.actH_lo; io.in_stride = p.dp; io.in_len = p.d;
+    io.sstab = nullptr; io.res = nullptr; io.gain = nullptr; io.gain2 = nullptr; io.ids = nullptr;
+    io.out = nullptr; io.out_hi = nullptr; io.out_lo = nullptr; io.out_stride = p.d; io.out_split = p.dp;
+    io.recurse = 0;
+    const LayerPtrs &L = p.layers[g.layer];
+    switch (g.kind) {
+        case PROJ:
+            io.in_hi = s.actR_hi; io.in_lo = s.actR_lo;
+            io.gain = L.g_in; io.out = s.x0; io.out_hi = s.actD_hi; io.out_lo = s.actD_lo;
+            break;
+        case QKV:
+            io.in_hi = s.actD_hi; io.in_lo = s.actD_lo; io.sstab = s.ssA;
+            io.out = s.qkv; io.out_stride = p.qdim + 2 * p.kvdim;
+            break;
+        case OPROJ:
+            io.in_hi = s.actO_hi; io.in_lo = s.actO_lo; io.in_stride = p.qp; io.in_len = p.qdim;
+            io.res = s.x0; io.gain = L.g_post; io.out = s.x1; io.out_hi = s.actP_hi; io.out_lo = s.actP_lo;
+            break;
+        case GATEUP:
+            io.in_hi = s.actP_hi; io.in_lo = s.actP_lo; io.sstab = s.ssB;
+            io.out_hi = s.actF_hi; io.out_lo = s.actF_lo; io.out_split = p.Fp;
+            break;
+        case DOWN:
+            io.in_hi = s.actF_hi; io.in_lo = s.actF_lo; io.in_stride = p.Fp; io.in_len = p.Fp;    // pad beyond F is zero
+            io.res = s.x1;
+            if (p.mode == 1 && g.layer + 1 < p.n_layers) {                                        // the result feeds the next layer
+                io.gain = p.layers[g.layer + 1].g_in; io.out = s.x0; io.out_hi = s.actD_hi; io.out_lo = s.actD_lo;
+            } else {
+                io.gain = p.g_final; io.out_hi = s.actH_hi; io.out_lo = s.actH_lo;
+                if (p.mode == 0) { io.gain2 = p.g_hnorm; io.recurse = 1; }
+            }
+            break;
+        default:                                                                                  // HEAD
+            io.sstab = s.ssC; io.ids = p.ids;
+            break;
+    }
+    const Geom &geo = c.misc->geo[g.kind];
+    if (PRE) g.pre = epi_prefetch(c, io, geo.v0 + (c.tid >> 3), c.tid & 7, epi_valid(c, g.kind, min(geo.cap, geo.v1 - geo.v0)));
+    if (c.tid == kConsumerThreads - 1) c.misc->io = io;
 }
 
 // One chunk (32 weight rows x 32 k) of a stage: four MMAs per activation set.
@@ -629,6 +672,21 @@ __device__ __forceinline__ void park(float (&acc)[2][2][4], float (&acd)[2][2][4
         }
 }
 
+// Eight products v * g of packed bf16 pairs as hi/lo parts, 16 bytes each.
+__device__ __forceinline__ void store_product8(bf16_t *hi, bf16_t *lo, int at, const uint32_t (&vw)[4], const uint32_t (&gw)[4]) {
+    uint32_t h[4], l[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        uint16_t h0, l0, h1, l1;
+        split_bf16(bf16lo_f32(vw[q]) * bf16lo_f32(gw[q]), h0, l0);
+        split_bf16(bf16hi_f32(vw[q]) * bf16hi_f32(gw[q]), h1, l1);
+        h[q] = (uint32_t)h0 | ((uint32_t)h1 << 16);
+        l[q] = (uint32_t)l0 | ((uint32_t)l1 << 16);
+    }
+    *reinterpret_cast<uint4 *>(hi + at) = make_uint4(h[0], h[1], h[2], h[3]);
+    *reinterpret_cast<uint4 *>(lo + at) = make_uint4(l[0], l[1], l[2], l[3]);
+}
+
 // The token embeddings of all rows over the first input vector in the staging area (projection with proj_split).
 __device__ __forceinline__ void restage_embeddings(const Cta &c, bf16_t *a_hi, bf16_t *a_lo, int st) {
     const MegaParams &p = *c.p;
@@ -638,17 +696,7 @@ __device__ __forceinline__ void restage_embeddings(const Cta &c, bf16_t *a_hi, b
         const int r = i / per_row, k = (i - r * per_row) * 8;
         const uint4 v = ldnc128(p.embed + (size_t)c.misc->tok[r] * p.d + k), g = ldnc128(p.g_enorm + k);
         const uint32_t vw[4] = {v.x, v.y, v.z, v.w}, gw[4] = {g.x, g.y, g.z, g.w};
-        uint32_t h[4], l[4];
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            uint16_t h0, l0, h1, l1;
-            split_bf16(bf16lo_f32(vw[q]) * bf16lo_f32(gw[q]), h0, l0);
-            split_bf16(bf16hi_f32(vw[q]) * bf16hi_f32(gw[q]), h1, l1);
-            h[q] = (uint32_t)h0 | ((uint32_t)h1 << 16);
-            l[q] = (uint32_t)l0 | ((uint32_t)l1 << 16);
-        }
-        *reinterpret_cast<uint4 *>(a_hi + (size_t)r * st + k) = make_uint4(h[0], h[1], h[2], h[3]);
-        *reinterpret_cast<uint4 *>(a_lo + (size_t)r * st + k) = make_uint4(l[0], l[1], l[2], l[3]);
+        store_product8(a_hi, a_lo, r * st + k, vw, gw);
     }
 }
 
@@ -668,9 +716,10 @@ __device__ __forceinline__ void restage_embeddings(const Cta &c, bf16_t *a_hi, b
 // stages of a phase) or by sixteen conflict-free 128-bit loads from the shared-memory stage (the rest), and the
 // warp's four k chunks of a stage are 8*(j >> 1) + 2*wi + (j & 1), j = 0..3.
 template <bool two_sets, bool TM, bool SPLIT>
-__device__ __forceinline__ void consume_tiles(Cta &c, const int kind, const ActSrc &act, EpiCtx &ex) {
+__device__ __forceinline__ void consume_tiles(Cta &c, const Phase &ph, const ActSrc &act, EpiCtx &ex) {
     const MegaParams &p = *c.p;
-    const Geom geo = geom(c, kind);
+    const int kind = ph.kind;
+    const Geom &geo = c.misc->geo[kind];
     const int R = c.R;
     const int g = c.lane >> 2, t = c.lane & 3;
     const int grp = c.warp >> 2, wi = c.warp & 3;
@@ -686,8 +735,8 @@ __device__ __forceinline__ void consume_tiles(Cta &c, const int kind, const ActS
     for (int vr0 = geo.v0; vr0 < geo.v1; vr0 += geo.cap, stage0 += geo.nks) {
         const int nv = min(geo.cap, geo.v1 - vr0);
         const int erow = c.tid >> 3, ecol = c.tid & 7;               // this thread's epilogue element
-        const bool evalid = erow < ((kind == GATEUP) ? min(nv, 16) : nv) && ecol < R;
-        const EpiPre pre = epi_prefetch(c, kind, ex, vr0 + erow, ecol, evalid);
+        const bool evalid = epi_valid(c, kind, nv);
+        const EpiPre pre = !two_sets && !TM && vr0 == geo.v0 ? ph.pre : epi_prefetch(c, c.misc->io, vr0 + erow, ecol, evalid);
         float acc[2][2][4], acd[2][2][4], acc0[2][4], acd0[2][4];
 #pragma unroll
         for (int i = 0; i < 2; ++i)
@@ -942,7 +991,7 @@ __device__ __forceinline__ void consume_tiles(Cta &c, const int kind, const ActS
 #pragma unroll
                     for (int w = 0; w < kConsumerWarps; ++w) b += rb[(size_t)w * kTileRows * R + (row + 16) * R + col];
                 }
-                epilogue(c, kind, ex, pre, vr0 + row, col, a, b);
+                epilogue(c, ph, ex, pre, vr0 + row, col, a, b);
             }
         }
         c.redbuf ^= 1;
@@ -990,44 +1039,43 @@ __device__ __forceinline__ void switch_layout(Cta &c) {
     c.parity = 0;
 }
 
-// Copies R rows of a hi/lo activation pair from global scratch into the shared staging area.
-// `len` elements per row (multiple of 8), rows `stride_s` apart in shared memory, starting at
-// element offset `dst_off`.
-// With remap_step >= 1 row r is read from global row src_row(r, remap_step): the projection of draft step 1
-// continues each sequence's last extend row.
+// Copies R rows of a hi/lo activation pair from global scratch into the shared staging area: `len` elements per row
+// (multiple of 8), rows `sstride` apart in shared memory. With remap_step >= 1 row r is read from global row
+// src_row(r, remap_step): the projection of draft step 1 continues each sequence's last extend row. A thread's pieces are 256
+// apart: their rows are counted on, not divided out (eight divisions per thread cost as much as the loads: 2400 cycles,
+// now 1700).
 template <int U>
-__device__ __forceinline__ void stage_hilo_impl(const Cta &c, const bf16_t *ghi, const bf16_t *glo, int gstride, int len, bf16_t *shi,
-                                                bf16_t *slo, int sstride, int dst_off, int remap_step) {
-    const int per_row = len / 8;
-    const int total = c.R * per_row;
-    // U units per thread and round: 2 U loads in flight before the first store waits
+__device__ __forceinline__ void stage_hilo(const Cta &c, const bf16_t *ghi, const bf16_t *glo, int gstride, int len, bf16_t *shi,
+                                           bf16_t *slo, int sstride, int remap_step) {
+    const int per_row = len >> 3;
+    int r = 0, k = c.tid;
+    auto wrap = [&]() { while (k >= per_row && r < c.R) { k -= per_row; ++r; } };
+    wrap();
+    // U pieces per thread and round: 2 U loads in flight before the first store waits
 #pragma unroll 1
-    for (int i0 = c.tid; i0 < total; i0 += U * kConsumerThreads) {
+    while (r < c.R) {
         uint4 a[U], b[U];
+        const int r0 = r, k0 = k;
 #pragma unroll
         for (int q = 0; q < U; ++q) {
-            int i = min(i0 + q * kConsumerThreads, total - 1);
-            int r = i / per_row, k = (i - r * per_row) * 8;
-            const int rs = remap_step > 0 ? src_row(c, r, remap_step) : r;
-            a[q] = ldcg128(ghi + (size_t)rs * gstride + k);
-            b[q] = ldcg128(glo + (size_t)rs * gstride + k);
+            const int rr = min(r, c.R - 1);                  // beyond the last row: the last one once more, not stored
+            const size_t src = (size_t)(remap_step > 0 ? src_row(c, rr, remap_step) : rr) * gstride + (r < c.R ? k * 8 : 0);
+            a[q] = ldcg128(ghi + src);
+            b[q] = ldcg128(glo + src);
+            k += kConsumerThreads;
+            wrap();
         }
+        r = r0; k = k0;
 #pragma unroll
         for (int q = 0; q < U; ++q) {
-            int i = i0 + q * kConsumerThreads;
-            if (i < total) {
-                int r = i / per_row, k = (i - r * per_row) * 8;
-                *reinterpret_cast<uint4 *>(shi + (size_t)r * sstride + dst_off + k) = a[q];
-                *reinterpret_cast<uint4 *>(slo + (size_t)r * sstride + dst_off + k) = b[q];
+            if (r < c.R) {
+                *reinterpret_cast<uint4 *>(shi + r * sstride + k * 8) = a[q];
+                *reinterpret_cast<uint4 *>(slo + r * sstride + k * 8) = b[q];
             }
+            k += kConsumerThreads;
+            wrap();
         }
     }
-}
-__device__ __forceinline__ void stage_hilo(const Cta &c, const bf16_t *ghi, const bf16_t *glo, int gstride, int len, bf16_t *shi,
-                                           bf16_t *slo, int sstride, int dst_off, int remap_step = 0) {
-    // several rows: twice as many loads per round, so that the copy stays at one or two L2 round trips
-    if (c.R * (len / 8) > 4 * kConsumerThreads) stage_hilo_impl<8>(c, ghi, glo, gstride, len, shi, slo, sstride, dst_off, remap_step);
-    else stage_hilo_impl<4>(c, ghi, glo, gstride, len, shi, slo, sstride, dst_off, remap_step);
 }
 
 __device__ __forceinline__ void flush_sq(const Cta &c, const SqAcc &q, float *tblA, float *tblB) {
@@ -1656,207 +1704,204 @@ __global__ void __launch_bounds__(TM ? kTmThreads : kThreads, 1) mega_kernel(con
 
     // ---------------- consumers: one loop over the phase program; every phase ends in a grid barrier
     setmaxnreg_inc<TM ? kTmConsumerRegs : kConsumerRegs>();
-    bf16_t *s_hi = reinterpret_cast<bf16_t *>(c.scr);
     EpiCtx ex;
     ex.best = 0ull;
-    Prog g;
+    Phase ph;
+    ph.pre = EpiPre{0.f, 0.f, 0.f, 0};
+    prog_begin(p, ph);
+    make_phase<!TWO && !TM>(c, ph);
+    bar_sync(1, kConsumerThreads);
 #pragma unroll 1
-    for (prog_begin(p, g); g.kind != DONE; prog_next(p, g)) {
-        const int kind = g.kind, step = g.step;
-        set_step_rows(c, step);
+    while (ph.kind != DONE) {
+        const int kind = ph.kind, step = ph.step;
         const int R = c.R;
-        const LayerPtrs &L = p.layers[g.layer];
-        const bool last_layer = (p.mode == 0) || (g.layer + 1 == p.n_layers);
         ex.sq.a = 0.f; ex.sq.b = 0.f;
-        ex.L = &L;
-        ex.step = step;
-        ex.to_next_layer = (p.mode == 1) && !last_layer;
-        ex.gnext = ex.to_next_layer ? p.layers[g.layer + 1].g_in : p.g_final;
         PROF(c, kind * 8);
-        if (p.n_stages2 > 0 && step == 1 && kind == PROJ) {
-            switch_layout(c);
-            s_hi = reinterpret_cast<bf16_t *>(c.scr);
-        }
+        if (p.n_stages2 > 0 && step == 1 && kind == PROJ) switch_layout(c);
         if (kind == ATTN) {
-            attention_phase<DH>(c, p.kvs[g.layer], step);
-            PROF(c, kind * 8 + 2);
-            grid_barrier(c);
-            continue;
-        }
-        if (kind == MERGE) {
-            merge_phase(c, p.kvs[g.layer], step);
-            PROF(c, kind * 8 + 2);
-            grid_barrier(c);
-            continue;
-        }
-        if (kind == EMBED) {
+            attention_phase<DH>(c, p.kvs[ph.layer], step);
+        } else if (kind == MERGE) {
+            merge_phase(c, p.kvs[ph.layer], step);
+        } else if (kind == EMBED) {
             // ---- target: x0 = Emb(tok), CTA-sliced over d; thread = (row slot tid>>3, activation row tid&7)
-            int r0 = (int)(((long long)c.cta * p.d) / c.grid), r1 = (int)(((long long)(c.cta + 1) * p.d) / c.grid);
-            for (int row = r0 + (c.tid >> 3); row < r1; row += kTileRows) {
+            const Geom &geo = c.misc->geo[OPROJ];          // the shares of d rows
+            const bf16_t *g_in = p.layers[0].g_in;
+            for (int row = geo.v0 + (c.tid >> 3); row < geo.v1; row += kTileRows) {
                 int col = c.tid & 7;
                 if (col < R) {
                     int tok = p.tokens[col];
                     if ((unsigned)tok >= (unsigned)p.V) { raise(c, kDevBadToken); tok = 0; }
                     float v = bf16bits_f32(p.embed[(size_t)tok * p.d + row]);
                     p.s.x0[(size_t)col * p.d + row] = v;
-                    store_split(p.s.actD_hi, p.s.actD_lo, (size_t)col * p.dp + row, v * bf16bits_f32(L.g_in[row]));
+                    store_split(p.s.actD_hi, p.s.actD_lo, (size_t)col * p.dp + row, v * bf16bits_f32(g_in[row]));
                     ex.sq.a += v * v;
                 }
             }
             flush_sq(c, ex.sq, p.s.ssA, nullptr);
-            PROF(c, kind * 8 + 2);
-            grid_barrier(c);
-            continue;
-        }
-
-        // ============ matrix phases: stage the input vector(s) in shared memory ...
-        const int klen = (kind == PROJ) ? (SPLIT && c.proj_split ? p.d : 2 * p.d) : (kind == OPROJ) ? p.qdim : (kind == DOWN) ? p.F : p.d;
-        const int st = ((klen + 31) & ~31) + 32;      // +64 B: rows land in different banks
-        bf16_t *a_hi = s_hi, *a_lo = s_hi + (size_t)R * st;
-        ActSrc act{a_hi, a_lo, st, true};
-        if (kind == PROJ) {
-            // ---- x0 = W_p [ rms(h) ; rms(Emb(tok)) ]
-            // loads that do not depend on each other are issued first: the previous step's argmax key,
-            // the partial sums that normalise the recursed state, and that state itself
-            unsigned long long key = 0ull;
-            if (step > 0 && c.tid < R) key = ldcg_u64(p.s.keys + (size_t)(step - 1) * kMaxRows + c.tid);
-            float pvc[kPartialRegs], pvd[kPartialRegs];
-            const bool renorm = step > 0 && c.warp < R;
-            if (renorm) {
-                const int col = src_row(c, c.warp, step);      // step 1 continues each sequence's last extend row
-                load_partials(c, p.s.ssC, col, pvc);
-                load_partials(c, p.s.ssD, col, pvd);
-            }
-            if (step > 0) stage_hilo(c, p.s.actR_hi, p.s.actR_lo, p.dp, p.d, a_hi, a_lo, st, 0, step);
-            if (renorm) {
-                // recursed state: h = (x2*g_final) * s_x; rms(h) adds s_h = rsqrt(s_x^2 * mean((x2 g)^2) + eps)
-                float sx = rsqrtf(reduce_partials(pvc) / (float)p.d + p.eps);
-                float sy = reduce_partials(pvd) / (float)p.d;
-                if (c.lane == 0) c.misc->scale0[c.warp] = sx * rsqrtf(sx * sx * sy + p.eps);
-            }
-            if (c.tid < R) {
-                int tok;
-                if (step == 0) {
-                    const int b = c.tid / p.M;         // a padding row's token is never looked at
-                    tok = (c.tid - b * p.M < seq_next(c, b)) ? p.tokens[c.tid] : 0;
-                } else {
-                    if ((key >> 32) == 0ull) raise(c, kDevAllNan);
-                    tok = (int)argmax_key_id(key);
-                    if (c.cta == 0) p.out_tokens[(size_t)c.tid * p.K + (step - 1)] = tok;
-                }
-                if ((unsigned)tok >= (unsigned)p.V) { raise(c, kDevBadToken); tok = 0; }
-                c.misc->tok[c.tid] = tok;
-            }
-            bar_sync(1, kConsumerThreads);
-#pragma unroll 1
-            for (int r = 0; r < R; ++r) {
-                float sqh = 0.f, sqe = 0.f;
-                const bf16_t *erow = p.embed + (size_t)c.misc->tok[r] * p.d;
-                for (int k = c.tid * 8; k < p.d; k += kConsumerThreads * 8) {
-                    uint4 ev = ldnc128(erow + k);
-                    uint4 gv = ldnc128(p.g_enorm + k);
-                    uint32_t ew[4] = {ev.x, ev.y, ev.z, ev.w}, gw[4] = {gv.x, gv.y, gv.z, gv.w};
-#pragma unroll
-                    for (int i = 0; i < 4; ++i) {
-                        float e0 = bf16lo_f32(ew[i]), e1 = bf16hi_f32(ew[i]);
-                        sqe += e0 * e0 + e1 * e1;
-                        if (!SPLIT || !c.proj_split) {
-                            store_split(a_hi, a_lo, (size_t)r * st + p.d + k + 2 * i, e0 * bf16lo_f32(gw[i]));
-                            store_split(a_hi, a_lo, (size_t)r * st + p.d + k + 2 * i + 1, e1 * bf16hi_f32(gw[i]));
-                        }
-                    }
-                    if (step == 0) {
-                        uint4 hv = ldnc128(p.h_last + (size_t)r * p.d + k);
-                        uint4 hg = ldnc128(p.g_hnorm + k);
-                        uint32_t hw[4] = {hv.x, hv.y, hv.z, hv.w}, hgw[4] = {hg.x, hg.y, hg.z, hg.w};
-#pragma unroll
-                        for (int i = 0; i < 4; ++i) {
-                            float h0 = bf16lo_f32(hw[i]), h1 = bf16hi_f32(hw[i]);
-                            sqh += h0 * h0 + h1 * h1;
-                            store_split(a_hi, a_lo, (size_t)r * st + k + 2 * i, h0 * bf16lo_f32(hgw[i]));
-                            store_split(a_hi, a_lo, (size_t)r * st + k + 2 * i + 1, h1 * bf16hi_f32(hgw[i]));
-                        }
-                    }
-                }
-                // block sums of the two squared norms of row r
-#pragma unroll
-                for (int o = 16; o > 0; o >>= 1) {
-                    sqh += __shfl_xor_sync(0xffffffffu, sqh, o);
-                    sqe += __shfl_xor_sync(0xffffffffu, sqe, o);
-                }
-                if (c.lane == 0) { c.misc->ssred[c.warp][r][0] = sqh; c.misc->ssred[c.warp][r][1] = sqe; }
-            }
-            bar_sync(1, kConsumerThreads);
-            if (c.tid < R) {
-                float sh = 0.f, se = 0.f;
-                for (int i = 0; i < kConsumerWarps; ++i) { sh += c.misc->ssred[i][c.tid][0]; se += c.misc->ssred[i][c.tid][1]; }
-                if (step == 0) c.misc->scale0[c.tid] = rsqrtf(sh / (float)p.d + p.eps);
-                c.misc->scale1[c.tid] = rsqrtf(se / (float)p.d + p.eps);
-            }
         } else {
-            // ---- the previous phase's output vector (hi/lo) and the sum of squares that normalises it
-            const bf16_t *ghi, *glo;
-            const float *sstab = nullptr;
-            int gstride = p.dp, glen = p.d;
-            switch (kind) {
-                case QKV:    ghi = p.s.actD_hi; glo = p.s.actD_lo; sstab = p.s.ssA; break;
-                case OPROJ:  ghi = p.s.actO_hi; glo = p.s.actO_lo; gstride = p.qp; glen = p.qdim; break;
-                case GATEUP: ghi = p.s.actP_hi; glo = p.s.actP_lo; sstab = p.s.ssB; break;
-                case DOWN:   ghi = p.s.actF_hi; glo = p.s.actF_lo; gstride = p.Fp; glen = p.Fp; break;   // pad beyond F is zero
-                default:     ghi = p.s.actH_hi; glo = p.s.actH_lo; sstab = p.s.ssC; break;               // HEAD
+            // ============ matrix phases: stage the input vector(s) in shared memory ...
+            const PhaseIo &io = c.misc->io;
+            const int klen = (kind == PROJ) ? (SPLIT && c.proj_split ? p.d : 2 * p.d) : io.in_len;
+            const int st = ((klen + 31) & ~31) + 32;      // +64 B: rows land in different banks
+            bf16_t *a_hi = reinterpret_cast<bf16_t *>(c.scr), *a_lo = a_hi + (size_t)R * st;
+            ActSrc act{a_hi, a_lo, st, true};
+            if (kind == PROJ) {
+                // ---- x0 = W_p [ rms(h) ; rms(Emb(tok)) ]. The chain key -> token -> embedding row is the phase's latency: the key
+                // is asked for first, the recursed state and the partial sums that normalise it arrive while the embedding
+                // row is on its way (one after the other they took 7500 cycles)
+                unsigned long long key = 0ull;
+                int tok = 0;
+                if (c.tid < R) {
+                    if (step > 0) key = ldcg_u64(p.s.keys + (size_t)(step - 1) * kMaxRows + c.tid);
+                    else {
+                        const int b = p.M > 1 ? c.tid / p.M : c.tid;       // a padding row's token is never looked at
+                        if (c.tid - b * p.M < seq_next(c, b)) tok = p.tokens[c.tid];
+                    }
+                }
+                const bool renorm = step > 0 && c.warp < R;
+                float pvc[kPartialRegs], pvd[kPartialRegs];
+                if (renorm) {
+                    const int col = src_row(c, c.warp, step);      // step 1 continues each sequence's last extend row
+                    load_partials(c, p.s.ssC, col, pvc);
+                    load_partials(c, p.s.ssD, col, pvd);
+                }
+                if (c.tid < R) {
+                    if (step > 0) {
+                        if ((key >> 32) == 0ull) raise(c, kDevAllNan);
+                        tok = (int)argmax_key_id(key);
+                        if (c.cta == 0) p.out_tokens[(size_t)c.tid * p.K + (step - 1)] = tok;
+                    }
+                    if ((unsigned)tok >= (unsigned)p.V) { raise(c, kDevBadToken); tok = 0; }
+                    c.misc->tok[c.tid] = tok;
+                }
+                bar_sync(1, kConsumerThreads);
+                // a thread's first two pieces of a row (all of it up to 4096 columns) are asked for together
+                constexpr int kStep = kConsumerThreads * 8;
+                const int k0 = c.tid * 8;
+                const bool both = !SPLIT || !c.proj_split;
+                uint4 e[2], eg[2];
+                auto fetch = [&](int r) {
+                    const bf16_t *erow = p.embed + (size_t)c.misc->tok[r] * p.d;
+#pragma unroll
+                    for (int q = 0; q < 2; ++q)
+                        if (k0 + q * kStep < p.d) { e[q] = ldnc128(erow + k0 + q * kStep); eg[q] = ldnc128(p.g_enorm + k0 + q * kStep); }
+                };
+                fetch(0);
+                if (step > 0) stage_hilo<2>(c, io.in_hi, io.in_lo, io.in_stride, p.d, a_hi, a_lo, st, step);
+                if (renorm) {
+                    // recursed state: h = (x2*g_final) * s_x; rms(h) adds s_h = rsqrt(s_x^2 * mean((x2 g)^2) + eps)
+                    float sx = rsqrtf(reduce_partials(pvc) / (float)p.d + p.eps);
+                    float sy = reduce_partials(pvd) / (float)p.d;
+                    if (c.lane == 0) c.misc->scale0[c.warp] = sx * rsqrtf(sx * sx * sy + p.eps);
+                }
+#pragma unroll 1
+                for (int r = 0; r < R; ++r) {
+                    float sqh = 0.f, sqe = 0.f;
+                    if (r > 0) fetch(r);
+#pragma unroll 1
+                    for (int kk = k0; kk < p.d; kk += 2 * kStep) {
+                        uint4 h[2], hg[2];
+#pragma unroll
+                        for (int q = 0; q < 2; ++q) {
+                            const int k = kk + q * kStep;
+                            if (k < p.d) {
+                                if (kk > k0) { e[q] = ldnc128(p.embed + (size_t)c.misc->tok[r] * p.d + k); eg[q] = ldnc128(p.g_enorm + k); }
+                                if (step == 0) { h[q] = ldnc128(p.h_last + (size_t)r * p.d + k); hg[q] = ldnc128(p.g_hnorm + k); }
+                            }
+                        }
+#pragma unroll
+                        for (int q = 0; q < 2; ++q) {
+                            const int k = kk + q * kStep;
+                            if (k < p.d) {
+                                const uint32_t ew[4] = {e[q].x, e[q].y, e[q].z, e[q].w}, egw[4] = {eg[q].x, eg[q].y, eg[q].z, eg[q].w};
+#pragma unroll
+                                for (int i = 0; i < 4; ++i) { const float e0 = bf16lo_f32(ew[i]), e1 = bf16hi_f32(ew[i]); sqe += e0 * e0 + e1 * e1; }
+                                if (both) store_product8(a_hi, a_lo, r * st + p.d + k, ew, egw);
+                                if (step == 0) {
+                                    const uint32_t hw[4] = {h[q].x, h[q].y, h[q].z, h[q].w}, hgw[4] = {hg[q].x, hg[q].y, hg[q].z, hg[q].w};
+#pragma unroll
+                                    for (int i = 0; i < 4; ++i) { const float h0 = bf16lo_f32(hw[i]), h1 = bf16hi_f32(hw[i]); sqh += h0 * h0 + h1 * h1; }
+                                    store_product8(a_hi, a_lo, r * st + k, hw, hgw);
+                                }
+                            }
+                        }
+                    }
+                    // block sums of the two squared norms of row r
+#pragma unroll
+                    for (int o = 16; o > 0; o >>= 1) {
+                        sqh += __shfl_xor_sync(0xffffffffu, sqh, o);
+                        sqe += __shfl_xor_sync(0xffffffffu, sqe, o);
+                    }
+                    if (c.lane == 0) { c.misc->ssred[c.warp][r][0] = sqh; c.misc->ssred[c.warp][r][1] = sqe; }
+                }
+                bar_sync(1, kConsumerThreads);
+                if (c.tid < R) {
+                    float sh = 0.f, se = 0.f;
+                    for (int i = 0; i < kConsumerWarps; ++i) { sh += c.misc->ssred[i][c.tid][0]; se += c.misc->ssred[i][c.tid][1]; }
+                    if (step == 0) c.misc->scale0[c.tid] = rsqrtf(sh / (float)p.d + p.eps);
+                    c.misc->scale1[c.tid] = rsqrtf(se / (float)p.d + p.eps);
+                }
+            } else {
+                // ---- the previous phase's output vector (hi/lo) and the sum of squares that normalises it
+                float pv[kPartialRegs];
+                const bool norm = io.sstab != nullptr && c.warp < R;
+                if (norm) load_partials(c, io.sstab, c.warp, pv);
+                if (kind == DOWN) act = ActSrc{io.in_hi, io.in_lo, io.in_stride, false};     // read from global memory inside the loop
+                // several rows: more loads per round, so that the copy stays at one or two L2 round trips
+                else if (R * (io.in_len >> 3) > 2 * kConsumerThreads) stage_hilo<8>(c, io.in_hi, io.in_lo, io.in_stride, io.in_len, a_hi, a_lo, st, 0);
+                else stage_hilo<2>(c, io.in_hi, io.in_lo, io.in_stride, io.in_len, a_hi, a_lo, st, 0);
+                if (norm) {
+                    float sc = rsqrtf(reduce_partials(pv) / (float)p.d + p.eps);
+                    if (c.lane == 0) c.misc->scale0[c.warp] = sc;
+                }
             }
-            float pv[kPartialRegs];
-            const bool norm = sstab != nullptr && c.warp < R;
-            if (norm) load_partials(c, sstab, c.warp, pv);       // in flight while the vector is staged
-            if (kind == DOWN) act = ActSrc{ghi, glo, gstride, false};     // read from global memory inside the loop
-            else stage_hilo(c, ghi, glo, gstride, glen, a_hi, a_lo, st, 0);
-            if (norm) {
-                float sc = rsqrtf(reduce_partials(pv) / (float)p.d + p.eps);
-                if (c.lane == 0) c.misc->scale0[c.warp] = sc;
-            }
-        }
-        if (kind == HEAD && c.tid < R) c.misc->outrow[c.tid] = out_row(c, c.tid, step);
-        bar_sync(1, kConsumerThreads);
-        if (kind == HEAD && p.out_h) {   // every CTA writes its slice of the post-final-norm hidden state
-            int r0 = (int)(((long long)c.cta * p.d) / c.grid), r1 = (int)(((long long)(c.cta + 1) * p.d) / c.grid);
-            for (int i = c.tid; i < R * (r1 - r0); i += kConsumerThreads) {
-                int r = i / (r1 - r0), k = r0 + (i - r * (r1 - r0));
-                const int orow = c.misc->outrow[r];
-                if (orow < 0) continue;                    // an extend row that is not its sequence's last
-                float y = bf16bits_f32(a_hi[(size_t)r * st + k]) + bf16bits_f32(a_lo[(size_t)r * st + k]);
-                size_t o = (p.mode == 0) ? ((size_t)orow * p.K + step) * p.d + k : (size_t)orow * p.d + k;
-                p.out_h[o] = f32_bf16bits(y * c.misc->scale0[r]);
-            }
-        }
-        PROF(c, kind * 8 + 1);
-
-        // ============ ... stream the weights ...
-        consume_tiles<TWO, TM, SPLIT>(c, kind, act, ex);
-
-        // ============ ... and publish what the next phase needs besides the vector
-        if (kind == PROJ) flush_sq(c, ex.sq, p.s.ssA, nullptr);
-        else if (kind == OPROJ) flush_sq(c, ex.sq, p.s.ssB, nullptr);
-        else if (kind == DOWN) flush_sq(c, ex.sq, ex.to_next_layer ? p.s.ssA : p.s.ssC, (p.mode == 0) ? p.s.ssD : nullptr);
-        else if (kind == HEAD) {
-            // reduce the per-thread maxima (thread = (row slot, col)) over the 32 row slots
-            unsigned long long k = ex.best;
-            unsigned long long o8 = __shfl_xor_sync(0xffffffffu, k, 8);
-            k = o8 > k ? o8 : k;
-            unsigned long long o16 = __shfl_xor_sync(0xffffffffu, k, 16);
-            k = o16 > k ? o16 : k;
-            if (c.lane < 8) c.misc->keyred[c.warp][c.lane] = k;
+            if (kind == HEAD && c.tid < R) c.misc->outrow[c.tid] = out_row(c, c.tid, step);
             bar_sync(1, kConsumerThreads);
-            if (c.tid < R) {
-                unsigned long long m = 0ull;
-                for (int w = 0; w < kConsumerWarps; ++w) m = c.misc->keyred[w][c.tid] > m ? c.misc->keyred[w][c.tid] : m;
-                const int orow = c.misc->outrow[c.tid];
-                if (m != 0ull && orow >= 0) atomicMax(p.s.keys + (size_t)step * kMaxRows + orow, m);
+            if (kind == HEAD && p.out_h) {   // every CTA writes its slice of the post-final-norm hidden state
+                const Geom &geo = c.misc->geo[OPROJ];                    // the shares of d rows
+                const int r = c.tid & 7, orow = r < R ? c.misc->outrow[r] : -1;      // -1: an extend row that is not its sequence's last
+                if (orow >= 0) {
+                    bf16_t *out = p.out_h + (p.mode == 0 ? (size_t)orow * p.K + step : (size_t)orow) * p.d;
+                    for (int k = geo.v0 + (c.tid >> 3); k < geo.v1; k += kTileRows) {
+                        float y = bf16bits_f32(a_hi[(size_t)r * st + k]) + bf16bits_f32(a_lo[(size_t)r * st + k]);
+                        out[k] = f32_bf16bits(y * c.misc->scale0[r]);
+                    }
+                }
             }
-            ex.best = 0ull;
-            if (p.n_stages2 > 0 && step == 0 && p.K > 1) bar_arrive(5, kThreads);      // see switch_layout
+            PROF(c, kind * 8 + 1);
+
+            // ============ ... stream the weights ...
+            consume_tiles<TWO, TM, SPLIT>(c, ph, act, ex);
+
+            // ============ ... and publish what the next phase needs besides the vector
+            if (kind == PROJ) flush_sq(c, ex.sq, p.s.ssA, nullptr);
+            else if (kind == OPROJ) flush_sq(c, ex.sq, p.s.ssB, nullptr);
+            else if (kind == DOWN) flush_sq(c, ex.sq, io.out ? p.s.ssA : p.s.ssC, io.recurse ? p.s.ssD : nullptr);
+            else if (kind == HEAD) {
+                // reduce the per-thread maxima (thread = (row slot, col)) over the 32 row slots
+                unsigned long long k = ex.best;
+                unsigned long long o8 = __shfl_xor_sync(0xffffffffu, k, 8);
+                k = o8 > k ? o8 : k;
+                unsigned long long o16 = __shfl_xor_sync(0xffffffffu, k, 16);
+                k = o16 > k ? o16 : k;
+                if (c.lane < 8) c.misc->keyred[c.warp][c.lane] = k;
+                bar_sync(1, kConsumerThreads);
+                if (c.tid < R) {
+                    unsigned long long m = 0ull;
+                    for (int w = 0; w < kConsumerWarps; ++w) m = c.misc->keyred[w][c.tid] > m ? c.misc->keyred[w][c.tid] : m;
+                    const int orow = c.misc->outrow[c.tid];
+                    if (m != 0ull && orow >= 0) atomicMax(p.s.keys + (size_t)step * kMaxRows + orow, m);
+                }
+                ex.best = 0ull;
+                if (p.n_stages2 > 0 && step == 0 && p.K > 1) bar_arrive(5, kThreads);      // see switch_layout
+            }
         }
         PROF(c, kind * 8 + 2);
-        grid_barrier(c);
+        grid_barrier(c, [&]() {
+            prog_next(p, ph);
+            set_step_rows(c, ph.step);
+            make_phase<!TWO && !TM>(c, ph);
+        });
     }
     PROF(c, DONE * 8);
     if (TM) {                                  // lets the mover's warp free the tensor memory
