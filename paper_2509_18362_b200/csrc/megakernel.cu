@@ -1113,7 +1113,8 @@ __device__ __forceinline__ void flush_sq(const Cta &c, const SqAcc &q, float *tb
 // the 64 K rows. The consumers add the positions this launch produced (earlier draft steps from
 // the pages, this call's rows from the QKV scratch, rotated and rounded to bf16 exactly as they
 // are stored) into the same stage buffer and then work from shared memory only.
-// Scratch: qs[M*Gq][dh] rotated, pre-scaled queries of one KV head, then the per-warp partials (o, m, l) of the
+// Scratch: rotated, pre-scaled queries of one KV head (split into bf16 parts when they are rotated: as fp32, split by every warp
+// that read them, a row's fragments took 1700 cycles), then the per-warp partials (o, m, l) of the
 // working warp groups.
 
 // One chunk of one KV head on the tensor cores, for every row of the call. K and V stay in the stage (16-byte piece w
@@ -1125,7 +1126,7 @@ __device__ __forceinline__ void flush_sq(const Cta &c, const SqAcc &q, float *tb
 // the same way, V fragments by transposing ldmatrix. The four warps' (o, m, l) are merged in warp order, then the
 // chunks in ascending order by the merge phase.
 template <int DH>
-__device__ __forceinline__ void attn_rows_mma(Cta &c, const bf16_t *sk, const bf16_t *sv, const float *qs, float *part,
+__device__ __forceinline__ void attn_rows_mma(Cta &c, const bf16_t *sk, const bf16_t *sv, const bf16_t *qs, float *part,
                                               int b, int kvh, int chunk, int base, int max_tokens, int rows) {
     const MegaParams &p = *c.p;
     constexpr int wstride = DH + 2;
@@ -1143,31 +1144,20 @@ __device__ __forceinline__ void attn_rows_mma(Cta &c, const bf16_t *sk, const bf
     const int vtok = tw + (c.lane & 7) + (((c.lane >> 3) & 1) << 3), vpc = c.lane >> 4;
     const uint32_t krow = sk_u + (uint32_t)ktok * (DH * 2), vrow = sv_u + (uint32_t)vtok * (DH * 2);
     const uint32_t ksw = (uint32_t)(ktok & 7), vsw = (uint32_t)(vtok & 7);
+    const int qh = min(c.lane & 7, Gq - 1);
 #pragma unroll 1
     for (int m = grp; m < M; m += 2) {
         const int npos = min(base + min(m, rows - 1), max_tokens - 1);   // last visible position of this row
-#pragma unroll 1
-        for (int h0 = 0; h0 < Gq; h0 += 8) {                             // eight query heads per pass
-            const int nh = min(8, Gq - h0);
-            // query fragments from the fp32 vectors: hi parts in rows 0-7, lo parts in rows 8-15
+        {
+            // query fragments: rows 0-7 the heads' hi parts, 8-15 their lo parts (a head that does not exist repeats the last one: not used)
             uint32_t qa[DH / 16][4];
             {
-                const float *qh = qs + ((size_t)(m * Gq + h0 + hrow)) * DH;
+                const uint32_t qrow = smem_u32(qs + (size_t)m * 2 * Gq * DH) + (uint32_t)((((c.lane >> 3) & 1) * Gq + qh) * DH * 2);
 #pragma unroll
-                for (int ks = 0; ks < DH / 16; ++ks) {
-                    float2 x0 = make_float2(0.f, 0.f), x1 = make_float2(0.f, 0.f);
-                    if (hrow < nh) {
-                        x0 = *reinterpret_cast<const float2 *>(qh + ks * 16 + kq);
-                        x1 = *reinterpret_cast<const float2 *>(qh + ks * 16 + kq + 8);
-                    }
-                    uint16_t h0a, l0a, h0b, l0b, h1a, l1a, h1b, l1b;
-                    split_bf16(x0.x, h0a, l0a); split_bf16(x0.y, h0b, l0b);
-                    split_bf16(x1.x, h1a, l1a); split_bf16(x1.y, h1b, l1b);
-                    qa[ks][0] = (uint32_t)h0a | ((uint32_t)h0b << 16);
-                    qa[ks][1] = (uint32_t)l0a | ((uint32_t)l0b << 16);
-                    qa[ks][2] = (uint32_t)h1a | ((uint32_t)h1b << 16);
-                    qa[ks][3] = (uint32_t)l1a | ((uint32_t)l1b << 16);
-                }
+                for (int ks = 0; ks < DH / 16; ++ks)
+                    asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];"
+                                 : "=r"(qa[ks][0]), "=r"(qa[ks][1]), "=r"(qa[ks][2]), "=r"(qa[ks][3])
+                                 : "r"(qrow + ((((uint32_t)(ks * 2) + (uint32_t)(c.lane >> 4)) ^ (uint32_t)(qh & 7)) << 4)));
             }
             // scores of this warp's 16 tokens (two n-tiles of 8)
             float s[2][4];
@@ -1230,37 +1220,46 @@ __device__ __forceinline__ void attn_rows_mma(Cta &c, const bf16_t *sk, const bf
             {
                 float *w = wp + ((size_t)wi * 8 + hrow) * wstride;
 #pragma unroll
-                for (int nt = 0; nt < DH / 8; ++nt) { w[nt * 8 + kq] = o[nt][0] + o[nt][2]; w[nt * 8 + kq + 1] = o[nt][1] + o[nt][3]; }
+                for (int nt = 0; nt < DH / 8; ++nt) *reinterpret_cast<float2 *>(w + nt * 8 + kq) = make_float2(o[nt][0] + o[nt][2], o[nt][1] + o[nt][3]);
                 if ((c.lane & 3) == 0) { w[DH] = mx; w[DH + 1] = psum; }
             }
             bar_sync(3 + grp, 128);
             const int gt = c.tid & 127;                      // thread within the group
-            if (gt < 32) {                                   // thread = (head gt >> 2, warp gt & 3): the warp's weight
+            if (gt < 32) {                                   // thread = (head gt >> 2, warp gt & 3): the warp's weight, the head's (m, l)
                 const int h = gt >> 2, w = gt & 3;
                 float mm = -INFINITY;
 #pragma unroll
                 for (int q = 0; q < 4; ++q) mm = fmaxf(mm, wp[((size_t)q * 8 + h) * wstride + DH]);
-                const float mw = wp[((size_t)w * 8 + h) * wstride + DH];
-                fw[w * 8 + h] = (mw == -INFINITY) ? 0.f : expf(mw - mm);
-                if (w == 0) fw[32 + 2 * h] = mm;
+                const float mw = wp[((size_t)w * 8 + h) * wstride + DH], lw = wp[((size_t)w * 8 + h) * wstride + DH + 1];
+                const float f = (mw == -INFINITY) ? 0.f : expf(mw - mm);
+                fw[w * 8 + h] = f;
+                float l = 0.f;
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    const float fq = __shfl_sync(0xffffffffu, f, (gt & ~3) + q), lq = __shfl_sync(0xffffffffu, lw, (gt & ~3) + q);
+                    l += fq * lq;
+                }
+                if (w == 0 && h < Gq) {
+                    float *dst = p.s.att_part + (((size_t)(b * M + m) * p.Hq + kvh * Gq + h) * p.max_chunks + chunk) * (DH + kPartPad);
+                    dst[DH] = mm;
+                    dst[DH + 1] = l;
+                }
             }
             bar_sync(3 + grp, 128);
-            for (int i = gt; i < nh * DH; i += 128) {
-                const int h = i / DH, e = i - h * DH;
-                float ov = 0.f, l = 0.f;
+            for (int i = gt; i < Gq * (DH / 2); i += 128) {  // two output elements
+                const int h = i / (DH / 2), e = (i - h * (DH / 2)) * 2;
+                float o0 = 0.f, o1 = 0.f;
 #pragma unroll
                 for (int w = 0; w < 4; ++w) {
-                    const float *pw = wp + ((size_t)w * 8 + h) * wstride;
+                    const float2 v = *reinterpret_cast<const float2 *>(wp + ((size_t)w * 8 + h) * wstride + e);
                     const float f = fw[w * 8 + h];
-                    ov += f * pw[e];
-                    l += f * pw[DH + 1];
+                    o0 += f * v.x;
+                    o1 += f * v.y;
                 }
-                const int r = b * M + m, hq = kvh * Gq + h0 + h;
-                float *dst = p.s.att_part + (((size_t)r * p.Hq + hq) * p.max_chunks + chunk) * (DH + kPartPad);
-                dst[e] = ov;
-                if (e == 0) { dst[DH] = fw[32 + 2 * h]; dst[DH + 1] = l; }
+                const int rr = b * M + m, hq = kvh * Gq + h;
+                *reinterpret_cast<float2 *>(p.s.att_part + (((size_t)rr * p.Hq + hq) * p.max_chunks + chunk) * (DH + kPartPad) + e) = make_float2(o0, o1);
             }
-            bar_sync(3 + grp, 128);                          // the group's buffer is free for its next pass
+            if (m + 2 < M) bar_sync(3 + grp, 128);           // the group's buffer is free for its next pass
         }
     }
 }
@@ -1358,7 +1357,7 @@ __device__ __forceinline__ void attention_phase(Cta &c, const KvPtrs &kv, int st
     const MegaParams &p = *c.p;
     constexpr int dh = DH, half = DH >> 1;
     const int Gq = p.Hq / p.Hkv, M = c.M;
-    float *qs = reinterpret_cast<float *>(c.scr);
+    bf16_t *qs = reinterpret_cast<bf16_t *>(c.scr);   // [M][hi, lo][Gq][dh], 16-byte piece w of head h at piece w ^ (h & 7)
     const float qscale = rsqrtf((float)dh);
     const int max_tokens = min(kv.max_pages * p.page, p.max_ctx);   // positions beyond are flagged, not touched
     const int upt = dh >> 3;
@@ -1381,7 +1380,7 @@ __device__ __forceinline__ void attention_phase(Cta &c, const KvPtrs &kv, int st
         constexpr int q4 = half / 4;
         for (int i = c.tid; i < M * Gq * q4; i += kConsumerThreads) {
             const int qi = i / q4, e = (i - qi * q4) * 4;
-            const int m = qi / Gq, hq = kvh * Gq + (qi - m * Gq);
+            const int m = M > 1 ? qi / Gq : 0, h = qi - m * Gq, hq = kvh * Gq + h;
             int pos = base + min(m, rows - 1);
             if (pos >= max_tokens) pos = max_tokens - 1;
             const float *q = p.s.qkv + (size_t)(b * M + m) * (p.qdim + 2 * p.kvdim) + hq * dh + e;
@@ -1397,16 +1396,25 @@ __device__ __forceinline__ void attention_phase(Cta &c, const KvPtrs &kv, int st
                 lo[u] = (x[u] * cc[u] - y[u] * ss[u]) * qscale;
                 hi[u] = (y[u] * cc[u] + x[u] * ss[u]) * qscale;
             }
-            *reinterpret_cast<float4 *>(qs + qi * dh + e) = make_float4(lo[0], lo[1], lo[2], lo[3]);
-            *reinterpret_cast<float4 *>(qs + qi * dh + e + half) = make_float4(hi[0], hi[1], hi[2], hi[3]);
+            bf16_t *qm = qs + (size_t)m * 2 * Gq * dh + h * dh;
+            auto put = [&](int at, const float (&v)[4]) {
+                uint16_t h0, h1, h2, h3, l0, l1, l2, l3;
+                split_bf16(v[0], h0, l0); split_bf16(v[1], h1, l1); split_bf16(v[2], h2, l2); split_bf16(v[3], h3, l3);
+                bf16_t *d = qm + (((at >> 3) ^ (h & 7)) << 3) + (at & 7);
+                *reinterpret_cast<uint2 *>(d) = make_uint2((uint32_t)h0 | ((uint32_t)h1 << 16), (uint32_t)h2 | ((uint32_t)h3 << 16));
+                *reinterpret_cast<uint2 *>(d + (size_t)Gq * dh) = make_uint2((uint32_t)l0 | ((uint32_t)l1 << 16), (uint32_t)l2 | ((uint32_t)l3 << 16));
+            };
+            put(e, lo);
+            put(e + half, hi);
         }
         PROF(c, ATTN * 8 + 3);
-        wait_bar(c, &c.full[slot], parity);
-        PROF(c, ATTN * 8 + 4);
+        // The rows of the chunk that are not committed are no copy's: they are put into the stage while the copies are on their way,
+        // each kind by other threads, so that its loads wait for nobody's (behind the wait, one kind after the other, they
+        // made the four items with a context's end the phase's last by 2800 cycles).
         // -- positions written earlier in this launch (previous draft steps): from the pages
         {
             const int lo = max(Lb, c0), hi = min(min(base, c0 + kAttnChunk), max_tokens);
-            for (int i = c.tid; i < (hi - lo) * upt; i += kConsumerThreads) {
+            for (int i = (c.tid + kConsumerThreads / 2) % kConsumerThreads; i < (hi - lo) * upt; i += kConsumerThreads) {
                 int tk = i / upt, w = i - tk * upt, j = lo + tk;
                 int page = bt[j / p.page];
                 if ((unsigned)page >= (unsigned)kv.num_pages) { raise(c, kDevBadPage); page = 0; }
@@ -1417,7 +1425,7 @@ __device__ __forceinline__ void attention_phase(Cta &c, const KvPtrs &kv, int st
             }
         }
         // -- this call's rows: rotate, round to bf16, put into the stage and append to the cache
-        for (int i = c.tid; i < M * half; i += kConsumerThreads) {
+        for (int i = (c.tid + kConsumerThreads / 4) % kConsumerThreads; i < M * half; i += kConsumerThreads) {
             int m = i / half, e = i - m * half;
             if (m >= rows) continue;                              // padding row: nothing to store
             int r = b * M + m, pos = base + m;
@@ -1441,16 +1449,17 @@ __device__ __forceinline__ void attention_phase(Cta &c, const KvPtrs &kv, int st
             kv.v_pages[o + e] = v0;
             kv.v_pages[o + e + half] = v1;
         }
+        wait_bar(c, &c.full[slot], parity);
+        PROF(c, ATTN * 8 + 4);
         bar_sync(1, kConsumerThreads);
         PROF(c, ATTN * 8 + 5);
 
-        float *part = qs + (((size_t)M * Gq * dh + 3) & ~(size_t)3);
+        float *part = reinterpret_cast<float *>(qs + (size_t)M * 2 * Gq * dh);
         attn_rows_mma<DH>(c, sk, sv, qs, part, b, kvh, chunk, base, max_tokens, rows);
-        bar_sync(1, kConsumerThreads);   // every warp has read what it needs from the stage
+        bar_sync(1, kConsumerThreads);   // every warp has read what it needs from the stage, the queries and the partials
         if (c.tid == 0) { volatile uint32_t *ud = &c.misc->use_done[slot]; *ud = *ud + 1; }   // see the mover of the tensor-memory path
         if (c.warp < kConsumerWarps / 2 && c.lane == 0) mbar_arrive(&c.empty[slot]);
         next_stage(c);
-        bar_sync(1, kConsumerThreads);   // the query / partial scratch is reused by the next item
     }
 }
 
@@ -1477,8 +1486,8 @@ __device__ __forceinline__ void merge_phase(Cta &c, const KvPtrs &kv, int step) 
     const int units = c.R * p.Hq;
     const int el = (c.tid % q4) * 4, cg = c.tid / q4;
     for (int u = c.cta; u < units; u += c.grid) {
-        const int r = u / p.Hq, hq = u - r * p.Hq;
-        const int b = r / M, m = r - b * M;
+        const int r = c.R > 1 ? u / p.Hq : 0, hq = u - r * p.Hq;
+        const int b = M > 1 ? r / M : r, m = r - b * M;
         const int pos = min(step_base(c, kv, b, step) + min(m, step_rows(c, b, step) - 1), max_tokens - 1);
         const int ncm = min(pos / kAttnChunk + 1, p.max_chunks);        // chunks visible to this row
         const float *src = p.s.att_part + ((size_t)r * p.Hq + hq) * p.max_chunks * stride;
@@ -1491,19 +1500,34 @@ __device__ __forceinline__ void merge_phase(Cta &c, const KvPtrs &kv, int step) 
         }
         bar_sync(1, kConsumerThreads);
         float mx = -INFINITY;
-        for (int i = 0; i < ncm; ++i) mx = fmaxf(mx, ms[i]);
-        float o0 = 0.f, o1 = 0.f, o2 = 0.f, o3 = 0.f, l = 0.f;
-        auto add = [&](int ch, const uint4 &v) {
-            const float mc = ms[ch];
-            const float f = (mc == -INFINITY) ? 0.f : expf(mc - mx);
-            o0 += f * __uint_as_float(v.x); o1 += f * __uint_as_float(v.y);
-            o2 += f * __uint_as_float(v.z); o3 += f * __uint_as_float(v.w);
-            l += f * ls[ch];
-        };
+        for (int i = c.lane; i < ncm; i += 32) mx = fmaxf(mx, ms[i]);
 #pragma unroll
-        for (int i = 0; i < kPre; ++i) if (cg + i * ncg < ncm) add(cg + i * ncg, pre[i]);
+        for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+        float o0 = 0.f, o1 = 0.f, o2 = 0.f, o3 = 0.f, l = 0.f;
+        // the threads of a chunk group work out the weights of its next q4 chunks side by side (each thread for itself, chunk
+        // after chunk, took 300 cycles a chunk); all of a warp's groups take the same turns
+        const int sub = c.tid % q4, cg_warp = (c.tid & ~31) / q4;
+        for (int t0 = 0; cg_warp + t0 * ncg < ncm; t0 += q4) {
+            const int mine = cg + (t0 + sub) * ncg;
+            const float mc = mine < ncm ? ms[mine] : -INFINITY, lc = mine < ncm ? ls[mine] : 0.f;
+            const float fc = (mc == -INFINITY) ? 0.f : expf(mc - mx);
+            auto add = [&](int j, const uint4 &v) {          // chunk cg + (t0 + j) ncg
+                const float f = __shfl_sync(0xffffffffu, fc, j, q4), lj = __shfl_sync(0xffffffffu, lc, j, q4);
+                if (cg + (t0 + j) * ncg >= ncm) return;
+                o0 += f * __uint_as_float(v.x); o1 += f * __uint_as_float(v.y);
+                o2 += f * __uint_as_float(v.z); o3 += f * __uint_as_float(v.w);
+                l += f * lj;
+            };
+            int j = 0;
+            if (t0 == 0) {
+#pragma unroll
+                for (int i = 0; i < kPre; ++i) add(i, pre[i]);
+                j = kPre;
+            }
 #pragma unroll 4
-        for (int ch = cg + kPre * ncg; ch < ncm; ch += ncg) add(ch, ldcg128(src + (size_t)ch * stride + el));
+            for (; j < q4 && cg_warp + (t0 + j) * ncg < ncm; ++j)
+                add(j, ldcg128(src + (size_t)min(cg + (t0 + j) * ncg, ncm - 1) * stride + el));
+        }
         if (tight) bar_sync(1, kConsumerThreads);    // every thread has read the maxima and sums
         *reinterpret_cast<float4 *>(red + cg * stride + el) = make_float4(o0, o1, o2, o3);
         if (el == 0) red[cg * stride + dh] = l;
