@@ -78,6 +78,12 @@ struct PhaseIo {
     int recurse;                     // down projection of a draft: publishes the recursed state as well
 };
 
+// A work item of the attention phase: sequence, KV head, 64-token chunk; the sequence's committed positions, its chunks, the
+// position of its row 0 and its rows that count.
+struct AttnItem { int b, kvh, chunk, Lb, nch, base, rows; };
+// A work unit of the merge phase: a row's query head, its chunk partials and how many of them it sees.
+struct MergeUnit { const float *src; int r, hq, ncm; };
+
 struct Misc {   // small shared-memory block
     uint64_t full[kMaxStages];
     uint64_t empty[kMaxStages];
@@ -96,6 +102,9 @@ struct Misc {   // small shared-memory block
     int seqlen[kMaxRows];   // committed length of every sequence and its number of extend rows, read once at kernel start:
     int next[kMaxRows];     // neither changes during a launch, and every phase that needs them saves an L2 round trip
     PhaseIo io;                      // of the current matrix phase
+    AttnItem item;                   // this CTA's first item of the current attention phase, and the phase's items
+    int n_items;
+    MergeUnit unit;                  // and its first unit of the current merge phase
     Geom geo[kMatrixKinds];          // filled once per launch: row shares and stage counts take divisions, 800 cycles at every phase start
     unsigned long long rowptr[kProducerWarps][32];   // tile row pointers, one line per producer warp
     int flag;
@@ -508,8 +517,9 @@ struct SqAcc {
 };
 
 // Operands of the epilogue that do not depend on the dot product (residual value, norm gains, the
-// token id of a head row): loaded when the tile starts, so their latency hides behind the stream.
-struct EpiPre { float resid, g0, g1; int id; };
+// token id of a head row): loaded when the tile starts, so their latency hides behind the stream (gains as they are: a
+// conversion would wait for them).
+struct EpiPre { float resid; bf16_t g0, g1; int id; };
 struct Phase : Prog {
     EpiPre pre;                      // of this thread's element of the first tile
 };
@@ -529,12 +539,12 @@ __device__ __forceinline__ void store_split(bf16_t *hi, bf16_t *lo, size_t idx, 
 
 __device__ __forceinline__ EpiPre epi_prefetch(const Cta &c, const PhaseIo &io, int row, int col, bool valid) {
     EpiPre e;
-    e.resid = 0.f; e.g0 = 0.f; e.g1 = 0.f; e.id = row;
+    e.resid = 0.f; e.g0 = 0; e.g1 = 0; e.id = row;
     if (!valid) return e;
     // the residual was written by this very thread: rows are shared out alike in every phase whose result has d rows
     if (io.res) e.resid = ldcg_f32(io.res + (size_t)col * c.p->d + row);
-    if (io.gain) e.g0 = bf16bits_f32(io.gain[row]);
-    if (io.gain2) e.g1 = bf16bits_f32(io.gain2[row]);
+    if (io.gain) e.g0 = io.gain[row];
+    if (io.gain2) e.g1 = io.gain2[row];
     if (io.ids) e.id = io.ids[row];
     return e;
 }
@@ -559,12 +569,12 @@ __device__ __forceinline__ void epilogue(const Cta &c, const Phase &ph, EpiCtx &
         }
         case PROJ: case OPROJ: case DOWN: {
             float r = io.res ? pre.resid + v : v;
-            float y = r * pre.g0;
+            float y = r * bf16bits_f32(pre.g0);
             x.sq.a += r * r;
             if (io.out) io.out[(size_t)col * io.out_stride + row] = r;
             store_split(io.out_hi, io.out_lo, (size_t)col * io.out_split + row, y);
             if (io.recurse) {
-                store_split(p.s.actR_hi, p.s.actR_lo, (size_t)col * p.dp + row, y * pre.g1);
+                store_split(p.s.actR_hi, p.s.actR_lo, (size_t)col * p.dp + row, y * bf16bits_f32(pre.g1));
                 x.sq.b += y * y;
             }
             break;
@@ -589,13 +599,27 @@ __device__ __forceinline__ void epilogue(const Cta &c, const Phase &ph, EpiCtx &
     }
 }
 
+__device__ __forceinline__ int attn_total(const Cta &c, const KvPtrs &kv, int step);
+__device__ __forceinline__ AttnItem attn_item(const Cta &c, const KvPtrs &kv, int step, int item);
+__device__ __forceinline__ MergeUnit merge_unit(const Cta &c, const KvPtrs &kv, int step, int u);
+
 // The phase of program position g (c.R is its row count already); every consumer thread calls it, between two CTA barriers.
 // PRE: the first tile's epilogue operands are kept from here on (with two sets of accumulators there are no registers for them).
 template <bool PRE>
 __device__ __forceinline__ void make_phase(const Cta &c, Phase &g) {
     const MegaParams &p = *c.p;
     const Scratch &s = p.s;
-    if (g.kind >= kMatrixKinds) return;
+    if (g.kind >= kMatrixKinds) {
+        // the geometry of the CTA's first piece of work takes divisions and the parameter block: 600 to 900 cycles
+        if (g.kind == ATTN && c.tid == kConsumerThreads - 1) {
+            const int total = attn_total(c, p.kvs[g.layer], g.step);
+            c.misc->n_items = total;
+            if (c.cta < total) c.misc->item = attn_item(c, p.kvs[g.layer], g.step, c.cta);
+        }
+        if (g.kind == MERGE && c.tid == kConsumerThreads - 1 && c.cta < c.R * p.Hq)
+            c.misc->unit = merge_unit(c, p.kvs[g.layer], g.step, c.cta);
+        return;
+    }
     PhaseIo io;
     io.in_hi = s.actH_hi; io.in_lo = s.actH_lo; io.in_stride = p.dp; io.in_len = p.d;
     io.sstab = nullptr; io.res = nullptr; io.gain = nullptr; io.gain2 = nullptr; io.ids = nullptr;
@@ -1264,8 +1288,6 @@ __device__ __forceinline__ void attn_rows_mma(Cta &c, const bf16_t *sk, const bf
     }
 }
 
-struct AttnItem { int b, kvh, chunk, Lb, nch, base, rows; };
-
 // Positions the cache of `kv` has slots for (positions beyond are flagged, never touched), the committed
 // length of a sequence brought into that range, the position of its row 0 in `step` and the chunks its
 // rows can see: every index the attention and merge phases form from seq_lens stays inside the block
@@ -1362,9 +1384,9 @@ __device__ __forceinline__ void attention_phase(Cta &c, const KvPtrs &kv, int st
     const int max_tokens = min(kv.max_pages * p.page, p.max_ctx);   // positions beyond are flagged, not touched
     const int upt = dh >> 3;
 
-    const int total = attn_total(c, kv, step);
+    const int total = c.misc->n_items;
     for (int item = c.cta; item < total; item += c.grid) {
-        const AttnItem it = attn_item(c, kv, step, item);
+        const AttnItem it = item == c.cta ? c.misc->item : attn_item(c, kv, step, item);
         const int b = it.b, kvh = it.kvh, chunk = it.chunk, Lb = it.Lb;
         const int base = it.base;                  // position of row m = 0
         const int rows = it.rows;                  // rows of this sequence that count (the rest is padding)
@@ -1471,13 +1493,23 @@ __device__ __forceinline__ void attention_phase(Cta &c, const KvPtrs &kv, int st
 // depends only on the number of visible chunks, i.e. on the row's position.
 // What bounds it is L2 latency: a thread requests its first chunks' vectors together with the maxima. (A unit used to be a
 // quarter of a head: four rows of 28 heads were four rounds on some CTAs, 6.2 us of a layer's 121; a 28-layer call with four rows 3391 -> 3253 us.)
+__device__ __forceinline__ MergeUnit merge_unit(const Cta &c, const KvPtrs &kv, int step, int u) {
+    const MegaParams &p = *c.p;
+    MergeUnit mu;
+    mu.r = u / p.Hq;
+    mu.hq = u - mu.r * p.Hq;
+    const int b = mu.r / c.M, m = mu.r - b * c.M;
+    const int pos = min(step_base(c, kv, b, step) + min(m, step_rows(c, b, step) - 1), kv_max_tokens(p, kv) - 1);
+    mu.ncm = min(pos / kAttnChunk + 1, p.max_chunks);        // chunks visible to this row
+    mu.src = p.s.att_part + ((size_t)mu.r * p.Hq + mu.hq) * p.max_chunks * (p.dh + kPartPad);
+    return mu;
+}
 __device__ __forceinline__ void merge_phase(Cta &c, const KvPtrs &kv, int step) {
     const MegaParams &p = *c.p;
-    const int dh = p.dh, M = c.M, stride = dh + kPartPad;
+    const int dh = p.dh, stride = dh + kPartPad;
     const int q4 = dh >> 2;                          // threads across a head (32 or 16)
     const int ncg = kConsumerThreads / q4;           // chunk groups (8 or 16)
-    constexpr int kPre = 4;                          // a thread's chunks requested before the maxima are known
-    const int max_tokens = min(kv.max_pages * p.page, p.max_ctx);
+    constexpr int kPre = 5;                          // a thread's chunks requested before the maxima are known (2560 positions at head dim 128)
     float *ms = reinterpret_cast<float *>(c.scr);    // [max_chunks] chunk maxima
     float *ls = ms + p.max_chunks;                   // [max_chunks] chunk denominators
     // [ncg][stride] partial sums (+ denominators), behind those where the staging area has the room, else in their place
@@ -1486,11 +1518,9 @@ __device__ __forceinline__ void merge_phase(Cta &c, const KvPtrs &kv, int step) 
     const int units = c.R * p.Hq;
     const int el = (c.tid % q4) * 4, cg = c.tid / q4;
     for (int u = c.cta; u < units; u += c.grid) {
-        const int r = c.R > 1 ? u / p.Hq : 0, hq = u - r * p.Hq;
-        const int b = M > 1 ? r / M : r, m = r - b * M;
-        const int pos = min(step_base(c, kv, b, step) + min(m, step_rows(c, b, step) - 1), max_tokens - 1);
-        const int ncm = min(pos / kAttnChunk + 1, p.max_chunks);        // chunks visible to this row
-        const float *src = p.s.att_part + ((size_t)r * p.Hq + hq) * p.max_chunks * stride;
+        const MergeUnit mu = u == c.cta ? c.misc->unit : merge_unit(c, kv, step, u);
+        const int r = mu.r, hq = mu.hq, ncm = mu.ncm;
+        const float *src = mu.src;
         uint4 pre[kPre];
 #pragma unroll
         for (int i = 0; i < kPre; ++i) pre[i] = ldcg128(src + (size_t)min(cg + i * ncg, ncm - 1) * stride + el);
@@ -1521,7 +1551,7 @@ __device__ __forceinline__ void merge_phase(Cta &c, const KvPtrs &kv, int step) 
             int j = 0;
             if (t0 == 0) {
 #pragma unroll
-                for (int i = 0; i < kPre; ++i) add(i, pre[i]);
+                for (int i = 0; i < kPre; ++i) if (cg_warp + i * ncg < ncm) add(i, pre[i]);
                 j = kPre;
             }
 #pragma unroll 4
@@ -1731,7 +1761,7 @@ __global__ void __launch_bounds__(TM ? kTmThreads : kThreads, 1) mega_kernel(con
     EpiCtx ex;
     ex.best = 0ull;
     Phase ph;
-    ph.pre = EpiPre{0.f, 0.f, 0.f, 0};
+    ph.pre = EpiPre{0.f, 0, 0, 0};
     prog_begin(p, ph);
     make_phase<!TWO && !TM>(c, ph);
     bar_sync(1, kConsumerThreads);
