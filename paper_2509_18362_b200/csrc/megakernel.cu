@@ -84,6 +84,10 @@ struct AttnItem { int b, kvh, chunk, Lb, nch, base, rows; };
 // A work unit of the merge phase: a row's query head, its chunk partials and how many of them it sees.
 struct MergeUnit { const float *src; int r, hq, ncm; };
 
+// The gate/up rows the producer asks to be brought into L2 while it waits (see ahead_begin): pieces asked for, pieces, and
+// when the next one is due.
+struct Ahead { const bf16_t *gate, *up; int i, n; unsigned long long due; };
+
 struct Misc {   // small shared-memory block
     uint64_t full[kMaxStages];
     uint64_t empty[kMaxStages];
@@ -105,6 +109,7 @@ struct Misc {   // small shared-memory block
     AttnItem item;                   // this CTA's first item of the current attention phase, and the phase's items
     int n_items;
     MergeUnit unit;                  // and its first unit of the current merge phase
+    Ahead ahead;
     Geom geo[kMatrixKinds];          // filled once per launch: row shares and stage counts take divisions, 800 cycles at every phase start
     unsigned long long rowptr[kProducerWarps][32];   // tile row pointers, one line per producer warp
     int flag;
@@ -394,9 +399,48 @@ __device__ __forceinline__ void tile_ptrs(Cta &c, int kind, const LayerPtrs &L, 
 // 4*j + rb = weight row g + 8*rb, k elements [32*ch + 8*t, +8) with ch = 8*(j >> 1) + 2*wi + (j & 1). A producer
 // instruction still copies 512 contiguous bytes of one weight row; the eight lanes of a quarter-warp land in eight
 // different 16-byte bank groups.
+// Between QKV and gate/up the consumers attend, merge and project (18000 cycles with their barriers) while the ring takes 4 us
+// of the stream: HBM would idle for 10 us of a layer. Meanwhile one producer thread asks for a quarter of the gate/up weights to be
+// brought into L2, at about the rate at which HBM serves an SM: of every tile but the first (the ring holds that) the first
+// kAheadRows of its 16 gate and 16 up rows, so that later every stage is part L2 hit, part HBM and the SM's copy path,
+// faster than its share of HBM, takes in both at once. Whole rows in one request each: by 128-byte lines or column
+// blocks, or a stretch of stages ahead of the ring, it loses time. 7B shape, us: draft of three steps 442 -> 409 (one row of 16 426, two
+// 420, six 415), 28 layers of one row 2648 -> 2450, of four rows 2994 -> 2866. 50 MB per layer stay well inside L2.
+constexpr int kAheadRows = 4;
+constexpr uint32_t kAheadNsPerKB = 18;
+__device__ __forceinline__ void ahead_begin(const Cta &c, const LayerPtrs &L) {
+    const Geom &g = c.misc->geo[GATEUP];
+    Ahead &a = c.misc->ahead;
+    a.gate = L.w_gate;
+    a.up = L.w_up;
+    a.i = 0;
+    a.n = 2 * ((g.v1 - g.v0 + g.cap - 1) / g.cap - 1);
+    a.due = 0;
+}
+// Until the stage is free or everything is asked for.
+__device__ __forceinline__ void ahead_while_waiting(const Cta &c, uint64_t *bar, uint32_t parity) {
+    const int d = c.p->d;
+    const Geom &g = c.misc->geo[GATEUP];
+    Ahead &a = c.misc->ahead;
+    int i = a.i;
+    unsigned long long due = a.due;
+    while (i < a.n && !mbar_test(bar, parity)) {
+        const unsigned long long now = global_timer_ns();
+        if (now < due) { __nanosleep(32); continue; }
+        const int row = g.v0 + (1 + (i >> 1)) * g.cap;
+        const uint32_t bytes = (uint32_t)min(kAheadRows, g.v1 - row) * (uint32_t)d * 2u;
+        prefetch_l2((i & 1 ? a.up : a.gate) + (size_t)row * d, bytes);
+        due = now + (bytes >> 10) * kAheadNsPerKB;
+        ++i;
+    }
+    a.i = i;
+    a.due = due;
+}
+
 template <bool TM>
 __device__ __forceinline__ void produce_phase(Cta &c, int kind, const LayerPtrs &L) {
     const MegaParams &p = *c.p;
+    if (!TM && kind == OPROJ && c.tid == kConsumerThreads) ahead_begin(c, L);
     const Geom g = geom(c, kind);
     const int pw = c.warp - kConsumerWarps;
     const unsigned char *cur[kRowsPerProducer], *nxt[kRowsPerProducer];
@@ -435,7 +479,10 @@ __device__ __forceinline__ void produce_phase(Cta &c, int kind, const LayerPtrs 
             const uint32_t parity = c.parity;
             bool ok = true;
             PROF_T0();
-            if (c.lane == 0) ok = wait_bar(c, &c.empty[slot], parity ^ 1u);
+            if (c.lane == 0) {
+                if (!TM && pw == 0 && (kind == OPROJ || (kind == GATEUP && vr0 == g.v0))) ahead_while_waiting(c, &c.empty[slot], parity ^ 1u);
+                ok = wait_bar(c, &c.empty[slot], parity ^ 1u);
+            }
             ok = __shfl_sync(0xffffffffu, ok, 0);
             PROF_ACC(c, 2, pw == 0 && c.lane == 0);
             if (!ok) return;   // abort: stop issuing copies
