@@ -7,7 +7,7 @@
 // the high part of activation row r and n = 2r + 1 the low part, so the pair carries an fp32
 // value) is small and re-read from L2 for every item. One CTA per SM walks a static list of work
 // items (row range, K range). Roles: warps 0-3 epilogue (TMEM -> registers -> global), warp 4 issues
-// the MMAs, warp 5 the TMA tile copies of X, warps 6-13 copy A with 16-byte cp.async, laid out as the MMA's
+// the MMAs, warp 5 the TMA tile copies of X, warp 14 see GemmArgs::ahead, warps 6-13 copy A with 16-byte cp.async, laid out as the MMA's
 // 128-byte-swizzled K-major tiles (64 K elements wide). Accumulators are double buffered in TMEM so the epilogue of one
 // item overlaps the MMAs of the next; in the epilogue of the last item the copy warps help.
 //
@@ -35,7 +35,7 @@
 namespace fmtp {
 
 constexpr int kGemmProducers = 256;          // eight copy warps
-constexpr int kGemmThreads = 192 + kGemmProducers;
+constexpr int kGemmThreads = 192 + kGemmProducers + 32;     // warp 14 asks for a later GEMM's weights
 constexpr int kGemmBK = 64;                 // K elements per swizzled block: one 128-byte row
 constexpr int kGemmTileM = 128;
 constexpr int kGemmTileBytes = kGemmTileM * 128;    // a tile's 64-wide block
@@ -75,7 +75,17 @@ struct GemmArgs {
     int n_stages, n_xstages;
     unsigned long long wait_limit_ns;   // every wait of the kernel gives up after this long
     int extra_arrivals;          // self-test only: arrivals a ring stage expects beyond the copies that are made
+    // Two row-major matrices [ahead_rows][ahead_ld] that a later GEMM streams by tiles of 128 rows: while this one runs, the first
+    // kAheadRows rows of every tile are asked into L2. Used by W_o for gate/up: its own weights are in the ring when attention
+    // ends, and until gate/up starts (merge, W_o, post: 15 us) HBM has nothing else to do. Then every stage of gate/up is part
+    // L2 hit, part HBM, and the copy path takes in both at once. 7B shape, four ragged sequences, five steps 728 -> 704 us (8 rows of 128
+    // 716, 16 707, 48 704, 64 709), 16 sequences 556 -> 552. At 64 rows it loses (64 ragged 905 -> 911, 16 x 4 rows of 28 layers
+    // 4178 -> 4212): there the activation block's re-reads fill the path between L2 and the SMs. So only with four-block stages.
+    const bf16_t *ahead[2];
+    int ahead_rows, ahead_ld;
 };
+constexpr int kAheadTileRows = 32;
+constexpr uint32_t kAheadPiece = 16384, kAheadPieceNs = 600;     // bytes of a request, and the time to the next one
 
 struct GemmSmem {
     uint64_t full[kGemmMaxStages], empty[kGemmMaxStages];
@@ -214,7 +224,29 @@ __global__ void __launch_bounds__(kGemmThreads, 1) skinny_gemm_kernel(const __gr
     const int n_my = gemm_my_items(n_items);
     auto tiles_of = [&](const GemmItem &gi) -> int { return g.epi == EPI_SWIGLU || gi.row_end - gi.row0 > kGemmTileM ? 2 : 1; };
 
-    if (warp >= 6) {
+    if (warp == 14) {
+        // ================= a later GEMM's weights into L2, one thread, until this CTA's last MMA is done
+        if (KA == 4 && lane == 0 && g.ahead[0]) {
+            const int tiles = (g.ahead_rows + kGemmTileM - 1) / kGemmTileM;
+            unsigned long long due = 0;
+            bool go = true;
+            for (int t = 2 * (int)blockIdx.x; t < 2 * tiles && go; t += (t & 1) ? 2 * (int)gridDim.x - 1 : 1) {      // both matrices of a tile, then the CTA's next tile
+                const int row = (t >> 1) * kGemmTileM;
+                const unsigned char *src = reinterpret_cast<const unsigned char *>(g.ahead[t & 1] + (size_t)row * g.ahead_ld);
+                const uint32_t bytes = (uint32_t)min(kAheadTileRows, g.ahead_rows - row) * (uint32_t)g.ahead_ld * 2u;
+                for (uint32_t at = 0; at < bytes && go; at += kAheadPiece) {
+                    while (go && global_timer_ns() < due) {
+                        go = !mbar_test(&sm->drain, 0);
+                        __nanosleep(100);
+                    }
+                    if (!go) break;
+                    prefetch_l2(src + at, min(kAheadPiece, bytes - at));
+                    due = global_timer_ns() + kAheadPieceNs;
+                }
+            }
+        }
+        __syncwarp();
+    } else if (warp >= 6) {
         // ================= weight copies: thread pt copies 16-byte column c of rows r0, r0 + 32, ... of a tile, KA K blocks at a
         // time: the blocks are immediate offsets on the source, so a pointer register is rewritten only once per stage (a
         // cp.async reads its address when it leaves the queue; rewriting it waits for that)
@@ -352,7 +384,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) skinny_gemm_kernel(const __gr
         __syncwarp();
     }
     unsigned long long (*last_max)[64] = reinterpret_cast<unsigned long long (*)[64]>(ring);     // EPI_ARGMAX: maxima of the last item, per warp quarter
-    if (warp < 4 || warp >= 6) {
+    if (warp < 4 || (warp >= 6 && warp < 14)) {
         // ================= epilogue: thread = one row of a tile (TMEM lane 32*(warp % 4) + lane), eight activation rows at a time.
         // One warp per scheduler would be a chain of latencies (64 rows, 3584-wide layer: 7 us of divides in gate/up, 18 us of
         // warp maxima in the output head when the rows went one after the other, 5 and 5 us by eights), and after the last item
