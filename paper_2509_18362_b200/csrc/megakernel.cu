@@ -830,6 +830,9 @@ __device__ __forceinline__ void consume_tiles(Cta &c, const Phase &ph, const Act
         // which half of the warps takes a stage depends only on the stage's index within the phase,
         // never on how many stages the CTA has seen before: the summation order of a row must not
         // depend on the batch or on earlier calls
+        // The stages that come by way of the slice ring are those the fast loop reads, the ones of sixteen chunks. The last of them
+        // may end 16 columns early (ffn = 496 mod 512): the input's rows are zero up to the next multiple of 32.
+        auto sixteen_chunks = [](const StageK &sk) -> bool { return sk.klen > 15 * 32; };
         // slice ring: slot (stage index mod 4) x warp of the owning group x activation row x 512 bytes
         const uint32_t slice_base = smem_u32(c.scr) + (uint32_t)(wi * R) * 512u;
         auto slice_slot = [&](int sa) -> uint32_t { return slice_base + (uint32_t)((sa & 3) * 4 * R) * 512u; };
@@ -846,7 +849,7 @@ __device__ __forceinline__ void consume_tiles(Cta &c, const Phase &ph, const Act
         const int first = ((stage0 & 1) == grp) ? 0 : 1;            // first stage this warp owns
         if (gfast && first < geo.nks) {
             const StageK s0 = stage_k(geo, first);
-            if (s0.klen == 512) slice_fetch(stage0 + first, s0);
+            if (sixteen_chunks(s0)) slice_fetch(stage0 + first, s0);
         }
         // the second input segment starts: every warp parks the sums of the first (whichever stages of it the warp owned)
         auto second_segment = [&]() {
@@ -985,7 +988,7 @@ __device__ __forceinline__ void consume_tiles(Cta &c, const Phase &ph, const Act
                         bool more = false;
                         if (ks + 2 < geo.nks) {
                             const StageK s2 = stage_k(geo, ks + 2);
-                            if (s2.klen == 512) { slice_fetch(stage0 + ks + 2, s2); more = true; }   // (a shorter last stage is read directly by the loop below)
+                            if (sixteen_chunks(s2)) { slice_fetch(stage0 + ks + 2, s2); more = true; }   // (a shorter last stage is read directly by the loop below)
                         }
                         if (more) asm volatile("cp.async.wait_group 1;" ::: "memory");
                         else asm volatile("cp.async.wait_group 0;" ::: "memory");
