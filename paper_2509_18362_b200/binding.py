@@ -24,7 +24,7 @@ FMTP_OK = 0
 DEV_BAD_TOKEN, DEV_BAD_PAGE, DEV_BAD_POS, DEV_TIMEOUT, DEV_ALL_NAN = 1, 2, 4, 8, 16
 
 EXPORTS = ["fmtp_create", "fmtp_destroy", "fmtp_workspace_bytes", "fmtp_set_workspace", "fmtp_strerror",
-           "fmtp_last_cuda_error", "fmtp_launch_count", "fmtp_tmem_launch_count", "fmtp_selftest_wait_timeout", "fmtp_selftest_inject_wait_timeout",
+           "fmtp_last_cuda_error", "fmtp_launch_count", "fmtp_tmem_launch_count", "fmtp_selftest_wait_timeout", "fmtp_selftest_inject_wait_timeout", "fmtp_selftest_ahead",
            "fastmtp_draft", "fastmtp_draft_host",
            "fastmtp_verify_accept", "fastmtp_verify_accept_host", "fastmtp_verify_accept_static", "fastmtp_accept_ids",
            "fastmtp_target_step"]
@@ -77,6 +77,9 @@ lib.fmtp_selftest_wait_timeout.argtypes = [_p, C.c_int, _p, _p]
 lib.fmtp_selftest_wait_timeout.restype = C.c_int
 lib.fmtp_selftest_inject_wait_timeout.argtypes = [_p, C.c_int, C.c_int]
 lib.fmtp_selftest_inject_wait_timeout.restype = C.c_int
+lib.fmtp_selftest_ahead.argtypes = [C.c_int, C.c_int, C.c_int, C.c_int, C.c_longlong, C.c_int, C.c_int, C.POINTER(C.c_int),
+                                    C.POINTER(C.c_longlong), C.POINTER(C.c_uint)]
+lib.fmtp_selftest_ahead.restype = C.c_int
 lib.fastmtp_draft.argtypes = [_p, C.POINTER(fmtp_mtp_w), _p, _p, _p, C.c_int, C.POINTER(fmtp_kv), C.c_int, C.c_int, _p,
                               C.c_int, _p, _p, _p, _p, _p]
 lib.fastmtp_draft.restype = C.c_int
@@ -152,6 +155,17 @@ def fmtp_selftest_wait_timeout(dev_status, limit_ms, dev_waited_ns=None, stream=
     rc = lib.fmtp_selftest_wait_timeout(_ptr(dev_status), int(limit_ms), _ptr(dev_waited_ns), _stream(stream))
     if rc != FMTP_OK:
         raise FastMTPError(rc, "fmtp_selftest_wait_timeout")
+
+
+def fmtp_selftest_ahead(batched, ffn, d, grid, l2_bytes, cta):
+    """Requests of one CTA for gate/up weights ahead of their phase, as (matrix, first element, bytes); see include/fastmtp.h."""
+    args = (int(batched), int(ffn), int(d), int(grid), int(l2_bytes), int(cta))
+    n = lib.fmtp_selftest_ahead(*args, 0, None, None, None)
+    if n < 0:
+        raise FastMTPError(n, "fmtp_selftest_ahead")
+    mat, at, size = (C.c_int * n)(), (C.c_longlong * n)(), (C.c_uint * n)()
+    lib.fmtp_selftest_ahead(*args, n, mat, at, size)
+    return list(zip(mat, at, size))
 
 
 STATIC_VERIFY_MAX_ROWS = 1024

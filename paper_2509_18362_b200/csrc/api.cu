@@ -4,6 +4,7 @@
 #include "../../include/fastmtp.h"
 #include "mega.cuh"
 #include "batched.cuh"
+#include "ahead.cuh"
 
 #include <cmath>
 #include <cstdlib>
@@ -17,6 +18,7 @@ struct fmtp_ctx {
     fmtp_shape shape;
     int n_sm;
     int smem_optin;
+    long long ahead_budget;    // bytes of weights a layer may ask into L2 ahead of their phase
     int KC;
     int dp, qp, Fp;
     int max_chunks;
@@ -241,6 +243,7 @@ int launch_mega(fmtp_ctx *c, MegaParams &p, cudaStream_t st) {
         cfg.smem = smem;
         cfg.grid = grid > c->n_sm ? c->n_sm : grid;
     }
+    p.ahead_limit = mega_ahead_limit(c->ahead_budget, cfg.grid, p.d);
     err = mega_launch(p, cfg.grid, st);
     if (err) return cuda_fail(c, (cudaError_t)err);
     c->launches++;
@@ -306,11 +309,12 @@ int fmtp_create(const fmtp_shape *sh, fmtp_ctx **out) {
     if (sh->d % 64 || sh->ffn % 16 || sh->n_q_heads % sh->n_kv_heads || sh->n_q_heads / sh->n_kv_heads > 8 ||
         sh->max_rows > 4096 || sh->n_layers > kMaxLayers)
         return FMTP_ESHAPE;
-    int dev = 0, major = 0, sms = 0, optin = 0;
+    int dev = 0, major = 0, sms = 0, optin = 0, l2 = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&major, cudaDevAttrComputeCapabilityMajor, dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&l2, cudaDevAttrL2CacheSize, dev);
     if (e != cudaSuccess || major < 10) return FMTP_ECUDA;
     fmtp_ctx *c = new (std::nothrow) fmtp_ctx();
     if (!c) return FMTP_ENOMEM;
@@ -318,6 +322,7 @@ int fmtp_create(const fmtp_shape *sh, fmtp_ctx **out) {
     c->shape = *sh;
     c->n_sm = sms;
     c->smem_optin = optin;
+    c->ahead_budget = ahead_budget(l2);
     c->KC = (sh->d % 512 == 0) ? 512 : (sh->d % 256 == 0) ? 256 : (sh->d % 128 == 0) ? 128 : 64;
     c->dp = (sh->d + 31) & ~31;
     c->qp = (sh->n_q_heads * sh->head_dim + 31) & ~31;
@@ -453,7 +458,7 @@ int fastmtp_draft(fmtp_ctx *c, const fmtp_mtp_w *w, const fmtp_bf16 *h_last, con
             std::memset(&bc, 0, sizeof(bc));
             bc.sh = c->bsh; bc.ws = c->bws;
             bc.rope_cos = c->s.rope_cos; bc.rope_sin = c->s.rope_sin;
-            bc.n_sm = c->n_sm; bc.smem_optin = c->smem_optin; bc.cache = &c->tmaps;
+            bc.n_sm = c->n_sm; bc.smem_optin = c->smem_optin; bc.ahead_budget = c->ahead_budget; bc.cache = &c->tmaps;
             bc.wait_limit_ns = kDefaultWaitNs;
             if (c->inject_which >= 2) { bc.wait_limit_ns = c->inject_limit_ns; bc.inject = c->inject_which; c->inject_which = 0; }
             bc.B = (B - b0 < kBatchRows) ? B - b0 : kBatchRows;
@@ -628,7 +633,7 @@ int fastmtp_target_step(fmtp_ctx *c, const fmtp_target_w *w, const int32_t *toke
             std::memset(&tc, 0, sizeof(tc));
             tc.sh = c->bsh; tc.ws = c->bws;
             tc.rope_cos = c->s.rope_cos; tc.rope_sin = c->s.rope_sin;
-            tc.n_sm = c->n_sm; tc.smem_optin = c->smem_optin; tc.cache = &c->tmaps; tc.wait_limit_ns = kDefaultWaitNs;
+            tc.n_sm = c->n_sm; tc.smem_optin = c->smem_optin; tc.ahead_budget = c->ahead_budget; tc.cache = &c->tmaps; tc.wait_limit_ns = kDefaultWaitNs;
             tc.B = Bg; tc.M = M; tc.n_layers = nl;
             tc.tokens = tokens + (size_t)b0 * M;
             tc.out_h = out_h ? out_h + (size_t)b0 * M * d : nullptr;

@@ -1273,7 +1273,7 @@ int batched_draft(const BatchedCall &c, cudaStream_t st, long long *launches) {
         // x += W_o o
         g = GemmArgs{};
         g.a[0] = c.layer.wo; g.a_rows[0] = d; g.n_seg = 1; g.epi = EPI_PARTIAL;
-        g.ahead[0] = c.layer.w_gate; g.ahead[1] = c.layer.w_up; g.ahead_rows = sh.F; g.ahead_ld = d;
+        g.ahead[0] = c.layer.w_gate; g.ahead[1] = c.layer.w_up; g.ahead_rows = sh.F; g.ahead_ld = d; g.ahead_limit = gemm_ahead_limit(c.ahead_budget, sh.F);
         if ((rc = gemm(g, rows, d, qdim, qdim, ws.xop0, ws.ld0))) return rc;
         if ((rc = post(g.splits, 1, 0, c.layer.g_post))) return rc;
         // act = silu(W_gate n) * (W_up n), written as the down projection's operand
@@ -1373,7 +1373,7 @@ int batched_target(const BatchedTargetCall &c, cudaStream_t st, long long *launc
         if ((rc = attention(sh, ws, kv, geo, R, c.n_sm, c.wait_limit_ns, 0, c.cache, st, launches))) return rc;
         g = GemmArgs{};
         g.a[0] = L.wo; g.a_rows[0] = d; g.n_seg = 1; g.epi = EPI_PARTIAL;
-        g.ahead[0] = L.w_gate; g.ahead[1] = L.w_up; g.ahead_rows = sh.F; g.ahead_ld = d;
+        g.ahead[0] = L.w_gate; g.ahead[1] = L.w_up; g.ahead_rows = sh.F; g.ahead_ld = d; g.ahead_limit = gemm_ahead_limit(c.ahead_budget, sh.F);
         if ((rc = gemm(g, d, qdim, qdim, ws.xop0, ws.ld0))) return rc;
         if ((rc = post(g.splits, 0, L.g_post))) return rc;
         g = GemmArgs{};

@@ -58,6 +58,7 @@ struct BatchedCall {
     BatchedWs ws;
     const float *rope_cos, *rope_sin;     // [max_ctx][dh/2]
     int n_sm, smem_optin;
+    long long ahead_budget;               // see ahead.cuh
     TmapCache *cache;
     unsigned long long wait_limit_ns;     // every device-side wait gives up after this long
     int inject;                           // self-test: a copy that is never made is expected by the call's first GEMM (2) or attention (3)
@@ -81,6 +82,7 @@ struct BatchedTargetCall {
     BatchedWs ws;
     const float *rope_cos, *rope_sin;
     int n_sm, smem_optin;
+    long long ahead_budget;               // see ahead.cuh
     TmapCache *cache;
     unsigned long long wait_limit_ns;
     int B, M, n_layers;                   // B * M <= kBatchRows rows

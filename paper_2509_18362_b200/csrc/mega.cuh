@@ -31,6 +31,9 @@ constexpr int kTmSlotCols = 64;
 
 typedef uint16_t bf16_t;
 
+// First of the rows of a matrix that CTA `cta` of `grid` has; the next CTA's first ends its share.
+__host__ __device__ inline int share_first(int cta, int rows, int grid) { return (int)(((long long)cta * rows) / grid); }
+
 struct LayerPtrs {
     const bf16_t *g_in, *wq, *wk, *wv, *wo, *g_post, *w_gate, *w_up, *w_down;
 };
@@ -74,6 +77,7 @@ struct MegaParams {
     int max_chunks;                   // capacity of att_part's chunk dimension
     int max_ctx;                      // rows of the rotary table
     unsigned long long wait_limit_ns; // every device-side wait gives up after this long (2 s outside the self-test)
+    int ahead_limit;                  // requests for gate/up weights a CTA may make per layer (mega_ahead_limit)
     int extra_arrivals;               // self-test only: arrivals the grid barrier expects beyond the CTAs that exist
     int use_tmem;                     // weight stages pass through tensor memory (stage = 32 rows x 512, every K a multiple of 512, R <= 4)
     // call

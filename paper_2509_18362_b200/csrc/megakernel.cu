@@ -37,6 +37,7 @@
 //     maximum per activation row and publishes it with one 64-bit atomicMax per CTA; logits are
 //     never written unless a debug buffer is passed.
 #include "mega.cuh"
+#include "ahead.cuh"
 #include "ptx.cuh"
 #include "umma.cuh"
 
@@ -326,8 +327,8 @@ __device__ __forceinline__ Geom make_geom(const Cta &c, int kind) {
         default:     g.rows = p.N;                    g.K = p.d;     break;
     }
     g.cap = (kind == GATEUP) ? kTileRows / 2 : kTileRows;
-    g.v0 = (int)(((long long)c.cta * g.rows) / c.grid);
-    g.v1 = (int)(((long long)(c.cta + 1) * g.rows) / c.grid);
+    g.v0 = share_first(c.cta, g.rows, c.grid);
+    g.v1 = share_first(c.cta + 1, g.rows, c.grid);
     g.kc = p.KC;
     g.rs = g.kc * 2;
     g.seglen = (kind == PROJ) ? p.d : g.K;
@@ -405,8 +406,7 @@ __device__ __forceinline__ void tile_ptrs(Cta &c, int kind, const LayerPtrs &L, 
 // kAheadRows of its 16 gate and 16 up rows, so that later every stage is part L2 hit, part HBM and the SM's copy path,
 // faster than its share of HBM, takes in both at once. Whole rows in one request each: by 128-byte lines or column
 // blocks, or a stretch of stages ahead of the ring, it loses time. 7B shape, us: draft of three steps 442 -> 409 (one row of 16 426, two
-// 420, six 415), 28 layers of one row 2648 -> 2450, of four rows 2994 -> 2866. 50 MB per layer stay well inside L2.
-constexpr int kAheadRows = 4;
+// 420, six 415), 28 layers of one row 2648 -> 2450, of four rows 2994 -> 2866.
 constexpr uint32_t kAheadNsPerKB = 18;
 __device__ __forceinline__ void ahead_begin(const Cta &c, const LayerPtrs &L) {
     const Geom &g = c.misc->geo[GATEUP];
@@ -414,7 +414,7 @@ __device__ __forceinline__ void ahead_begin(const Cta &c, const LayerPtrs &L) {
     a.gate = L.w_gate;
     a.up = L.w_up;
     a.i = 0;
-    a.n = 2 * ((g.v1 - g.v0 + g.cap - 1) / g.cap - 1);
+    a.n = mega_ahead_count(g.v0, g.v1, g.cap, c.p->ahead_limit);
     a.due = 0;
 }
 // Until the stage is free or everything is asked for.
@@ -427,10 +427,9 @@ __device__ __forceinline__ void ahead_while_waiting(const Cta &c, uint64_t *bar,
     while (i < a.n && !mbar_test(bar, parity)) {
         const unsigned long long now = global_timer_ns();
         if (now < due) { __nanosleep(32); continue; }
-        const int row = g.v0 + (1 + (i >> 1)) * g.cap;
-        const uint32_t bytes = (uint32_t)min(kAheadRows, g.v1 - row) * (uint32_t)d * 2u;
-        prefetch_l2((i & 1 ? a.up : a.gate) + (size_t)row * d, bytes);
-        due = now + (bytes >> 10) * kAheadNsPerKB;
+        const AheadReq r = mega_ahead_req(g.v0, g.v1, g.cap, d, i);
+        prefetch_l2((r.mat ? a.up : a.gate) + r.at, r.bytes);
+        due = now + (r.bytes >> 10) * kAheadNsPerKB;
         ++i;
     }
     a.i = i;

@@ -29,6 +29,7 @@
 #pragma once
 #include "umma.cuh"
 #include "batched.cuh"
+#include "ahead.cuh"
 #include <cuda.h>
 #include <cstring>
 
@@ -76,16 +77,16 @@ struct GemmArgs {
     unsigned long long wait_limit_ns;   // every wait of the kernel gives up after this long
     int extra_arrivals;          // self-test only: arrivals a ring stage expects beyond the copies that are made
     // Two row-major matrices [ahead_rows][ahead_ld] that a later GEMM streams by tiles of 128 rows: while this one runs, the first
-    // kAheadRows rows of every tile are asked into L2. Used by W_o for gate/up: its own weights are in the ring when attention
+    // kAheadTileRows rows of these are asked into L2, as far as the time and ahead.cuh's bound allow. Used by W_o for gate/up: its own weights are in the ring when attention
     // ends, and until gate/up starts (merge, W_o, post: 15 us) HBM has nothing else to do. Then every stage of gate/up is part
     // L2 hit, part HBM, and the copy path takes in both at once. 7B shape, four ragged sequences, five steps 728 -> 704 us (8 rows of 128
     // 716, 16 707, 48 704, 64 709), 16 sequences 556 -> 552. At 64 rows it loses (64 ragged 905 -> 911, 16 x 4 rows of 28 layers
     // 4178 -> 4212): there the activation block's re-reads fill the path between L2 and the SMs. So only with four-block stages.
     const bf16_t *ahead[2];
     int ahead_rows, ahead_ld;
+    uint32_t ahead_limit;        // bytes a CTA may ask for per tile (gemm_ahead_limit)
 };
-constexpr int kAheadTileRows = 32;
-constexpr uint32_t kAheadPiece = 16384, kAheadPieceNs = 600;     // bytes of a request, and the time to the next one
+constexpr uint32_t kAheadPieceNs = 600;     // from a request to the next one
 
 struct GemmSmem {
     uint64_t full[kGemmMaxStages], empty[kGemmMaxStages];
@@ -227,20 +228,21 @@ __global__ void __launch_bounds__(kGemmThreads, 1) skinny_gemm_kernel(const __gr
     if (warp == 14) {
         // ================= a later GEMM's weights into L2, one thread, until this CTA's last MMA is done
         if (KA == 4 && lane == 0 && g.ahead[0]) {
-            const int tiles = (g.ahead_rows + kGemmTileM - 1) / kGemmTileM;
+            uint32_t left = g.ahead_limit * (uint32_t)gemm_ahead_tiles((int)blockIdx.x, g.ahead_rows, (int)gridDim.x);
+            const int end = 2 * ((g.ahead_rows + kAheadTile - 1) / kAheadTile);
             unsigned long long due = 0;
             bool go = true;
-            for (int t = 2 * (int)blockIdx.x; t < 2 * tiles && go; t += (t & 1) ? 2 * (int)gridDim.x - 1 : 1) {      // both matrices of a tile, then the CTA's next tile
-                const int row = (t >> 1) * kGemmTileM;
-                const unsigned char *src = reinterpret_cast<const unsigned char *>(g.ahead[t & 1] + (size_t)row * g.ahead_ld);
-                const uint32_t bytes = (uint32_t)min(kAheadTileRows, g.ahead_rows - row) * (uint32_t)g.ahead_ld * 2u;
-                for (uint32_t at = 0; at < bytes && go; at += kAheadPiece) {
+            for (int t = 2 * (int)blockIdx.x; t < end && left && go; t = gemm_ahead_next(t, (int)gridDim.x)) {
+                const AheadReq r = gemm_ahead_share(t, g.ahead_rows, g.ahead_ld, left);
+                left -= r.bytes;
+                const unsigned char *src = reinterpret_cast<const unsigned char *>(g.ahead[r.mat] + r.at);
+                for (uint32_t at = 0; at < r.bytes && go; at += kAheadPiece) {
                     while (go && global_timer_ns() < due) {
                         go = !mbar_test(&sm->drain, 0);
                         __nanosleep(100);
                     }
                     if (!go) break;
-                    prefetch_l2(src + at, min(kAheadPiece, bytes - at));
+                    prefetch_l2(src + at, min(kAheadPiece, r.bytes - at));
                     due = global_timer_ns() + kAheadPieceNs;
                 }
             }
