@@ -77,7 +77,6 @@ struct MegaParams {
     int max_chunks;                   // capacity of att_part's chunk dimension
     int max_ctx;                      // rows of the rotary table
     unsigned long long wait_limit_ns; // every device-side wait gives up after this long (2 s outside the self-test)
-    int ahead_limit;                  // requests for gate/up weights a CTA may make per layer (mega_ahead_limit)
     int extra_arrivals;               // self-test only: arrivals the grid barrier expects beyond the CTAs that exist
     int use_tmem;                     // weight stages pass through tensor memory (stage = 32 rows x 512, every K a multiple of 512, R <= 4)
     // call
@@ -100,6 +99,7 @@ struct MegaParams {
     LayerPtrs layers[kMaxLayers];
     KvPtrs kvs[kMaxLayers];
     Scratch s;
+    int ahead_limit;                  // requests for gate/up weights a CTA may make per layer (mega_ahead_limit); read once per launch
 };
 
 // Shared-memory bytes the kernel needs for these parameters.

@@ -409,12 +409,10 @@ __device__ __forceinline__ void tile_ptrs(Cta &c, int kind, const LayerPtrs &L, 
 // 420, six 415), 28 layers of one row 2648 -> 2450, of four rows 2994 -> 2866.
 constexpr uint32_t kAheadNsPerKB = 18;
 __device__ __forceinline__ void ahead_begin(const Cta &c, const LayerPtrs &L) {
-    const Geom &g = c.misc->geo[GATEUP];
     Ahead &a = c.misc->ahead;
     a.gate = L.w_gate;
     a.up = L.w_up;
     a.i = 0;
-    a.n = mega_ahead_count(g.v0, g.v1, g.cap, c.p->ahead_limit);
     a.due = 0;
 }
 // Until the stage is free or everything is asked for.
@@ -1687,7 +1685,11 @@ __global__ void __launch_bounds__(TM ? kTmThreads : kThreads, 1) mega_kernel(con
         c.misc->aborted = 0;
         mbar_fence_init();
     }
-    if (c.tid >= 32 && c.tid < 32 + kMatrixKinds) c.misc->geo[c.tid - 32] = make_geom(c, c.tid - 32);
+    if (c.tid >= 32 && c.tid < 32 + kMatrixKinds) {
+        const Geom g = make_geom(c, c.tid - 32);
+        c.misc->geo[c.tid - 32] = g;
+        if (c.tid == 32 + GATEUP) c.misc->ahead.n = mega_ahead_count(g.v0, g.v1, g.cap, p.ahead_limit);
+    }
     if (c.tid < p.B) {
         c.misc->seqlen[c.tid] = p.kvs[0].seq_lens[c.tid];
         c.misc->next[c.tid] = (p.mode == 0 && p.n_ext) ? min(max(p.n_ext[c.tid], 1), p.M) : p.M;
