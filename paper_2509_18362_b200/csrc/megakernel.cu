@@ -1556,9 +1556,8 @@ __device__ __forceinline__ void merge_phase(Cta &c, const KvPtrs &kv, int step) 
     const int dh = p.dh, stride = dh + kPartPad;
     const int q4 = dh >> 2;                          // threads across a head (32 or 16)
     const int ncg = kConsumerThreads / q4;           // chunk groups (8 or 16)
-    constexpr int kPre = 5;                          // a thread's chunks requested before the maxima are known (2560 positions at head dim 128)
-    constexpr int kLater = 4;                        // and the later ones at once (one by one, behind the last one's shuffles, a call at 65536 positions
-                                                     // took 796 instead of 691 us)
+    constexpr int kPre = 5;                          // a thread's chunks requested at once, the first ones before the maxima are known (2560 positions
+                                                     // at head dim 128)
     float *ms = reinterpret_cast<float *>(c.scr);    // [max_chunks] chunk maxima
     float *ls = ms + p.max_chunks;                   // [max_chunks] chunk denominators
     // [ncg][stride] partial sums (+ denominators), behind those where the staging area has the room, else in their place
@@ -1571,8 +1570,13 @@ __device__ __forceinline__ void merge_phase(Cta &c, const KvPtrs &kv, int step) 
         const int r = mu.r, hq = mu.hq, ncm = mu.ncm;
         const float *src = mu.src;
         uint4 pre[kPre];
+        // (a chunk beyond the last is the last one once more: with a condition on each they go out one by one, 807 instead of 690 us
+        // for a call at 65536 positions)
+        auto fetch = [&](int n) {
 #pragma unroll
-        for (int i = 0; i < kPre; ++i) pre[i] = ldcg128(src + (size_t)min(cg + i * ncg, ncm - 1) * stride + el);
+            for (int i = 0; i < kPre; ++i) pre[i] = ldcg128(src + (size_t)min(cg + (n + i) * ncg, ncm - 1) * stride + el);
+        };
+        fetch(0);
         for (int i = c.tid; i < ncm; i += kConsumerThreads) {
             ms[i] = ldcg_f32(src + (size_t)i * stride + dh);
             ls[i] = ldcg_f32(src + (size_t)i * stride + dh + 1);
@@ -1597,19 +1601,11 @@ __device__ __forceinline__ void merge_phase(Cta &c, const KvPtrs &kv, int step) 
                 o2 += f * __uint_as_float(v.z); o3 += f * __uint_as_float(v.w);
                 l += f * lj;
             };
-            int j = 0;
-            if (t0 == 0) {
-#pragma unroll
-                for (int i = 0; i < kPre; ++i) if (cg_warp + i * ncg < ncm) add(i, pre[i]);
-                j = kPre;
-            }
 #pragma unroll 1
-            for (; j < q4 && cg_warp + (t0 + j) * ncg < ncm; j += kLater) {
-                uint4 v[kLater];
+            for (int j = 0; j < q4 && cg_warp + (t0 + j) * ncg < ncm; j += kPre) {
+                if (t0 + j > 0) fetch(t0 + j);
 #pragma unroll
-                for (int q = 0; q < kLater; ++q) v[q] = ldcg128(src + (size_t)min(cg + (t0 + j + q) * ncg, ncm - 1) * stride + el);
-#pragma unroll
-                for (int q = 0; q < kLater; ++q) if (j + q < q4) add(j + q, v[q]);
+                for (int i = 0; i < kPre; ++i) if (j + i < q4 && cg_warp + (t0 + j + i) * ncg < ncm) add(j + i, pre[i]);
             }
         }
         if (tight) bar_sync(1, kConsumerThreads);    // every thread has read the maxima and sums
