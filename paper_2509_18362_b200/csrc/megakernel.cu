@@ -393,20 +393,15 @@ __device__ __forceinline__ void tile_ptrs(Cta &c, int kind, const LayerPtrs &L, 
     for (int i = 0; i < kRowsPerProducer; ++i) out[i] = reinterpret_cast<const unsigned char *>(tbl[pw + i * kProducerWarps]);
 }
 
-// Stage layout with tensor-memory staging (TM): the stage is the image of its tensor-memory slot, 128 lane rows x
-// 256 bytes, stored as two 16 KB tiles of 128-byte rows with the 128-byte swizzle the tcgen05 descriptors describe
-// (16-byte piece c of lane row L at c ^ (L & 7)). Lane row 32*wi + 4*g + t belongs to thread (g, t) of the consumer
-// warps wi and wi + 4 and holds, in fragment order, the sixteen 16-byte pieces that thread multiplies: piece
-// 4*j + rb = weight row g + 8*rb, k elements [32*ch + 8*t, +8) with ch = 8*(j >> 1) + 2*wi + (j & 1). A producer
-// instruction still copies 512 contiguous bytes of one weight row; the eight lanes of a quarter-warp land in eight
-// different 16-byte bank groups.
 // Between QKV and gate/up the consumers attend, merge and project (18000 cycles with their barriers) while the ring takes 4 us
-// of the stream: HBM would idle for 10 us of a layer. Meanwhile one producer thread asks for a quarter of the gate/up weights to be
-// brought into L2, at about the rate at which HBM serves an SM: of every tile but the first (the ring holds that) the first
-// kAheadRows of its 16 gate and 16 up rows, so that later every stage is part L2 hit, part HBM and the SM's copy path,
-// faster than its share of HBM, takes in both at once. Whole rows in one request each: by 128-byte lines or column
-// blocks, or a stretch of stages ahead of the ring, it loses time. 7B shape, us: draft of three steps 442 -> 409 (one row of 16 426, two
-// 420, six 415), 28 layers of one row 2648 -> 2450, of four rows 2994 -> 2866.
+// of the stream: HBM would idle for 10 us of a layer. Meanwhile one producer thread asks for gate/up weights to be brought into L2:
+// of every tile but the first (the ring holds that) the first kAheadRows of its 16 gate and 16 up rows (ahead.cuh), 59 of a 7B layer's
+// 272 MB, so that later every stage is part L2 hit, part HBM and the SM's copy path, faster than its share of HBM, takes in both
+// at once. The pace is 57 GB/s an SM, a little above HBM's share (44): at 64 GB/s the requests hold up what the
+// consumers read (415 us), at 44 they end too late (2476 us for 28 layers). Whole rows in one request each: by 128-byte lines or column blocks, or a
+// stretch of stages ahead of the ring, it loses time; with the first tile as well it is the same within 0.6 %.
+// 7B shape, us, calls back to back on one set of buffers, none / one / two / four / six rows of 16: draft of three steps 437 / 427 / 419 / 408 / 410,
+// with four extend rows 458 / 450 / 445 / 441 / 448; 28 layers of one row 2620 / 2568 / 2529 / 2454 / 2455, of four 2998 / 2964 / 2935 / 2888 / 2874.
 constexpr uint32_t kAheadNsPerKB = 18;
 __device__ __forceinline__ void ahead_begin(const Cta &c, const LayerPtrs &L) {
     Ahead &a = c.misc->ahead;
@@ -434,6 +429,13 @@ __device__ __forceinline__ void ahead_while_waiting(const Cta &c, uint64_t *bar,
     a.due = due;
 }
 
+// Stage layout with tensor-memory staging (TM): the stage is the image of its tensor-memory slot, 128 lane rows x
+// 256 bytes, stored as two 16 KB tiles of 128-byte rows with the 128-byte swizzle the tcgen05 descriptors describe
+// (16-byte piece c of lane row L at c ^ (L & 7)). Lane row 32*wi + 4*g + t belongs to thread (g, t) of the consumer
+// warps wi and wi + 4 and holds, in fragment order, the sixteen 16-byte pieces that thread multiplies: piece
+// 4*j + rb = weight row g + 8*rb, k elements [32*ch + 8*t, +8) with ch = 8*(j >> 1) + 2*wi + (j & 1). A producer
+// instruction still copies 512 contiguous bytes of one weight row; the eight lanes of a quarter-warp land in eight
+// different 16-byte bank groups.
 template <bool TM>
 __device__ __forceinline__ void produce_phase(Cta &c, int kind, const LayerPtrs &L) {
     const MegaParams &p = *c.p;
@@ -824,9 +826,6 @@ __device__ __forceinline__ void consume_tiles(Cta &c, const Phase &ph, const Act
 #pragma unroll
         for (int s8 = 0; s8 < 8; ++s8) xo[s8] = (uint32_t)(32 * wi + c.lane) * 128u + (((uint32_t)s8 ^ ((uint32_t)c.lane & 7u)) << 4);
         const bool gfast = !act.in_smem && 16 * R * 512 <= c.scr_bytes;      // the slice ring must fit the staging area
-        // which half of the warps takes a stage depends only on the stage's index within the phase,
-        // never on how many stages the CTA has seen before: the summation order of a row must not
-        // depend on the batch or on earlier calls
         // The stages that come by way of the slice ring are those the fast loop reads, the ones of sixteen chunks. The last of them
         // may end 16 columns early (ffn = 496 mod 512): the input's rows are zero up to the next multiple of 32.
         auto sixteen_chunks = [](const StageK &sk) -> bool { return sk.klen > 15 * 32; };
@@ -843,6 +842,9 @@ __device__ __forceinline__ void consume_tiles(Cta &c, const Phase &ph, const Act
                 asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst + (uint32_t)r * 512u), "l"(src + (size_t)r * act.stride) : "memory");
             asm volatile("cp.async.commit_group;" ::: "memory");
         };
+        // which half of the warps takes a stage depends only on the stage's index within the phase,
+        // never on how many stages the CTA has seen before: the summation order of a row must not
+        // depend on the batch or on earlier calls
         const int first = ((stage0 & 1) == grp) ? 0 : 1;            // first stage this warp owns
         if (gfast && first < geo.nks) {
             const StageK s0 = stage_k(geo, first);
@@ -861,86 +863,84 @@ __device__ __forceinline__ void consume_tiles(Cta &c, const Phase &ph, const Act
 #pragma unroll 1
         for (int ks = 0; ks < geo.nks; ++ks) {
             if (kind == PROJ && ks == geo.nks_seg) second_segment();
-            {
-                // the first kTmSlots stages of a phase come through tensor memory (they land while the consumers are still
-                // busy with the previous phase's end), the rest is read from the shared-memory stage directly
-                const bool via_tmem = stage0 + ks < kTmSlots;
-                if (((stage0 + ks) & 1) == grp) {
-                    const StageK sk = stage_k(geo, ks);
-                    uint32_t w0[32], w1[32];
-                    const int ts = c.tslot, slot = c.slot;
-                    PROF_T0();
-                    if (via_tmem) {
-                        wait_bar(c, &c.misc->tfull[ts], c.tparity);
-                        PROF_ACC(c, 0, c.tid == 0);
-                        tc_fence_after_sync();
-                        const uint32_t ta = c.tmem + ((uint32_t)(32 * wi) << 16) + (uint32_t)(ts * kTmSlotCols);
-                        tmem_ld32_issue(ta, w0);
-                        tmem_ld32_issue(ta + 32, w1);
-                    } else {
-                        wait_bar(c, &c.full[slot], c.parity);
-                        PROF_ACC(c, 0, c.tid == 0);
-                    }
-                    uint4 bq[kCpw];
-                    if (act.in_smem) {
-                        const uint32_t ab = smem_u32(abase + aoff0 + (size_t)sk.koff);
-#pragma unroll
-                        for (int j = 0; j < kCpw; ++j) bq[j] = has0 ? lds128_u32(ab + (8 * (j >> 1) + 2 * wi + (j & 1)) * 64) : zero;
-                    } else {
-                        if (ks + 2 < geo.nks) slice_fetch(stage0 + ks + 2, stage_k(geo, ks + 2));
-                        if (ks + 2 < geo.nks) asm volatile("cp.async.wait_group 1;" ::: "memory");
-                        else asm volatile("cp.async.wait_group 0;" ::: "memory");
-                        __syncwarp();
-                        const uint32_t sl = slice_slot(stage0 + ks) + (uint32_t)(arow * 512 + ((g & 1) * 4 + t) * 16);
-#pragma unroll
-                        for (int j = 0; j < kCpw; ++j) bq[j] = has0 ? lds128_u32(sl + j * 128) : zero;
-                    }
-                    if (via_tmem) {
-                        tmem_ld_wait();
-                        tc_fence_before_sync();
-                        __syncwarp();
-                        if (c.lane == 0) mbar_arrive(&c.misc->tempty[ts]);       // the slot's data is in registers
-                    } else {
-                        // the stage has the slot's layout: lane row 32*wi + lane, piece s of it at (s & 7) ^ (lane & 7) in tile s >> 3
-                        const uint32_t lb = smem_u32(c.ring + (size_t)slot * p.stage_bytes);
-#pragma unroll
-                        for (int s8 = 0; s8 < 8; ++s8) {
-                            const uint4 a = lds128_u32(lb + xo[s8]);
-                            const uint4 b = lds128_u32(lb + xo[s8] + 16384u);
-                            w0[4 * s8] = a.x; w0[4 * s8 + 1] = a.y; w0[4 * s8 + 2] = a.z; w0[4 * s8 + 3] = a.w;
-                            w1[4 * s8] = b.x; w1[4 * s8 + 1] = b.y; w1[4 * s8 + 2] = b.z; w1[4 * s8 + 3] = b.w;
-                        }
-                    }
-#pragma unroll
-                    for (int j = 0; j < 2; ++j) {
-                        Frag f;
-                        f.u0 = make_uint4(w0[16 * j + 0], w0[16 * j + 1], w0[16 * j + 2], w0[16 * j + 3]);
-                        f.v0 = make_uint4(w0[16 * j + 4], w0[16 * j + 5], w0[16 * j + 6], w0[16 * j + 7]);
-                        f.u1 = make_uint4(w0[16 * j + 8], w0[16 * j + 9], w0[16 * j + 10], w0[16 * j + 11]);
-                        f.v1 = make_uint4(w0[16 * j + 12], w0[16 * j + 13], w0[16 * j + 14], w0[16 * j + 15]);
-                        mma_chunk(acc, f, bq[j]);
-                    }
-#pragma unroll
-                    for (int j = 0; j < 2; ++j) {
-                        Frag f;
-                        f.u0 = make_uint4(w1[16 * j + 0], w1[16 * j + 1], w1[16 * j + 2], w1[16 * j + 3]);
-                        f.v0 = make_uint4(w1[16 * j + 4], w1[16 * j + 5], w1[16 * j + 6], w1[16 * j + 7]);
-                        f.u1 = make_uint4(w1[16 * j + 8], w1[16 * j + 9], w1[16 * j + 10], w1[16 * j + 11]);
-                        f.v1 = make_uint4(w1[16 * j + 12], w1[16 * j + 13], w1[16 * j + 14], w1[16 * j + 15]);
-                        mma_chunk(acc, f, bq[2 + j]);
-                    }
-                    if (!via_tmem) {
-                        __syncwarp();
-                        if (c.lane == 0) {
-                            // counted before the arrival, so that the count of a use is never written after the slot's next use
-                            if (wi == 0) { volatile uint32_t *ud = &c.misc->use_done[slot]; *ud = *ud + 1; }   // see the mover
-                            mbar_arrive(&c.empty[slot]);
-                        }
-                    }
-                    PROF_ACC(c, 1, c.tid == 0);
+            // the first kTmSlots stages of a phase come through tensor memory (they land while the consumers are still
+            // busy with the previous phase's end), the rest is read from the shared-memory stage directly
+            const bool via_tmem = stage0 + ks < kTmSlots;
+            if (((stage0 + ks) & 1) == grp) {
+                const StageK sk = stage_k(geo, ks);
+                uint32_t w0[32], w1[32];
+                const int ts = c.tslot, slot = c.slot;
+                PROF_T0();
+                if (via_tmem) {
+                    wait_bar(c, &c.misc->tfull[ts], c.tparity);
+                    PROF_ACC(c, 0, c.tid == 0);
+                    tc_fence_after_sync();
+                    const uint32_t ta = c.tmem + ((uint32_t)(32 * wi) << 16) + (uint32_t)(ts * kTmSlotCols);
+                    tmem_ld32_issue(ta, w0);
+                    tmem_ld32_issue(ta + 32, w1);
+                } else {
+                    wait_bar(c, &c.full[slot], c.parity);
+                    PROF_ACC(c, 0, c.tid == 0);
                 }
-                if (via_tmem) next_tslot(c);
+                uint4 bq[kCpw];
+                if (act.in_smem) {
+                    const uint32_t ab = smem_u32(abase + aoff0 + (size_t)sk.koff);
+#pragma unroll
+                    for (int j = 0; j < kCpw; ++j) bq[j] = has0 ? lds128_u32(ab + (8 * (j >> 1) + 2 * wi + (j & 1)) * 64) : zero;
+                } else {
+                    if (ks + 2 < geo.nks) slice_fetch(stage0 + ks + 2, stage_k(geo, ks + 2));
+                    if (ks + 2 < geo.nks) asm volatile("cp.async.wait_group 1;" ::: "memory");
+                    else asm volatile("cp.async.wait_group 0;" ::: "memory");
+                    __syncwarp();
+                    const uint32_t sl = slice_slot(stage0 + ks) + (uint32_t)(arow * 512 + ((g & 1) * 4 + t) * 16);
+#pragma unroll
+                    for (int j = 0; j < kCpw; ++j) bq[j] = has0 ? lds128_u32(sl + j * 128) : zero;
+                }
+                if (via_tmem) {
+                    tmem_ld_wait();
+                    tc_fence_before_sync();
+                    __syncwarp();
+                    if (c.lane == 0) mbar_arrive(&c.misc->tempty[ts]);       // the slot's data is in registers
+                } else {
+                    // the stage has the slot's layout: lane row 32*wi + lane, piece s of it at (s & 7) ^ (lane & 7) in tile s >> 3
+                    const uint32_t lb = smem_u32(c.ring + (size_t)slot * p.stage_bytes);
+#pragma unroll
+                    for (int s8 = 0; s8 < 8; ++s8) {
+                        const uint4 a = lds128_u32(lb + xo[s8]);
+                        const uint4 b = lds128_u32(lb + xo[s8] + 16384u);
+                        w0[4 * s8] = a.x; w0[4 * s8 + 1] = a.y; w0[4 * s8 + 2] = a.z; w0[4 * s8 + 3] = a.w;
+                        w1[4 * s8] = b.x; w1[4 * s8 + 1] = b.y; w1[4 * s8 + 2] = b.z; w1[4 * s8 + 3] = b.w;
+                    }
+                }
+#pragma unroll
+                for (int j = 0; j < 2; ++j) {
+                    Frag f;
+                    f.u0 = make_uint4(w0[16 * j + 0], w0[16 * j + 1], w0[16 * j + 2], w0[16 * j + 3]);
+                    f.v0 = make_uint4(w0[16 * j + 4], w0[16 * j + 5], w0[16 * j + 6], w0[16 * j + 7]);
+                    f.u1 = make_uint4(w0[16 * j + 8], w0[16 * j + 9], w0[16 * j + 10], w0[16 * j + 11]);
+                    f.v1 = make_uint4(w0[16 * j + 12], w0[16 * j + 13], w0[16 * j + 14], w0[16 * j + 15]);
+                    mma_chunk(acc, f, bq[j]);
+                }
+#pragma unroll
+                for (int j = 0; j < 2; ++j) {
+                    Frag f;
+                    f.u0 = make_uint4(w1[16 * j + 0], w1[16 * j + 1], w1[16 * j + 2], w1[16 * j + 3]);
+                    f.v0 = make_uint4(w1[16 * j + 4], w1[16 * j + 5], w1[16 * j + 6], w1[16 * j + 7]);
+                    f.u1 = make_uint4(w1[16 * j + 8], w1[16 * j + 9], w1[16 * j + 10], w1[16 * j + 11]);
+                    f.v1 = make_uint4(w1[16 * j + 12], w1[16 * j + 13], w1[16 * j + 14], w1[16 * j + 15]);
+                    mma_chunk(acc, f, bq[2 + j]);
+                }
+                if (!via_tmem) {
+                    __syncwarp();
+                    if (c.lane == 0) {
+                        // counted before the arrival, so that the count of a use is never written after the slot's next use
+                        if (wi == 0) { volatile uint32_t *ud = &c.misc->use_done[slot]; *ud = *ud + 1; }   // see the mover
+                        mbar_arrive(&c.empty[slot]);
+                    }
+                }
+                PROF_ACC(c, 1, c.tid == 0);
             }
+            if (via_tmem) next_tslot(c);
             next_stage(c);
         }
         } else {
@@ -955,73 +955,71 @@ __device__ __forceinline__ void consume_tiles(Cta &c, const Phase &ph, const Act
 #pragma unroll 1
         for (; ks < geo.nks; ks += 2, skip_stages(2)) {
             if (!parked && ks >= geo.nks_seg) { second_segment(); parked = true; }
-            {
-                const int slot = c.slot;
-                const uint32_t parity = c.parity;
-                PROF_T0();
-                wait_bar(c, &c.full[slot], parity);
-                PROF_ACC(c, 0, c.tid == 0);
+            const int slot = c.slot;
+            const uint32_t parity = c.parity;
+            PROF_T0();
+            wait_bar(c, &c.full[slot], parity);
+            PROF_ACC(c, 0, c.tid == 0);
 
-                const StageK sk = stage_k(geo, ks);
-                const int nchunk = (sk.klen + 31) >> 5;
-                const uint32_t sb = ring0 + (uint32_t)slot * (uint32_t)p.stage_bytes;
-                const int par = g & 1;                    // odd rows: 64-byte halves swapped
-                const int kbase = sk.koff - (SPLIT && kind == PROJ && c.proj_split && ks >= geo.nks_seg ? geo.seglen : 0);
-                if (nchunk == 16 && (act.in_smem || gfast)) {
-                    // the stage width of the large shapes: this warp's chunks
-                    // wi, wi + 4, wi + 8, wi + 12 in two batches of two, all loads of a batch issued before its MMAs,
-                    // nothing predicated (see the producer: this loop sets the stream rate)
-                    uint4 bq[kCpw], dq[two_sets ? kCpw : 1];
-                    if (act.in_smem) {
-                        const uint32_t ab = act0 + (uint32_t)kbase * 2u, db = ab + (uint32_t)act.stride * 8u;
+            const StageK sk = stage_k(geo, ks);
+            const int nchunk = (sk.klen + 31) >> 5;
+            const uint32_t sb = ring0 + (uint32_t)slot * (uint32_t)p.stage_bytes;
+            const int par = g & 1;                    // odd rows: 64-byte halves swapped
+            const int kbase = sk.koff - (SPLIT && kind == PROJ && c.proj_split && ks >= geo.nks_seg ? geo.seglen : 0);
+            if (nchunk == 16 && (act.in_smem || gfast)) {
+                // the stage width of the large shapes: this warp's chunks
+                // wi, wi + 4, wi + 8, wi + 12 in two batches of two, all loads of a batch issued before its MMAs,
+                // nothing predicated (see the producer: this loop sets the stream rate)
+                uint4 bq[kCpw], dq[two_sets ? kCpw : 1];
+                if (act.in_smem) {
+                    const uint32_t ab = act0 + (uint32_t)kbase * 2u, db = ab + (uint32_t)act.stride * 8u;
 #pragma unroll
-                        for (int j = 0; j < kCpw; ++j) {
-                            bq[j] = has0 ? lds128_u32(ab + j * 256) : zero;
-                            if (two_sets) dq[two_sets ? j : 0] = has1 ? lds128_u32(db + j * 256) : zero;
-                        }
-                    } else {
-                        // request the slices of the next owned stage, then wait for this stage's (requested one owned
-                        // stage ago) and read the fragments from the slice ring
-                        bool more = false;
-                        if (ks + 2 < geo.nks) {
-                            const StageK s2 = stage_k(geo, ks + 2);
-                            if (sixteen_chunks(s2)) { slice_fetch(stage0 + ks + 2, s2); more = true; }   // (a shorter last stage is read directly by the loop below)
-                        }
-                        if (more) asm volatile("cp.async.wait_group 1;" ::: "memory");
-                        else asm volatile("cp.async.wait_group 0;" ::: "memory");
-                        __syncwarp();
-                        const uint32_t sl = slice_slot(stage0 + ks) + (uint32_t)(arow * 512 + ((g & 1) * 4 + t) * 16);
-#pragma unroll
-                        for (int j = 0; j < kCpw; ++j) {
-                            bq[j] = has0 ? lds128_u32(sl + j * 128) : zero;
-                            if (two_sets) dq[two_sets ? j : 0] = has1 ? lds128_u32(sl + 4 * 512 + j * 128) : zero;
-                        }
-                    }
-#pragma unroll
-                    for (int b2 = 0; b2 < 2; ++b2) {
-                        const int ch = wi + 8 * b2;
-                        Frag f0 = load_frag(sb + (ch ^ par) * 64, rs);
-                        Frag f1 = load_frag(sb + ((ch + 4) ^ par) * 64, rs);
-                        mma_chunk(acc, f0, bq[2 * b2]);
-                        if (two_sets) mma_chunk(acd, f0, dq[two_sets ? 2 * b2 : 0]);
-                        mma_chunk(acc, f1, bq[2 * b2 + 1]);
-                        if (two_sets) mma_chunk(acd, f1, dq[two_sets ? 2 * b2 + 1 : 0]);
+                    for (int j = 0; j < kCpw; ++j) {
+                        bq[j] = has0 ? lds128_u32(ab + j * 256) : zero;
+                        if (two_sets) dq[two_sets ? j : 0] = has1 ? lds128_u32(db + j * 256) : zero;
                     }
                 } else {
-#pragma unroll 1
-                    for (int ch = wi; ch < nchunk; ch += 4) {
-                        Frag f0 = load_frag(sb + (ch ^ par) * 64, rs);
-                        uint4 b0 = zero, d0 = zero;
-                        if (has0) b0 = act.in_smem ? lds128(abase + aoff0 + kbase + ch * 32) : ldcg128(abase + aoff0 + kbase + ch * 32);
-                        if (has1) d0 = act.in_smem ? lds128(abase + aoff1 + kbase + ch * 32) : ldcg128(abase + aoff1 + kbase + ch * 32);
-                        mma_chunk(acc, f0, b0);
-                        if (two_sets) mma_chunk(acd, f0, d0);
+                    // request the slices of the next owned stage, then wait for this stage's (requested one owned
+                    // stage ago) and read the fragments from the slice ring
+                    bool more = false;
+                    if (ks + 2 < geo.nks) {
+                        const StageK s2 = stage_k(geo, ks + 2);
+                        if (sixteen_chunks(s2)) { slice_fetch(stage0 + ks + 2, s2); more = true; }   // (a shorter last stage is read directly by the loop below)
+                    }
+                    if (more) asm volatile("cp.async.wait_group 1;" ::: "memory");
+                    else asm volatile("cp.async.wait_group 0;" ::: "memory");
+                    __syncwarp();
+                    const uint32_t sl = slice_slot(stage0 + ks) + (uint32_t)(arow * 512 + ((g & 1) * 4 + t) * 16);
+#pragma unroll
+                    for (int j = 0; j < kCpw; ++j) {
+                        bq[j] = has0 ? lds128_u32(sl + j * 128) : zero;
+                        if (two_sets) dq[two_sets ? j : 0] = has1 ? lds128_u32(sl + 4 * 512 + j * 128) : zero;
                     }
                 }
-                __syncwarp();
-                if (c.lane == 0) mbar_arrive(&c.empty[slot]);
-                PROF_ACC(c, 1, c.tid == 0);
+#pragma unroll
+                for (int b2 = 0; b2 < 2; ++b2) {
+                    const int ch = wi + 8 * b2;
+                    Frag f0 = load_frag(sb + (ch ^ par) * 64, rs);
+                    Frag f1 = load_frag(sb + ((ch + 4) ^ par) * 64, rs);
+                    mma_chunk(acc, f0, bq[2 * b2]);
+                    if (two_sets) mma_chunk(acd, f0, dq[two_sets ? 2 * b2 : 0]);
+                    mma_chunk(acc, f1, bq[2 * b2 + 1]);
+                    if (two_sets) mma_chunk(acd, f1, dq[two_sets ? 2 * b2 + 1 : 0]);
+                }
+            } else {
+#pragma unroll 1
+                for (int ch = wi; ch < nchunk; ch += 4) {
+                    Frag f0 = load_frag(sb + (ch ^ par) * 64, rs);
+                    uint4 b0 = zero, d0 = zero;
+                    if (has0) b0 = act.in_smem ? lds128(abase + aoff0 + kbase + ch * 32) : ldcg128(abase + aoff0 + kbase + ch * 32);
+                    if (has1) d0 = act.in_smem ? lds128(abase + aoff1 + kbase + ch * 32) : ldcg128(abase + aoff1 + kbase + ch * 32);
+                    mma_chunk(acc, f0, b0);
+                    if (two_sets) mma_chunk(acd, f0, d0);
+                }
             }
+            __syncwarp();
+            if (c.lane == 0) mbar_arrive(&c.empty[slot]);
+            PROF_ACC(c, 1, c.tid == 0);
         }
         if (!parked) second_segment();
         if (ks > geo.nks) {                       // one stage too far
@@ -1219,119 +1217,117 @@ __device__ __forceinline__ void attn_rows_mma(Cta &c, const bf16_t *sk, const bf
 #pragma unroll 1
     for (int m = grp; m < M; m += 2) {
         const int npos = min(base + min(m, rows - 1), max_tokens - 1);   // last visible position of this row
+        // query fragments: rows 0-7 the heads' hi parts, 8-15 their lo parts (a head that does not exist repeats the last one: not used)
+        uint32_t qa[DH / 16][4];
         {
-            // query fragments: rows 0-7 the heads' hi parts, 8-15 their lo parts (a head that does not exist repeats the last one: not used)
-            uint32_t qa[DH / 16][4];
-            {
-                const uint32_t qrow = smem_u32(qs + (size_t)m * 2 * Gq * DH) + (uint32_t)((((c.lane >> 3) & 1) * Gq + qh) * DH * 2);
+            const uint32_t qrow = smem_u32(qs + (size_t)m * 2 * Gq * DH) + (uint32_t)((((c.lane >> 3) & 1) * Gq + qh) * DH * 2);
 #pragma unroll
-                for (int ks = 0; ks < DH / 16; ++ks)
-                    asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];"
-                                 : "=r"(qa[ks][0]), "=r"(qa[ks][1]), "=r"(qa[ks][2]), "=r"(qa[ks][3])
-                                 : "r"(qrow + ((((uint32_t)(ks * 2) + (uint32_t)(c.lane >> 4)) ^ (uint32_t)(qh & 7)) << 4)));
-            }
-            // scores of this warp's 16 tokens (two n-tiles of 8)
-            float s[2][4];
-            s[0][0] = s[0][1] = s[0][2] = s[0][3] = 0.f;
-            s[1][0] = s[1][1] = s[1][2] = s[1][3] = 0.f;
-#pragma unroll
-            for (int ks = 0; ks < DH / 16; ++ks) {
-                uint32_t b00, b01, b10, b11;
+            for (int ks = 0; ks < DH / 16; ++ks)
                 asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];"
-                             : "=r"(b00), "=r"(b01), "=r"(b10), "=r"(b11) : "r"(krow + ((((uint32_t)(ks * 2 + kpc)) ^ ksw) << 4)));
-                mma_bf16(s[0], qa[ks][0], qa[ks][1], qa[ks][2], qa[ks][3], b00, b01);
-                mma_bf16(s[1], qa[ks][0], qa[ks][1], qa[ks][2], qa[ks][3], b10, b11);
-            }
-            // thread: head hrow, tokens tw + nt*8 + kq + {0,1}; hi-part product in [0],[1], lo-part in [2],[3]
-            float sc[4], mx = -INFINITY;
-#pragma unroll
-            for (int nt = 0; nt < 2; ++nt)
-#pragma unroll
-                for (int j = 0; j < 2; ++j) {
-                    float v = s[nt][j] + s[nt][j + 2];
-                    if (c0 + tw + nt * 8 + kq + j > npos) v = -INFINITY;
-                    sc[nt * 2 + j] = v;
-                    mx = fmaxf(mx, v);
-                }
-            mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 1));
-            mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 2));
-            float psum = 0.f;
-            uint32_t pa[4];
-            {
-                float pr[4];
-#pragma unroll
-                for (int i = 0; i < 4; ++i) { pr[i] = (sc[i] == -INFINITY) ? 0.f : expf(sc[i] - mx); psum += pr[i]; }
-                uint16_t h0, l0, h1, l1, h2, l2, h3, l3;
-                split_bf16(pr[0], h0, l0); split_bf16(pr[1], h1, l1); split_bf16(pr[2], h2, l2); split_bf16(pr[3], h3, l3);
-                pa[0] = (uint32_t)h0 | ((uint32_t)h1 << 16);      // row hrow,     tokens kq, kq+1
-                pa[1] = (uint32_t)l0 | ((uint32_t)l1 << 16);      // row hrow + 8
-                pa[2] = (uint32_t)h2 | ((uint32_t)h3 << 16);      // row hrow,     tokens 8+kq, 8+kq+1
-                pa[3] = (uint32_t)l2 | ((uint32_t)l3 << 16);
-            }
-            psum += __shfl_xor_sync(0xffffffffu, psum, 1);
-            psum += __shfl_xor_sync(0xffffffffu, psum, 2);
-            // o[head][dim] = sum over the warp's tokens of p * V. Beyond the row's context the stage holds later rows' values or
-            // what nothing has written, which need not be finite: a probability of 0 meets a 0 there (masked in registers,
-            // and not by zeros in the stage besides: that cost 0.3 % of a draft)
-            const int seen = npos + 1 - (c0 + tw);
-            const uint32_t keep0 = (kq < seen ? 0xffffu : 0u) | (kq + 1 < seen ? 0xffff0000u : 0u);
-            const uint32_t keep1 = (kq + 8 < seen ? 0xffffu : 0u) | (kq + 9 < seen ? 0xffff0000u : 0u);
-            float o[DH / 8][4];
-#pragma unroll
-            for (int nt = 0; nt < DH / 8; ++nt) o[nt][0] = o[nt][1] = o[nt][2] = o[nt][3] = 0.f;
-#pragma unroll
-            for (int nt = 0; nt < DH / 8; nt += 2) {
-                uint32_t b00, b01, b10, b11;
-                asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];"
-                             : "=r"(b00), "=r"(b01), "=r"(b10), "=r"(b11) : "r"(vrow + ((((uint32_t)(nt + vpc)) ^ vsw) << 4)));
-                mma_bf16(o[nt], pa[0], pa[1], pa[2], pa[3], b00 & keep0, b01 & keep1);
-                mma_bf16(o[nt + 1], pa[0], pa[1], pa[2], pa[3], b10 & keep0, b11 & keep1);
-            }
-            // ---- merge the group's four warps (fixed order) -> chunk partial in global memory
-            {
-                float *w = wp + ((size_t)wi * 8 + hrow) * wstride;
-#pragma unroll
-                for (int nt = 0; nt < DH / 8; ++nt) *reinterpret_cast<float2 *>(w + nt * 8 + kq) = make_float2(o[nt][0] + o[nt][2], o[nt][1] + o[nt][3]);
-                if ((c.lane & 3) == 0) { w[DH] = mx; w[DH + 1] = psum; }
-            }
-            bar_sync(3 + grp, 128);
-            const int gt = c.tid & 127;                      // thread within the group
-            if (gt < 32) {                                   // thread = (head gt >> 2, warp gt & 3): the warp's weight, the head's (m, l)
-                const int h = gt >> 2, w = gt & 3;
-                float mm = -INFINITY;
-#pragma unroll
-                for (int q = 0; q < 4; ++q) mm = fmaxf(mm, wp[((size_t)q * 8 + h) * wstride + DH]);
-                const float mw = wp[((size_t)w * 8 + h) * wstride + DH], lw = wp[((size_t)w * 8 + h) * wstride + DH + 1];
-                const float f = (mw == -INFINITY) ? 0.f : expf(mw - mm);
-                fw[w * 8 + h] = f;
-                float l = 0.f;
-#pragma unroll
-                for (int q = 0; q < 4; ++q) {
-                    const float fq = __shfl_sync(0xffffffffu, f, (gt & ~3) + q), lq = __shfl_sync(0xffffffffu, lw, (gt & ~3) + q);
-                    l += fq * lq;
-                }
-                if (w == 0 && h < Gq) {
-                    float *dst = p.s.att_part + (((size_t)(b * M + m) * p.Hq + kvh * Gq + h) * p.max_chunks + chunk) * (DH + kPartPad);
-                    dst[DH] = mm;
-                    dst[DH + 1] = l;
-                }
-            }
-            bar_sync(3 + grp, 128);
-            for (int i = gt; i < Gq * (DH / 2); i += 128) {  // two output elements
-                const int h = i / (DH / 2), e = (i - h * (DH / 2)) * 2;
-                float o0 = 0.f, o1 = 0.f;
-#pragma unroll
-                for (int w = 0; w < 4; ++w) {
-                    const float2 v = *reinterpret_cast<const float2 *>(wp + ((size_t)w * 8 + h) * wstride + e);
-                    const float f = fw[w * 8 + h];
-                    o0 += f * v.x;
-                    o1 += f * v.y;
-                }
-                const int rr = b * M + m, hq = kvh * Gq + h;
-                *reinterpret_cast<float2 *>(p.s.att_part + (((size_t)rr * p.Hq + hq) * p.max_chunks + chunk) * (DH + kPartPad) + e) = make_float2(o0, o1);
-            }
-            if (m + 2 < M) bar_sync(3 + grp, 128);           // the group's buffer is free for its next pass
+                             : "=r"(qa[ks][0]), "=r"(qa[ks][1]), "=r"(qa[ks][2]), "=r"(qa[ks][3])
+                             : "r"(qrow + ((((uint32_t)(ks * 2) + (uint32_t)(c.lane >> 4)) ^ (uint32_t)(qh & 7)) << 4)));
         }
+        // scores of this warp's 16 tokens (two n-tiles of 8)
+        float s[2][4];
+        s[0][0] = s[0][1] = s[0][2] = s[0][3] = 0.f;
+        s[1][0] = s[1][1] = s[1][2] = s[1][3] = 0.f;
+#pragma unroll
+        for (int ks = 0; ks < DH / 16; ++ks) {
+            uint32_t b00, b01, b10, b11;
+            asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];"
+                         : "=r"(b00), "=r"(b01), "=r"(b10), "=r"(b11) : "r"(krow + ((((uint32_t)(ks * 2 + kpc)) ^ ksw) << 4)));
+            mma_bf16(s[0], qa[ks][0], qa[ks][1], qa[ks][2], qa[ks][3], b00, b01);
+            mma_bf16(s[1], qa[ks][0], qa[ks][1], qa[ks][2], qa[ks][3], b10, b11);
+        }
+        // thread: head hrow, tokens tw + nt*8 + kq + {0,1}; hi-part product in [0],[1], lo-part in [2],[3]
+        float sc[4], mx = -INFINITY;
+#pragma unroll
+        for (int nt = 0; nt < 2; ++nt)
+#pragma unroll
+            for (int j = 0; j < 2; ++j) {
+                float v = s[nt][j] + s[nt][j + 2];
+                if (c0 + tw + nt * 8 + kq + j > npos) v = -INFINITY;
+                sc[nt * 2 + j] = v;
+                mx = fmaxf(mx, v);
+            }
+        mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 1));
+        mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 2));
+        float psum = 0.f;
+        uint32_t pa[4];
+        {
+            float pr[4];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) { pr[i] = (sc[i] == -INFINITY) ? 0.f : expf(sc[i] - mx); psum += pr[i]; }
+            uint16_t h0, l0, h1, l1, h2, l2, h3, l3;
+            split_bf16(pr[0], h0, l0); split_bf16(pr[1], h1, l1); split_bf16(pr[2], h2, l2); split_bf16(pr[3], h3, l3);
+            pa[0] = (uint32_t)h0 | ((uint32_t)h1 << 16);      // row hrow,     tokens kq, kq+1
+            pa[1] = (uint32_t)l0 | ((uint32_t)l1 << 16);      // row hrow + 8
+            pa[2] = (uint32_t)h2 | ((uint32_t)h3 << 16);      // row hrow,     tokens 8+kq, 8+kq+1
+            pa[3] = (uint32_t)l2 | ((uint32_t)l3 << 16);
+        }
+        psum += __shfl_xor_sync(0xffffffffu, psum, 1);
+        psum += __shfl_xor_sync(0xffffffffu, psum, 2);
+        // o[head][dim] = sum over the warp's tokens of p * V. Beyond the row's context the stage holds later rows' values or
+        // what nothing has written, which need not be finite: a probability of 0 meets a 0 there (masked in registers,
+        // and not by zeros in the stage besides: that cost 0.3 % of a draft)
+        const int seen = npos + 1 - (c0 + tw);
+        const uint32_t keep0 = (kq < seen ? 0xffffu : 0u) | (kq + 1 < seen ? 0xffff0000u : 0u);
+        const uint32_t keep1 = (kq + 8 < seen ? 0xffffu : 0u) | (kq + 9 < seen ? 0xffff0000u : 0u);
+        float o[DH / 8][4];
+#pragma unroll
+        for (int nt = 0; nt < DH / 8; ++nt) o[nt][0] = o[nt][1] = o[nt][2] = o[nt][3] = 0.f;
+#pragma unroll
+        for (int nt = 0; nt < DH / 8; nt += 2) {
+            uint32_t b00, b01, b10, b11;
+            asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];"
+                         : "=r"(b00), "=r"(b01), "=r"(b10), "=r"(b11) : "r"(vrow + ((((uint32_t)(nt + vpc)) ^ vsw) << 4)));
+            mma_bf16(o[nt], pa[0], pa[1], pa[2], pa[3], b00 & keep0, b01 & keep1);
+            mma_bf16(o[nt + 1], pa[0], pa[1], pa[2], pa[3], b10 & keep0, b11 & keep1);
+        }
+        // ---- merge the group's four warps (fixed order) -> chunk partial in global memory
+        {
+            float *w = wp + ((size_t)wi * 8 + hrow) * wstride;
+#pragma unroll
+            for (int nt = 0; nt < DH / 8; ++nt) *reinterpret_cast<float2 *>(w + nt * 8 + kq) = make_float2(o[nt][0] + o[nt][2], o[nt][1] + o[nt][3]);
+            if ((c.lane & 3) == 0) { w[DH] = mx; w[DH + 1] = psum; }
+        }
+        bar_sync(3 + grp, 128);
+        const int gt = c.tid & 127;                      // thread within the group
+        if (gt < 32) {                                   // thread = (head gt >> 2, warp gt & 3): the warp's weight, the head's (m, l)
+            const int h = gt >> 2, w = gt & 3;
+            float mm = -INFINITY;
+#pragma unroll
+            for (int q = 0; q < 4; ++q) mm = fmaxf(mm, wp[((size_t)q * 8 + h) * wstride + DH]);
+            const float mw = wp[((size_t)w * 8 + h) * wstride + DH], lw = wp[((size_t)w * 8 + h) * wstride + DH + 1];
+            const float f = (mw == -INFINITY) ? 0.f : expf(mw - mm);
+            fw[w * 8 + h] = f;
+            float l = 0.f;
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const float fq = __shfl_sync(0xffffffffu, f, (gt & ~3) + q), lq = __shfl_sync(0xffffffffu, lw, (gt & ~3) + q);
+                l += fq * lq;
+            }
+            if (w == 0 && h < Gq) {
+                float *dst = p.s.att_part + (((size_t)(b * M + m) * p.Hq + kvh * Gq + h) * p.max_chunks + chunk) * (DH + kPartPad);
+                dst[DH] = mm;
+                dst[DH + 1] = l;
+            }
+        }
+        bar_sync(3 + grp, 128);
+        for (int i = gt; i < Gq * (DH / 2); i += 128) {  // two output elements
+            const int h = i / (DH / 2), e = (i - h * (DH / 2)) * 2;
+            float o0 = 0.f, o1 = 0.f;
+#pragma unroll
+            for (int w = 0; w < 4; ++w) {
+                const float2 v = *reinterpret_cast<const float2 *>(wp + ((size_t)w * 8 + h) * wstride + e);
+                const float f = fw[w * 8 + h];
+                o0 += f * v.x;
+                o1 += f * v.y;
+            }
+            const int rr = b * M + m, hq = kvh * Gq + h;
+            *reinterpret_cast<float2 *>(p.s.att_part + (((size_t)rr * p.Hq + hq) * p.max_chunks + chunk) * (DH + kPartPad) + e) = make_float2(o0, o1);
+        }
+        if (m + 2 < M) bar_sync(3 + grp, 128);           // the group's buffer is free for its next pass
     }
 }
 

@@ -76,12 +76,14 @@ struct GemmArgs {
     int n_stages, n_xstages;
     unsigned long long wait_limit_ns;   // every wait of the kernel gives up after this long
     int extra_arrivals;          // self-test only: arrivals a ring stage expects beyond the copies that are made
-    // Two row-major matrices [ahead_rows][ahead_ld] that a later GEMM streams by tiles of 128 rows: while this one runs, the first
-    // kAheadTileRows rows of these are asked into L2, as far as the time and ahead.cuh's bound allow. Used by W_o for gate/up: its own weights are in the ring when attention
+    // Two row-major matrices [ahead_rows][ahead_ld] that a later GEMM streams by tiles of 128 rows: while this one runs, its CTAs ask for the
+    // first kAheadTileRows rows of each to be brought into L2 (ahead.cuh), until their own last MMA is done: a GEMM of few tiles, and so few
+    // CTAs, gets no further than its first tiles. Used by W_o for gate/up: its own weights are in the ring when attention
     // ends, and until gate/up starts (merge, W_o, post: 15 us) HBM has nothing else to do. Then every stage of gate/up is part
-    // L2 hit, part HBM, and the copy path takes in both at once. 7B shape, four ragged sequences, five steps 728 -> 704 us (8 rows of 128
-    // 716, 16 707, 48 704, 64 709), 16 sequences 556 -> 552. At 64 rows it loses (64 ragged 905 -> 911, 16 x 4 rows of 28 layers
-    // 4178 -> 4212): there the activation block's re-reads fill the path between L2 and the SMs. So only with four-block stages.
+    // L2 hit, part HBM, and the copy path takes in both at once. 7B shape, none / 8 / 16 / 32 / 48 / 64 rows of 128, us: four ragged
+    // sequences, five steps 727 / 715 / 706 / 703 / 703 / 703, 16 sequences with extend rows 556 / 554 / 552 / 552 / 552 / 552. At 64 rows it
+    // gives nothing (64 ragged sequences 909 -> 907, 16 x 4 rows of 28 layers 4182 -> 4194): there the activation block's re-reads
+    // fill the path between L2 and the SMs. So only with four-block stages.
     const bf16_t *ahead[2];
     int ahead_rows, ahead_ld;
     uint32_t ahead_limit;        // bytes a CTA may ask for per tile (gemm_ahead_limit)
