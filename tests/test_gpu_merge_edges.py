@@ -8,10 +8,10 @@ pytestmark = pytest.mark.gpu
 
 
 @pytest.mark.parametrize("dh,L", [
-    # chunks of 64 positions dealt over 8 (head dimension 128) or 16 groups of threads. The first five rounds, the later ones by
-    # fours, and a new turn of weights after 32 or 16 rounds: 256 chunks at either head dimension
-    (128, [64 * 40 - 2, 64 * 40, 64 * 41, 64 * 71, 64 * 72, 64 * 73]),
-    (64, [64 * 80 - 2, 64 * 80, 64 * 81, 64 * 143, 64 * 144, 64 * 145]),
+    # chunks of 64 positions dealt over 8 (head dimension 128) or 16 groups of threads, which take five rounds at a time; a new turn
+    # of weights after 32 or 16 rounds: 256 chunks at either head dimension
+    (128, [64 * 40 - 2, 64 * 40, 64 * 41, 64 * 79, 64 * 80, 64 * 81]),
+    (64, [64 * 80 - 2, 64 * 80, 64 * 81, 64 * 159, 64 * 160, 64 * 161]),
     (128, [64 * 256 - 2, 64 * 256, 64 * 257, 64 * 296 + 5]),
     (64, [64 * 256 - 2, 64 * 256, 64 * 257, 64 * 336 + 5]),
     (128, [64 * 520 + 1]),
