@@ -170,7 +170,8 @@ int fmtp_selftest_inject_wait_timeout(fmtp_ctx *ctx, int limit_ms, int which);
 /* Diagnostic (no counterpart in the paper, host only, needs no GPU): the requests by which CTA `cta` of `grid` asks gate/up
  * weights of a layer [ffn, d] into an L2 cache of l2_bytes ahead of their phase, as the kernels make them if there is time for all:
  * batched = 0 the persistent kernel, 1 the batched path (grid: the CTAs of W_o's GEMM). Request i is bytes[i] bytes from
- * element at[i] of mat[i] (0 gate, 1 up) on. Returns their number and stores the first max_requests of them. */
+ * element at[i] of mat[i] (0 gate, 1 up) on. Returns their number and stores the first max_requests of them.
+ * FMTP_EINVAL for a size that is not positive or above 2^22, a negative l2_bytes, a cta that does not exist or a missing array. */
 int fmtp_selftest_ahead(int batched, int ffn, int d, int grid, long long l2_bytes, int cta, int max_requests, int *mat, long long *at,
                         unsigned int *bytes);
 

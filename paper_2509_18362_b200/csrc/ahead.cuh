@@ -12,8 +12,11 @@ struct AheadReq { int mat; long long at; uint32_t bytes; };
 // All CTAs' requests of a layer together stay within 9/16 of L2 (75 MB): what is pushed out again before its tile comes is read
 // twice. The 7B shape asks for 59 MB (persistent kernel) and 68 (batched path). Without the bound a layer of d = 8192 with ffn
 // 28672 asked for 232 MB: drafts of three steps at 2048 and 16384 positions 1212 and 1359 us, with it 1166 and 1312, without
-// any request 1171 and 1297; d = 5120 with ffn 27648 at 16384 919 / 900 / 894. Bounds of 32, 48, 64 and 80 MB are within 1 % of each other.
-__host__ __device__ inline long long ahead_budget(long long l2_bytes) { return l2_bytes / 16 * 9; }
+// any request 1171 and 1297; d = 5120 with ffn 27648 at 16384 919 / 900 / 894. Bounds of 32, 48, 64 and 80 MB are within 1.5 % of each other.
+__host__ __device__ inline long long ahead_budget(long long l2_bytes) {
+    const long long share = l2_bytes / 16 * 9, most = 1ll << 30;      // (32-bit counts below)
+    return share < most ? share : most;
+}
 
 // ---- persistent kernel: the first kAheadRows of the gate and of the up rows of every tile but the CTA's first, whole rows, a
 // request each. Rows v0 .. v1 of ffn are the CTA's, a tile has `cap` of them.

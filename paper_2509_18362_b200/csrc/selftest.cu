@@ -46,7 +46,9 @@ extern "C" int fmtp_selftest_wait_timeout(uint32_t *dev_status, int limit_ms, un
 
 extern "C" int fmtp_selftest_ahead(int batched, int ffn, int d, int grid, long long l2_bytes, int cta, int max_requests, int *mat,
                                    long long *at, unsigned int *bytes) {
-    if (ffn < 1 || d < 1 || grid < 1 || cta < 0 || cta >= grid || max_requests < 0 || (max_requests > 0 && (!mat || !at || !bytes))) return FMTP_EINVAL;
+    const int most = 1 << 22;                                         // keeps every product of the lists inside its type
+    if (ffn < 1 || ffn > most || d < 1 || d > most || grid < 1 || grid > most || l2_bytes < 0 || cta < 0 || cta >= grid) return FMTP_EINVAL;
+    if (max_requests < 0 || (max_requests > 0 && (!mat || !at || !bytes))) return FMTP_EINVAL;
     const long long budget = fmtp::ahead_budget(l2_bytes);
     int n = 0;
     auto put = [&](const fmtp::AheadReq &r) {

@@ -5,7 +5,7 @@ import pytest
 from paper_2509_18362_b200 import binding as Bd
 
 L2 = 132644864           # what the driver reports for a B200
-HUGE = 1 << 40           # no bound
+HUGE = 1 << 40           # no bound that any shape here meets
 SHARE = {False: (4, 16), True: (32, 128)}      # rows asked for of a tile's rows
 
 
@@ -69,8 +69,17 @@ def test_the_7b_shape_keeps_all_requests(batched, total):
     assert not batched or sum(size for one in few for _, _, size in one) == total
 
 
+def test_any_size_of_l2_gives_a_list():
+    for l2 in (1, 15, 1 << 31, 1 << 40, (1 << 63) - 1):
+        for batched in (0, 1):
+            total = sum(size for _, _, size in Bd.fmtp_selftest_ahead(batched, 1 << 22, 64, 1, l2, 0))
+            assert total <= max(l2 * 9 // 16, 0)
+            assert l2 < 1 << 31 or total == (1 << 22) * 64 * 2 * 2 // 4 - (0 if batched else 2 * 4 * 64 * 2)
+
+
 def test_no_room_and_bad_arguments():
     assert Bd.fmtp_selftest_ahead(0, 18944, 3584, 148, 0, 3) == [] and Bd.fmtp_selftest_ahead(1, 18944, 3584, 148, 0, 3) == []
-    for args in ((0, 0, 64, 1, L2, 0), (0, 64, 64, 0, L2, 0), (1, 64, 64, 4, L2, 4), (1, 64, 64, 4, L2, -1)):
+    for args in ((0, 0, 64, 1, L2, 0), (0, 64, 64, 0, L2, 0), (1, 64, 64, 4, L2, 4), (1, 64, 64, 4, L2, -1), (0, 64, 64, 4, -1, 0),
+                 (0, 64, 1 << 29, 1, L2, 0), (1, (1 << 31) - 1, 64, 1, L2, 0)):
         with pytest.raises(Bd.FastMTPError):
             Bd.fmtp_selftest_ahead(*args)
